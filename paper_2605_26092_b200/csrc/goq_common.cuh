@@ -85,10 +85,9 @@ __device__ __forceinline__ uint32_t gather_meta(uint32_t w) {
     return ((w >> 3) & 1u) | ((w >> 6) & 2u) | ((w >> 9) & 4u) | ((w >> 12) & 8u) | ((w >> 15) & 16u) |
            ((w >> 18) & 32u);
 }
+// bit i -> bit 4i + 3: the two halves of three bits move apart, then one multiply spreads each half (the products do not meet)
 __host__ __device__ inline uint32_t scatter_meta(uint32_t meta) {
-    uint32_t r = 0;
-    for (int i = 0; i < 6; ++i) r |= ((meta >> i) & 1u) << (4 * i + 3);
-    return r;
+    return (((meta & 7u) | ((meta & 56u) << 9)) * 0x248u) & 0x888888u;
 }
 // nibble i of the result = nibble (i XOR s) of m
 __device__ __forceinline__ uint32_t xor_permute_nibbles(uint32_t m, int s) {
