@@ -34,142 +34,172 @@ __device__ __forceinline__ double lattice_value(int c, int wbits) {
     const double mag = __longlong_as_double((long long)(1023 - e) << 52);   // 2^-e
     return sg ? -mag : mag;
 }
-// Nearest lattice state in linear distance; exact ties go to the state of smaller magnitude. |v| <= 1. Between two
-// neighbouring magnitudes 2^E and 2^(E+1) the midpoint is 1.5 * 2^E, so the choice is read off the exponent field and the
-// top of the mantissa of |v|; below the smallest magnitude the neighbours are that state and zero. The positive side has
-// no +2^-emax (that bin is the zero): its smallest state is 2^-(emax-1), met by zero at the midpoint 2^-emax.
-__device__ __forceinline__ int rtn_code(double v, int wbits) {
-    const int emax = (1 << (wbits - 1)) - 1;
-    const long long bits = __double_as_longlong(fabs(v));
-    const int E = (int)((bits >> 52) & 0x7FF) - 1023;                              // |v| = m 2^E, 1 <= m < 2
-    const bool upper = (bits & 0xFFFFFFFFFFFFFll) > (1ll << 51);                   // m > 1.5: the larger neighbour
-    const int e = -E - (upper ? 1 : 0);                                            // magnitude 2^-e
-    const double a = fabs(v);
-    if (v < 0.0) {
-        if (!(a > __longlong_as_double((long long)(1023 - emax - 1) << 52))) return emax;   // at or below 2^-(emax+1): zero
-        return (1 << (wbits - 1)) | min(e, emax);
+// ---- GEO quantizer -----------------------------------------------------------------------------------------
+// A lane owns a whole micro-block (8 weights), so all four pair patterns stay inside the thread; the LPG = group / 8 lanes
+// of a macro-block share its sums. Everything is flat: macro-blocks do not straddle rows, so lane l of a warp takes
+// micro-block base + l whatever the shape. Bound: the float64 pipe (about 110 operations per micro-block) and the memory
+// system, near each other. What keeps float64 work down without changing one result:
+//   - codes need no division (rtn_codes);
+//   - every product has a power of two as a factor, hence is exact; ||b2||^2 = ||b1||^2 (b2 is a signed permutation
+//     of b1), <w, b2> is the sum of the chosen patterns' |d|;
+// Sums are added in a fixed order: elements 0..3 and 4..7 of a micro-block apart, each over the lanes from the farthest
+// partner down, then the halves.
+// Measured, 11008 x 4096 W3 g128: 92 us (one lane per four weights, with a float64 quotient per weight and a warp-wide float64
+// reduction for every sum: 438 us). 62 registers and 32 warps an SM: latency, not a pipe, is what is left (float64 pipe ~30 %).
+template <int LPG>
+__device__ __forceinline__ double group_sum2(double p0, double p1) {
+    if constexpr (LPG == 1) {
+        return p0 + p1;
+    } else {
+        constexpr int o0 = LPG / 2;
+        const bool up = (threadIdx.x & o0) != 0;   // the first step splits the halves over the lanes: one exchange instead of two
+        double v = (up ? p1 : p0) + __shfl_xor_sync(kFull, up ? p0 : p1, o0);
+#pragma unroll
+        for (int o = o0 / 2; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        return v + __shfl_xor_sync(kFull, v, o0);
     }
-    if (!(a > __longlong_as_double((long long)(1023 - emax) << 52))) return emax;           // at or below 2^-emax: zero
-    return min(e, emax - 1);
 }
 
-// b2 of the four elements a lane holds (elements 4*(lane&1) .. +3 of its micro-block) under record (s, flags):
-// for each pair (i, j = i XOR s), i < j, with flag f (1 iff eta = -1):  y_i = -eta x_j,  y_j = eta x_i   (Theorem 1)
-__device__ __forceinline__ void exchange4(const double (&x)[4], int s, unsigned flags, int half, double (&y)[4]) {
-    double xo[4];   // the neighbouring lane's elements (the other half of the micro-block): fetched by every lane, whatever its pattern
+// Codes of a micro-block, a nibble each: nearest lattice state in linear distance, exact ties to the state of smaller
+// magnitude (Section 3.2). Between 2^-(e+1) and 2^-e the midpoint is 0.75 * 2^-e; the zero meets the smallest negative
+// magnitude at 2^-(emax+1) and the smallest positive one (there is no +2^-emax) at 2^-emax. `th` holds these midpoints times
+// s_norm, rounded DOWN to fp32: for an fp32 number a, a > t and a > round_down(t) are the same, so every decision is the
+// exact one and nothing is divided. A code is a sum of predicates: e counts the midpoints |w| does not exceed, and the sign bit
+// is set only below the negative zero bin (between it and 0, |w| exceeds no midpoint of either sign and e = emax, the zero).
+template <int WB> struct Midpoints {
+    static constexpr int emax = (1 << (WB - 1)) - 1;
+    float both[emax > 1 ? emax - 1 : 1], last_neg, last_pos, zero_neg;
+};
+template <int WB>
+__device__ __forceinline__ Midpoints<WB> midpoints(float s) {
+    constexpr int emax = Midpoints<WB>::emax;
+    Midpoints<WB> m;
+    float t = 0.75f;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) xo[a] = __shfl_xor_sync(kFull, x[a], 1);
+    for (int i = 0; i < emax - 1; ++i, t *= 0.5f) m.both[i] = __fmul_rd(t, s);
+    m.last_neg = __fmul_rd(t, s);
+    m.last_pos = __fmul_rd(1.0f / (float)(1 << emax), s);
+    m.zero_neg = __fmul_rd(1.0f / (float)(2 << emax), s);
+    return m;
+}
+template <int WB>
+__device__ __forceinline__ uint32_t rtn_codes(const float (&w)[8], const Midpoints<WB>& m) {
+    constexpr int emax = Midpoints<WB>::emax;
+    uint32_t code = 0;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        if (s < 4) {   // the partner stays inside the lane's half of the micro-block
-            const int b = a ^ s;
-            const int i = min(a, b) + 4 * half;                 // lower index of the pair inside the micro-block
-            int p = 0;                                          // pairs are numbered in ascending order of their lower index
-            for (int q = 0; q < i; ++q) p += (q < (q ^ s));
-            const double eta = ((flags >> p) & 1u) ? -1.0 : 1.0;
-            const double xb = (b == 0) ? x[0] : (b == 1) ? x[1] : (b == 2) ? x[2] : x[3];
-            y[a] = (a < b) ? -eta * xb : eta * xb;
-        } else {       // s = 4: the partner is the same position in the other half
-            const double eta = ((flags >> a) & 1u) ? -1.0 : 1.0;
-            y[a] = half ? eta * xo[a] : -eta * xo[a];
+    for (int i = 0; i < 8; ++i) {
+        const float a = fabsf(w[i]);
+        const bool neg = w[i] < -m.zero_neg;
+#pragma unroll
+        for (int q = 0; q < emax - 1; ++q)
+            if (!(a > m.both[q])) code += 1u << (4 * i);
+        if (!(a > (neg ? m.last_neg : m.last_pos))) code += 1u << (4 * i);
+        if (neg) code += (1u << (WB - 1)) << (4 * i);
+    }
+    return code;
+}
+// The values of eight codes as the high words of doubles (the low words are zero). W <= 3: sign/exponent bytes by table.
+template <int WB>
+__device__ __forceinline__ void code_values(uint32_t code, double (&x)[8]) {
+    if constexpr (WB <= 3) {
+        // W3 codes 0..7: +1 +.5 +.25 0 -1 -.5 -.25 -.125;  W2 codes 0..3: +1 0 -1 -.5
+        constexpr uint32_t t0 = WB == 3 ? 0x00D0E0F0u : 0xE0F000F0u, t1 = WB == 3 ? 0xC0D0E0F0u : 0u;
+        constexpr uint32_t s0 = WB == 3 ? 0x003F3F3Fu : 0xBFBF003Fu, s1 = WB == 3 ? 0xBFBFBFBFu : 0u;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t sel = h ? code >> 16 : code;
+            const uint32_t t = __byte_perm(t0, t1, sel), sg = __byte_perm(s0, s1, sel);
+            const uint32_t v01 = __byte_perm(t, sg, 0x5140), v23 = __byte_perm(t, sg, 0x7362);
+            x[4 * h + 0] = __hiloint2double((int)(v01 << 16), 0);
+            x[4 * h + 1] = __hiloint2double((int)(v01 & 0xFFFF0000u), 0);
+            x[4 * h + 2] = __hiloint2double((int)(v23 << 16), 0);
+            x[4 * h + 3] = __hiloint2double((int)(v23 & 0xFFFF0000u), 0);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t c = (code >> (4 * i)) & 15u;
+            x[i] = __hiloint2double(c == 7u ? 0 : (int)(((1023u - (c & 7u)) << 20) | ((c & 8u) << 28)), 0);
         }
     }
 }
 
-// One warp per macro-block of `group` weights (lane l holds elements 4l .. 4l+3; lanes beyond group/4 idle).
-__global__ void __launch_bounds__(kWarps * 32)
+template <int WB, int LPG, bool K1>
+__global__ void __launch_bounds__(kWarps * 32, 4)
 quantize_geo_kernel(const float* __restrict__ w, uint8_t* __restrict__ codes, uint8_t* __restrict__ meta,
-                    uint16_t* __restrict__ coef, int n_out, int k_in, int group, int wbits, int k1) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nj = k_in / group;
-    const long long blk = (long long)blockIdx.x * kWarps + warp;
-    if (blk >= (long long)n_out * nj) return;
-    const int row = (int)(blk / nj), j = (int)(blk % nj);
-    const bool on = lane * 4 < group;
-    const size_t base = (size_t)row * k_in + (size_t)j * group + lane * 4;
-    const int emax = (1 << (wbits - 1)) - 1, half = lane & 1;
-    double wv[4] = {0, 0, 0, 0};
-    if (on) {
-        const float4 f = *reinterpret_cast<const float4*>(w + base);
-        wv[0] = f.x; wv[1] = f.y; wv[2] = f.z; wv[3] = f.w;
+                    uint16_t* __restrict__ coef, long long n_micro) {
+    const int in_group = threadIdx.x & (LPG - 1);
+    const long long mb = (long long)blockIdx.x * (kWarps * 32) + threadIdx.x;   // this lane's micro-block
+    const bool on = mb < n_micro;
+    float wf[8];
+    {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        if (on) {
+            const float4* src = reinterpret_cast<const float4*>(w) + mb * 2;
+            a = __ldcs(src); b = __ldcs(src + 1);
+        }
+        wf[0] = a.x; wf[1] = a.y; wf[2] = a.z; wf[3] = a.w;
+        wf[4] = b.x; wf[5] = b.y; wf[6] = b.z; wf[7] = b.w;
     }
-    // Section 3.2: s_norm = ||w||_inf, v = w / s_norm, b1 = Q(v)
-    const double s_norm = warp_max(fmax(fmax(fabs(wv[0]), fabs(wv[1])), fmax(fabs(wv[2]), fabs(wv[3]))));
-    int cd[4];
-    double x[4];
+    // Section 3.2: s_norm = ||w||_inf, b1 = Q(w / s_norm)
+    float s = 0.f;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        cd[a] = (s_norm == 0.0) ? emax : rtn_code(wv[a] / s_norm, wbits);
-        x[a] = on ? lattice_value(cd[a], wbits) : 0.0;
+    for (int i = 0; i < 8; ++i) s = fmaxf(s, fabsf(wf[i]));
+#pragma unroll
+    for (int o = LPG / 2; o; o >>= 1) s = fmaxf(s, __shfl_xor_sync(kFull, s, o));
+    const uint32_t code = rtn_codes<WB>(wf, midpoints<WB>(s));
+    double x[8], p[2] = {0.0, 0.0}, n2 = 0.0;
+    code_values<WB>(code, x);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        p[i >> 2] = fma((double)wf[i], x[i], p[i >> 2]);   // exact product
+        n2 = fma(x[i], x[i], n2);
     }
-    // Eq. 1: r = w - (<w, b1> / ||b1||^2) b1 (zero-norm bypass: an all-zero block keeps c1 = 0)
-    const double nb1 = warp_sum(x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
-    const double wb1 = warp_sum(wv[0] * x[0] + wv[1] * x[1] + wv[2] * x[2] + wv[3] * x[3]);
-    const double c1 = nb1 == 0.0 ? 0.0 : wb1 / nb1;
-    double r[4];
+    float nb = (float)n2;   // ||b1||^2: a multiple of 2^(-2 emax), at most 128, so exact in fp32 whatever the order
 #pragma unroll
-    for (int a = 0; a < 4; ++a) r[a] = wv[a] - c1 * x[a];
-
-    unsigned rec = 0;
+    for (int o = LPG / 2; o; o >>= 1) nb += __shfl_xor_sync(kFull, nb, o);
+    // zero-norm bypass: an all-zero block keeps c1 = c2 = 0
+    const double c1 = nb == 0.f ? 0.0 : group_sum2<LPG>(p[0], p[1]) / (double)nb;
     double c2 = 0.0;
-    if (!k1) {
-        // Section 3.3, steps 1-2: d = x_i r_j - x_j r_i per pair, eta* = sgn d, A_s = sum |d|, s* = first maximiser
-        double d[4][2];     // patterns 1..3: the two pairs inside this half; pattern 4: handled below
-        double a_s[4];
+    uint32_t rec = 0;
+    if constexpr (!K1) {
+        // Eq. 1: r = w - c1 b1. Section 3.3, steps 1-2: d = x_i r_j - x_j r_i per pair, eta* = sgn d, A_s = sum |d|, s* = first maximiser
+        double r[8];
 #pragma unroll
-        for (int s = 1; s <= 3; ++s) {
+        for (int i = 0; i < 8; ++i) r[i] = fma(-c1, x[i], (double)wf[i]);
+        double best = -1.0;
+#pragma unroll
+        for (int sp = 1; sp <= 4; ++sp) {
+            double d[4];
             int n = 0;
-            double sum = 0.0;
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const int b = a ^ s;
-                if (a < b) { d[s - 1][n] = x[a] * r[b] - x[b] * r[a]; sum += fabs(d[s - 1][n]); ++n; }
+            for (int i = 0; i < 8; ++i) {
+                const int j = i ^ sp;   // pairs in ascending order of their lower index
+                // exact products; the added zero keeps d from being -0, so that its sign bit is "d < 0"
+                if (i < j) { d[n] = fma(x[i], r[j], fma(-x[j], r[i], 0.0)); ++n; }
             }
-            // the micro-block's four pairs: two here, two in the neighbouring lane; added in pair order
-            const double other = __shfl_xor_sync(kFull, sum, 1);
-            a_s[s - 1] = half ? other + sum : sum + other;
+            const double a = sp < 4 ? (fabs(d[0]) + fabs(d[1])) + (fabs(d[2]) + fabs(d[3]))
+                                    : ((fabs(d[0]) + fabs(d[1])) + fabs(d[2])) + fabs(d[3]);
+            uint32_t f = 0;   // flag of pair p at bit 2 + p
+#pragma unroll
+            for (int q = 3; q >= 0; --q) f = __funnelshift_l((uint32_t)__double2hiint(d[q]), f, 1);
+            f = f * 4u + (uint32_t)(sp - 1);
+            if (a > best) { best = a; rec = f; }
         }
-        double d4[4];
-        {
-            double sum = 0.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const double xo = __shfl_xor_sync(kFull, x[a], 1), ro = __shfl_xor_sync(kFull, r[a], 1);
-                d4[a] = half ? (xo * r[a] - x[a] * ro) : (x[a] * ro - xo * r[a]);   // (i, j) = (lower half, upper half)
-                sum += fabs(d4[a]);
-            }
-            a_s[3] = sum;
-        }
-        int s_star = 0;
-#pragma unroll
-        for (int s = 1; s < 4; ++s) if (a_s[s] > a_s[s_star]) s_star = s;
-        // sign flags of the chosen pattern. The exchange with the neighbouring lane is made by every lane (patterns differ
-        // from micro-block to micro-block, and a warp-wide shuffle must not sit in a branch only some lanes take).
-        unsigned mine = 0;
-#pragma unroll
-        for (int s = 0; s < 3; ++s)
-            if (s == s_star) mine = (d[s][0] < 0.0 ? 1u : 0u) | (d[s][1] < 0.0 ? 2u : 0u);
-        const unsigned other = __shfl_xor_sync(kFull, mine, 1);
-        unsigned flags = half ? (other | (mine << 2)) : (mine | (other << 2));
-        if (s_star == 3) {
-            flags = 0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) flags |= (d4[a] < 0.0 ? 1u : 0u) << a;
-        }
-        rec = (s_norm == 0.0) ? 0u : ((unsigned)s_star | (flags << 2));
-        // step 3 and Eq. 2: b2 from the record, c2 = <w, b2> / ||b2||^2
-        double y[4];
-        exchange4(x, (int)(rec & 3u) + 1, rec >> 2, half, y);
-        const double nb2 = warp_sum(y[0] * y[0] + y[1] * y[1] + y[2] * y[2] + y[3] * y[3]);
-        const double wb2 = warp_sum(wv[0] * y[0] + wv[1] * y[1] + wv[2] * y[2] + wv[3] * y[3]);
-        c2 = nb2 == 0.0 ? 0.0 : wb2 / nb2;
+        // step 3 and Eq. 2: with eta = sgn d, <w, b2> of the micro-block is the chosen pattern's sum |d| (<b1, b2> = 0)
+        const double wb2 = group_sum2<LPG>(best, 0.0);
+        c2 = nb == 0.f ? 0.0 : wb2 / (double)nb;
+        if (nb == 0.f) rec = 0;   // s_norm = 0 iff b1 = 0: the largest weight never rounds to zero
     }
-    if (on) {
-        *reinterpret_cast<uint32_t*>(codes + base) = (uint32_t)cd[0] | ((uint32_t)cd[1] << 8) | ((uint32_t)cd[2] << 16) | ((uint32_t)cd[3] << 24);
-        if (!half) meta[((size_t)row * k_in + (size_t)j * group) / 8 + lane / 2] = (uint8_t)rec;
-    }
-    if (lane == 0) {
-        uint16_t* c = coef + ((size_t)row * nj + j) * 2;
+    if (!on) return;
+    const uint32_t even = code & 0x0F0F0F0Fu, odd = (code >> 4) & 0x0F0F0F0Fu;   // nibbles -> bytes
+    const uint32_t lo = __byte_perm(even, odd, 0x5140), hi = __byte_perm(even, odd, 0x7362);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(codes) + mb * 2;
+    if ((reinterpret_cast<uintptr_t>(codes) & 7u) == 0) *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+    else { dst[0] = lo; dst[1] = hi; }
+    meta[mb] = (uint8_t)rec;
+    if (in_group == 0) {
+        uint16_t* c = coef + mb / LPG * 2;
         c[0] = __half_as_ushort(__double2half(c1));
         c[1] = __half_as_ushort(__double2half(c2));
     }
@@ -284,10 +314,28 @@ quantize_act_kernel(const T* __restrict__ x, int k, const float* __restrict__ am
 }  // namespace quant
 
 // ---- launchers -----------------------------------------------------------------------------------------------
+template <int WB, int LPG>
+static void launch_geo(const Geometry& g, const float* w, uint8_t* codes, uint8_t* meta, uint16_t* coef, cudaStream_t st) {
+    const long long n_micro = (long long)g.n_out * (g.k_in / 8);
+    constexpr int kPerBlock = quant::kWarps * 32;
+    const unsigned blocks = (unsigned)((n_micro + kPerBlock - 1) / kPerBlock);
+    if (g.k1) quant::quantize_geo_kernel<WB, LPG, true><<<blocks, quant::kWarps * 32, 0, st>>>(w, codes, meta, coef, n_micro);
+    else quant::quantize_geo_kernel<WB, LPG, false><<<blocks, quant::kWarps * 32, 0, st>>>(w, codes, meta, coef, n_micro);
+}
+template <int WB>
+static void launch_geo_group(const Geometry& g, const float* w, uint8_t* codes, uint8_t* meta, uint16_t* coef, cudaStream_t st) {
+    switch (g.group) {
+        case 8: launch_geo<WB, 1>(g, w, codes, meta, coef, st); break;
+        case 16: launch_geo<WB, 2>(g, w, codes, meta, coef, st); break;
+        case 32: launch_geo<WB, 4>(g, w, codes, meta, coef, st); break;
+        case 64: launch_geo<WB, 8>(g, w, codes, meta, coef, st); break;
+        default: launch_geo<WB, 16>(g, w, codes, meta, coef, st); break;
+    }
+}
 cudaError_t launch_quantize_geo(const Geometry& g, const float* w, uint8_t* codes, uint8_t* meta, uint16_t* coef, cudaStream_t st) {
-    const long long blocks = (long long)g.n_out * (g.k_in / g.group);
-    quant::quantize_geo_kernel<<<(unsigned)((blocks + quant::kWarps - 1) / quant::kWarps), quant::kWarps * 32, 0, st>>>(
-        w, codes, meta, coef, g.n_out, g.k_in, g.group, g.wbits, g.k1);
+    if (g.wbits == 2) launch_geo_group<2>(g, w, codes, meta, coef, st);
+    else if (g.wbits == 3) launch_geo_group<3>(g, w, codes, meta, coef, st);
+    else launch_geo_group<4>(g, w, codes, meta, coef, st);
     return cudaGetLastError();
 }
 cudaError_t launch_solve_ref(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib,
