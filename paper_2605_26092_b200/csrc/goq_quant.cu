@@ -206,68 +206,208 @@ quantize_geo_kernel(const float* __restrict__ w, uint8_t* __restrict__ codes, ui
 }
 
 // ---- REF mode (Eq. 3) --------------------------------------------------------------------------------------
-// c* = (A^T A + lambda I)^-1 A^T Y with A = [X_q b1, X_q b2] (M x 2), Y = X_q w, per row and macro-block.
-// CTA = 8 warps = 8 rows of one macro-block column j: the calibration tile X_q[m0 .. m0+31][j g .. (j+1) g) is staged
-// in shared memory once per 32 observations and shared by the 8 rows; lane l of a warp owns observation m0 + l and
-// runs the three g-long dot products; the five entries of the normal equations accumulate in float64.
-constexpr int kRefObs = 32;
-__global__ void __launch_bounds__(kWarps * 32)
+// c* = (A^T A + lambda I)^-1 A^T Y with A = [X_q b1, X_q b2] (M x 2), Y = X_q w, per row and macro-block column j, in float64.
+// The calibration rows enter only through the Gram matrix G = X_q^T X_q of the column (g x g), which all output rows share:
+//   b1^T G b1, b1^T G b2, b2^T G b2, b1^T G w, b2^T G w  are the five entries of the normal equations. With H = the lower
+// triangle of G and half its diagonal, G = H + H^T and b^T G c = b.(H c) + (H b).c, so a row costs the three triangular products
+// H b1, H b2, H w: 1.5 g^2 multiply-adds whatever M is, against 3 M g for the observations one by one. With M <= g / 2 the
+// latter is the cheaper (DIRECT), and is used.
+// Both are matrix products with the columns' G (or X) as the shared operand and run on the float64 tensor pipe
+// (mma.m8n8k4): same rate as scalar float64 on this part, but an eighth of the operand traffic and no conversions of shared
+// values in the inner loop. CTA = 16 warps on one macro-block column and a range of 8-row tiles; G is formed once per CTA.
+// Bound: the float64 pipe.
+constexpr int kRefWarps = 16;
+constexpr int kRefChunk = 64;   // observations staged at a time while G is formed
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
+}
+template <int NB> struct RefSmem {   // NB = group / 8
+    static constexpr int kStride = NB * 8 + 4;                         // floats per staged row: fragment reads are conflict-free
+    static constexpr int kFrags = NB * (NB + 1);                       // 4 x 8 operand fragments of H (of X: at most NB * NB)
+    static constexpr size_t kBytes = (size_t)kFrags * 32 * sizeof(double) + (size_t)kRefWarps * 16 * kStride * sizeof(float);
+};
+template <int WB, int NB, bool DIRECT>
+__global__ void __launch_bounds__(kRefWarps * 32, 1)
 solve_ref_kernel(const float* __restrict__ w, const uint8_t* __restrict__ codes, const uint8_t* __restrict__ meta,
                  const float* __restrict__ xc, int m, double lambda, uint16_t* __restrict__ coef, double* __restrict__ c_out,
-                 int n_out, int k_in, int group, int wbits) {
-    __shared__ float xs[kRefObs][kBlockK + 1];
-    __shared__ float ws[kWarps][kBlockK], b1s[kWarps][kBlockK], b2s[kWarps][kBlockK];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nj = k_in / group, j = blockIdx.x, row = blockIdx.y * kWarps + warp;
-    const bool row_ok = row < n_out;
-    // this row's w, b1, b2 of the macro-block (b2 by the recorded exchange, Section 3.3)
-    for (int t = lane; t < group / 8; t += 32) {
-        double x[8], y[8];
-        const size_t o = (size_t)(row_ok ? row : 0) * k_in + (size_t)j * group + t * 8;
-        for (int i = 0; i < 8; ++i) x[i] = lattice_value(codes[o + i], wbits);
-        const unsigned rec = meta[o / 8];
-        const int s = (int)(rec & 3u) + 1;
-        int p = 0;
-        for (int i = 0; i < 8; ++i) {
-            const int q = i ^ s;
-            if (i < q) {
-                const double eta = ((rec >> (2 + p)) & 1u) ? -1.0 : 1.0;
-                y[i] = -eta * x[q];
-                y[q] = eta * x[i];
-                ++p;
+                 int n_out, int k_in) {
+    constexpr int G = NB * 8, kStride = RefSmem<NB>::kStride;
+    extern __shared__ __align__(16) unsigned char smem_ref[];
+    double* frag = reinterpret_cast<double*>(smem_ref);
+    float* stage = reinterpret_cast<float*>(frag + RefSmem<NB>::kFrags * 32);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lr = lane >> 2, lc = lane & 3;
+    const int nj = k_in / G, j = blockIdx.x;
+    const float* xj = xc + (size_t)j * G;
+
+    if constexpr (DIRECT) {   // operand = the observations: fragment (block of 8 observations, 4 channels), element (channel, observation)
+        for (int i = threadIdx.x; i < ((m + 7) / 8) * 8 * G; i += kRefWarps * 32) {
+            const int o = i / G, k = i - o * G;
+            frag[((o >> 3) * (2 * NB) + (k >> 2)) * 32 + (o & 7) * 4 + (k & 3)] = o < m ? (double)xj[(size_t)o * k_in + k] : 0.0;
+        }
+        __syncthreads();
+    } else {
+        // G, lower block triangle, element blocks of 8 x 8. Up to 8 block rows: warp w takes block row w. With 16: warp w < 8 takes
+        // blocks 0..7 of row 15 - w, warp 8 + v the rest of row 15 - v and row v (8 or 9 blocks each).
+        constexpr int kAcc = NB < 8 ? NB : 8;
+        const int v = warp & 7;
+        const bool second = NB == 16 && warp >= 8;
+        const int row_a = NB == 16 ? 15 - v : warp, b0 = second ? 8 : 0;   // blocks b0 .. of row_a, and blocks 0..v of row v
+        double acc_a[kAcc][2], acc_b[kAcc][2];
+#pragma unroll
+        for (int b = 0; b < kAcc; ++b) acc_a[b][0] = acc_a[b][1] = acc_b[b][0] = acc_b[b][1] = 0.0;
+        for (int o0 = 0; o0 < m; o0 += kRefChunk) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < kRefChunk * G; i += kRefWarps * 32) {
+                const int o = i / G, k = i - o * G;
+                stage[o * kStride + k] = (o0 + o < m) ? xj[(size_t)(o0 + o) * k_in + k] : 0.f;
+            }
+            __syncthreads();
+            if (warp < NB) {
+#pragma unroll 1
+                for (int s = 0; s < kRefChunk / 4; ++s) {
+                    const float* xs = stage + (s * 4 + lc) * kStride + lr;
+                    const double fa = (double)xs[row_a * 8];
+#pragma unroll
+                    for (int b = 0; b < kAcc; ++b)
+                        if (b0 + b <= row_a) dmma(acc_a[b], fa, (double)xs[(b0 + b) * 8]);
+                    if (second) {
+                        const double fb = (double)xs[v * 8];
+#pragma unroll
+                        for (int b = 0; b < kAcc; ++b)
+                            if (b <= v) dmma(acc_b[b], fb, (double)xs[b * 8]);
+                    }
+                }
             }
         }
-        for (int i = 0; i < 8; ++i) {
-            ws[warp][t * 8 + i] = row_ok ? w[o + i] : 0.f;
-            b1s[warp][t * 8 + i] = (float)x[i];   // PoT values: exact in float
-            b2s[warp][t * 8 + i] = (float)y[i];
+        if (warp < NB) {
+            // element (row lr, columns 2 lc, 2 lc + 1) of block (ib, b) -> H as an operand fragment: element (k, i)
+            auto put = [&](int ib, int b, const double (&c)[2]) {
+                const int k = 2 * lc;
+                double2 h = make_double2(c[0], c[1]);
+                if (ib == b) {
+                    h.x = k > lr ? 0.0 : (k == lr ? 0.5 * h.x : h.x);
+                    h.y = k + 1 > lr ? 0.0 : (k + 1 == lr ? 0.5 * h.y : h.y);
+                }
+                *reinterpret_cast<double2*>(frag + (ib * (ib + 1) + 2 * b + (k >> 2)) * 32 + lr * 4 + (k & 3)) = h;
+            };
+#pragma unroll
+            for (int b = 0; b < kAcc; ++b) if (b0 + b <= row_a) put(row_a, b0 + b, acc_a[b]);
+            if (second) {
+#pragma unroll
+                for (int b = 0; b < kAcc; ++b) if (b <= v) put(v, b, acc_b[b]);
+            }
         }
-    }
-    double g11 = 0, g12 = 0, g22 = 0, r1 = 0, r2 = 0;
-    for (int m0 = 0; m0 < m; m0 += kRefObs) {
         __syncthreads();
-        for (int i = threadIdx.x; i < kRefObs * group; i += kWarps * 32) {
-            const int o = i / group, k = i - o * group;
-            xs[o][k] = (m0 + o < m) ? xc[(size_t)(m0 + o) * k_in + (size_t)j * group + k] : 0.f;
-        }
-        __syncthreads();
-        double u1 = 0, u2 = 0, t = 0;
-        for (int k = 0; k < group; ++k) {
-            const double xv = xs[lane][k];
-            u1 += xv * b1s[warp][k];
-            u2 += xv * b2s[warp][k];
-            t += xv * ws[warp][k];
-        }
-        g11 += u1 * u1; g12 += u1 * u2; g22 += u2 * u2; r1 += u1 * t; r2 += u2 * t;
     }
-    g11 = warp_sum(g11); g12 = warp_sum(g12); g22 = warp_sum(g22); r1 = warp_sum(r1); r2 = warp_sum(r2);
-    if (lane == 0 && row_ok) {
-        const double a = g11 + lambda, d = g22 + lambda, det = a * d - g12 * g12;
-        const double c1 = (d * r1 - g12 * r2) / det, c2 = (a * r2 - g12 * r1) / det;
-        const size_t o = ((size_t)row * nj + j) * 2;
-        coef[o] = __half_as_ushort(__double2half(c1));
-        coef[o + 1] = __half_as_ushort(__double2half(c2));
-        if (c_out) { c_out[o] = c1; c_out[o + 1] = c2; }
+
+    const int n_rt = (n_out + 7) / 8;
+    const int rt_lo = (int)((long long)n_rt * blockIdx.y / gridDim.y), rt_hi = (int)((long long)n_rt * (blockIdx.y + 1) / gridDim.y);
+    // this warp's eight rows: b1 and b2 as a bf16 pair (PoT values are exact in it), and w
+    uint32_t* vb = reinterpret_cast<uint32_t*>(stage + warp * 16 * kStride);
+    float* vw = stage + warp * 16 * kStride + 8 * kStride;
+    auto low = [](uint32_t p) { return (double)__uint_as_float(p << 16); };
+    auto high = [](uint32_t p) { return (double)__uint_as_float(p & 0xFFFF0000u); };
+    const bool codes8 = (reinterpret_cast<uintptr_t>(codes) & 7u) == 0;
+    for (int rt = rt_lo + warp; rt < rt_hi; rt += kRefWarps) {
+        __syncwarp();
+        for (int i = lane; i < 8 * NB; i += 32) {
+            const int r = i / NB, t = i - r * NB, row = rt * 8 + r;
+            uint32_t* dst = vb + r * kStride + t * 8;
+            if (row < n_out) {   // b2 by the recorded exchange (Section 3.3)
+                const size_t o = (size_t)row * k_in + (size_t)j * G + t * 8;
+                uint32_t cw[2];
+                if (codes8) { const uint2 q = *reinterpret_cast<const uint2*>(codes + o); cw[0] = q.x; cw[1] = q.y; }
+                else {
+                    cw[0] = codes[o] | (codes[o + 1] << 8) | (codes[o + 2] << 16) | ((uint32_t)codes[o + 3] << 24);
+                    cw[1] = codes[o + 4] | (codes[o + 5] << 8) | (codes[o + 6] << 16) | ((uint32_t)codes[o + 7] << 24);
+                }
+                const uint32_t rec = meta[o / 8], s = (rec & 3u) + 1u, flips = flip_mask(rec);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) dst[e] = __float_as_uint((float)lattice_value((int)((cw[e >> 2] >> (8 * (e & 3))) & 255u), WB)) >> 16;
+                uint32_t y[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) y[e] = dst[e ^ s] ^ (((flips >> e) & 1u) << 15);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) dst[e] |= y[e] << 16;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) dst[e] = 0u;
+            }
+        }
+        for (int i = lane; i < 8 * G; i += 32) {
+            const int r = i / G, k = i - r * G, row = rt * 8 + r;
+            vw[r * kStride + k] = row < n_out ? w[(size_t)row * k_in + (size_t)j * G + k] : 0.f;
+        }
+        __syncwarp();
+        double g11 = 0, g12 = 0, g22 = 0, r1 = 0, r2 = 0;
+        const uint32_t* fb = vb + lr * kStride + lc;
+        const float* fw = vw + lr * kStride + lc;
+        const int n_blocks = DIRECT ? (m + 7) / 8 : NB;
+        // two blocks of 8 output columns at a time: they share the row operands
+#pragma unroll 1
+        for (int ib = 0; ib < n_blocks; ib += 2) {
+            double c[2][3][2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) c[h][q][0] = c[h][q][1] = 0.0;
+            const bool two = NB > 1 && ib + 1 < n_blocks;
+            const double* f0 = frag + (DIRECT ? ib * 2 * NB : ib * (ib + 1)) * 32 + lane;
+            const double* f1 = frag + (DIRECT ? (ib + 1) * 2 * NB : (ib + 1) * (ib + 2)) * 32 + lane;
+            const int s0 = DIRECT ? 2 * NB : 2 * (ib + 1), s1 = DIRECT ? 2 * NB : 2 * (ib + 2);
+#pragma unroll 2
+            for (int s = 0; s < s0; ++s) {
+                const uint32_t p = fb[4 * s];
+                const double a1 = low(p), a2 = high(p), a3 = (double)fw[4 * s];
+                const double b0 = f0[s * 32];
+                dmma(c[0][0], a1, b0); dmma(c[0][1], a2, b0); dmma(c[0][2], a3, b0);
+                if (two) {
+                    const double b1 = f1[s * 32];
+                    dmma(c[1][0], a1, b1); dmma(c[1][1], a2, b1); dmma(c[1][2], a3, b1);
+                }
+            }
+            if (two && !DIRECT) {
+#pragma unroll
+                for (int s = s1 - 2; s < s1; ++s) {
+                    const double b1 = f1[s * 32];
+                    const uint32_t p = fb[4 * s];
+                    dmma(c[1][0], low(p), b1); dmma(c[1][1], high(p), b1); dmma(c[1][2], (double)fw[4 * s], b1);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1 && !two) break;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const double p = c[h][0][e], q = c[h][1][e], t = c[h][2][e];
+                    if constexpr (DIRECT) {
+                        g11 = fma(p, p, g11); g12 = fma(p, q, g12); g22 = fma(q, q, g22); r1 = fma(p, t, r1); r2 = fma(q, t, r2);
+                    } else {
+                        const int at = lr * kStride + (ib + h) * 8 + 2 * lc + e;
+                        const double b1 = low(vb[at]), b2 = high(vb[at]), ww = (double)vw[at];
+                        g11 = fma(b1, p, g11); g22 = fma(b2, q, g22);
+                        g12 = fma(b1, q, fma(b2, p, g12));
+                        r1 = fma(b1, t, fma(ww, p, r1));
+                        r2 = fma(b2, t, fma(ww, q, r2));
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            g11 += __shfl_xor_sync(kFull, g11, o); g12 += __shfl_xor_sync(kFull, g12, o); g22 += __shfl_xor_sync(kFull, g22, o);
+            r1 += __shfl_xor_sync(kFull, r1, o); r2 += __shfl_xor_sync(kFull, r2, o);
+        }
+        if constexpr (!DIRECT) { g11 *= 2.0; g22 *= 2.0; }
+        const int row = rt * 8 + lr;
+        if (lc == 0 && row < n_out) {
+            const double a = g11 + lambda, d = g22 + lambda, det = a * d - g12 * g12;
+            const double c1 = (d * r1 - g12 * r2) / det, c2 = (a * r2 - g12 * r1) / det;
+            const size_t o = ((size_t)row * nj + j) * 2;
+            coef[o] = __half_as_ushort(__double2half(c1));
+            coef[o + 1] = __half_as_ushort(__double2half(c2));
+            if (c_out) { c_out[o] = c1; c_out[o + 1] = c2; }
+        }
     }
 }
 
@@ -338,12 +478,47 @@ cudaError_t launch_quantize_geo(const Geometry& g, const float* w, uint8_t* code
     else launch_geo_group<4>(g, w, codes, meta, coef, st);
     return cudaGetLastError();
 }
+template <int WB, int NB>
+static cudaError_t launch_ref(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib,
+                              int m, double lambda, uint16_t* coef, double* c_out, cudaStream_t st) {
+    const bool direct = 2 * m <= NB * 8;
+    auto kernel = direct ? quant::solve_ref_kernel<WB, NB, true> : quant::solve_ref_kernel<WB, NB, false>;
+    const size_t smem = quant::RefSmem<NB>::kBytes;
+    static SmemAttrCache cache[2];
+    if (cudaError_t e = ensure_dynamic_smem(kernel, smem, cache[direct ? 1 : 0])) return e;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 148;
+    // Row chunks per column: every CTA forms its column's G again, so few chunks save work and many fill the chip. Take the
+    // split whose waves cost least in float64 tensor clocks (4 per m8n8k4 and SM, a row tile's loads and epilogue about 400).
+    const int cols = g.k_in / g.group, tiles = (g.n_out + 7) / 8, slots = sms;
+    const double form = direct ? 500.0 : 4.0 * (NB * (NB + 1) / 2) * ((m + 63) / 64 * 16) + 1500.0;
+    const double tile = 12.0 * (direct ? (m + 7) / 8 * 2 * NB : NB * (NB + 1)) + 400.0;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int c = 1; c <= tiles && c <= 65535 && c <= 4 * slots; ++c) {
+        const double waves = (double)(((long long)cols * c + slots - 1) / slots);
+        const double cost = waves * (form + ((tiles + c - 1) / c + quant::kRefWarps - 1) / quant::kRefWarps * quant::kRefWarps * tile);
+        if (c == 1 || cost < best_cost) { best = c; best_cost = cost; }
+    }
+    kernel<<<dim3(cols, best), quant::kRefWarps * 32, smem, st>>>(w, codes, meta, x_calib, m, lambda, coef, c_out, g.n_out, g.k_in);
+    return cudaGetLastError();
+}
+template <int WB>
+static cudaError_t launch_ref_group(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib,
+                                    int m, double lambda, uint16_t* coef, double* c_out, cudaStream_t st) {
+    switch (g.group) {
+        case 8: return launch_ref<WB, 1>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+        case 16: return launch_ref<WB, 2>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+        case 32: return launch_ref<WB, 4>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+        case 64: return launch_ref<WB, 8>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+        default: return launch_ref<WB, 16>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+    }
+}
 cudaError_t launch_solve_ref(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib,
                              int m, double lambda, uint16_t* coef, double* c_out, cudaStream_t st) {
-    dim3 grid(g.k_in / g.group, (g.n_out + quant::kWarps - 1) / quant::kWarps);
-    quant::solve_ref_kernel<<<grid, quant::kWarps * 32, 0, st>>>(w, codes, meta, x_calib, m, lambda, coef, c_out, g.n_out, g.k_in,
-                                                                 g.group, g.wbits);
-    return cudaGetLastError();
+    if (g.wbits == 2) return launch_ref_group<2>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+    if (g.wbits == 3) return launch_ref_group<3>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
+    return launch_ref_group<4>(g, w, codes, meta, x_calib, m, lambda, coef, c_out, st);
 }
 cudaError_t launch_quantize_act(const void* x, int x_dtype, int m, int k, int abits, const float* amax, int8_t* xq, float* sx,
                                 cudaStream_t st) {

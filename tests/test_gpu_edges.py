@@ -1,0 +1,100 @@
+"""Kernels at the sizes where they can go wrong: edges of tiles, remainders, the smallest and largest of a dispatch's range,
+against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import synth_inputs as si
+from oracle import goq_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def goq():
+    from paper_2605_26092_b200 import build
+    build.build()
+    from paper_2605_26092_b200 import goq as g
+    g.lib()
+    assert torch.cuda.is_available()
+    return g
+
+
+def _unaligned(a, shift):
+    """The array on the device, `shift` elements behind an aligned address."""
+    t = torch.from_numpy(np.ascontiguousarray(a))
+    buf = torch.empty(t.numel() + shift, dtype=t.dtype, device="cuda")
+    buf[shift:] = t.reshape(-1).cuda()
+    return buf[shift:]
+
+
+@pytest.mark.parametrize("b", [2, 3, 4])
+@pytest.mark.parametrize("n,k,g,shift", [(1, 8, 8, 0), (16, 128, 128, 0), (17, 136, 8, 0), (15, 240, 16, 3), (33, 384, 64, 1), (40, 96, 32, 0)])
+def test_pack_edges(goq, n, k, g, b, shift):
+    """Rows and columns that end inside a record, code and record arrays at odd addresses: the fields come back unchanged."""
+    rng = np.random.default_rng(n + k + b)
+    codes = rng.integers(0, 1 << b, size=(n, k), dtype=np.uint8)
+    meta = rng.integers(0, 64, size=(n, k // 8), dtype=np.uint8)
+    coef = rng.standard_normal((n, k // g, 2)).astype(np.float16)
+    d = goq.desc(n, k, g, b)
+    packed = torch.full((goq.packed_bytes(d),), 0xA5, dtype=torch.uint8, device="cuda")
+    goq.pack(d, _unaligned(codes, shift), _unaligned(meta, shift), _unaligned(coef.view(np.int16), shift), packed)
+    b1 = torch.empty((n, k), dtype=torch.uint8, device="cuda")
+    b2 = torch.empty((n, k), dtype=torch.uint8, device="cuda")
+    cf = torch.empty((n, k // g, 2), dtype=torch.int16, device="cuda")
+    goq.unpack(d, packed, b1, b2, cf)
+    torch.cuda.synchronize()
+    assert np.array_equal(b1.cpu().numpy(), codes)
+    assert np.array_equal(cf.cpu().numpy().view(np.uint16), coef.view(np.uint16))
+    ref = O.decode_b2(codes, meta, b)
+    got = b2.cpu().numpy()
+    val = np.where(got == 0x80, 0.0, np.where(got & 8, -1.0, 1.0) * 2.0 ** -(got & 7).astype(np.float64))
+    assert np.array_equal(val, ref)
+
+
+@pytest.mark.parametrize("b", [2, 3, 4])
+@pytest.mark.parametrize("g", [8, 16, 32, 64, 128])
+def test_geo_quantizer_on_the_midpoints(goq, g, b):
+    """Weights on, just above and just below every decision boundary of the lattice (midpoints times the block's largest, which
+    is not a power of two), at ordinary, subnormal-threatening and large scales: codes equal to the oracle's."""
+    rng = np.random.default_rng(g + b)
+    n, k = 24, 2 * g
+    emax = (1 << (b - 1)) - 1
+    mids = [0.75 * 2.0 ** -e for e in range(emax)] + [2.0 ** -emax, 2.0 ** -(emax + 1)]
+    w = np.zeros((n, k), dtype=np.float32)
+    for r in range(n):
+        top = np.float32(rng.uniform(0.5, 1.0)) * np.float32(2.0 ** [0, -40, -120, 90][r % 4])
+        v = (rng.choice(mids, size=k) * np.float64(top)).astype(np.float32)
+        step = rng.integers(-1, 2, size=k)
+        v = np.where(step > 0, np.nextafter(v, np.float32(np.inf)), np.where(step < 0, np.nextafter(v, np.float32(0)), v))
+        w[r] = v * rng.choice(np.array([-1, 1], dtype=np.float32), size=k)
+        w[r, ::g] = top * (1 if r % 2 else -1)
+    codes_o, _, _ = O.quantize_geo(w, g, b)
+    d = goq.desc(n, k, g, b)
+    codes = torch.empty((n, k), dtype=torch.uint8, device="cuda")
+    meta = torch.empty((n, k // 8), dtype=torch.uint8, device="cuda")
+    coef = torch.empty((n, k // g, 2), dtype=torch.int16, device="cuda")
+    goq.quantize_geo(d, torch.from_numpy(w).cuda(), codes, meta, coef)
+    torch.cuda.synchronize()
+    assert np.array_equal(codes.cpu().numpy(), codes_o)
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [(1, 8, 8, 3, 4), (9, 24, 8, 2, 5), (130, 48, 16, 4, 9), (8, 64, 32, 3, 16), (31, 96, 32, 3, 17),
+                                       (200, 192, 64, 3, 32), (7, 128, 64, 2, 33), (300, 256, 128, 3, 64), (129, 384, 128, 3, 65),
+                                       (2500, 128, 128, 4, 200)])
+def test_ref_solve_edges(goq, n, k, g, b, m):
+    """Both sides of the line between the observation form and the Gram form (m = g / 2), row tiles and observation chunks that
+    do not fill, every group size. float64 normal equations: 1e-9 as in the general test."""
+    w = si.gaussian_weights(n, k, seed=n + m).astype(np.float32)
+    codes, meta, _ = O.quantize_geo(w, g, b)
+    x = si.f32_activations(m, k, seed=m).astype(np.float32)
+    c_ref = O.solve_ref(w, codes, meta, x, g, b, lam=1e-2)
+    d = goq.desc(n, k, g, b)
+    coef = torch.zeros((n, k // g, 2), dtype=torch.int16, device="cuda")
+    c64 = torch.full((n, k // g, 2), np.nan, dtype=torch.float64, device="cuda")
+    goq.solve_ref(d, torch.from_numpy(w).cuda(), torch.from_numpy(codes).cuda(), torch.from_numpy(meta).cuda(),
+                  torch.from_numpy(x).cuda(), m, 1e-2, coef, c64)
+    torch.cuda.synchronize()
+    got = c64.cpu().numpy()
+    assert np.allclose(got, c_ref, rtol=1e-9, atol=1e-11)
+    assert np.array_equal(coef.cpu().numpy().view(np.uint16), got.astype(np.float16).view(np.uint16))
