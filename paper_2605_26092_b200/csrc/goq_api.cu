@@ -11,6 +11,8 @@ namespace {
 
 std::atomic<int> g_gemv_variant{0};
 std::atomic<int> g_wait_limit{0};   // 0: the kernels' own bound on device-side waits
+constexpr int kGemmExactMaxTokens = 32;     // goq_gemm: fp32-accurate results up to here
+constexpr int kGemmMidMaxTokens = 256;
 constexpr int kGemmViaGemvMaxTokens = 32;   // above: the tcgen05 GEMM (split-K) is faster than 16-token GEMV launches
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
@@ -83,6 +85,7 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
         size_t need = 0;
         if (goq::gemv_stream_supported(g)) need = goq::gemv_stream_workspace(g);
         if (m <= 4 && goq::gemv_seq_supported(g, m) && goq::gemv_seq_workspace(1) > need) need = goq::gemv_seq_workspace(1);
+        if (goq::gemm_mid_supported(g, m, true) && goq::gemm_mid_workspace(g, m, true) > need) need = goq::gemm_mid_workspace(g, m, true);
         return need;
     }
     if (op == GOQ_OP_GEMM) {
@@ -90,6 +93,9 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
         size_t need = goq::gemm_tc_supported(g) ? goq::gemm_tc_workspace(g, m) : 0;
         if (m <= kGemmViaGemvMaxTokens && goq::gemv_stream_supported(g) && goq::gemv_stream_workspace(g) > need)
             need = goq::gemv_stream_workspace(g);
+        for (int exact = 0; exact < 2; ++exact)
+            if (goq::gemm_mid_supported(g, m, exact != 0) && goq::gemm_mid_workspace(g, m, exact != 0) > need)
+                need = goq::gemm_mid_workspace(g, m, exact != 0);
         return need;
     }
     return 0;
@@ -125,6 +131,12 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         return GOQ_ERR_ALIGNMENT;
     if (goq_status s = check_arch()) return s;
     const int variant = g_gemv_variant.load(std::memory_order_relaxed);
+    if (variant == 4) {
+        if (!goq::gemm_mid_supported(g, batch, true)) return GOQ_ERR_UNSUPPORTED;
+        if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
+        if (ws_bytes < goq::gemm_mid_workspace(g, batch, true)) return GOQ_ERR_WORKSPACE;
+        return from_cuda(goq::launch_gemm_mid(g, packed, x_bf16, batch, y, y_dtype, ws, true, (cudaStream_t)stream));
+    }
     bool use_stream = goq::gemv_stream_supported(g) && (variant == 0 || variant == 3);
     if (variant == 3 && !use_stream) return GOQ_ERR_UNSUPPORTED;
     if (use_stream) {
@@ -161,6 +173,18 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (!y) return GOQ_ERR_INVALID_ARG;
         if (goq_status s = check_arch()) return s;
         const int variant = g_gemv_variant.load(std::memory_order_relaxed);
+        // More tokens than one streaming GEMV takes, fewer than fill the prefill kernel's 128 x 512 tiles: the tensor-core kernel
+        // that splits the packed records evenly over the SMs. Up to 32 tokens with both bases as exact operands (fp32 accuracy),
+        // above with w_hat rounded once to fp16. Measured, W3 g128, us (this kernel / streaming launches or prefill kernel):
+        // 8192 x 8192: 43 / 72 at 32 tokens, 43 / 92 at 64, 65 / 95 at 256, 92 / 121 at 512; 4096 x 4096: 23 / 31, 27 / 52,
+        // 44 / 53, 50 / 67; 1024 x 8192: 20 / 23, 27 / 75, 70 / 75, 57 / 118.
+        const bool exact = m <= kGemmExactMaxTokens;
+        // Above 256 tokens it decodes the weights once per 256 tokens, so it is for calls whose 128 x 512 tiles would leave half of
+        // the SMs without one (1024 x 8192 W4, 777 tokens: 49 / 122; 4096 x 4096, 1024 tokens: 64 / 69; 16384 x 2048, 640: 153 / 78).
+        const bool mid_wanted = variant == 4 || (variant == 0 && m > 16 && (m <= kGemmMidMaxTokens || goq::gemm_tc_tiles(g, m) * 2 <= 148));
+        if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
+            return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
+        if (variant == 4) return GOQ_ERR_UNSUPPORTED;
         // Few tokens (17..32): the streaming GEMV kernel, 16 tokens per launch (36 us each on 8192 x 8192, so 72 us at
         // 32 tokens), against ~89 us for the tensor-core kernel with split-K, which takes over from 33 tokens.
         if (m <= kGemmViaGemvMaxTokens && variant == 0 && goq::gemv_stream_supported(g)) {

@@ -25,9 +25,7 @@
 //
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, skips the remaining work,
 // still frees its tensor memory and records GOQ_ERR_TIMEOUT in the status word.
-#include <cuda.h>
-#include <cuda_fp16.h>
-#include "goq_common.cuh"
+#include "goq_tc_core.cuh"
 #include "goq_internal.h"
 
 namespace goq {
@@ -41,209 +39,6 @@ constexpr int kExpanders = 8;   // expander warps; each owns one 16-row unit rec
 constexpr int kThreads = (2 + kExpanders) * 32;
 constexpr int kATileBytes = kTileN * kChunkK * 2;   // 16 KiB, the weight operand tile of a stage
 constexpr int kBTileBytes = kTileM * kChunkK * 2;   // 64 KiB
-constexpr int kLutCopies = 8;   // record table, one copy per lane & 7: lookups are bank-conflict free (shared-memory
-                                // bandwidth, shared with the tensor core's operand reads, bounds this kernel)
-constexpr int kLutBytes = 64 * kLutCopies * 16;
-constexpr int kSpin = 1 << 22;
-
-__device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t n) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(b)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(b)) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(s32(b)), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-    for (int it = 0; it < kSpin; ++it) {
-        if (mbar_try(b, parity)) return true;
-        if ((it & 63) == 63 && *abort_flag) return false;
-    }
-    *abort_flag = 1;
-    return false;
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s32(dst)),
-                 "l"(src), "r"(bytes), "r"(s32(bar)) : "memory");
-}
-// 2-D tiled TMA load (no multicast): coordinates {c0 = k element, c1 = token row}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(s32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(s32(bar)) : "memory");
-}
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-    uint32_t d;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-    return d;
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-    uint32_t v;
-    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ uint32_t after_wait(uint32_t addr) {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %1;" : "=r"(r) : "r"(addr) : "memory");
-    return r;
-}
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-__device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
-// ---- tensor memory and MMA ---------------------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc_512(uint32_t* smem_slot) {  // whole warp
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s32(smem_slot)) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_512(uint32_t taddr) {  // whole warp
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(taddr) : "memory");
-}
-// K-major operand tile with 128-byte swizzle: rows of 128 bytes, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);        // start address
-    d |= (uint64_t)1 << 16;                          // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                // stride byte offset between 8-row groups
-    d |= (uint64_t)1 << 46;                          // descriptor version for sm_100
-    d |= (uint64_t)2 << 61;                          // SWIZZLE_128B
-    return d;
-}
-// kind::f16 instruction descriptor: fp32 accumulate, fp16 x fp16 (format fields 0), both K-major, M = 128, N = 256
-constexpr uint32_t kIdesc = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(bar)) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-
-// ---- record decode (same tables as the decode GEMV) --------------------------------------------
-// High byte of the fp16 number of every PoT state, by code (the low byte of a power of two is zero).
-template <int WB> struct PotBytes;
-template <> struct PotBytes<3> {  // +1 +.5 +.25 0 -1 -.5 -.25 -.125
-    static constexpr uint32_t H0 = 0x0034383Cu, H1 = 0xB0B4B8BCu;
-};
-template <> struct PotBytes<2> {  // +1 0 -1 -.5
-    static constexpr uint32_t H0 = 0xB8BC003Cu, H1 = 0u;
-};
-// W4: code = sign << 3 | e, value (-1)^sign 2^-e (fp16 high byte (15 - e) << 2), sign 0 with e = 7 is the zero state
-struct PotBytes4 {
-    static constexpr uint32_t PH0 = 0x3034383Cu, PH1 = 0x0024282Cu, NH0 = 0xB0B4B8BCu, NH1 = 0xA0A4A8ACu;
-};
-constexpr uint32_t kHashMul = 0x01008420u;  // (record bits in place) * kHashMul >> 26 is a bijection onto 0..63
-
-struct ExchangeLut { uint32_t v[64][4]; };
-constexpr ExchangeLut make_exchange_lut() {
-    ExchangeLut t{};
-    for (uint32_t meta = 0; meta < 64; ++meta) {
-        const int s = (int)(meta & 3u) + 1;
-        // flips: bit i = 1 iff b2 element i has the opposite sign of the b1 element routed to it
-        uint32_t flips = 0;
-        int p = 0;
-        for (int i = 0; i < 8; ++i) {
-            const int j = i ^ s;
-            if (i < j) {
-                const uint32_t f = (meta >> (2 + p)) & 1u;  // 1 iff eta = -1
-                flips |= (f ^ 1u) << i;                     // y_i = -eta x_j
-                flips |= f << j;                            // y_j =  eta x_i
-                ++p;
-            }
-        }
-        uint32_t sel_a = 0, sel_b = 0, f_a = 0, f_b = 0, spread = 0;
-        for (int i = 0; i < 4; ++i) {
-            sel_a |= (uint32_t)(i ^ s) << (4 * i);
-            sel_b |= (uint32_t)((4 + i) ^ s) << (4 * i);
-            f_a |= ((flips >> i) & 1u) << (8 * i + 7);
-            f_b |= ((flips >> (4 + i)) & 1u) << (8 * i + 7);
-        }
-        for (int i = 0; i < 6; ++i) spread |= ((meta >> i) & 1u) << (4 * i + 3);
-        const uint32_t slot = (uint32_t)(spread * kHashMul) >> 26;
-        t.v[slot][0] = sel_a; t.v[slot][1] = sel_b; t.v[slot][2] = f_a; t.v[slot][3] = f_b;
-    }
-    return t;
-}
-__constant__ ExchangeLut c_lut = make_exchange_lut();
-
-__device__ __forceinline__ uint32_t hmul2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t r;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-    return r;
-}
-// Eight weights of one micro-block -> w_hat = c1*b1 + c2*b2 in fp16, four f16x2 words. c1, c2: the coefficient in both
-// halves of a register. b1 and b2 are built as fp16 directly (table high byte over a zero low byte), c1*b1 is a
-// power-of-two scaling (exact) and the fused multiply-add rounds once: the same value as fp32 arithmetic rounded
-// to fp16, for a quarter of the instructions.
-// W <= 3: the exchange record sits in the spare bit of the word's nibbles and is hashed into the table slot. W = 4: the
-// nibbles are full (the sign is bit 3), the record comes from the unit's byte plane (`record`) and the table is filled
-// in record order; the high byte is taken from a positive or a negative table per weight, chosen by a byte mask that
-// prmt's sign-replicate mode makes of the sign bits (top bit of each byte of w: odd weights; of w << 4: even weights).
-template <int WB>
-__device__ __forceinline__ void expand_what(uint32_t w, uint32_t record, uint32_t lut_lane, uint32_t c1, uint32_t c2, uint32_t (&out)[4]) {
-    const uint32_t m = w & 0x77777777u, mh = m >> 16;
-    uint32_t ha, hb, slot_off;
-    if constexpr (WB <= 3) {
-        ha = prmt(PotBytes<WB>::H0, PotBytes<WB>::H1, m);
-        hb = prmt(PotBytes<WB>::H0, PotBytes<WB>::H1, mh);
-        slot_off = (((w - m) * kHashMul) >> 19) & 0x1F80u;
-    } else {
-        const uint32_t s_odd = prmt(w, 0u, 0xBA98u), s_even = prmt(w << 4, 0u, 0xBA98u);
-        const uint32_t ma = prmt(s_even, s_odd, 0x5140u), mb = prmt(s_even, s_odd, 0x7362u);   // weights 0..3, 4..7
-        ha = (prmt(PotBytes4::PH0, PotBytes4::PH1, m) & ~ma) | (prmt(PotBytes4::NH0, PotBytes4::NH1, m) & ma);
-        hb = (prmt(PotBytes4::PH0, PotBytes4::PH1, mh) & ~mb) | (prmt(PotBytes4::NH0, PotBytes4::NH1, mh) & mb);
-        slot_off = (record & 63u) << 7;
-    }
-    const uint4 e = lds128(slot_off | lut_lane);  // table is 8 KiB aligned, lut_lane selects the copy
-    const uint32_t qa = prmt(ha, hb, e.x) ^ e.z, qb = prmt(ha, hb, e.y) ^ e.w;   // b2: permuted, pair signs applied
-    // bytes {0, h[2q], 0, h[2q+1]}: weights 2q, 2q+1 as one f16x2 word
-    const uint32_t R[4] = {prmt(ha, 0u, 0x1404u), prmt(ha, 0u, 0x3424u), prmt(hb, 0u, 0x1404u), prmt(hb, 0u, 0x3424u)};
-    const uint32_t Q[4] = {prmt(qa, 0u, 0x1404u), prmt(qa, 0u, 0x3424u), prmt(qb, 0u, 0x1404u), prmt(qb, 0u, 0x3424u)};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) out[q] = hfma2(c2, Q[q], hmul2(c1, R[q]));
-}
 
 struct GemmParams {
     const uint8_t* packed;
@@ -313,17 +108,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
         mbar_init(&epi_bar[1], 4);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < 64 * kLutCopies; i += kThreads) {
-        uint32_t slot = (uint32_t)(i / kLutCopies);
-        if constexpr (WB == 4) {   // table in record order: entry `record` is the hashed table's entry of that record
-            uint32_t spread = 0;
-            for (int b = 0; b < 6; ++b) spread |= ((slot >> b) & 1u) << (4 * b + 3);
-            slot = (spread * kHashMul) >> 26;
-        }
-        const uint32_t* e = c_lut.v[slot];
-        *reinterpret_cast<uint4*>(lut + (size_t)i * 16) = make_uint4(e[0], e[1], e[2], e[3]);
-    }
-    if (warp == 1) tmem_alloc_512(&tmem_base_slot);
+    fill_lut<WB>(lut, tid, kThreads);
+    if (warp == 1) tmem_alloc<512>(&tmem_base_slot);
     // Everything above needs nothing from the activation pre-pass, which may still be running (programmatic dependent
     // launch: this grid is scheduled as soon as the pre-pass lets it); what follows reads what the pre-pass wrote.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -389,8 +175,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
 #pragma unroll
                 for (int ks = 0; ks < kChunkK / 16; ++ks) {
                     const uint32_t acc = (chunk > 0 || ks > 0) ? 1u : 0u;
-                    umma_f16(tmem_base, adesc + 2 * ks, bdesc0 + 2 * ks, acc);         // tokens   0..255
-                    if (n_half == 2) umma_f16(tmem_base + 256, adesc + 2 * ks, bdesc1 + 2 * ks, acc);   // tokens 256..511
+                    umma_f16(tmem_base, adesc + 2 * ks, bdesc0 + 2 * ks, idesc_f16(256), acc);         // tokens   0..255
+                    if (n_half == 2) umma_f16(tmem_base + 256, adesc + 2 * ks, bdesc1 + 2 * ks, idesc_f16(256), acc);   // tokens 256..511
                 }
                 umma_commit(&empty[s]);
             }
@@ -566,7 +352,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
     __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tmem_dealloc_512(tmem_base);
+        tmem_dealloc<512>(tmem_base);
     }
     if (tid == 0 && abort_flag) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
@@ -576,6 +362,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
 // xh[tok][k] = fp16(x[tok][k] * 2^s), inv_scale[tok] = 2^-s, s chosen from the exponent field of the token's largest
 // magnitude (an all-zero token gets the largest scale, harmlessly; inf / nan stay inf / nan).
 constexpr int kPrepThreads = 256;
+constexpr int kPrepHold = 6;   // 16-byte vectors a thread keeps: rows up to 12288
 // Blocks beyond the tokens compute the per-channel scales of the weight operand, one 16-row tile each: w_hat is
 // formed in fp16, whose normal range ends at 2^-14, so every channel's coefficients are multiplied by the power of two
 // that puts the channel's largest |c1|, |c2| in [2^6, 2^7) (exact in fp16) and the epilogue divides it out again.
@@ -586,6 +373,7 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
                                                                 int groups_per_block, uint32_t* __restrict__ row_scale,
                                                                 float* __restrict__ row_inv) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the GEMM's CTAs may set themselves up meanwhile
+    asm volatile("griddepcontrol.wait;" ::: "memory");                // (launched as a dependent itself: what precedes it is complete)
     if ((int)blockIdx.x >= m_total) {
         __shared__ uint32_t part_max[kPrepThreads / 16][16];
         const int T = (int)blockIdx.x - m_total, r = threadIdx.x & 15, part = threadIdx.x >> 4;
@@ -611,18 +399,28 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
         }
         return;
     }
+    // one token: the row stays in registers between the maximum and the conversion (rows longer than kPrepHold vectors a
+    // thread are read twice), so the pass costs one trip to memory
     const int tok = blockIdx.x, tid = threadIdx.x;
     const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)tok * k_in);
     uint4* out = reinterpret_cast<uint4*>(xh + (size_t)tok * k_in);
     const int n_vec = k_in / 8;   // k_in is a multiple of 8 (checked by the launcher)
     __shared__ uint32_t warp_max[kPrepThreads / 32];
     uint32_t amax = 0;
-    for (int i = tid; i < n_vec; i += kPrepThreads) {
-        const uint4 v = __ldg(&row[i]);
+    auto largest = [&](const uint4& v) {
         const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) amax = max(amax, max(in32[j] & 0x7FFFu, (in32[j] >> 16) & 0x7FFFu));
+    };
+    uint4 held[kPrepHold];
+#pragma unroll
+    for (int h = 0; h < kPrepHold; ++h) {
+        const int i = tid + h * kPrepThreads;
+        held[h] = i < n_vec ? __ldg(&row[i]) : make_uint4(0u, 0u, 0u, 0u);
     }
+#pragma unroll
+    for (int h = 0; h < kPrepHold; ++h) largest(held[h]);
+    for (int i = tid + kPrepHold * kPrepThreads; i < n_vec; i += kPrepThreads) largest(__ldg(&row[i]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
     if ((tid & 31) == 0) warp_max[tid >> 5] = amax;
@@ -632,15 +430,18 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
     int sfield = 268 - (int)(amax >> 7);   // exponent field of 2^s: the largest magnitude lands in [2^14, 2^15)
     sfield = sfield < 1 ? 1 : (sfield > 253 ? 253 : sfield);
     const float mult = __uint_as_float((uint32_t)sfield << 23);
-    for (int i = tid; i < n_vec; i += kPrepThreads) {
-        const uint4 v = __ldg(&row[i]);
+    auto convert = [&](int i, const uint4& v) {
         const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
         uint32_t o32[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             o32[j] = pack_f16x2(__uint_as_float(in32[j] << 16) * mult, __uint_as_float(in32[j] & 0xFFFF0000u) * mult);
         out[i] = make_uint4(o32[0], o32[1], o32[2], o32[3]);
-    }
+    };
+#pragma unroll
+    for (int h = 0; h < kPrepHold; ++h)
+        if (tid + h * kPrepThreads < n_vec) convert(tid + h * kPrepThreads, held[h]);
+    for (int i = tid + kPrepHold * kPrepThreads; i < n_vec; i += kPrepThreads) convert(i, __ldg(&row[i]));
     if (tid == 0) inv_scale[tok] = __uint_as_float((uint32_t)(254 - sfield) << 23);
 }
 
@@ -658,6 +459,48 @@ static EncodeTiledFn encode_tiled_fn() {
             fn = (EncodeTiledFn)ptr;
     }
     return fn;
+}
+
+// fp16 activations [m][k_in] as boxes of 64 k x `rows` tokens, 128-byte swizzle
+cudaError_t encode_x_map(CUtensorMap* map, void* xh, int k_in, int m, int rows) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)k_in, (cuuint64_t)m};
+    const cuuint64_t strides[1] = {(cuuint64_t)k_in * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)rows};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, xh, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;   // distinct code: the tensor map could not be encoded
+}
+bool packed_map_supported(const Geometry& g) {
+    return g.unit_bytes / 8 <= 256 && (unsigned long long)g.k_blocks * g.unit_bytes / 8 < (1ull << 31);
+}
+cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)g.k_blocks * g.unit_bytes / 8, (cuuint64_t)g.n_tiles};
+    const cuuint64_t strides[1] = {(cuuint64_t)g.k_blocks * g.unit_bytes};
+    const cuuint32_t box[2] = {(cuuint32_t)g.unit_bytes / 8, 8};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<void*>(packed), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
+}
+// The activation pre-pass alone, as a programmatic dependent of what precedes it: its launch overlaps the tail of that kernel.
+cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(m);
+    cfg.blockDim = dim3(kPrepThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, x_to_f16_kernel, (const uint16_t*)x, k_in, xh, inv_scale, m, (const uint8_t*)nullptr, 0, 0, 0,
+                              (uint32_t*)nullptr, (float*)nullptr);
 }
 
 static int sm_count_cached() {
@@ -691,20 +534,11 @@ template <int WB>
 static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, int* status,
                              float* inv_scale, uint32_t* row_scale, float* row_inv, uint16_t* xh, int* tile_counter, float* partial,
                              cudaStream_t st) {
-    EncodeTiledFn enc = encode_tiled_fn();
-    if (!enc) return cudaErrorNotSupported;
     if (g.k_in % 8 != 0) return cudaErrorInvalidValue;
     x_to_f16_kernel<<<m + g.n_tiles, kPrepThreads, 0, st>>>((const uint16_t*)x, g.k_in, xh, inv_scale, m, (const uint8_t*)packed,
                                                            g.unit_bytes, g.k_blocks, g.groups_per_block, row_scale, row_inv);
     CUtensorMap map;
-    const cuuint64_t dims[2] = {(cuuint64_t)g.k_in, (cuuint64_t)m};
-    const cuuint64_t strides[1] = {(cuuint64_t)g.k_in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kChunkK, 256};
-    const cuuint32_t estr[2] = {1, 1};
-    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, xh, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidTexture;  // distinct code: the tensor map could not be encoded
+    if (cudaError_t e = encode_x_map(&map, xh, g.k_in, m, 256)) return e;
     const size_t smem = smem_bytes(g);
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_tc_kernel<WB>, smem, smem_attr)) return e;
@@ -775,6 +609,7 @@ TcScratch tc_scratch(const Geometry& g, int m) {
     return t;
 }
 }  // namespace
+int gemm_tc_tiles(const Geometry& g, int m) { return (g.n_pad + tc::kTileN - 1) / tc::kTileN * ((m + tc::kTileM - 1) / tc::kTileM); }
 size_t gemm_tc_workspace(const Geometry& g, int m) { return tc_scratch(g, m).total; }
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws,
                            cudaStream_t st) {

@@ -98,3 +98,33 @@ def test_ref_solve_edges(goq, n, k, g, b, m):
     got = c64.cpu().numpy()
     assert np.allclose(got, c_ref, rtol=1e-9, atol=1e-11)
     assert np.array_equal(coef.cpu().numpy().view(np.uint16), got.astype(np.float16).view(np.uint16))
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [
+    (1, 8, 8, 3, 17), (129, 136, 8, 3, 33), (127, 256, 16, 4, 32), (128, 128, 128, 3, 64),
+    (4000, 384, 128, 3, 65), (257, 1152, 64, 3, 256), (300, 640, 128, 4, 257), (1000, 4096, 32, 3, 511),
+    (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 20)])
+def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
+    """The kernel between decode and prefill: channel tiles and token tiles that do not fill, one unit in all, one tile shared by
+    many SMs and several tiles an SM, both operand forms (exact up to 32 tokens), every bit width; twice, bit for bit.
+    Bounds: two exact operands with fp32 sums 2e-5 (as every fp32-accumulating kernel), w_hat rounded once to fp16 5e-4."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b)
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+    prev = goq.set_gemv_variant(4)
+    try:
+        out = []
+        for _ in range(2):
+            y = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+            goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+            torch.cuda.synchronize()
+            assert goq.workspace_status(ws) == goq.OK
+            out.append(y.cpu().numpy())
+    finally:
+        goq.set_gemv_variant(prev)
+    assert np.array_equal(out[0], out[1])
+    exact = m <= 32
+    check_parity(out[0].astype(np.float64), y_ref, 2e-5 if exact else 5e-4, 1e-4 if exact else 2e-3)
