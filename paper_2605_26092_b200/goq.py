@@ -8,7 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
-from ctypes import POINTER, Structure, c_char_p, c_int, c_int32, c_size_t, c_void_p
+from ctypes import POINTER, Structure, byref, c_char_p, c_int, c_int32, c_size_t, c_void_p
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libgoq.so")
@@ -120,14 +120,43 @@ def status_string(status: int) -> str:
 
 
 def _ptr(t):
-    return None if t is None else c_void_p(t.data_ptr() if hasattr(t, "data_ptr") else int(t))
+    """Device address of a tensor (or an integer address) as a plain int: the argument types are declared, so ctypes converts."""
+    if t is None:
+        return None
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        return int(t)
+
+
+def _current_stream_slow():
+    import torch
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _pick_stream_getter():
+    # A decode step makes a call every few microseconds; torch.cuda.current_stream() builds a Stream object each time (about 2 us).
+    import torch
+    stream = torch.cuda.current_stream().cuda_stream   # also initialises CUDA
+    try:
+        raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        if raw(device()) == stream:
+            return lambda: raw(device())
+    except (AttributeError, RuntimeError):
+        pass
+    return _current_stream_slow
+
+
+_current_stream = None
 
 
 def _stream(stream=None):
+    global _current_stream
     if stream is not None:
-        return c_void_p(int(stream))
-    import torch
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+        return int(stream)
+    if _current_stream is None:
+        _current_stream = _pick_stream_getter()
+    return _current_stream()
 
 
 def _check(status: int, where: str):
@@ -136,24 +165,24 @@ def _check(status: int, where: str):
 
 
 def packed_bytes(d: Desc) -> int:
-    return lib().goq_packed_bytes(ctypes.byref(d))
+    return lib().goq_packed_bytes(byref(d))
 
 
 def algorithmic_bytes(d: Desc) -> int:
-    return lib().goq_algorithmic_bytes(ctypes.byref(d))
+    return lib().goq_algorithmic_bytes(byref(d))
 
 
 def workspace_bytes(d: Desc, op: int, m: int) -> int:
-    return lib().goq_workspace_bytes(ctypes.byref(d), op, m)
+    return lib().goq_workspace_bytes(byref(d), op, m)
 
 
 def workspace_init(ws, stream=None):
-    _check(lib().goq_workspace_init(_ptr(ws), ws.numel() * ws.element_size(), _stream(stream)), "goq_workspace_init")
+    _check(lib().goq_workspace_init(_ptr(ws), ws.nbytes, _stream(stream)), "goq_workspace_init")
 
 
 def workspace_status(ws, stream=None) -> int:
     out = c_int(0)
-    _check(lib().goq_workspace_status(_ptr(ws), _stream(stream), ctypes.byref(out)), "goq_workspace_status")
+    _check(lib().goq_workspace_status(_ptr(ws), _stream(stream), byref(out)), "goq_workspace_status")
     return out.value
 
 
@@ -178,25 +207,26 @@ def set_wait_limit(polls: int) -> int:
 
 
 def pack(d: Desc, codes, meta, coef_f16, packed, stream=None):
-    _check(lib().goq_pack(ctypes.byref(d), _ptr(codes), _ptr(meta), _ptr(coef_f16), _ptr(packed),
-                          packed.numel() * packed.element_size(), _stream(stream)), "goq_pack")
+    _check(lib().goq_pack(byref(d), _ptr(codes), _ptr(meta), _ptr(coef_f16), _ptr(packed),
+                          packed.nbytes, _stream(stream)), "goq_pack")
 
 
 def unpack(d: Desc, packed, codes_b1=None, codes_b2=None, coef_f16=None, stream=None):
-    _check(lib().goq_unpack(ctypes.byref(d), _ptr(packed), _ptr(codes_b1), _ptr(codes_b2), _ptr(coef_f16),
+    _check(lib().goq_unpack(byref(d), _ptr(packed), _ptr(codes_b1), _ptr(codes_b2), _ptr(coef_f16),
                             _stream(stream)), "goq_unpack")
 
 
 def gemv(d: Desc, packed, x_bf16, batch: int, y, y_dtype: int, ws=None, stream=None):
-    wsb = 0 if ws is None else ws.numel() * ws.element_size()
-    _check(lib().goq_gemv(ctypes.byref(d), _ptr(packed), _ptr(x_bf16), batch, _ptr(y), y_dtype, _ptr(ws), wsb,
-                          _stream(stream)), "goq_gemv")
+    wsb = 0 if ws is None else ws.nbytes
+    status = (_lib or lib()).goq_gemv(byref(d), _ptr(packed), _ptr(x_bf16), batch, _ptr(y), y_dtype, _ptr(ws), wsb, _stream(stream))
+    if status != OK:
+        raise GoqError(status, "goq_gemv")
 
 
 def gemv_static(d: Desc, packed, x_bf16, batch: int, y, y_dtype: int, stream=None):
     """goq_gemv_static: the decode GEMV with the library's built-in scratch array (no scratch argument).
     For callers that cannot allocate device memory; calls that may overlap on the GPU must not share it."""
-    _check(lib().goq_gemv_static(ctypes.byref(d), _ptr(packed), _ptr(x_bf16), batch, _ptr(y), y_dtype,
+    _check(lib().goq_gemv_static(byref(d), _ptr(packed), _ptr(x_bf16), batch, _ptr(y), y_dtype,
                                  _stream(stream)), "goq_gemv_static")
 
 
@@ -206,24 +236,24 @@ def quantize_activations(x, x_dtype: int, m: int, k: int, xq, sx, amax=None, abi
 
 
 def gemm_i8_requant(d: Desc, packed, x, m: int, sx, cq, sc, y, amax, yq=None, sy=None, stream=None):
-    _check(lib().goq_gemm_i8_requant(ctypes.byref(d), _ptr(packed), _ptr(x), m, _ptr(sx), _ptr(cq), _ptr(sc), _ptr(y),
+    _check(lib().goq_gemm_i8_requant(byref(d), _ptr(packed), _ptr(x), m, _ptr(sx), _ptr(cq), _ptr(sc), _ptr(y),
                                      _ptr(amax), _ptr(yq), _ptr(sy), _stream(stream)), "goq_gemm_i8_requant")
 
 
 def quantize_geo(d: Desc, w, codes, meta, coef_f16, stream=None):
-    _check(lib().goq_quantize_geo(ctypes.byref(d), _ptr(w), _ptr(codes), _ptr(meta), _ptr(coef_f16), _stream(stream)),
+    _check(lib().goq_quantize_geo(byref(d), _ptr(w), _ptr(codes), _ptr(meta), _ptr(coef_f16), _stream(stream)),
            "goq_quantize_geo")
 
 
 def solve_ref(d: Desc, w, codes, meta, x_calib, m: int, lam: float, coef_f16, c_f64=None, stream=None):
-    _check(lib().goq_solve_ref(ctypes.byref(d), _ptr(w), _ptr(codes), _ptr(meta), _ptr(x_calib), m, float(lam),
+    _check(lib().goq_solve_ref(byref(d), _ptr(w), _ptr(codes), _ptr(meta), _ptr(x_calib), m, float(lam),
                                _ptr(coef_f16), _ptr(c_f64), _stream(stream)), "goq_solve_ref")
 
 
 def gemv_static_status(stream=None) -> int:
     """goq_gemv_static_status: status word of the library's built-in scratch array (synchronises the stream)."""
     out = c_int(0)
-    _check(lib().goq_gemv_static_status(_stream(stream), ctypes.byref(out)), "goq_gemv_static_status")
+    _check(lib().goq_gemv_static_status(_stream(stream), byref(out)), "goq_gemv_static_status")
     return out.value
 
 
@@ -256,7 +286,7 @@ def sequence_order(seq):
 
 def gemv_sequence(seq, ws, stream=None):
     """goq_gemv_sequence: a chain of decode GEMVs in one persistent kernel. `seq` comes from make_sequence."""
-    _check(lib().goq_gemv_sequence(seq, len(seq), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)),
+    _check(lib().goq_gemv_sequence(seq, len(seq), _ptr(ws), ws.nbytes, _stream(stream)),
            "goq_gemv_sequence")
 
 
@@ -265,18 +295,18 @@ def gemv_sequence_host(seq, x_host, x_stage, y_host, y_stage, ws, stream=None):
     block out. x_host / y_host are (pinned) host tensors, x_stage / y_stage the device blocks the items point into."""
     xb, yb = x_stage.numel() * x_stage.element_size(), y_stage.numel() * y_stage.element_size()
     _check(lib().goq_gemv_sequence_host(seq, len(seq), _ptr(x_host), _ptr(x_stage), xb, _ptr(y_host), _ptr(y_stage), yb,
-                                        _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)),
+                                        _ptr(ws), ws.nbytes, _stream(stream)),
            "goq_gemv_sequence_host")
 
 
 def gemm(d: Desc, packed, x, m: int, x_dtype: int, y=None, y_dtype: int = F32, sx=None, cq=None, sc=None,
          acc=None, ws=None, stream=None):
-    wsb = 0 if ws is None else ws.numel() * ws.element_size()
-    _check(lib().goq_gemm(ctypes.byref(d), _ptr(packed), _ptr(x), m, x_dtype, _ptr(sx), _ptr(cq), _ptr(sc),
+    wsb = 0 if ws is None else ws.nbytes
+    _check(lib().goq_gemm(byref(d), _ptr(packed), _ptr(x), m, x_dtype, _ptr(sx), _ptr(cq), _ptr(sc),
                           _ptr(y), y_dtype, _ptr(acc), _ptr(ws), wsb, _stream(stream)), "goq_gemm")
 
 
 def gemv_host(d: Desc, packed, x_host, batch: int, y_host, y_dtype: int, x_stage, y_stage, ws=None, stream=None):
-    wsb = 0 if ws is None else ws.numel() * ws.element_size()
-    _check(lib().goq_gemv_host(ctypes.byref(d), _ptr(packed), _ptr(x_host), batch, _ptr(y_host), y_dtype,
+    wsb = 0 if ws is None else ws.nbytes
+    _check(lib().goq_gemv_host(byref(d), _ptr(packed), _ptr(x_host), batch, _ptr(y_host), y_dtype,
                                _ptr(x_stage), _ptr(y_stage), _ptr(ws), wsb, _stream(stream)), "goq_gemv_host")
