@@ -125,10 +125,10 @@ goq_status goq_unpack(const goq_desc* desc, const void* packed, uint8_t* codes_b
  *   ws       scratch of goq_workspace_bytes(desc, GOQ_OP_GEMV, batch) bytes, 256-byte aligned,
  *            initialised once with goq_workspace_init (may be NULL if the size is 0)
  * Each PoT term is applied to the activation as an exponent shift; sums are fp32. Up to 4 tokens
- * whose activations fit the chain kernel's staging buffer run as a one-linear goq_gemv_sequence
+ * whose activations fit the staging buffer in shared memory take goq_gemv_sequence's arithmetic
  * (integer operands: same rounding and saturation of non-finite activations as stated there);
  * the other cases take the bf16-operand streaming kernel.
- * Stream order: the streaming kernel starts fetching `packed` before earlier work on the stream has
+ * Stream order: the kernels start fetching `packed` before earlier work on the stream has
  * finished (programmatic dependent launch), so the packed weights must not be written by work that
  * is still in flight on the stream when the call is issued (synchronise after goq_pack, or put
  * other work in between). x and y follow plain stream order. */

@@ -84,7 +84,6 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
     if (op == GOQ_OP_GEMV && m <= 16) {
         size_t need = 0;
         if (goq::gemv_stream_supported(g)) need = goq::gemv_stream_workspace(g);
-        if (m <= 4 && goq::gemv_seq_supported(g, m) && goq::gemv_seq_workspace(1) > need) need = goq::gemv_seq_workspace(1);
         if (goq::gemm_mid_supported(g, m, true) && goq::gemm_mid_workspace(g, m, true) > need) need = goq::gemm_mid_workspace(g, m, true);
         return need;
     }
@@ -143,15 +142,10 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
         if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;
         if (!goq::stream_hash_is_bijective()) return GOQ_ERR_UNSUPPORTED;
-        // Up to 4 tokens whose activations fit the chain kernel's staging buffer: that kernel as a one-linear chain
-        // is the faster one. A refused cooperative launch falls through to the streaming kernel.
-        if (variant == 0 && batch <= 4 && goq::gemv_seq_supported(g, batch) && ws_bytes >= goq::gemv_seq_workspace(1)) {
-            goq::SeqCall c{g, packed, x_bf16, y, batch, y_dtype, 0};
-            if (goq::launch_gemv_seq(&c, 1, g.wbits, g.group, g.unit_bytes, ws, g_wait_limit.load(std::memory_order_relaxed),
-                                     (cudaStream_t)stream) == cudaSuccess)
-                return GOQ_OK;
-            (void)cudaGetLastError();
-        }
+        // Up to 4 tokens whose activations fit beside the ring: integer operands, a third of the decode's instructions
+        if (variant == 0 && goq::gemv_one_supported(g, batch))
+            return from_cuda(goq::launch_gemv_one(g, packed, x_bf16, batch, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed),
+                                                  (cudaStream_t)stream));
         return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
     }
     bool use_mma = goq::linear_mma_supported(g);

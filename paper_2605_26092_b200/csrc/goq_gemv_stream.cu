@@ -362,13 +362,16 @@ size_t gemv_stream_workspace(const Geometry& g) { return stream_ws_layout(g).tot
 size_t gemv_stream_zeroed_prefix(const Geometry& g) { return stream_ws_layout(g).counters_off + (size_t)g.n_tiles * 4; }
 
 bool stream_hash_is_bijective() {
-    bool seen[64] = {};
-    for (uint32_t meta = 0; meta < 64; ++meta) {
-        uint32_t s = record_slot(meta);
-        if (seen[s]) return false;
-        seen[s] = true;
-    }
-    return true;
+    static const bool ok = [] {
+        bool seen[64] = {};
+        for (uint32_t meta = 0; meta < 64; ++meta) {
+            uint32_t s = record_slot(meta);
+            if (seen[s]) return false;
+            seen[s] = true;
+        }
+        return true;
+    }();
+    return ok;
 }
 
 static int sm_count() {

@@ -71,6 +71,12 @@ size_t gemv_seq_zeroed_prefix(int n_items);
 cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, int unit_bytes, void* ws, int spin_limit,
                             cudaStream_t st);
 
+// One decode GEMV of at most 4 tokens with the chain kernel's arithmetic, as a programmatic dependent launch (goq_gemv_one.cu).
+// `ws` as for launch_gemv_stream (only the status word and the zero-kept counter area are used).
+bool gemv_one_supported(const Geometry& g, int m);
+cudaError_t launch_gemv_one(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
+                            int spin_limit, cudaStream_t st);
+
 // Prefill GEMM on tcgen05 tensor cores (wbits <= 3). `ws` holds gemm_tc_workspace(g, m) bytes: status word and
 // (split-K) tile counters in the common areas, then the per-token scales, the fp16 copy of the m x k_in activations
 // and the split-K partial tiles.

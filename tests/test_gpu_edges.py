@@ -128,3 +128,39 @@ def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
     assert np.array_equal(out[0], out[1])
     exact = m <= 32
     check_parity(out[0].astype(np.float64), y_ref, 2e-5 if exact else 5e-4, 1e-4 if exact else 2e-3)
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [(1, 32, 32, 3, 1), (16, 128, 128, 2, 4), (2368, 128, 128, 3, 3), (2369, 128, 64, 3, 1), (37888, 256, 32, 2, 2),
+                                       (16, 12288, 128, 3, 4), (129, 3200, 64, 3, 3), (4736, 4096, 128, 3, 1)])
+def test_single_decode_gemv_edges(goq, n, k, g, b, m):
+    """The single-linear integer-operand kernel: one record in all, one record an SM, a tile spread over all SMs, several tiles an SM,
+    ranges that need all or few of the k-blocks; back to back on one scratch buffer, whose counter area must stay zero, and equal
+    to the same linear in a chain bit for bit. Bound 2e-5 as for every fp32-accumulating kernel."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xs = [si.bf16_activations(m, k, seed=s) for s in range(3)]
+    ws = goq.new_workspace(d, goq.OP_GEMV, m)
+    ys = [torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda") for _ in xs]
+    xd = [dev(x) for x in xs]
+    for x, y in zip(xd, ys):
+        goq.gemv(d, packed, x, m, y, goq.F32, ws=ws)
+    torch.cuda.synchronize()
+    assert goq.workspace_status(ws) == goq.OK and not ws[256:256 + 65536].any()
+    rows = si.sample_rows(n, min(n, 200), seed=1)
+    for x, y in zip(xs, ys):
+        y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(x), g, b, rows=rows)
+        got = y.cpu().numpy().astype(np.float64)[:, rows]
+        if n > 1:
+            check_parity(got, y_ref, 2e-5, 1e-4)
+        else:
+            # One output has no norm over channels to average in, and it may be small by cancellation. An activation is rounded at
+            # half of 2^-14 of the largest of its block, so the output is off by at most 2^-15 max|x| sum |w_hat|.
+            w = np.abs(O.decode_b1(codes, b) * np.repeat(coef[..., 0].astype(np.float64), g, 1)
+                       + O.decode_b2(codes, meta, b) * np.repeat(coef[..., 1].astype(np.float64), g, 1)).sum()
+            assert np.abs(got - y_ref).max() <= 2.0 ** -15 * np.abs(si.bf16_bits_to_f64(x)).max() * w
+    seq_ws = torch.zeros(goq.sequence_workspace_bytes(1), dtype=torch.uint8, device="cuda")
+    yc = torch.empty((m, n), dtype=torch.float32, device="cuda")
+    goq.gemv_sequence(goq.make_sequence([(d, packed, xd[0], m, yc, goq.F32, False)]), seq_ws)
+    torch.cuda.synchronize()
+    assert torch.equal(yc, ys[0])
