@@ -124,10 +124,9 @@ goq_status goq_unpack(const goq_desc* desc, const void* packed, uint8_t* codes_b
  *   y        out [batch][n_out], y_dtype GOQ_BF16 or GOQ_F32
  *   ws       scratch of goq_workspace_bytes(desc, GOQ_OP_GEMV, batch) bytes, 256-byte aligned,
  *            initialised once with goq_workspace_init (may be NULL if the size is 0)
- * Each PoT term is applied to the activation as an exponent shift; sums are fp32. Up to 4 tokens
- * whose activations fit the staging buffer in shared memory take goq_gemv_sequence's arithmetic
- * (integer operands: same rounding and saturation of non-finite activations as stated there);
- * the other cases take the bf16-operand streaming kernel.
+ * Each PoT term is applied to the activation as an exponent shift (a bf16 operand of the tensor core);
+ * sums are fp32. Large linears (W2, W3) at up to 4 tokens take goq_gemv_sequence's arithmetic
+ * (integer operands: same rounding and saturation of non-finite activations as stated there).
  * Stream order: the kernels start fetching `packed` before earlier work on the stream has
  * finished (programmatic dependent launch), so the packed weights must not be written by work that
  * is still in flight on the stream when the call is issued (synchronise after goq_pack, or put
@@ -303,8 +302,8 @@ goq_status goq_gemv_sequence_host(const goq_gemv_item* items, int n_items, const
 int goq_last_cuda_error(void);
 
 /* Force a kernel variant (benchmarks and tests only): 0 = automatic, 1 = scalar exponent-add
- * kernel, 2 = tensor-core fragment kernel, 3 = streaming tensor-core kernel, 4 = mid-batch tcgen05 kernel (in goq_gemv its
- * form with exact operands). Process-wide. Returns the previous value. */
+ * kernel, 2 = tensor-core fragment kernel, 3 = streaming tensor-core kernel, 4 = mid-batch tcgen05 kernel (goq_gemm),
+ * 5 = integer-operand kernel of one linear (goq_gemv). Process-wide. Returns the previous value. */
 int goq_set_gemv_variant(int variant);
 
 /* Bound, in polls, of every device-side wait of goq_gemv_sequence (tests only; 0 restores the kernel's own bound).

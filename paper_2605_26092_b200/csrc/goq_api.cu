@@ -84,7 +84,6 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
     if (op == GOQ_OP_GEMV && m <= 16) {
         size_t need = 0;
         if (goq::gemv_stream_supported(g)) need = goq::gemv_stream_workspace(g);
-        if (goq::gemm_mid_supported(g, m, true) && goq::gemm_mid_workspace(g, m, true) > need) need = goq::gemm_mid_workspace(g, m, true);
         return need;
     }
     if (op == GOQ_OP_GEMM) {
@@ -130,24 +129,24 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         return GOQ_ERR_ALIGNMENT;
     if (goq_status s = check_arch()) return s;
     const int variant = g_gemv_variant.load(std::memory_order_relaxed);
-    if (variant == 4) {
-        if (!goq::gemm_mid_supported(g, batch, true)) return GOQ_ERR_UNSUPPORTED;
-        if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
-        if (ws_bytes < goq::gemm_mid_workspace(g, batch, true)) return GOQ_ERR_WORKSPACE;
-        return from_cuda(goq::launch_gemm_mid(g, packed, x_bf16, batch, y, y_dtype, ws, true, (cudaStream_t)stream));
-    }
-    bool use_stream = goq::gemv_stream_supported(g) && (variant == 0 || variant == 3);
-    if (variant == 3 && !use_stream) return GOQ_ERR_UNSUPPORTED;
+    const bool use_stream = goq::gemv_stream_supported(g) && (variant == 0 || variant == 3 || variant == 5);
+    if ((variant == 3 || variant == 5) && !use_stream) return GOQ_ERR_UNSUPPORTED;
     if (use_stream) {
         if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
         if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;
         if (!goq::stream_hash_is_bijective()) return GOQ_ERR_UNSUPPORTED;
-        // Up to 4 tokens whose activations fit beside the ring: integer operands, a third of the decode's instructions
-        if (variant == 0 && goq::gemv_one_supported(g, batch))
+        // Up to 4 tokens on a large linear: integer operands, half the decode's instructions; below, the fragment kernel's shorter
+        // start and end count for more. Measured, us, integer / fragment, at 1 token: 4096 units (1024 x 8192) 5.2 / 4.9,
+        // 8192 (4096 x 4096) 6.1 / 6.3; at 4 tokens: 6.2 / 4.9, 7.3 / 6.3, 22016 (11008 x 4096) 13.2 / 15.4.
+        const bool one = goq::gemv_one_supported(g, batch) && (variant == 5 || (variant == 0 && g.n_units > (batch == 1 ? 6000u : 12000u)));
+        if (variant == 5 && !one) return GOQ_ERR_UNSUPPORTED;
+        if (one)
             return from_cuda(goq::launch_gemv_one(g, packed, x_bf16, batch, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed),
                                                   (cudaStream_t)stream));
-        return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
+        if (variant == 3) return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
     }
+    if (variant == 0 && goq::gemv_mma_supported(g, batch))
+        return from_cuda(goq::launch_gemv_mma(g, packed, x_bf16, batch, y, y_dtype, (cudaStream_t)stream));
     bool use_mma = goq::linear_mma_supported(g);
     if (variant == 1) use_mma = false;
     if (variant == 2 && !use_mma) return GOQ_ERR_UNSUPPORTED;
@@ -179,26 +178,23 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
             return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
         if (variant == 4) return GOQ_ERR_UNSUPPORTED;
-        // Few tokens (17..32): the streaming GEMV kernel, 16 tokens per launch (36 us each on 8192 x 8192, so 72 us at
-        // 32 tokens), against ~89 us for the tensor-core kernel with split-K, which takes over from 33 tokens.
-        if (m <= kGemmViaGemvMaxTokens && variant == 0 && goq::gemv_stream_supported(g)) {
-            if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
-            if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;
-            if (!goq::stream_hash_is_bijective()) return GOQ_ERR_UNSUPPORTED;
+        // What the mid-batch kernel does not take up to 32 tokens: the decode GEMV, 16 tokens per launch
+        if (m <= kGemmViaGemvMaxTokens && variant == 0 && goq::gemv_mma_supported(g, 16)) {
+            if (goq::gemv_stream_supported(g)) {
+                if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
+                if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;
+                if (!goq::stream_hash_is_bijective()) return GOQ_ERR_UNSUPPORTED;
+            }
             const size_t ybytes = (y_dtype == GOQ_F32) ? 4 : 2;
             for (int t0 = 0; t0 < m; t0 += 16) {
                 const int nb = (m - t0 < 16) ? (m - t0) : 16;
-                cudaError_t e = goq::launch_gemv_stream(g, packed, (const uint16_t*)x + (size_t)t0 * g.k_in, nb,
-                                                        (uint8_t*)y + (size_t)t0 * g.n_out * ybytes, y_dtype, ws,
-                                                        (cudaStream_t)stream);
+                cudaError_t e = goq::launch_gemv_mma(g, packed, (const uint16_t*)x + (size_t)t0 * g.k_in, nb,
+                                                     (uint8_t*)y + (size_t)t0 * g.n_out * ybytes, y_dtype, (cudaStream_t)stream);
                 if (e != cudaSuccess) return from_cuda(e);
             }
             return GOQ_OK;
         }
-        // W4 has no streaming GEMV: up to 32 tokens its mma.sync kernel is the faster one (41 us at 16 tokens on
-        // 8192 x 8192 against ~92 us for the tensor-core kernel), so the tensor-core kernel takes W4 from 33 tokens on
-        const bool w4_few = g.wbits == 4 && m <= kGemmViaGemvMaxTokens && variant == 0 && goq::linear_mma_supported(g);
-        if (goq::gemm_tc_supported(g) && variant != 2 && !w4_few) {
+        if (goq::gemm_tc_supported(g) && variant != 2) {
             if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
             if (ws_bytes < goq::gemm_tc_workspace(g, m)) return GOQ_ERR_WORKSPACE;
             return from_cuda(goq::launch_gemm_tc(g, packed, x, m, y, y_dtype, ws, (cudaStream_t)stream));

@@ -143,8 +143,12 @@ def test_single_decode_gemv_edges(goq, n, k, g, b, m):
     ws = goq.new_workspace(d, goq.OP_GEMV, m)
     ys = [torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda") for _ in xs]
     xd = [dev(x) for x in xs]
-    for x, y in zip(xd, ys):
-        goq.gemv(d, packed, x, m, y, goq.F32, ws=ws)
+    prev = goq.set_gemv_variant(5)
+    try:
+        for x, y in zip(xd, ys):
+            goq.gemv(d, packed, x, m, y, goq.F32, ws=ws)
+    finally:
+        goq.set_gemv_variant(prev)
     torch.cuda.synchronize()
     assert goq.workspace_status(ws) == goq.OK and not ws[256:256 + 65536].any()
     rows = si.sample_rows(n, min(n, 200), seed=1)
@@ -164,3 +168,20 @@ def test_single_decode_gemv_edges(goq, n, k, g, b, m):
     goq.gemv_sequence(goq.make_sequence([(d, packed, xd[0], m, yc, goq.F32, False)]), seq_ws)
     torch.cuda.synchronize()
     assert torch.equal(yc, ys[0])
+
+
+@pytest.mark.parametrize("b", [2, 3, 4])
+@pytest.mark.parametrize("n,k,g,m", [(1, 32, 32, 1), (17, 160, 32, 8), (256, 256, 64, 9), (40, 640, 128, 5), (33, 896, 128, 16), (16, 16384, 128, 16),
+                                     (600, 4096, 64, 3), (1200, 2080, 32, 12), (2400, 2048, 128, 7)])
+def test_fragment_gemv_edges(goq, n, k, g, m, b):
+    """The decode GEMV on bf16 fragments: rows and columns that end inside a record, fewer k-blocks than warps, one CTA per tile and
+    clusters of two to eight, odd batches; fp32 and bf16 outputs, twice, bit for bit. fp32 sums of exact products: 2e-5."""
+    from tests.gpu_util import check_bf16_output, check_parity, pack_weights, run_gemv
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m + b)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b)
+    y = run_gemv(d, packed, xb, goq.F32)
+    check_parity(y, y_ref, 2e-5, 1e-4)
+    assert np.array_equal(y, run_gemv(d, packed, xb, goq.F32))
+    check_bf16_output(run_gemv(d, packed, xb, goq.BF16), y_ref, 1e-4)
