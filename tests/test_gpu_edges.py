@@ -185,3 +185,35 @@ def test_fragment_gemv_edges(goq, n, k, g, m, b):
     check_parity(y, y_ref, 2e-5, 1e-4)
     assert np.array_equal(y, run_gemv(d, packed, xb, goq.F32))
     check_bf16_output(run_gemv(d, packed, xb, goq.BF16), y_ref, 1e-4)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("m,k,abits", [(1, 1, 8), (9, 4, 8), (3, 1024, 8), (17, 1028, 8), (2, 5000, 4), (5, 4096, 2), (3, 4100, 6), (4, 771, 8)])
+def test_activation_quantizer_edges(goq, m, k, abits, dtype):
+    """Rows of every path (a warp, a CTA, more than the registers hold, not a multiple of four), quotients on and next to the halves
+    where the fp32 estimate cannot decide, the largest and smallest scales: integers and scales equal to the oracle's."""
+    rng = np.random.default_rng(m * k + abits)
+    qmax = 2 ** (abits - 1) - 1
+    x = rng.standard_normal((m, k)).astype(np.float32)
+    for r in range(m):
+        top = np.float32([3.0, 1.7e-30, 2.9e38, 1e-39, 0.3333][r % 5])
+        half = (rng.integers(0, 2 * qmax, size=k) - qmax + 0.5) * (np.float64(top) / qmax)
+        half = half.astype(np.float32)
+        step = rng.integers(-2, 3, size=k)
+        half = np.where(step > 0, np.nextafter(half, np.float32(np.inf)), np.where(step < 0, np.nextafter(half, np.float32(-np.inf)), half))
+        x[r] = np.clip(np.where(rng.random(k) < 0.7, half, x[r] * top / 5), -top, top)
+        x[r, r % k] = top
+    if dtype == "bf16":
+        bits = si.f32_to_bf16_bits(x)
+        x = si.bf16_bits_to_f64(bits).astype(np.float32)
+        xd, code = torch.from_numpy(bits.view(np.int16)).cuda(), goq.BF16
+    else:
+        xd, code = torch.from_numpy(x).cuda(), goq.F32
+    xq_ref, sx_ref = O.quantize_activations_int(x, abits)
+    for amax in (None, torch.from_numpy(np.abs(x).max(axis=1)).cuda()):
+        xq = torch.full((m, k), 99, dtype=torch.int8, device="cuda")
+        sx = torch.zeros(m, dtype=torch.float32, device="cuda")
+        goq.quantize_activations(xd, code, m, k, xq, sx, amax=amax, abits=abits)
+        torch.cuda.synchronize()
+        assert np.array_equal(xq.cpu().numpy(), xq_ref)
+        assert np.array_equal(sx.cpu().numpy(), sx_ref)
