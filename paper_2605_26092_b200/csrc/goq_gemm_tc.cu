@@ -473,6 +473,18 @@ cudaError_t encode_x_map(CUtensorMap* map, void* xh, int k_in, int m, int rows) 
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;   // distinct code: the tensor map could not be encoded
 }
+// int8 activations [m][k_in] as boxes of 128 k x `rows` tokens, 128-byte swizzle
+cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int rows) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)k_in, (cuuint64_t)m};
+    const cuuint64_t strides[1] = {(cuuint64_t)k_in};
+    const cuuint32_t box[2] = {128, (cuuint32_t)rows};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
+}
 bool packed_map_supported(const Geometry& g) {
     return g.unit_bytes / 8 <= 256 && (unsigned long long)g.k_blocks * g.unit_bytes / 8 < (1ull << 31);
 }
