@@ -391,6 +391,7 @@ gemm_a8_mma_kernel(const uint8_t* __restrict__ packed, int unit_bytes, const int
 cudaError_t launch_gemm_a8(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx,
                            const int8_t* cq, const float* sc, void* y, int y_dtype, int32_t* acc, float* amax, cudaStream_t st) {
     auto* words = (const uint8_t*)packed;
+    if (gemm_i8tc_supported(g, m)) return launch_gemm_i8tc(g, packed, x, m, sx, cq, sc, y, y_dtype, acc, amax, nullptr, st);
     if (g.group >= 32 && g.wbits <= 3) {
         dim3 grid2((g.n_tiles + kA8Warps - 1) / kA8Warps, (m + kA8Tok - 1) / kA8Tok), block2(kA8Warps * 32);
 #define GOQ_A8_LAUNCH(WB_, CPG_)                                                                                          \

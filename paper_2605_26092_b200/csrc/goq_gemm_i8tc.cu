@@ -3,7 +3,7 @@
 //   ACC_b[m,n] = sum_j c~_b[n,j] sum_{k in j} x~[m,k] v_b[n,k],   v_b = 2^emax b_b in {0, +-1, .. +-2^emax}
 //
 // The coefficient changes every macro-block while a tensor-core accumulator does not, so it goes into the operand: c~ v needs 11 bits
-// (W3), two int8 digits: c~ v = B h + l, B = 16 (W2, W3) or 128 (W4), ACC = B sum x h + sum x l. All integers, summed modulo 2^32;
+// (W3), two int8 digits: c~ v = B h + l, B = 16 (W2, W3) or 192 (W4), ACC = B sum x h + sum x l. All integers, summed modulo 2^32;
 // the result is below 2^31 by the host's bound, so it is the same bits in any order. Four digit planes (two bases x two digits) of
 // 64 channels make one N = 256 operand; a CTA's tile is 128 tokens x 128 channels, its four accumulators all of tensor memory.
 // Against per-macro-block sums on mma.sync (goq_gemm_a8.cu) this doubles the multiply-adds and takes the coefficient stage, eight
@@ -12,13 +12,14 @@
 // Digits come from byte tables: 256 entries, one per value of c~, of the digits of c~ v for every code, looked up per row and
 // macro-block (16 bytes: h and l of eight codes); a weight is then two byte permutes. b2 = the same lookup routed by the exchange
 // record; its pair signs negate bytes. For B = 16 both digits are chosen non-zero, so a byte's negation is (~q) + 1 without a
-// carry into the next byte; for B = 128 the addition masks the top bits.
+// carry into the next byte; for B = 192 the addition masks the top bits.
 //
-// Roles (27 warps, persistent CTAs): 0-7 epilogue (a thread is a token: ACC or y, four channels a store), 8 packed records (one 2-D TMA
-// copy per 128 channels x 128 k), 9 activation tiles (TMA), 10 MMA issue, 11-26 decode, warp (e, v) rows 8 v .. of record e of every
-// k-block. Bound: shared-memory bandwidth (operand reads of the MMAs, digit stores, table lookups).
-// Every mbarrier wait is bounded; there is no scratch and hence no status word on this path: a CTA that gives up leaves its outputs
-// unwritten.
+// Roles (27 warps, persistent CTAs): 0-7 epilogue (a thread is a token: ACC or y, eight channels a store), 8 packed records (one 2-D TMA
+// copy per 64 channels x 128 k), 9 activation tiles (TMA), 10 MMA issue, 11-26 decode: two groups of eight alternate k-blocks, warp (e, v)
+// of a group takes rows 8 v .. of record e. Bound: shared-memory bandwidth (per 64 x 256 x 128: operand reads of the MMAs ~770 clocks, digit
+// stores, lookups and copies ~900). With 128 x 128 tiles the second part was twice that and the kernel ran at its sum (98 %).
+// Every mbarrier wait is bounded; a CTA that gives up leaves its outputs unwritten and reports GOQ_ERR_TIMEOUT where it is given a
+// status word.
 #include "goq_tc_core.cuh"
 #include "goq_internal.h"
 
@@ -29,8 +30,8 @@ using namespace tc;
 
 constexpr int kEpiWarps = 8, kPkWarp = 8, kXWarp = 9, kMmaWarp = 10, kDec0 = 11, kDecWarps = 16;
 constexpr int kThreads = (kDec0 + kDecWarps) * 32;
-constexpr int kTokens = 128, kChannels = 128, kStages = 2, kMaxPk = 3;
-constexpr int kABytes = kTokens * 128, kBHalf = 256 * 128, kBBytes = 2 * kBHalf, kStageBytes = kABytes + kBBytes;
+constexpr int kTokens = 128, kChannels = 64, kStages = 3, kMaxPk = 4;
+constexpr int kABytes = kTokens * 128, kBBytes = 256 * 128, kStageBytes = kBBytes + 2 * kABytes;
 constexpr int kLut8Bytes = 64 * 16 * 8;   // record table: 8-byte entries, 16 copies
 
 struct Params {
@@ -40,7 +41,9 @@ struct Params {
     void* y;
     int32_t* acc;
     float* amax;
+    int* status;
     int unit_bytes, meta_off, k_blocks, groups_in, n_out, m, y_dtype, tiles_x, tiles, n_pk;
+    int tt;   // M = 128 operands per tile: 1 or 2
 };
 
 // kind::i8: s8 x s8 -> s32, both K-major, M = 128, N = 256
@@ -60,6 +63,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
 }
+// 32 bytes a thread: a whole sector, and half the address-divergent requests of two 16-byte stores
+__device__ __forceinline__ void st_global_v8(float* d, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(d), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]),
+                 "f"(v[6]), "f"(v[7]) : "memory");
+}
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
     uint2 v;
     asm("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
@@ -69,7 +77,8 @@ __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
     asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
-template <int WB> struct Digits { static constexpr int base_log2 = WB == 4 ? 7 : 4, entry = WB == 4 ? 32 : 16; };
+// W4: |c~ v| <= 2^14 = 85.3 * 192, and |l| <= 96: both digits and their negatives are int8 for every c~, -128 included
+template <int WB> struct Digits { static constexpr int base = WB == 4 ? 192 : 16, entry = WB == 4 ? 32 : 16; };
 // integer of code c (W4: sign << 3 | e): +-2^(emax - e)
 template <int WB>
 __device__ __forceinline__ int code_int(int c) {
@@ -80,8 +89,8 @@ __device__ __forceinline__ int code_int(int c) {
 }
 template <int WB>
 __device__ __forceinline__ void split_digits(int v, int& h, int& l) {
-    constexpr int B = 1 << Digits<WB>::base_log2;
-    h = (v + B / 2) >> Digits<WB>::base_log2;
+    constexpr int B = Digits<WB>::base;
+    h = (v + B / 2 + 256 * B) / B - 256;   // floor
     l = v - B * h;
     if constexpr (WB <= 3) {   // both non-zero
         if (l == 0) { h += 1; l = -B; }
@@ -101,9 +110,9 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     unsigned char* lut = stages + kStages * kStageBytes;
     unsigned char* ctab = lut + kLut8Bytes;                              // [c~ as a byte][h of 8 codes, l of 8 codes (W4: +, - of each)]
     unsigned char* pk_ring = ctab + 256 * Digits<WB>::entry;
-    const int pk_bytes = 8 * p.unit_bytes;
-    __shared__ uint64_t full[kStages], empty[kStages], pk_full[kMaxPk], pk_empty[kMaxPk], tm_full, tm_empty[2];
-    __shared__ float2 sc_s[2][kChannels];   // per-channel scales of the current tile and the next
+    const int pk_bytes = 4 * p.unit_bytes;
+    __shared__ uint64_t full[kStages], empty[kStages], pk_full[kMaxPk], pk_empty[kMaxPk], tm_full[2], tm_empty[2];
+    __shared__ float2 sc_s[2][2][kChannels];   // per-channel scales of the current tile and the next, a copy per token half
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
 
@@ -114,21 +123,20 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     struct { int tile, kb, slot, round, issued; } pk = {(int)blockIdx.x, 0, 0, 0, 0};
     auto pk_issue = [&]() {
         mbar_expect_tx(&pk_full[pk.slot], (uint32_t)pk_bytes);   // (rows past the last tile arrive as zeros)
-        tma_load_2d(pk_ring + pk.slot * pk_bytes, &packed_map, pk.kb * (p.unit_bytes >> 3), (pk.tile % p.tiles_x) * 8, &pk_full[pk.slot]);
+        tma_load_2d(pk_ring + pk.slot * pk_bytes, &packed_map, pk.kb * (p.unit_bytes >> 3), (pk.tile % p.tiles_x) * 4, &pk_full[pk.slot]);
         if (++pk.kb == p.k_blocks) { pk.kb = 0; pk.tile += (int)gridDim.x; }
         ++pk.issued;
         if (++pk.slot == p.n_pk) { pk.slot = 0; ++pk.round; }
     };
     if (warp == kPkWarp && lane == 0) {
-        for (int i = 0; i < kMaxPk; ++i) { mbar_init(&pk_full[i], 1); mbar_init(&pk_empty[i], kDecWarps); }
+        for (int i = 0; i < kMaxPk; ++i) { mbar_init(&pk_full[i], 1); mbar_init(&pk_empty[i], 8); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         while (pk.issued < units && pk.round == 0) pk_issue();
     }
     if (tid == 0) {
         abort_flag = 0;
-        for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], kDecWarps + 1); mbar_init(&empty[i], 1); }
-        mbar_init(&tm_full, 1);
-        for (int i = 0; i < 2; ++i) mbar_init(&tm_empty[i], kEpiWarps / 2);
+        for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 8 + 1); mbar_init(&empty[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&tm_full[i], 1); mbar_init(&tm_empty[i], kEpiWarps / 2); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // record table: byte selector of b2's first half (the second half's is this XOR 0x4444) and the flips of both halves, bit 7 and bit 6
@@ -181,49 +189,50 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
                     const int s = u % kStages;
                     if (u >= kStages) ok = mbar_wait(&empty[s], ((u / kStages) - 1) & 1, &abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(&full[s], (uint32_t)kABytes);
-                    tma_load_2d(stages + s * kStageBytes, &x_map, kb * kBlockK, (tile / p.tiles_x) * kTokens, &full[s]);
+                    mbar_expect_tx(&full[s], (uint32_t)(p.tt * kABytes));
+                    for (int i = 0; i < p.tt; ++i)
+                        tma_load_2d(stages + s * kStageBytes + kBBytes + i * kABytes, &x_map, kb * kBlockK, ((tile / p.tiles_x) * p.tt + i) * kTokens, &full[s]);
                 }
             if (!ok || abort_flag)   // as in the mid-batch kernel: a millisecond, which no copy takes
                 for (int i = 0; i < 1000; ++i) __nanosleep(1000);
         }
     } else if (warp == kMmaWarp) {
-        const uint64_t adesc0 = smem_desc_sw128(s32(stages)), bdesc0 = smem_desc_sw128(s32(stages + kABytes));
+        const uint64_t bdesc0 = smem_desc_sw128(s32(stages)), adesc0 = smem_desc_sw128(s32(stages + kBBytes));
         const bool leader = elect_one();
         bool ok = true, ready = false;
-        int u = 0;
+        int s = 0;
+        uint32_t par = 0;
         for (int i = 0; i < my_tiles && ok; ++i) {
-            for (int kb = 0; kb < p.k_blocks; ++kb, ++u) {
-                const int s = u % kStages;
-                if (!ready) ok = mbar_wait(&full[s], (u / kStages) & 1, &abort_flag);
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!ready) ok = mbar_wait(&full[s], par, &abort_flag);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                ready = mbar_test(&full[(u + 1) % kStages], ((u + 1) / kStages) & 1);
+                const int s_next = s + 1 == kStages ? 0 : s + 1;
+                const uint32_t par_next = s_next == 0 ? par ^ 1u : par;
+                ready = mbar_test(&full[s_next], par_next);
                 const uint64_t ad = adesc0 + (uint32_t)(s * (kStageBytes >> 4)), bd = bdesc0 + (uint32_t)(s * (kStageBytes >> 4));
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {   // 64 channels x 4 digit planes each
+                for (int h = 0; h < p.tt; ++h) {   // 128 tokens each
                     if (kb == 0 && i > 0) {
-                        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_empty[hf], (i - 1) & 1, &abort_flag));
+                        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_empty[h], (i - 1) & 1, &abort_flag));
                         if (!ok) break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     if (leader) {
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            umma_i8(tmem_base + hf * 256, ad + 2 * ks, bd + hf * (kBHalf >> 4) + 2 * ks, (kb > 0 || ks > 0) ? 1u : 0u);
+                            umma_i8(tmem_base + h * 256, ad + h * (kABytes >> 4) + 2 * ks, bd + 2 * ks, (kb > 0 || ks > 0) ? 1u : 0u);
+                        if (kb == p.k_blocks - 1) umma_commit(&tm_full[h]);
                     }
                 }
                 if (!ok) break;
-                if (leader) {
-                    umma_commit(&empty[s]);
-                    if (kb == p.k_blocks - 1) umma_commit(&tm_full);
-                }
+                if (leader) umma_commit(&empty[s]);
                 __syncwarp();
+                s = s_next; par = par_next;
             }
         }
     } else if (warp >= kDec0) {
         // ------------------------------ decode: packed records -> digit planes ------------------------------
-        const int e = (warp - kDec0) >> 1, v = (warp - kDec0) & 1, g = lane >> 2, t = lane & 3;
+        const int group = (warp - kDec0) >> 3, e = ((warp - kDec0) >> 1) & 3, v = (warp - kDec0) & 1, g = lane >> 2, t = lane & 3;
         const uint32_t lut_lane = s32(lut) + (uint32_t)(lane & 15) * 8, ctab_a = s32(ctab);
         // Row r of a plane: 128 bytes, 16-byte piece j at j ^ (r & 7). Odd rows take their words in the order c ^ 2: the four rows of a
         // half warp's store then cover all eight pieces.
@@ -231,8 +240,10 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         uint32_t off[4];
 #pragma unroll
         for (int ci = 0; ci < 4; ++ci)
-            off[ci] = (uint32_t)(kABytes + (e >> 2) * kBHalf + ((e & 3) * 16 + v * 8 + g) * 128 + (((2 * (ci ^ flip) + (t >> 1)) ^ g) << 4) + (t & 1) * 8);
+            off[ci] = (uint32_t)((e * 16 + v * 8 + g) * 128 + (((2 * (ci ^ flip) + (t >> 1)) ^ g) << 4) + (t & 1) * 8);
         int tile = blockIdx.x, kb = 0;
+        auto step = [&]() { if (++kb == p.k_blocks) { kb = 0; tile += gridDim.x; } };
+        if (group) step();
         uint32_t next_c[GPB];
         auto fetch = [&]() {   // (c~_1, c~_2) of this lane's row, the k-block's macro-blocks; then step on
             const int row = (tile % p.tiles_x) * kChannels + e * 16 + v * 8 + g;
@@ -241,17 +252,17 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
                 const int j = kb * GPB + jj;
                 next_c[jj] = (row < p.n_out && j < p.groups_in) ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(p.cq) + (size_t)row * p.groups_in + j) : 0u;
             }
-            if (++kb == p.k_blocks) { kb = 0; tile += gridDim.x; }
+            step(); step();
         };
-        fetch();
+        if (group < units) fetch();
         bool ok = true;
-        int slot = 0;
-        uint32_t pk_par = 0;
-        for (int u = 0; u < units; ++u) {
+        int slot = group, s = group;   // n_pk >= 2
+        uint32_t pk_par = 0, st_par = 1;   // st_par: parity of the stage's previous release (the first round passes at once)
+        for (int u = group; u < units; u += 2) {
             uint32_t cc[GPB];
 #pragma unroll
             for (int jj = 0; jj < GPB; ++jj) cc[jj] = next_c[jj];
-            if (u + 1 < units) fetch();
+            if (u + 2 < units) fetch();
             ok = __all_sync(0xFFFFFFFFu, mbar_wait(&pk_full[slot], pk_par, &abort_flag));
             if (!ok) break;
             const uint32_t unit = after_wait(s32(pk_ring) + slot * pk_bytes + e * p.unit_bytes);
@@ -261,8 +272,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             const bool odd = flip != 0;
             const uint32_t w[4] = {odd ? wv.z : wv.x, odd ? wv.w : wv.y, odd ? wv.x : wv.z, odd ? wv.y : wv.w};
             if constexpr (WB == 4) mv = odd ? __funnelshift_l(mv, mv, 16) : mv;
-            const int s = u % kStages;
-            if (u >= kStages) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], ((u / kStages) - 1) & 1, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], st_par, &abort_flag));
             if (!ok) break;
             const uint32_t at = s32(stages) + (uint32_t)(s * kStageBytes);
 #pragma unroll
@@ -308,28 +318,32 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
             __syncwarp();
             if (lane == 0) { mbar_arrive(&full[s]); mbar_arrive(&pk_empty[slot]); }
-            if (++slot == p.n_pk) { slot = 0; pk_par ^= 1u; }
+            slot += 2;
+            if (slot >= p.n_pk) { slot -= p.n_pk; pk_par ^= 1u; }
+            s += 2;
+            if (s >= kStages) { s -= kStages; st_par ^= 1u; }
         }
     } else {
         // ------------------------------ epilogue: a thread is a token, a warp 32 tokens x 64 channels ------------------------------
-        const int quarter = warp & 3, hf = warp >> 2;
+        const int quarter = warp & 3, h2 = warp >> 2;
         constexpr float kInvScale = 1.0f / (float)(1u << ((1u << (WB - 1)) - 1u));
-        constexpr int kB = Digits<WB>::base_log2;
+        constexpr uint32_t kB = Digits<WB>::base;
         bool ok = true;
         int tile = blockIdx.x;
+        if (h2 < p.tt)
         for (int i = 0; i < my_tiles; ++i, tile += gridDim.x) {
-            const int ch0 = (tile % p.tiles_x) * kChannels + hf * 64, tok = (tile / p.tiles_x) * kTokens + quarter * 32 + lane;
-            float2* sc = sc_s[i & 1] + hf * 64;
-            // every warp of a channel half writes the same values; the previous tile's readers of this buffer are two tiles behind
+            const int ch0 = (tile % p.tiles_x) * kChannels, tok = ((tile / p.tiles_x) * p.tt + h2) * kTokens + quarter * 32 + lane;
+            float2* sc = sc_s[h2][i & 1];
+            // every warp of a token half writes the same values; the readers of this buffer's previous use are two tiles behind
             if (p.y) {
                 for (int c = lane; c < 64; c += 32) sc[c] = ch0 + c < p.n_out ? *reinterpret_cast<const float2*>(p.sc + (size_t)(ch0 + c) * 2) : make_float2(0.f, 0.f);
             }
             __syncwarp();
             const float sxk = (p.sx && tok < p.m ? p.sx[tok] : 1.f) * kInvScale;
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full, i & 1, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[h2], i & 1, &abort_flag));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + hf * 256;
+            const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + h2 * 256;
             const bool f32 = p.y_dtype == GOQ_F32;
             float vmax = 0.f;
 #pragma unroll 1
@@ -340,8 +354,8 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    a2[j] = (int)(((uint32_t)a1[j] << kB) + (uint32_t)a2[j]);
-                    a1[j] = (int)(((uint32_t)h[j] << kB) + (uint32_t)l[j]);
+                    a2[j] = (int)((uint32_t)a1[j] * kB + (uint32_t)a2[j]);
+                    a1[j] = (int)((uint32_t)h[j] * kB + (uint32_t)l[j]);
                 }
                 if (tok >= p.m || ch0 + c0 >= p.n_out) continue;
                 const size_t o = (size_t)tok * p.n_out + ch0 + c0;
@@ -370,9 +384,8 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
                     }
                     if (f32) {
                         float* d = reinterpret_cast<float*>(p.y) + o;
-                        if (all8 && (reinterpret_cast<uintptr_t>(p.y) & 15u) == 0) {
-                            *reinterpret_cast<float4*>(d) = make_float4(y[0], y[1], y[2], y[3]);
-                            *reinterpret_cast<float4*>(d + 4) = make_float4(y[4], y[5], y[6], y[7]);
+                        if (all8 && (reinterpret_cast<uintptr_t>(p.y) & 31u) == 0) {
+                            st_global_v8(d, y);
                         } else {
 #pragma unroll
                             for (int j = 0; j < 8; ++j) if (ch0 + c0 + j < p.n_out) d[j] = y[j];
@@ -390,7 +403,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tm_empty[hf]);
+            if (lane == 0) mbar_arrive(&tm_empty[h2]);
             // requantising epilogue (Section 3.5): the token's largest output magnitude; non-negative floats order like their bits
             if (p.amax && p.y && tok < p.m) atomicMax(reinterpret_cast<int*>(p.amax) + tok, __float_as_int(vmax));
         }
@@ -400,6 +413,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem_dealloc<512>(tmem_base);
     }
+    if (tid == 0 && abort_flag && p.status) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
 
 static int sm_count() {
@@ -412,7 +426,7 @@ static int sm_count() {
 }
 template <int WB, int GPB>
 static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& x_map, const CUtensorMap& packed_map, cudaStream_t st) {
-    const size_t fixed = 1024 + (size_t)kStages * kStageBytes + kLut8Bytes + 256 * Digits<WB>::entry, pk = (size_t)8 * g.unit_bytes;
+    const size_t fixed = 1024 + (size_t)kStages * kStageBytes + kLut8Bytes + 256 * Digits<WB>::entry, pk = (size_t)4 * g.unit_bytes;
     p.n_pk = (int)((224 * 1024 - fixed) / pk);
     if (p.n_pk > kMaxPk) p.n_pk = kMaxPk;
     const size_t smem = fixed + p.n_pk * pk;
@@ -436,16 +450,20 @@ static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& x_map
 bool gemm_i8tc_supported(const Geometry& g, int m) { return g.group >= 32 && g.k_in % 16 == 0 && tc::packed_map_supported(g) && m >= 1; }
 
 cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx, const int8_t* cq, const float* sc,
-                             void* y, int y_dtype, int32_t* acc, float* amax, cudaStream_t st) {
+                             void* y, int y_dtype, int32_t* acc, float* amax, int* status, cudaStream_t st) {
     CUtensorMap xm, pm;
     if (cudaError_t e = tc::encode_i8_map(&xm, x, g.k_in, m, i8tc::kTokens)) return e;
-    if (cudaError_t e = tc::encode_packed_map(&pm, packed, g)) return e;
+    if (cudaError_t e = tc::encode_packed_map(&pm, packed, g, 4)) return e;
     i8tc::Params p;
     p.packed = (const uint8_t*)packed; p.cq = cq; p.sx = sx; p.sc = sc; p.y = y; p.acc = acc; p.amax = amax;
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.k_blocks = g.k_blocks; p.groups_in = g.k_in / g.group; p.n_out = g.n_out;
     p.m = m; p.y_dtype = y_dtype;
     p.tiles_x = (g.n_pad + i8tc::kChannels - 1) / i8tc::kChannels;
-    p.tiles = p.tiles_x * ((m + i8tc::kTokens - 1) / i8tc::kTokens);
+    const int half_tiles = (m + i8tc::kTokens - 1) / i8tc::kTokens;
+    // 256 tokens a tile halve the decode; 128 where that would leave SMs without a tile
+    p.tt = p.tiles_x * ((half_tiles + 1) / 2) >= i8tc::sm_count() ? 2 : 1;
+    p.tiles = p.tiles_x * ((half_tiles + p.tt - 1) / p.tt);
+    p.status = status;
 #define GOQ_I8TC(WB_)                                                                                                       \
     (g.groups_per_block == 1 ? i8tc::launch<WB_, 1>(g, p, xm, pm, st) : g.groups_per_block == 2 ? i8tc::launch<WB_, 2>(g, p, xm, pm, st) \
                                                                                                : i8tc::launch<WB_, 4>(g, p, xm, pm, st))

@@ -463,7 +463,7 @@ static bool make_plan(const Geometry& g, int m, bool two, Plan* p) {
 template <int WB, bool TWO, int GL>
 static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, cudaStream_t st) {
     CUtensorMap map, pmap;
-    if (cudaError_t e = encode_packed_map(&pmap, packed, g)) return e;
+    if (cudaError_t e = encode_packed_map(&pmap, packed, g, 8)) return e;
     if (cudaError_t e = encode_x_map(&map, ws + pl.xh_off, g.k_in, m, pl.n_cols)) return e;
     Params p;
     p.packed = (const uint8_t*)packed;

@@ -245,9 +245,9 @@ __device__ __forceinline__ void fill_lut(unsigned char* lut, int tid, int n_thre
 // host side, defined in goq_gemm_tc.cu
 cudaError_t encode_x_map(CUtensorMap* map, void* xh, int k_in, int m, int rows);
 cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int rows);
-// packed records as boxes of one k-block x 8 row tiles (8-byte elements; rows past the end read as zeros)
+// packed records as boxes of one k-block x `row_tiles` row tiles (8-byte elements; rows past the end read as zeros)
 bool packed_map_supported(const Geometry& g);
-cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g);
+cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g, int row_tiles);
 cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st);
 
 }  // namespace tc
