@@ -149,8 +149,9 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
  *      acc  out, optional: [2][m][n_out] int32, ACC_b[m][n] = sum_j cq[n][j][b] * sum_{k in j} x[m][k] * (2^emax b_b[n][k])
  *      y    out, optional: [m][n_out] = sx[m] * 2^-emax * (sc[n][0]*ACC_1 + sc[n][1]*ACC_2)
  *    At least one of acc, y must be given. Returns GOQ_ERR_OVERFLOW_BOUND if k_in*127*127*2^emax >= 2^31 (W3: k_in up
- *    to 16642; W4, emax = 7: k_in up to 1040). wbits = 4 and groups of 16 run on the packed-dot-product kernel, wbits <= 3
- *    with groups of 32 or more on the int8 tensor-core kernel. */
+ *    to 16642; W4, emax = 7: k_in up to 1040). Groups of 16 run on the packed-dot-product kernel, larger ones on the int8
+ *    tensor cores. Needs no scratch; if ws is given, a give-up of a bounded wait is reported in its status word. Weights are
+ *    fetched early, as in goq_gemv. */
 goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int m, int x_dtype,
                     const float* sx, const int8_t* cq, const float* sc, void* y, int y_dtype,
                     int32_t* acc, void* ws, size_t ws_bytes, void* stream);

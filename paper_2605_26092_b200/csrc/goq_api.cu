@@ -221,7 +221,8 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         const long long bound = (long long)g.k_in * 127 * 127 * (1ll << ((1 << (g.wbits - 1)) - 1));
         if (bound >= (1ll << 31)) return GOQ_ERR_OVERFLOW_BOUND;
         if (goq_status s = check_arch()) return s;
-        return from_cuda(goq::launch_gemm_a8(g, packed, (const int8_t*)x, m, sx, cq, sc, y, y_dtype, acc, nullptr,
+        int* status = (ws && aligned(ws, 256) && ws_bytes >= goq::kWsStatusBytes) ? (int*)ws : nullptr;   // needs no scratch; reports there if it may
+        return from_cuda(goq::launch_gemm_a8(g, packed, (const int8_t*)x, m, sx, cq, sc, y, y_dtype, acc, nullptr, status,
                                              (cudaStream_t)stream));
     }
     return GOQ_ERR_INVALID_ARG;
@@ -241,7 +242,7 @@ goq_status goq_gemm_i8_requant(const goq_desc* desc, const void* packed, const i
     if (goq_status s = check_arch()) return s;
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaError_t e = cudaMemsetAsync(amax, 0, (size_t)m * sizeof(float), st)) return from_cuda(e);
-    if (cudaError_t e = goq::launch_gemm_a8(g, packed, x, m, sx, cq, sc, y, GOQ_F32, nullptr, amax, st)) return from_cuda(e);
+    if (cudaError_t e = goq::launch_gemm_a8(g, packed, x, m, sx, cq, sc, y, GOQ_F32, nullptr, amax, nullptr, st)) return from_cuda(e);
     if (yq) return from_cuda(goq::launch_quantize_act(y, GOQ_F32, m, g.n_out, 8, amax, yq, sy, st));
     return GOQ_OK;
 }

@@ -100,7 +100,8 @@ cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x
 // Integer-activation layer.
 // amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch).
 cudaError_t launch_gemm_a8(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx,
-                           const int8_t* cq, const float* sc, void* y, int y_dtype, int32_t* acc, float* amax, cudaStream_t st);
+                           const int8_t* cq, const float* sc, void* y, int y_dtype, int32_t* acc, float* amax, int* status,
+                           cudaStream_t st);
 
 // The same on tcgen05 (goq_gemm_i8tc.cu), group >= 32, any wbits.
 bool gemm_i8tc_supported(const Geometry& g, int m);

@@ -217,3 +217,36 @@ def test_activation_quantizer_edges(goq, m, k, abits, dtype):
         torch.cuda.synchronize()
         assert np.array_equal(xq.cpu().numpy(), xq_ref)
         assert np.array_equal(sx.cpu().numpy(), sx_ref)
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [(1, 32, 32, 3, 1), (16, 32, 32, 2, 127), (63, 96, 32, 4, 128), (64, 128, 64, 3, 129), (65, 192, 64, 4, 255),
+                                       (130, 320, 64, 2, 256), (200, 1024, 128, 3, 257), (72, 416, 32, 3, 300), (8, 1024, 128, 4, 700),
+                                       (4800, 128, 64, 3, 600), (192, 3072, 64, 3, 40000 // 64)])
+@pytest.mark.parametrize("out", ["f32", "bf16"])
+def test_int8_tensor_core_gemm_edges(goq, n, k, g, b, m, out):
+    """The int8 layer on the tensor cores: channel and token tiles that do not fill, one and two token halves a tile, fewer and more tiles
+    than SMs, every bit width and group, coefficients over the whole byte (-128 and 0 among them): accumulators bit-exact, outputs
+    those accumulators give in fp32 (2^-22 of the two terms' magnitudes), bf16 within its rounding."""
+    from tests.gpu_util import dev, pack_weights
+    rng = np.random.default_rng(n + k + m)
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    cq = rng.integers(-128, 128, size=(n, k // g, 2)).astype(np.int8)
+    cq[0, 0] = (-128, 0)
+    x = rng.integers(-127, 128, size=(m, k)).astype(np.int8)
+    x[m // 2] = 127
+    sx = rng.uniform(0.5, 2, size=m).astype(np.float32)
+    sc = rng.uniform(-1, 1, size=(n, 2)).astype(np.float32)
+    y = torch.zeros((m, n), dtype=torch.float32 if out == "f32" else torch.bfloat16, device="cuda")
+    acc = torch.zeros((2, m, n), dtype=torch.int32, device="cuda")
+    goq.gemm(d, packed, dev(x), m, goq.I8, y=y, y_dtype=goq.F32 if out == "f32" else goq.BF16, sx=dev(sx), cq=dev(cq), sc=dev(sc), acc=acc)
+    torch.cuda.synchronize()
+    rows = si.sample_rows(n, min(n, 256), seed=1)
+    a1, a2, _ = O.linear_i32(codes[rows], meta[rows], cq[rows], sc[rows], x, sx, g, b)
+    got = acc.cpu().numpy()
+    assert np.array_equal(got[0][:, rows], a1) and np.array_equal(got[1][:, rows], a2)
+    emax = (1 << (b - 1)) - 1
+    t = [sx[:, None].astype(np.float64) * 2.0 ** -emax * sc[rows, i].astype(np.float64) * a for i, a in enumerate((a1, a2))]
+    yh = y.float().cpu().numpy().astype(np.float64)[:, rows]
+    bound = 2.0 ** -21 * (np.abs(t[0]) + np.abs(t[1])) + (0.0 if out == "f32" else 2.0 ** -8 * np.abs(t[0] + t[1]))
+    assert np.all(np.abs(yh - t[0] - t[1]) <= bound)
