@@ -58,6 +58,8 @@ struct Item {
     int xsrc;                                // earlier item whose output this item's x lies in (read from that item's tagged copy), or -1
     unsigned int xoff;                       // first 64-bit word of x inside that copy
     int tag_out;                             // a later item reads this item's output: keep the tagged copy
+    int xid;                                 // items that read the same activations have the same number: staged once for all of them
+    int x_shared;                            // another item has this number too: stage every k-block, not just this CTA's
     unsigned int uq, ur;                     // units / G and units % G for the launch's G CTAs (the kernel never divides)
 };
 struct Params {
@@ -73,7 +75,7 @@ struct Params {
 
 constexpr int kPartWords = 128;              // 64-bit (value, tag) words of one posted part: 16 rows x 8 tokens
 constexpr int kTagWords = 4 * (kMaxKBlocks * kBlockK / 2);   // per item: four tokens of the widest input a linear can take
-constexpr int kXBatch = 3;                   // 16-byte activation chunks a lane holds while it polls their tags
+constexpr int kXBatch = 4;                   // 16-byte activation chunks a lane holds while it polls their tags
 
 template <int WB, int CPG, int NG, bool K1>
 __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_constant__ Params p) {
@@ -328,13 +330,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
     uint32_t phases = 0;              // bit 0: dependency barrier, bit 1: activation barrier, bit 2: buffer hand-shake, bit 3: activation buffer in use
     unsigned seq = 0;                 // tile parts this CTA has opened so far (same in every warp): indexes the reduction slots
     bool alive = true;
+    int staged = -1;                  // number of the activations in the buffer in use
 
     for (int i = 0; i < p.n_items && alive; ++i) {
         const Item& it = p.item[i];
         const Walk wk = make_walk(it, cta, p.g_magic);
         if (wk.L == 0) continue;   // nothing of this linear belongs to this CTA (the control warp reports it finished)
         const int kb = it.k_blocks, k_pad = kb * kBlockK, plane = k_pad + kXPad, m = it.m;
-        if (p.x_double) phases ^= 8u;
+        // q, k and v (gate and up) read the same activations: they are staged for the first of them and stay
+        const bool stage = it.xid != staged;
+        if (stage && p.x_double) phases ^= 8u;
         const int x_sel = (int)((phases >> 3) & 1u);
         unsigned char* xb = xq + (size_t)x_sel * p.xbuf_bytes;
         float* xsc = xscale + x_sel * (kMaxKBlocks * 4 * NG);
@@ -345,79 +350,76 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
         if (it.depends && i > 0) {
             if (!wait_a(dep_addr, phases & 1u, &abort_flag, spin)) { alive = false; break; }
             phases ^= 1u;
-        } else if (!p.x_double) {   // one buffer: every warp must have left the previous linear
+        } else if (stage && !p.x_double) {   // one buffer: every warp must have left the previous linear
             __syncwarp();
             if (lane == 0) arrive_a(free_addr);
             if (!wait_a(free_addr, (phases >> 2) & 1u, &abort_flag, spin)) { alive = false; break; }
             phases ^= 4u;
         }
-        {
-            // 16-byte chunks of 8 bf16; 16 chunks = one k-block of one token: Q = rne(x 2^s), the block's largest magnitude in [2^14, 2^15)
-            const int cpt = k_pad / 8, total = cpt * m;
-            auto convert = [&](const uint4 v, const bool in, const int r, const int k0) {
-                convert_chunk<WB>(v, in, xb + (size_t)(2 * r) * plane + k0, plane, xsc + (k0 >> 7) * (4 * NG) + r);
-            };
-            if (it.xsrc < 0) {   // activations from outside the chain, or ordered by the counter wait above
-                for (int c0 = warp * 32; c0 < total; c0 += kNW * 32) {
-                    const int c = c0 + lane;
-                    const bool in = c < total;
-                    const int r = in ? (int)mul_shift32((unsigned)c >> 4, it.kb_magic) : 0, k0 = in ? (c - r * cpt) * 8 : 0;   // cpt = 16 k_blocks
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (in && k0 < it.k_in) v = __ldcg(reinterpret_cast<const uint4*>(it.x + (size_t)r * it.k_in + k0));   // L2: written by other SMs
-                    convert(v, in, r, k0);
-                }
-            } else {
-                // Activations that an earlier linear of this launch produces: read from its tagged copy, word by word,
-                // until every word carries this launch's tag. That is the whole dependency wait: a chunk is converted as soon
-                // as the tiles it comes from are finished, wherever they were finished.
-                const unsigned tag = tag_s;
-                const uint2* tg = p.tags + (size_t)it.xsrc * kTagWords + it.xoff;
-                const int tstride = p.item[it.xsrc].n_tiles * 8;
-                const int bound = spin < kGlobalSpin ? spin : kGlobalSpin;
-                for (int cb = warp * 32; cb < total && alive; cb += kNW * 32 * kXBatch) {
-                    uint4 v[kXBatch];
-                    bool need[kXBatch];
+        if (stage) {
+            staged = it.xid;
+            // 16-byte chunks of 8 bf16; 16 chunks = one k-block of one token. A CTA whose range is shorter than a tile's row of records
+            // needs only that many k-blocks. Chunks go round the lanes token by token; kXBatch of them are fetched at a time.
+            const unsigned kb0 = it.x_shared ? 0u : wk.a - (unsigned)wk.Ta * (unsigned)kb;
+            const unsigned cw = (it.x_shared ? (unsigned)kb : min(wk.L, (unsigned)kb)) * 16u;   // chunks per token
+            unsigned r = 0, c = (unsigned)warp * 32u + (unsigned)lane;   // this lane's next chunk
+            auto settle = [&]() { while (r < (unsigned)m && c >= cw) { c -= cw; ++r; } };
+            settle();
+            const unsigned tag = tag_s;
+            const uint2* tg = it.xsrc < 0 ? nullptr : p.tags + (size_t)it.xsrc * kTagWords + it.xoff;
+            const unsigned tstride = it.xsrc < 0 ? 0u : (unsigned)p.item[it.xsrc].n_tiles * 8u;
+            const int bound = spin < kGlobalSpin ? spin : kGlobalSpin;
+            while (__any_sync(0xFFFFFFFFu, r < (unsigned)m)) {
+                uint4 v[kXBatch];
+                unsigned at[kXBatch], need = 0;   // token << 16 | first k; bit u: chunk u is still to be fetched
 #pragma unroll
-                    for (int u = 0; u < kXBatch; ++u) {
-                        const int c = cb + u * (kNW * 32) + lane;
-                        const int r = c < total ? (int)mul_shift32((unsigned)c >> 4, it.kb_magic) : 0, k0 = c < total ? (c - r * cpt) * 8 : 0;
-                        need[u] = c < total && k0 < it.k_in;
-                        v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    }
+                for (int u = 0; u < kXBatch; ++u) {
+                    unsigned kk = kb0 + (c >> 4);
+                    if (kk >= (unsigned)kb) kk -= (unsigned)kb;
+                    const unsigned k0 = kk * kBlockK + (c & 15u) * 8u;
+                    at[u] = r < (unsigned)m ? (r << 16) | k0 : 0xFFFFFFFFu;
+                    if (r < (unsigned)m && k0 < (unsigned)it.k_in) need |= 1u << u;
+                    v[u] = make_uint4(0u, 0u, 0u, 0u);
+                    c += kNW * 32u;
+                    settle();
+                }
+                if (it.xsrc < 0) {   // activations from outside the chain, or ordered by the counter wait above
+#pragma unroll
+                    for (int u = 0; u < kXBatch; ++u)
+                        if (need & (1u << u)) v[u] = __ldcg(reinterpret_cast<const uint4*>(it.x + (size_t)(at[u] >> 16) * it.k_in + (at[u] & 0xFFFFu)));   // L2: written by other SMs
+                } else {
+                    // Activations that an earlier linear of this launch produces: read from its tagged copy, word by word,
+                    // until every word carries this launch's tag. That is the whole dependency wait: a chunk is converted as soon
+                    // as the tiles it comes from are finished, wherever they were finished.
                     int spins = 0;
                     for (;;) {
-                        bool ok = true;
 #pragma unroll
                         for (int u = 0; u < kXBatch; ++u)
-                            if (need[u]) {
-                                const int c = cb + u * (kNW * 32) + lane;
-                                const int r = (int)mul_shift32((unsigned)c >> 4, it.kb_magic), k0 = (c - r * cpt) * 8;
-                                const uint2* src = tg + (size_t)r * tstride + (k0 >> 1);
+                            if (need & (1u << u)) {
+                                const uint2* src = tg + ((at[u] >> 16) * tstride + ((at[u] & 0xFFFFu) >> 1));
                                 unsigned long long w0, w1, w2, w3;
                                 asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(src) : "memory");
                                 asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w2), "=l"(w3) : "l"(src + 2) : "memory");
                                 if ((unsigned)(w0 >> 32) == tag && (unsigned)(w1 >> 32) == tag && (unsigned)(w2 >> 32) == tag && (unsigned)(w3 >> 32) == tag) {
                                     v[u] = make_uint4((unsigned)w0, (unsigned)w1, (unsigned)w2, (unsigned)w3);
-                                    need[u] = false;
-                                } else {
-                                    ok = false;
+                                    need &= ~(1u << u);
                                 }
                             }
-                        if (__all_sync(0xFFFFFFFFu, ok)) break;
+                        if (__all_sync(0xFFFFFFFFu, need == 0u)) break;
                         ++spins;
                         if (__any_sync(0xFFFFFFFFu, abort_flag != 0) || spins > bound) { abort_flag = 1; alive = false; break; }   // the whole warp or nobody
                     }
                     if (!alive) break;
-#pragma unroll
-                    for (int u = 0; u < kXBatch; ++u) {
-                        const int c = cb + u * (kNW * 32) + lane;
-                        const bool in = c < total;
-                        const int r = in ? (int)mul_shift32((unsigned)c >> 4, it.kb_magic) : 0, k0 = in ? (c - r * cpt) * 8 : 0;
-                        if (cb + u * (kNW * 32) < total) convert(v[u], in, r, k0);   // warp-uniform: the conversion shuffles
-                    }
                 }
-                if (!alive) break;
+#pragma unroll
+                for (int u = 0; u < kXBatch; ++u)
+                    if (__any_sync(0xFFFFFFFFu, at[u] != 0xFFFFFFFFu)) {   // warp-uniform: the conversion shuffles
+                        const unsigned rr = at[u] >> 16, k0 = at[u] & 0xFFFFu;
+                        const bool in = at[u] != 0xFFFFFFFFu;
+                        convert_chunk<WB>(v[u], in, xb + (size_t)(2u * rr) * plane + k0, plane, xsc + (k0 >> 7) * (4 * NG) + rr);
+                    }
             }
+            if (!alive) break;
             __syncwarp();
             if (lane == 0) arrive_a(xbar_addr);
             if (!wait_a(xbar_addr, (phases >> 1) & 1u, &abort_flag, spin)) { alive = false; break; }
@@ -762,6 +764,15 @@ cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, i
                 it.xoff = order[(size_t)j].word_offset;
                 p.item[it.xsrc].tag_out = 1;
             }
+        }
+    }
+    // Neighbouring items that read the same activations share their staging: same address, shape and source, no barrier between.
+    for (int j = 0; j < n; ++j) {
+        chain::Item &a = p.item[j], &b = p.item[j > 0 ? j - 1 : 0];
+        a.xid = j; a.x_shared = 0;
+        if (j > 0 && !a.depends && a.x == b.x && a.k_in == b.k_in && a.m == b.m && a.xsrc == b.xsrc && a.xoff == b.xoff) {
+            a.xid = b.xid;
+            a.x_shared = b.x_shared = 1;
         }
     }
     const int cpg = group / 32;

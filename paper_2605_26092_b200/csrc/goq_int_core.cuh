@@ -206,11 +206,11 @@ template <int WB>
 __device__ __forceinline__ void convert_chunk(const uint4 v, const bool in, unsigned char* hi, int plane, float* scale) {
     const int lane = threadIdx.x & 31;
     const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
-    uint32_t amax = 0;
+    // magnitudes order like their bit patterns: two at a time
+    uint32_t amax = __vmaxu2(__vmaxu2(in32[0] & 0x7FFF7FFFu, in32[1] & 0x7FFF7FFFu), __vmaxu2(in32[2] & 0x7FFF7FFFu, in32[3] & 0x7FFF7FFFu));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) amax = max(amax, max(in32[j] & 0x7FFFu, (in32[j] >> 16) & 0x7FFFu));
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
+    for (int o = 1; o < 16; o <<= 1) amax = __vmaxu2(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
+    amax = max(amax & 0xFFFFu, amax >> 16);
     int sfield = 268 - (int)(amax >> 7);
     sfield = sfield < 1 ? 1 : (sfield > 253 ? 253 : sfield);
     const float mult = __uint_as_float((uint32_t)sfield << 23);

@@ -250,3 +250,45 @@ def test_int8_tensor_core_gemm_edges(goq, n, k, g, b, m, out):
     yh = y.float().cpu().numpy().astype(np.float64)[:, rows]
     bound = 2.0 ** -21 * (np.abs(t[0]) + np.abs(t[1])) + (0.0 if out == "f32" else 2.0 ** -8 * np.abs(t[0] + t[1]))
     assert np.all(np.abs(yh - t[0] - t[1]) <= bound)
+
+
+@pytest.mark.parametrize("k,n,inner,m,g,b", [(256, 64, 512, 1, 64, 3), (1024, 256, 2816, 4, 128, 3), (128, 128, 256, 3, 32, 2), (4096, 1024, 11008, 4, 128, 3),
+                                             (2048, 2048, 4096, 7, 128, 3), (512, 128, 1408, 2, 128, 2)])
+def test_chain_shares_staged_activations(goq, k, n, inner, m, g, b):
+    """Two decoder layers as a chain: q, k, v read one input, gate and up another, so their activations are staged once; linears with
+    fewer records than SMs (CTAs that skip one of the sharers), ranges that need only some k-blocks, one and two activation
+    buffers. Every linear against the oracle on the bits it read (fp32 sums of rounded activations, bf16 out), three launches equal."""
+    from tests.gpu_util import check_bf16_output, dev, pack_weights
+    shapes = [(k, k), (n, k), (n, k), (k, k), (inner, k), (inner, k), (k, inner)]
+    x0 = si.bf16_activations(m, k, seed=5)
+    x = dev(x0)
+    items, layers, ys = [], [], []
+    for layer in range(2):
+        base = 7 * layer
+        reads = [base - 1] * 3 + [base + (2 if n == k else 0), base + 3, base + 3, base + 5]
+        for j, (no, ki) in enumerate(shapes):
+            codes, meta, coef = si.random_quantized(no, ki, g, b, seed=layer * 7 + j)
+            coef = (coef.astype(np.float64) * (1.5 / np.sqrt(ki)) / max(1e-9, np.std(coef.astype(np.float64)))).astype(np.float16)
+            d, packed = pack_weights(no, ki, g, b, codes, meta, coef)
+            y = torch.zeros((m, no), dtype=torch.bfloat16, device="cuda")
+            src = reads[j]
+            items.append((d, packed, x if src < 0 else ys[src], m, y, goq.BF16, False))
+            layers.append((codes, meta, coef, src))
+            ys.append(y)
+    seq = goq.make_sequence(items)
+    ws = torch.zeros(goq.sequence_workspace_bytes(len(items)), dtype=torch.uint8, device="cuda")
+    runs = []
+    for _ in range(3):
+        for y in ys:
+            y.zero_()
+        goq.gemv_sequence(seq, ws)
+        torch.cuda.synchronize()
+        assert goq.workspace_status(ws) == goq.OK
+        runs.append([y.view(torch.int16).cpu().numpy().view(np.uint16).copy() for y in ys])
+    for r in runs[1:]:
+        assert all(np.array_equal(a, c) for a, c in zip(runs[0], r))
+    for (codes, meta, coef, src), got in zip(layers, runs[0]):
+        xin = si.bf16_bits_to_f64(x0 if src < 0 else runs[0][src])
+        rows = si.sample_rows(codes.shape[0], min(codes.shape[0], 64), seed=2)
+        y_ref = O.linear_f64(codes, meta, coef, xin, g, b, rows=rows)
+        check_bf16_output(si.bf16_bits_to_f64(got)[:, rows], y_ref, 1e-4)
