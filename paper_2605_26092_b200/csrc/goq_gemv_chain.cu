@@ -75,6 +75,7 @@ struct Params {
 
 constexpr int kPartWords = 128;              // 64-bit (value, tag) words of one posted part: 16 rows x 8 tokens
 constexpr int kTagWords = 4 * (kMaxKBlocks * kBlockK / 2);   // per item: four tokens of the widest input a linear can take
+constexpr int kBelow = 4;                   // CTAs whose posted parts the control warp fetches at a time
 constexpr int kXBatch = 4;                   // 16-byte activation chunks a lane holds while it polls their tags
 
 template <int WB, int CPG, int NG, bool K1>
@@ -214,34 +215,55 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                     if (!whole && finisher) {
                         bool good = true;
                         unsigned bc = wk.a, remc = rem_a;   // upper boundary of CTA cc's range (= lower boundary of CTA cc + 1)
-                        for (int cc = cta - 1; cc >= 0 && bc > r_lo && good; --cc) {
-                            const unsigned borrow = remc < ur ? 1u : 0u;
-                            const unsigned ac = bc - uq - borrow;
-                            remc = remc - ur + (borrow ? (unsigned)G : 0u);
-                            if (ac != bc) {   // CTA cc has records of this tile; they are its first tile's if its range starts inside
-                                const uint2* pc = p.parts + (((size_t)i * G + cc) * 2 + (ac >= r_lo ? 0 : 1)) * kPartWords + lane;
-                                int spins = 0;
-                                for (;;) {
-                                    uint2 w[NG][2];
-                                    bool all = true;
+                        // up to kBelow CTAs' words in flight at a time (small linears: a tile may lie in many CTAs)
+                        for (int cc = cta - 1; cc >= 0 && bc > r_lo && good;) {
+                            const uint2* pc[kBelow];
+                            int np = 0;
 #pragma unroll
-                                    for (int cg = 0; cg < NG; ++cg)
-#pragma unroll
-                                        for (int hh = 0; hh < 2; ++hh) {
-                                            asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(w[cg][hh].x), "=r"(w[cg][hh].y)
-                                                         : "l"(pc + (cg * 2 + hh) * 32) : "memory");
-                                            all = all && w[cg][hh].y == tag;
-                                        }
-                                    if (__all_sync(0xFFFFFFFFu, all)) {
-#pragma unroll
-                                        for (int cg = 0; cg < NG; ++cg) { below[cg][0] += __uint_as_float(w[cg][0].x); below[cg][1] += __uint_as_float(w[cg][1].x); }
-                                        break;
-                                    }
-                                    ++spins;
-                                    if (__any_sync(0xFFFFFFFFu, abort_flag != 0) || spins > kGlobalSpin || spins > spin) { abort_flag = 1; good = false; break; }
+                            for (int u = 0; u < kBelow; ++u) {
+                                pc[u] = nullptr;
+                                while (cc >= 0 && bc > r_lo) {   // next CTA below that has records of this tile; they are its first tile's if its range starts inside
+                                    const unsigned borrow = remc < ur ? 1u : 0u;
+                                    const unsigned ac = bc - uq - borrow;
+                                    remc = remc - ur + (borrow ? (unsigned)G : 0u);
+                                    const bool has = ac != bc;
+                                    if (has) pc[u] = p.parts + (((size_t)i * G + cc) * 2 + (ac >= r_lo ? 0 : 1)) * kPartWords + lane;
+                                    bc = ac;
+                                    --cc;
+                                    if (has) { np = u + 1; break; }
                                 }
                             }
-                            bc = ac;
+                            uint2 w[kBelow][NG][2];
+                            int spins = 0;
+                            for (;;) {
+                                bool all = true;
+#pragma unroll
+                                for (int u = 0; u < kBelow; ++u)
+                                    if (u < np) {
+#pragma unroll
+                                        for (int cg = 0; cg < NG; ++cg)
+#pragma unroll
+                                            for (int hh = 0; hh < 2; ++hh)
+                                                asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(w[u][cg][hh].x), "=r"(w[u][cg][hh].y)
+                                                             : "l"(pc[u] + (cg * 2 + hh) * 32) : "memory");
+                                    }
+#pragma unroll
+                                for (int u = 0; u < kBelow; ++u)
+                                    if (u < np) {
+#pragma unroll
+                                        for (int cg = 0; cg < NG; ++cg) all = all && w[u][cg][0].y == tag && w[u][cg][1].y == tag;
+                                    }
+                                if (__all_sync(0xFFFFFFFFu, all)) break;
+                                ++spins;
+                                if (__any_sync(0xFFFFFFFFu, abort_flag != 0) || spins > kGlobalSpin || spins > spin) { abort_flag = 1; good = false; break; }
+                            }
+                            if (!good) break;
+#pragma unroll
+                            for (int u = 0; u < kBelow; ++u)   // nearest CTA first: a fixed order
+                                if (u < np) {
+#pragma unroll
+                                    for (int cg = 0; cg < NG; ++cg) { below[cg][0] += __uint_as_float(w[u][cg][0].x); below[cg][1] += __uint_as_float(w[u][cg][1].x); }
+                                }
                         }
                         if (!good) { ok = false; break; }
                     }
@@ -300,11 +322,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                 if (!ok) break;
                 seq += (unsigned)wk.P;
             }
-            // this CTA has finished linear i: the warp's stores are ordered before lane 0's fetch-add, which releases them
+            // this CTA has finished linear i: the warp's stores are ordered before lane 0's fetch-add, which releases them. Only where the
+            // next linear waits for the counter (a release costs the warp the round trip of all its stores).
             __syncwarp();
             if (lane == 0) {
                 if (i < p.n_items - 1) {
-                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&p.done[i]) : "memory");
+                    if (p.item[i + 1].depends) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&p.done[i]) : "memory");
                 } else {   // the CTA that completes the last linear last leaves the counters zero for the next call
                     const int prev = atomic_add_acq_rel_gpu(&p.done[i], 1);
                     if (prev == G - 1) {
