@@ -6,10 +6,9 @@
 //
 // Work split. A unit is 128 output channels x one 128-wide k-block (eight unit records). The units of a call are numbered
 // token tile by token tile, channel tile by channel tile, k-block by k-block; CTA c of G takes [U c / G, U (c+1) / G): equal
-// work for every SM whatever the shape (8192 x 8192: 4096 units on 148 SMs). A channel tile shared by several CTAs is finished
-// by the one that arrives last: every CTA parks its fp32 partial tile, and the last one adds the parts in CTA order
-// (deterministic) and stores. A range's last tile is the one whose other parts are long parked, so the sum is made after the
-// CTA's own work by all of its threads.
+// work for every SM whatever the shape (8192 x 8192: 4096 units on 148 SMs). Every CTA parks its fp32 part of a channel tile that it
+// shares with others; a small second kernel adds the parts in CTA order (deterministic). A range's last part is drained by all
+// warps.
 //
 // Roles (23 warps). Warps 0-3: coefficient scales ahead of each tile, then the epilogue (tensor memory -> y or the parked part).
 // Warp 4: packed records into a ring (one 2-D TMA copy per unit). Warp 5: activation tiles (2-D TMA, 128-byte swizzle). Warp 6:
@@ -44,7 +43,6 @@ struct Params {
     void* y;
     const float* inv_scale;   // [m] 2^-s of each token
     int* status;
-    int* counters;            // [tile][4 channel quarters], zero on entry, left zero
     float* partial;           // [CTA][2][n_cols][128]
     int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m, y_dtype, group_log2, gpb;
     int n_cols;               // tokens per tile (MMA N): a multiple of 16, at most 256
@@ -108,7 +106,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
     __shared__ uint32_t row_max[kTileN];    // (start) largest |c| of the first part's channels, as fp16 bits
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
-    __shared__ SharedTile fin[2];
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     const int G = gridDim.x, cta = blockIdx.x;
@@ -228,8 +225,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         // The whole warp runs the loop and one elected lane issues: descriptors stay in uniform registers. A wait that succeeds
         // still takes a trip through the (busy) shared-memory pipe, ~250 clocks, so the next stage is probed before this one's
         // MMAs are issued.
-        describe_shared(fin, lane, u0, u1, p.units, p.k_blocks, G);   // (there is time before the first stage)
-        __syncwarp();
         const uint32_t idesc = idesc_f16((uint32_t)p.n_cols), acc_step = 256u / (uint32_t)p.na;
         const uint64_t adesc0 = smem_desc_sw128(s32(a_tiles)), bdesc0 = smem_desc_sw128(s32(b_tiles));
         const bool leader = elect_one();
@@ -413,11 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem_dealloc<kTmemCols>(tmem_base);
     }
-    if (abort_flag) {
-        if (tid == 0) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
-        return;
-    }
-    finish_shared<kThreads>(fin, p.partial, park_floats, p.counters, p.tiles_x, p.n_cols, p.m, p.inv_scale, out);
+    if (tid == 0 && abort_flag) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
 
 // ---- host side ------------------------------------------------------------------------------------
@@ -441,7 +432,7 @@ static bool make_plan(const Geometry& g, int m, bool two, Plan* p) {
     p->n_cols = ((m + p->t_tiles - 1) / p->t_tiles + 15) & ~15;   // equal token tiles
     p->tiles_x = (g.n_pad + kTileN - 1) / kTileN;
     const long long units = (long long)p->t_tiles * p->tiles_x * g.k_blocks;
-    if (units >= (1ll << 30) || (size_t)p->t_tiles * p->tiles_x * 4 * sizeof(int) > kWsCounterBytes) return false;
+    if (units >= (1ll << 30)) return false;
     p->units = (int)units;
     p->grid = (int)(units < sm_count() ? units : sm_count());
     // rings: up to six k-blocks of packed records, then as many operand stages as fit (at least three)
@@ -470,7 +461,6 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     p.y = y;
     p.inv_scale = (const float*)(ws + pl.inv_off);
     p.status = (int*)ws;
-    p.counters = (int*)(ws + kWsStatusBytes);
     p.partial = (float*)(ws + pl.partial_off);
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.k_blocks = g.k_blocks; p.n_tiles = g.n_tiles; p.n_out = g.n_out;
     p.m = m; p.y_dtype = y_dtype; p.gpb = g.groups_per_block;
@@ -494,7 +484,13 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_mid_kernel<WB, TWO, GL>, p, map, pmap);
+    if (cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_mid_kernel<WB, TWO, GL>, p, map, pmap)) return e;
+    if (p.units % pl.grid == 0 && (p.units / pl.grid) % g.k_blocks == 0) return cudaSuccess;   // whole tiles only
+    const FinishParams f = {p.partial, p.inv_scale, y, y_dtype, g.n_out, m, pl.n_cols, pl.tiles_x, g.k_blocks, pl.units, pl.grid};
+    cfg.gridDim = dim3(pl.tiles_x * pl.t_tiles, (pl.n_cols + kFinishTokens - 1) / kFinishTokens);
+    cfg.blockDim = dim3(kFinishThreads);
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, finish_kernel, f);
 }
 
 template <int WB, bool TWO>
@@ -506,7 +502,7 @@ static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed,
 
 bool gemm_mid_supported(const Geometry& g, int m, bool exact) {
     mid::Plan p;
-    return g.k_in % 8 == 0 && tc::packed_map_supported(g) && (size_t)g.n_tiles * 4 <= kWsCounterBytes && mid::make_plan(g, m, exact && !g.k1, &p);
+    return g.k_in % 8 == 0 && tc::packed_map_supported(g) && mid::make_plan(g, m, exact && !g.k1, &p);
 }
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact) {
     mid::Plan p;

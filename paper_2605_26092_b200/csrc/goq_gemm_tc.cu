@@ -415,11 +415,15 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
     uint4 held[kPrepHold];
 #pragma unroll
     for (int h = 0; h < kPrepHold; ++h) {
+        if (h * kPrepThreads >= n_vec) break;
         const int i = tid + h * kPrepThreads;
         held[h] = i < n_vec ? __ldg(&row[i]) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
-    for (int h = 0; h < kPrepHold; ++h) largest(held[h]);
+    for (int h = 0; h < kPrepHold; ++h) {
+        if (h * kPrepThreads >= n_vec) break;
+        largest(held[h]);
+    }
     for (int i = tid + kPrepHold * kPrepThreads; i < n_vec; i += kPrepThreads) largest(__ldg(&row[i]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
@@ -439,8 +443,10 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
         out[i] = make_uint4(o32[0], o32[1], o32[2], o32[3]);
     };
 #pragma unroll
-    for (int h = 0; h < kPrepHold; ++h)
+    for (int h = 0; h < kPrepHold; ++h) {
+        if (h * kPrepThreads >= n_vec) break;
         if (tid + h * kPrepThreads < n_vec) convert(tid + h * kPrepThreads, held[h]);
+    }
     for (int i = tid + kPrepHold * kPrepThreads; i < n_vec; i += kPrepThreads) convert(i, __ldg(&row[i]));
     if (tid == 0) inv_scale[tok] = __uint_as_float((uint32_t)(254 - sfield) << 23);
 }

@@ -3,8 +3,9 @@
 //
 // Units are numbered token tile by token tile, channel tile by channel tile, k-block by k-block; CTA c of G takes
 // [U c / G, U (c+1) / G). A CTA parks the part of a tile it has only a share of (its range's first and last tile at most) as fp32
-// [token][128 channels] in scratch. At its end it counts itself in at both tiles; the CTA that comes last adds all parts in CTA
-// order, with all its threads, and stores.
+// [token][128 channels] in scratch; `finish_kernel`, launched behind as a programmatic dependent, adds the parts of every shared
+// tile in CTA order and stores. (Adding in the CTA that came last instead needs no second launch, but leaves the sum of a tile to
+// one SM: 1024 x 8192 at 256 tokens, where eight tiles have 19 parts of 128 KB each, took 71 us, now 28.)
 #pragma once
 #include "goq_tc_core.cuh"
 
@@ -23,28 +24,6 @@ __device__ __forceinline__ Part part_at(int u, int u1, int k_blocks) {
     p.kb = u - p.tile * k_blocks;
     p.n = min(k_blocks - p.kb, u1 - u);
     return p;
-}
-
-// device-scope fetch-add: releases this thread's earlier writes (and those ordered before it by a barrier), acquires the others'
-__device__ __forceinline__ int atomic_add_acq_rel(int* addr, int v) {
-    int old;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(addr), "r"(v) : "memory");
-    return old;
-}
-
-// The range's first and last tile: the CTAs that share it, where the first of them keeps its part (every other sharer starts
-// inside the tile, so it is that CTA's first part), and which channel quarters this CTA has to finish.
-struct SharedTile { int tile, c_lo, c_hi, first_slot, last_of[4]; };
-
-// Filled by lanes 0 and 1 of a warp that has time before the main loop (the divisions are slow).
-__device__ __forceinline__ void describe_shared(SharedTile (&fin)[2], int lane, int u0, int u1, int units, int k_blocks, int n_ctas) {
-    if (lane >= 2) return;
-    const int tile = (lane ? u1 - 1 : u0) / k_blocks;
-    const int c_lo = (int)((((long long)tile * k_blocks + 1) * n_ctas - 1) / units);
-    fin[lane].tile = tile;
-    fin[lane].c_lo = c_lo;
-    fin[lane].c_hi = (int)((((long long)(tile + 1) * k_blocks) * n_ctas - 1) / units);
-    fin[lane].first_slot = range_begin(c_lo, units, n_ctas) == tile * k_blocks ? 0 : 1;
 }
 
 // y[token][channel..channel + 3], vector stores where the output allows them
@@ -83,49 +62,46 @@ struct Output {
     }
 };
 
-// After the CTA's own work, by all its threads (contains barriers). park_floats: floats of one parked part, two parts a CTA.
-// scale: per-token factor of the sums (nullptr: 1).
-template <int THREADS>
-__device__ __forceinline__ void finish_shared(SharedTile (&fin)[2], const float* partial, size_t park_floats, int* counters,
-                                              int tiles_x, int n_cols, int m, const float* scale, const Output& out) {
-    const int tid = threadIdx.x;
-    if (tid < 8) {   // the parked parts are ordered before by the caller's barrier; the fetch-add releases them
-        const int f = tid >> 2, quarter = tid & 3;
-        bool mine = false;
-        if (fin[f].c_hi > fin[f].c_lo && !(f == 1 && fin[0].tile == fin[1].tile)) {
-            int* counter = &counters[fin[f].tile * 4 + quarter];
-            mine = atomic_add_acq_rel(counter, 1) == fin[f].c_hi - fin[f].c_lo;
-            if (mine) *counter = 0;
-        }
-        fin[f].last_of[quarter] = mine ? 1 : 0;
+struct FinishParams {
+    const float* partial;   // [CTA][2][n_cols][128]: a CTA's first part, its last one
+    const float* scale;     // per-token factor of the sums
+    void* y;
+    int y_dtype, n_out, m, n_cols, tiles_x, k_blocks, units, n_ctas;
+};
+constexpr int kFinishThreads = 256, kFinishTokens = 16;   // of a CTA: 16 tokens of a tile, two tokens x four channels a thread
+
+// grid: (channel tiles x token tiles, token slices). Bound by the parts' way through L2.
+static __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const FinishParams p) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int tile = blockIdx.x, ch = (threadIdx.x & 31) * 4;
+    // the CTAs that share the tile, and where the first of them keeps its part (every other one starts inside the tile, so it is
+    // that CTA's first)
+    const int c_lo = (int)((((long long)tile * p.k_blocks + 1) * p.n_ctas - 1) / p.units);
+    const int c_hi = (int)((((long long)(tile + 1) * p.k_blocks) * p.n_ctas - 1) / p.units);
+    if (c_lo == c_hi) return;   // one CTA had the whole tile and has stored it
+    const int slot = range_begin(c_lo, p.units, p.n_ctas) == tile * p.k_blocks ? 0 : 1;
+    const int tok0 = (tile / p.tiles_x) * p.n_cols, cols = min(p.n_cols, p.m - tok0);
+    const int col = blockIdx.y * kFinishTokens + (threadIdx.x >> 5);
+    if (col >= cols) return;
+    const int col2 = min(col + kFinishTokens / 2, cols - 1);
+    const size_t park = (size_t)p.n_cols * kTileN, stride = 2 * park;
+    const float* lo = p.partial + ((size_t)c_lo * 2 + slot) * park + ch;
+    const float* rest = p.partial + (size_t)(c_lo + 1) * stride + ch;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float4 f0 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col * kTileN));
+    float4 f1 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col2 * kTileN));
+    const float s0 = __ldcg(p.scale + tok0 + col), s1 = __ldcg(p.scale + tok0 + col2);
+#pragma unroll 8
+    for (int c = c_lo + 1; c <= c_hi; ++c, rest += stride) {   // CTA order
+        const float4 a = __ldcg(reinterpret_cast<const float4*>(rest + (size_t)col * kTileN));
+        const float4 b = __ldcg(reinterpret_cast<const float4*>(rest + (size_t)col2 * kTileN));
+        f0.x += a.x; f0.y += a.y; f0.z += a.z; f0.w += a.w;
+        f1.x += b.x; f1.y += b.y; f1.z += b.z; f1.w += b.w;
     }
-    __syncthreads();
-    for (int f = 0; f < 2; ++f) {
-        if (!(fin[f].last_of[0] | fin[f].last_of[1] | fin[f].last_of[2] | fin[f].last_of[3])) continue;
-        const int tile = fin[f].tile, c_lo = fin[f].c_lo, c_hi = fin[f].c_hi;
-        const int tok0 = (tile / tiles_x) * n_cols, elems = min(n_cols, m - tok0) * 32, ch0 = (tile % tiles_x) * kTileN;
-        const float4* first_part = reinterpret_cast<const float4*>(partial + ((size_t)c_lo * 2 + fin[f].first_slot) * park_floats);
-        const float4* other = reinterpret_cast<const float4*>(partial);
-        const size_t stride = park_floats / 2;   // two parts a CTA, four floats a vector
-        for (int idx0 = tid; idx0 < elems; idx0 += THREADS * 2) {   // two elements (four channels of a token) a thread in flight
-            const int idx[2] = {idx0, min(idx0 + THREADS, elems - 1)};
-            float4 f0 = __ldcg(first_part + idx[0]), f1 = __ldcg(first_part + idx[1]);
-#pragma unroll 4
-            for (int c = c_lo + 1; c <= c_hi; ++c) {   // CTA order
-                const float4 a = __ldcg(other + c * stride + idx[0]), b = __ldcg(other + c * stride + idx[1]);
-                f0.x += a.x; f0.y += a.y; f0.z += a.z; f0.w += a.w;
-                f1.x += b.x; f1.y += b.y; f1.z += b.z; f1.w += b.w;
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int col = idx[j] >> 5, c4 = (idx[j] & 31) * 4;
-                if (idx0 + j * THREADS >= elems || !fin[f].last_of[c4 >> 5]) continue;
-                const float s = scale ? __ldcg(scale + tok0 + col) : 1.0f;
-                const float4 v = j ? f1 : f0;
-                out.store4(tok0 + col, ch0 + c4, make_float4(v.x * s, v.y * s, v.z * s, v.w * s));
-            }
-        }
-    }
+    const Output out = {p.y, p.y_dtype, p.n_out};
+    const int ch0 = (tile % p.tiles_x) * kTileN + ch;
+    out.store4(tok0 + col, ch0, make_float4(f0.x * s0, f0.y * s0, f0.z * s0, f0.w * s0));
+    if (col + kFinishTokens / 2 < cols) out.store4(tok0 + col2, ch0, make_float4(f1.x * s1, f1.y * s1, f1.z * s1, f1.w * s1));
 }
 
 }  // namespace streamk
