@@ -172,9 +172,11 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         // 8192 x 8192: 43 / 72 at 32 tokens, 43 / 92 at 64, 65 / 95 at 256, 92 / 121 at 512; 4096 x 4096: 23 / 31, 27 / 52,
         // 44 / 53, 50 / 67; 1024 x 8192: 20 / 23, 27 / 75, 70 / 75, 57 / 118.
         const bool exact = m <= kGemmExactMaxTokens;
-        // Above 256 tokens it decodes the weights once per 256 tokens, so it is for calls whose 128 x 512 tiles would leave half of
-        // the SMs without one (1024 x 8192 W4, 777 tokens: 49 / 122; 4096 x 4096, 1024 tokens: 64 / 69; 16384 x 2048, 640: 153 / 78).
-        const bool mid_wanted = variant == 4 || (variant == 0 && m > 16 && (m <= kGemmMidMaxTokens || goq::gemm_tc_tiles(g, m) * 2 <= 148));
+        // Above 256 tokens it decodes the weights once per 256 tokens, but spreads any number of tiles evenly; the two kernels'
+        // estimates decide. Measured, us, this kernel / prefill kernel: 1024 x 8192 W4 at 777 tokens 35 / 102, at 4096 107 / 137;
+        // 4096 x 4096 at 1024 51 / 56, at 1280 65 / 59; 11008 x 4096 at 512 67 / 69, at 1280 137 / 125; 16000 x 512 at 512 38 / 24.
+        const bool mid_wanted = variant == 4 || (variant == 0 && m > 16 && (m <= kGemmMidMaxTokens || !goq::gemm_tc_supported(g) ||
+                                                                            goq::gemm_mid_us(g, m) <= goq::gemm_tc_us(g, m)));
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
             return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
         if (variant == 4) return GOQ_ERR_UNSUPPORTED;

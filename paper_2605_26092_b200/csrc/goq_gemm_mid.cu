@@ -174,13 +174,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
                     if (c0 + j < cols) __stcg(park + (size_t)(c0 + j) * kTileN, v[j] * inv_row);
-            } else if (ch < p.n_out) {
+            } else {
+                // the tokens' factors at once: loaded one by one between the stores they made a tile's drain longer than its main
+                // loop (16 of them are always there to read)
+                float4 s[4];
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (c0 + j < cols) {
-                        const float f = v[j] * (__ldcg(&p.inv_scale[tok0 + c0 + j]) * inv_row);
-                        out.store1(tok0 + c0 + j, ch, f);
-                    }
+                for (int j = 0; j < 4; ++j) s[j] = __ldcg(reinterpret_cast<const float4*>(p.inv_scale + tok0 + c0) + j);
+                const float sc[16] = {s[0].x, s[0].y, s[0].z, s[0].w, s[1].x, s[1].y, s[1].z, s[1].w,
+                                      s[2].x, s[2].y, s[2].z, s[2].w, s[3].x, s[3].y, s[3].z, s[3].w};
+                if (ch < p.n_out) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (c0 + j < cols) out.store1(tok0 + c0 + j, ch, v[j] * (sc[j] * inv_row));
+                }
             }
         }
     };
@@ -503,6 +509,15 @@ static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed,
 bool gemm_mid_supported(const Geometry& g, int m, bool exact) {
     mid::Plan p;
     return g.k_in % 8 == 0 && tc::packed_map_supported(g) && mid::make_plan(g, m, exact && !g.k1, &p);
+}
+// Estimated time of a call: a unit's decode plus a share that grows with its tokens, or the drain of its tile by four warps where
+// the tile has few k-blocks, and 14 us for the pre-pass, the start and the shared tiles. (W3, us a unit: 0.75 at 64 tokens, 1.4 at
+// 256; 0.15 more at W4; 16 us for the drain of 256 tokens.)
+float gemm_mid_us(const Geometry& g, int m) {
+    mid::Plan p;
+    if (!mid::make_plan(g, m, false, &p)) return 1e30f;
+    const float unit = 0.55f + 0.0032f * (float)p.n_cols + (g.wbits == 4 ? 0.15f : 0.f), drain = 0.0625f * (float)p.n_cols / (float)g.k_blocks;
+    return 14.f + (float)((p.units + p.grid - 1) / p.grid) * (unit > drain ? unit : drain);
 }
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact) {
     mid::Plan p;

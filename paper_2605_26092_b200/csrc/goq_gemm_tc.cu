@@ -2,7 +2,7 @@
 //
 // Eq. 4 of the paper with the coefficients folded into the weight operand:
 //   y[m,n] = sum_k x[m,k] * w_hat[n,k],   w_hat[n,k] = c1[n,j] b1[n,k] + c2[n,j] b2[n,k]   (Section 3.1)
-// Each CTA computes a 128 (output channels) x 512 (tokens) tile. Per 64-wide k-chunk
+// Each CTA computes a tile of 128 output channels x up to 512 tokens (two halves of at most 256). Per 64-wide k-chunk
 //   - a producer thread bulk-copies the packed unit records of the 128 rows (cp.async.bulk, 8 records per
 //     128 k) and loads the 512 x 64 bf16 activation tile with two 2-D TMA copies (128-byte swizzle);
 //   - eight expander warps decode the records (same byte-table decode and record lookup as the GEMV:
@@ -48,11 +48,12 @@ struct GemmParams {
     const float* row_inv;        // [n_pad] its inverse
     int* status;
     int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m_total, y_dtype, group_log2;
-    // Tile schedule (1-D grid). CTAs [0, n_full) take 128 x 512 tiles, numbered channel-tile fastest; the remaining
-    // CTAs take the last tiles as halves of 256 tokens each, so that a last wave that would fill less than half of
+    // Tile schedule (1-D grid). CTAs [0, n_full) take whole tiles (2 * half tokens), numbered channel-tile fastest; the remaining
+    // CTAs take the last tiles as token halves, so that a last wave that would fill less than half of
     // the SMs runs for half as long on twice as many.
     // With at most 256 tokens in all, every tile is one half (halves_per_tile = 1).
     int n_full, n_tiles_x, halves_per_tile;
+    int half;   // tokens of a half tile (MMA N): a multiple of 16, at most 256
     // Split-K (only with at most 256 tokens, where the tiles alone would leave most SMs idle): n_split CTAs share a
     // tile, each takes kb_per_split k-blocks and parks its fp32 partial tile in `partial`; the CTA that arrives last
     // at the tile's counter adds the partials in split order (the result does not depend on timing), scales and
@@ -91,12 +92,12 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
     const int bid = blockIdx.x;
     const int unit_id = bid / p.n_split, split = bid - unit_id * p.n_split;   // n_split > 1 only when every tile is one half
     const int tile = unit_id < p.n_full ? unit_id : p.n_full + (unit_id - p.n_full) / p.halves_per_tile;
-    const int n_half = unit_id < p.n_full ? 2 : 1;   // token halves (of 256) this CTA computes
-    const int kb0 = split * p.kb_per_split;            // this CTA's k-blocks: [kb0, kb0 + nkb)
-    const int nkb = min(p.kb_per_split, p.k_blocks - kb0);
     const int tile_x = tile % p.n_tiles_x;
     const int T0 = tile_x * (kTileN / kTileRows);  // first 16-row tile of this CTA
-    const int tok0 = (tile / p.n_tiles_x) * kTileM + (unit_id < p.n_full ? 0 : ((unit_id - p.n_full) % p.halves_per_tile) * 256);
+    const int tok0 = (tile / p.n_tiles_x) * 2 * p.half + (unit_id < p.n_full ? 0 : ((unit_id - p.n_full) % p.halves_per_tile) * p.half);
+    const int n_half = unit_id < p.n_full && tok0 + p.half < p.m_total ? 2 : 1;   // token halves this CTA computes
+    const int kb0 = split * p.kb_per_split;            // this CTA's k-blocks: [kb0, kb0 + nkb)
+    const int nkb = tok0 < p.m_total ? min(p.kb_per_split, p.k_blocks - kb0) : 0;
     const int n_chunks = 2 * nkb;
 
     if (tid == 0) {
@@ -112,8 +113,12 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
     if (warp == 1) tmem_alloc<512>(&tmem_base_slot);
     // Everything above needs nothing from the activation pre-pass, which may still be running (programmatic dependent
     // launch: this grid is scheduled as soon as the pre-pass lets it); what follows reads what the pre-pass wrote.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next call's pre-pass gets in place behind this grid)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = tid; i < kTileM; i += kThreads) inv_s[i] = (tok0 + i < p.m_total) ? __ldcg(&p.inv_scale[tok0 + i]) : 1.0f;
+    for (int i = tid; i < kTileM; i += kThreads) {
+        const int col = i & 255, tok = tok0 + (i >> 8) * p.half + col;
+        inv_s[i] = (col < p.half && tok < p.m_total) ? __ldcg(&p.inv_scale[tok]) : 1.0f;
+    }
     for (int i = tid; i < kTileN; i += kThreads) {
         const bool in = T0 * kTileRows + i < p.n_tiles * kTileRows;
         row_s[i] = in ? __ldcg(&p.row_scale[T0 * kTileRows + i]) : 0x3C003C00u;   // 1.0
@@ -145,10 +150,10 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
                     if (chunk >= kStages) ok = mbar_wait(&empty[s], ((chunk / kStages) - 1) & 1, &abort_flag);
                     if (!ok) break;
                     b_issued = chunk + 1;
-                    mbar_expect_tx(&full_b[s], (uint32_t)n_half * (kBTileBytes / 2));
+                    mbar_expect_tx(&full_b[s], (uint32_t)(n_half * p.half) * (kChunkK * 2));
                     tma_load_2d(b_tiles + s * kBTileBytes, &x_map, (2 * kb0 + chunk) * kChunkK, tok0, &full_b[s]);
                     if (n_half == 2)
-                        tma_load_2d(b_tiles + s * kBTileBytes + kBTileBytes / 2, &x_map, (2 * kb0 + chunk) * kChunkK, tok0 + 256, &full_b[s]);
+                        tma_load_2d(b_tiles + s * kBTileBytes + kBTileBytes / 2, &x_map, (2 * kb0 + chunk) * kChunkK, tok0 + p.half, &full_b[s]);
                 }
             }
             if (!ok || abort_flag) {
@@ -163,6 +168,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
             bool ok = true;
+            const uint32_t idesc = idesc_f16((uint32_t)p.half);
             for (int chunk = 0; chunk < n_chunks; ++chunk) {
                 const int s = chunk % kStages;
                 const uint32_t par = (chunk / kStages) & 1;
@@ -175,8 +181,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
 #pragma unroll
                 for (int ks = 0; ks < kChunkK / 16; ++ks) {
                     const uint32_t acc = (chunk > 0 || ks > 0) ? 1u : 0u;
-                    umma_f16(tmem_base, adesc + 2 * ks, bdesc0 + 2 * ks, idesc_f16(256), acc);         // tokens   0..255
-                    if (n_half == 2) umma_f16(tmem_base + 256, adesc + 2 * ks, bdesc1 + 2 * ks, idesc_f16(256), acc);   // tokens 256..511
+                    umma_f16(tmem_base, adesc + 2 * ks, bdesc0 + 2 * ks, idesc, acc);         // first half's tokens
+                    if (n_half == 2) umma_f16(tmem_base + 256, adesc + 2 * ks, bdesc1 + 2 * ks, idesc, acc);   // second half's
                 }
                 umma_commit(&empty[s]);
             }
@@ -278,8 +284,9 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
                     }
                 }
             };
+            const int n_cb = (p.half + 31) / 32;
 #pragma unroll 1
-            for (int cb = 0; cb < 8 && ok; ++cb) {
+            for (int cb = 0; cb < n_cb && ok; ++cb) {
                 uint32_t v[32];
                 const int col0 = col_half * 256 + cb * 32;
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)col0, v);
@@ -310,17 +317,17 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
                 }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const int jt = q * 8 + i, tok = tok0 + col0 + jt;
-                    if (tok < p.m_total) store4(tok, *reinterpret_cast<const float4*>(&st[jt * kTileN + 4 * lane]));
+                    const int jt = q * 8 + i, tok = tok0 + col_half * p.half + cb * 32 + jt;
+                    if (cb * 32 + jt < p.half && tok < p.m_total) store4(tok, *reinterpret_cast<const float4*>(&st[jt * kTileN + 4 * lane]));
                 }
             }
             if (p.n_split > 1 && ok) {
                 // Every warp's partial rows are on their way: make them visible, meet, and let one thread count this CTA
-                // in. The epilogue barrier has been through eight phases, so the next two have parities 0 and 1.
+                // in. The epilogue barrier has been through n_cb phases.
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&epi_bar[0]);
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[0], 0, &abort_flag));
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[0], n_cb & 1, &abort_flag));
                 if (ok) {
                     if (lane == 0) {
                         if (q == 0) {
@@ -329,7 +336,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
                         }
                         mbar_arrive(&epi_bar[0]);
                     }
-                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[0], 1, &abort_flag));
+                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[0], (n_cb + 1) & 1, &abort_flag));
                 }
                 if (ok && split_last) {
                     const float* part = p.partial + (size_t)tile * p.n_split * (256 * kTileN);
@@ -506,10 +513,12 @@ cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geomet
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
 }
-// The activation pre-pass alone, as a programmatic dependent of what precedes it: its launch overlaps the tail of that kernel.
-cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st) {
+// The activation pre-pass (and, with `row_tiles` blocks more, the channel scales) as a programmatic dependent of what precedes it:
+// its launch overlaps the tail of that kernel.
+static cudaError_t launch_pre_pass(const void* x, int k_in, int m, int row_tiles, uint16_t* xh, float* inv_scale, const void* packed,
+                                   int unit_bytes, int k_blocks, int gpb, uint32_t* row_scale, float* row_inv, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(m);
+    cfg.gridDim = dim3(m + row_tiles);
     cfg.blockDim = dim3(kPrepThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -517,8 +526,11 @@ cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, x_to_f16_kernel, (const uint16_t*)x, k_in, xh, inv_scale, m, (const uint8_t*)nullptr, 0, 0, 0,
-                              (uint32_t*)nullptr, (float*)nullptr);
+    return cudaLaunchKernelEx(&cfg, x_to_f16_kernel, (const uint16_t*)x, k_in, xh, inv_scale, m, (const uint8_t*)packed, unit_bytes,
+                              k_blocks, gpb, row_scale, row_inv);
+}
+cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st) {
+    return launch_pre_pass(x, k_in, m, 0, xh, inv_scale, nullptr, 0, 0, 0, nullptr, nullptr, st);
 }
 
 static int sm_count_cached() {
@@ -529,6 +541,30 @@ static int sm_count_cached() {
             n = 148;
     }
     return n;
+}
+// Token tiles of a call, equally wide (600 tokens: 2 of 320, not 512 and 88). More of them than 512 tokens each allow where that
+// makes the waves over the SMs clearly shorter (a call with few channel tiles leaves SMs idle): a CTA takes, for each k-block,
+// the weights' decode plus a share that grows with its tokens (4096 x 4096 W3, us a k-block: 1.1 at 128 tokens, 1.3 at 256, 1.6 at
+// 512), and about 8 us to start and to drain. 2000 x 11008 at 2048 tokens: 8 tiles 142 us, 4 tiles 176. Where every SM has work
+// anyway more tiles only decode more (4096 x 4096 at 4096 tokens: 9 tiles 153 us, 8 tiles 141), hence the margin of 8 %.
+static float wave_us(int k_blocks, int tokens) { return 8.f + (float)k_blocks * (0.95f + 0.00135f * (float)tokens); }
+struct TokenTiles { int n, half, n_full, n_tail; float us; };   // tiles of 2 * half tokens; n_full CTAs take whole tiles, n_tail tiles go as halves
+static TokenTiles token_tiles(const Geometry& g, int m) {
+    const int sms = sm_count_cached(), tiles_x = (g.n_pad + kTileN - 1) / kTileN;
+    TokenTiles best = {};
+    if (m <= 256) { best.n = 1; best.half = (m + 15) & ~15; best.n_tail = tiles_x; return best; }
+    const int n0 = (m + kTileM - 1) / kTileM;
+    for (int n = n0; n <= n0 + 4; ++n) {
+        TokenTiles t;
+        t.half = ((m + 2 * n - 1) / (2 * n) + 15) & ~15;
+        t.n = (m + 2 * t.half - 1) / (2 * t.half);
+        const int tiles = tiles_x * t.n, tail = tiles % sms;   // tiles of the last, partial wave
+        t.n_tail = (tiles > sms && 2 * tail <= sms) ? tail : 0;
+        t.n_full = tiles - t.n_tail;
+        t.us = (float)((t.n_full + sms - 1) / sms) * wave_us(g.k_blocks, 2 * t.half) + (t.n_tail ? 4.f + wave_us(g.k_blocks, t.half) : 0.f);
+        if (best.n == 0 || t.us < 0.975f * best.us) best = t;
+    }
+    return best;
 }
 // Split-K factor for a call (1 = none): only with at most 256 tokens, when the channel tiles alone would leave at
 // least half of the SMs idle, and never below four k-blocks per CTA.
@@ -553,10 +589,11 @@ static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* 
                              float* inv_scale, uint32_t* row_scale, float* row_inv, uint16_t* xh, int* tile_counter, float* partial,
                              cudaStream_t st) {
     if (g.k_in % 8 != 0) return cudaErrorInvalidValue;
-    x_to_f16_kernel<<<m + g.n_tiles, kPrepThreads, 0, st>>>((const uint16_t*)x, g.k_in, xh, inv_scale, m, (const uint8_t*)packed,
-                                                           g.unit_bytes, g.k_blocks, g.groups_per_block, row_scale, row_inv);
+    if (cudaError_t e = launch_pre_pass(x, g.k_in, m, g.n_tiles, xh, inv_scale, packed, g.unit_bytes, g.k_blocks, g.groups_per_block,
+                                        row_scale, row_inv, st)) return e;
     CUtensorMap map;
-    if (cudaError_t e = encode_x_map(&map, xh, g.k_in, m, 256)) return e;
+    const TokenTiles tt = token_tiles(g, m);
+    if (cudaError_t e = encode_x_map(&map, xh, g.k_in, m, tt.half)) return e;
     const size_t smem = smem_bytes(g);
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_tc_kernel<WB>, smem, smem_attr)) return e;
@@ -577,18 +614,16 @@ static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* 
     int lg = 3;
     while ((1 << lg) < g.group) ++lg;
     p.group_log2 = lg;
-    const int tiles_x = (g.n_pad + kTileN - 1) / kTileN, tiles = tiles_x * ((m + kTileM - 1) / kTileM);
-    const int sm_count = sm_count_cached();
-    const int tail = tiles % sm_count;   // tiles of the last, partial wave
-    const int split = (tiles > sm_count && tail > 0 && 2 * tail <= sm_count) ? tail : 0;
+    const int tiles_x = (g.n_pad + kTileN - 1) / kTileN, tiles = tiles_x * tt.n;
     p.n_tiles_x = tiles_x;
+    p.half = tt.half;
     p.halves_per_tile = (m <= 256) ? 1 : 2;
-    p.n_full = (m <= 256) ? 0 : tiles - split;
+    p.n_full = tt.n_full;
     p.n_split = split_factor(g, m);
     p.kb_per_split = (g.k_blocks + p.n_split - 1) / p.n_split;
     p.partial = partial;
     p.tile_counter = tile_counter;
-    const int n_ctas = (m <= 256) ? tiles * p.n_split : p.n_full + 2 * split;
+    const int n_ctas = (m <= 256) ? tiles * p.n_split : p.n_full + 2 * tt.n_tail;
     // Programmatic dependent launch on the pre-pass just enqueued: the CTAs fill their tables, allocate tensor memory
     // and initialise their barriers while it runs, and wait (griddepcontrol.wait) before the first read of its outputs.
     cudaLaunchConfig_t cfg = {};
@@ -627,7 +662,8 @@ TcScratch tc_scratch(const Geometry& g, int m) {
     return t;
 }
 }  // namespace
-int gemm_tc_tiles(const Geometry& g, int m) { return (g.n_pad + tc::kTileN - 1) / tc::kTileN * ((m + tc::kTileM - 1) / tc::kTileM); }
+// estimated time of a call of more than 256 tokens (pre-pass and launch 9 us)
+float gemm_tc_us(const Geometry& g, int m) { return 9.f + tc::token_tiles(g, m).us; }
 size_t gemm_tc_workspace(const Geometry& g, int m) { return tc_scratch(g, m).total; }
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws,
                            cudaStream_t st) {

@@ -86,13 +86,14 @@ cudaError_t launch_gemv_one(const Geometry& g, const void* packed, const void* x
 // and the split-K partial tiles.
 bool gemm_tc_supported(const Geometry& g);
 size_t gemm_tc_workspace(const Geometry& g, int m);
-int gemm_tc_tiles(const Geometry& g, int m);   // its 128 x 512 tiles
+float gemm_tc_us(const Geometry& g, int m);   // estimated time, more than 256 tokens
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype,
                            void* ws, cudaStream_t st);
 
 // The same layer for a few to a few hundred tokens (goq_gemm_mid.cu), any group, wbits 2..4. exact: the two bases as separate
 // operands without rounding (fp32 accuracy), else w_hat rounded once to fp16. `ws` holds gemm_mid_workspace bytes.
 bool gemm_mid_supported(const Geometry& g, int m, bool exact);
+float gemm_mid_us(const Geometry& g, int m);   // estimated time
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact);
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
                             bool exact, cudaStream_t st);

@@ -130,6 +130,30 @@ def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
     check_parity(out[0].astype(np.float64), y_ref, 2e-5 if exact else 5e-4, 1e-4 if exact else 2e-3)
 
 
+@pytest.mark.parametrize("variant,n,k,g,b,m", [
+    (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
+    (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
+def test_prefill_gemm_token_tiles(goq, variant, n, k, g, b, m):
+    """Equal token tiles narrower than 512: one token more than a half tile holds, a last tile that does not fill, tiles left over
+    as halves (9600 and 9500 channels on 148 SMs), few channel tiles in many token tiles; in the mid-batch kernel ranges of several
+    whole tiles, drained by four warps. Every token's row is written once. Bound: w_hat rounded once to fp16, 5e-4."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b)
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+    prev = goq.set_gemv_variant(variant)
+    try:
+        y = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+        goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+        assert goq.workspace_status(ws) == goq.OK
+    finally:
+        goq.set_gemv_variant(prev)
+    check_parity(y.cpu().numpy().astype(np.float64), y_ref, 5e-4, 2e-3)
+
+
 @pytest.mark.parametrize("n,k,g,b,m", [(1, 32, 32, 3, 1), (16, 128, 128, 2, 4), (2368, 128, 128, 3, 3), (2369, 128, 64, 3, 1), (37888, 256, 32, 2, 2),
                                        (16, 12288, 128, 3, 4), (129, 3200, 64, 3, 3), (4736, 4096, 128, 3, 1)])
 def test_single_decode_gemv_edges(goq, n, k, g, b, m):
