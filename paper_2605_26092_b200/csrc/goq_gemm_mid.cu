@@ -278,7 +278,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         for (int u = u0; u < u1 && ok; ++q) {
             const Part part = part_at(u, u1, p.k_blocks);
             const bool valid = (part.tile % p.tiles_x) * 8 + e < p.n_tiles;
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&sc_full[q & 1], (q >> 1) & 1, &abort_flag));
+            // a part with a unit of this group's: it cannot end, nor this barrier's next phase begin, before that unit is decoded
+            if (part.n > 1 || (i & 1) == group) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&sc_full[q & 1], (q >> 1) & 1, &abort_flag));
             const uint32_t rs_a = row_s[q & 1][e * 16 + g], rs_b = row_s[q & 1][e * 16 + 8 + g];
             __half2 cf[2] = {u2h(0u), u2h(0u)};   // {c1, c2} of rows g and g + 8, scaled (exactly: by a power of two)
             auto load_coef = [&](uint32_t unit, int jj) {
@@ -395,7 +396,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
             u += part.n;
         }
     }
-    __syncwarp();
+    // The epilogue warps come here once every earlier part is drained: from then on the barrier of the last part is in the phase that
+    // is waited for (the warps that run ahead would find the phase before the last completed and take it for this one).
+    __syncthreads();
     // ---- the range's last part: every warp drains its quarter's columns, in turn with the others of that quarter ----
     const int last_tile = (u1 - 1) / p.k_blocks, q_last = last_tile - u0 / p.k_blocks;
     const Part last = part_at(max(u0, last_tile * p.k_blocks), u1, p.k_blocks);

@@ -151,7 +151,15 @@ def test_prefill_gemm_token_tiles(goq, variant, n, k, g, b, m):
         assert goq.workspace_status(ws) == goq.OK
     finally:
         goq.set_gemv_variant(prev)
-    check_parity(y.cpu().numpy().astype(np.float64), y_ref, 5e-4, 2e-3)
+    got = y.cpu().numpy().astype(np.float64)
+    if n > 1:
+        check_parity(got, y_ref, 5e-4, 2e-3)
+    else:
+        # One output has no norm over channels to average in, and it may be small by cancellation. Each w_hat is off by at most its
+        # fp16 rounding, 2^-11 of itself (the sums in fp32 add far less), so the output by at most 2^-11 sum |x| |w_hat|.
+        w = np.abs(O.decode_b1(codes, b) * np.repeat(coef[..., 0].astype(np.float64), g, 1)
+                   + O.decode_b2(codes, meta, b) * np.repeat(coef[..., 1].astype(np.float64), g, 1))
+        assert (np.abs(got - y_ref) <= 2.0 ** -11 * np.abs(si.bf16_bits_to_f64(xb)) @ w.T).all()
 
 
 @pytest.mark.parametrize("n,k,g,b,m", [(1, 32, 32, 3, 1), (16, 128, 128, 2, 4), (2368, 128, 128, 3, 3), (2369, 128, 64, 3, 1), (37888, 256, 32, 2, 2),
