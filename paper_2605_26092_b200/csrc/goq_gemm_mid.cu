@@ -444,11 +444,15 @@ static bool make_plan(const Geometry& g, int m, bool two, Plan* p) {
     if (units >= (1ll << 30)) return false;
     p->units = (int)units;
     p->grid = (int)(units < sm_count() ? units : sm_count());
-    // rings: up to six k-blocks of packed records, then as many operand stages as fit (at least three)
+    // Rings: four k-blocks of packed records, then as many operand stages as fit (at least three): a fourth stage counts for more
+    // than a fifth record block (8192 x 8192 at 192 tokens 46.5 -> 43.7 us). Six blocks where that is most of a CTA's range, read
+    // while the pre-pass still runs, and for the exact form, whose stages are larger anyway.
     const size_t budget = 227 * 1024 - 4 * 1024 - 8192 - kLutBytes;   // static variables, alignment of the table, the table
     const size_t stage = (size_t)(two ? 2 : 1) * kChunkBytes + (size_t)p->n_cols * 128, pk = (size_t)8 * g.unit_bytes;
-    p->n_pk = 6;
-    while (p->n_pk > 2 && p->n_pk * pk + 3 * stage > budget) --p->n_pk;
+    p->n_pk = two || p->units <= 12 * p->grid ? 6 : 4;
+    // (an even number, so that a slot comes round to the same group of decoding warps: with one phase bit a barrier, another group
+    // might take the slot's records before for its own)
+    while (p->n_pk > 2 && p->n_pk * pk + 3 * stage > budget) p->n_pk -= 2;
     if (p->n_pk * pk + 3 * stage > budget) return false;
     p->n_stages = (int)((budget - p->n_pk * pk) / stage);
     if (p->n_stages > kMaxStages) p->n_stages = kMaxStages;
