@@ -5,8 +5,9 @@
 // The coefficient changes every macro-block while a tensor-core accumulator does not, so it goes into the operand: c~ v needs 11 bits
 // (W3), two int8 digits: c~ v = B h + l, B = 16 (W2, W3) or 192 (W4), ACC = B sum x h + sum x l. All integers, summed modulo 2^32;
 // the result is below 2^31 by the host's bound, so it is the same bits in any order. Four digit planes (two bases x two digits) of
-// 64 channels make one N = 256 operand; a CTA's tile is 128 tokens x 128 channels, its four accumulators all of tensor memory.
-// Against per-macro-block sums on mma.sync (goq_gemm_a8.cu) this doubles the multiply-adds and takes the coefficient stage, eight
+// 64 channels make one N = 256 operand; a CTA's tile is 256 tokens (two M = 128 halves) x 64 channels, its accumulators all of tensor
+// memory.
+// Against per-macro-block sums in registers (mma.sync) this doubles the multiply-adds and takes the coefficient stage, eight
 // integer multiply-adds per four MMAs, out of the loop.
 //
 // Digits come from byte tables: 256 entries, one per value of c~, of the digits of c~ v for every code, looked up per row and
