@@ -438,9 +438,13 @@ struct Plan {
 };
 static bool make_plan(const Geometry& g, int m, bool two, Plan* p) {
     p->t_tiles = (m + 255) / 256;
-    p->n_cols = ((m + p->t_tiles - 1) / p->t_tiles + 15) & ~15;   // equal token tiles
     p->tiles_x = (g.n_pad + kTileN - 1) / kTileN;
-    const long long units = (long long)p->t_tiles * p->tiles_x * g.k_blocks;
+    long long units = (long long)p->t_tiles * p->tiles_x * g.k_blocks;
+    // One to four units an SM and wide parts: parking and summing them costs more than the decode, and half as much for a narrower
+    // tile: twice the token tiles (us at 256 tokens: 2048 x 2048 21.6 -> 18.8, 1024 x 8192 28.5 -> 25.9, 1500 x 4096 24.0 -> 22.6; with
+    // seven units, 4096 x 4096, 26.1 -> 26.8; with less than one, 512 x 2048, 13.6 -> 14.5; 1500 x 4096 at 64 tokens 15.8 -> 18.6).
+    if (m > 128 && units >= sm_count() && units < 4 * sm_count()) { p->t_tiles *= 2; units *= 2; }
+    p->n_cols = ((m + p->t_tiles - 1) / p->t_tiles + 15) & ~15;   // equal token tiles
     if (units >= (1ll << 30)) return false;
     p->units = (int)units;
     p->grid = (int)(units < sm_count() ? units : sm_count());

@@ -103,7 +103,7 @@ def test_ref_solve_edges(goq, n, k, g, b, m):
 @pytest.mark.parametrize("n,k,g,b,m", [
     (1, 8, 8, 3, 17), (129, 136, 8, 3, 33), (127, 256, 16, 4, 32), (128, 128, 128, 3, 64),
     (4000, 384, 128, 3, 65), (257, 1152, 64, 3, 256), (300, 640, 128, 4, 257), (1000, 4096, 32, 3, 511),
-    (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 20)])
+    (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 20), (1100, 2304, 128, 3, 200)])
 def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
     """The kernel between decode and prefill: channel tiles and token tiles that do not fill, one unit in all, one tile shared by
     many SMs and several tiles an SM, both operand forms (exact up to 32 tokens), every bit width; twice, bit for bit.
