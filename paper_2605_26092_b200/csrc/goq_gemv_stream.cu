@@ -411,7 +411,7 @@ static cudaError_t launch_stream(const Geometry& g, const StreamParams& p0, cuda
                         (size_t)(2 * n_stages + 2) * sizeof(uint64_t) + (size_t)p.x_smem_bytes;
     auto kernel = p.x_smem_bytes ? gemv_stream_kernel<WB, NT, CPG, true> : gemv_stream_kernel<WB, NT, CPG, false>;
     static SmemAttrCache smem_attr[2];
-    if (cudaError_t e = ensure_dynamic_smem(kernel, 160 * 1024, smem_attr[p.x_smem_bytes ? 1 : 0])) return e;
+    if (cudaError_t e = ensure_dynamic_smem(kernel, smem > 160 * 1024 ? smem : (size_t)160 * 1024, smem_attr[p.x_smem_bytes ? 1 : 0])) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kStreamThreads);
