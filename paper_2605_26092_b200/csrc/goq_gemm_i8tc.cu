@@ -30,6 +30,7 @@ namespace i8tc {
 using namespace tc;
 
 constexpr int kEpiWarps = 8, kPkWarp = 8, kXWarp = 9, kMmaWarp = 10, kDec0 = 11, kDecWarps = 16;
+constexpr int kDecGroups = 2;   // decoding groups: group i takes the k-blocks u with u % 2 == i
 constexpr int kThreads = (kDec0 + kDecWarps) * 32;
 constexpr int kTokens = 128, kChannels = 64, kStages = 3, kMaxPk = 4;
 constexpr int kABytes = kTokens * 128, kBBytes = 256 * 128, kStageBytes = kBBytes + 2 * kABytes;
@@ -78,6 +79,16 @@ __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
     asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
+// Slots of the packed-record ring: as many as fit. A multiple of the decoding groups, so that a slot always comes round to the same
+// group: a barrier has one phase bit, and a group that does not wait for every phase of a slot may find the one before the last
+// completed, take it for its own and decode the records it left.
+constexpr int kSmemBytes = 227 * 1024 - 2 * 1024;   // the static variables take less than 2 KiB
+constexpr int fixed_bytes(int lut_entry) { return 1024 + kStages * kStageBytes + kLut8Bytes + 256 * lut_entry; }
+constexpr int ring_slots(int unit_bytes, int lut_entry) {
+    const int n = (kSmemBytes - fixed_bytes(lut_entry)) / (4 * unit_bytes);
+    return (n < kMaxPk ? n : kMaxPk) / kDecGroups * kDecGroups;
+}
+
 // W4: |c~ v| <= 2^14 = 85.3 * 192, and |l| <= 96: both digits and their negatives are int8 for every c~, -128 included
 template <int WB> struct Digits { static constexpr int base = WB == 4 ? 192 : 16, entry = WB == 4 ? 32 : 16; };
 // integer of code c (W4: sign << 3 | e): +-2^(emax - e)
@@ -113,7 +124,9 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     unsigned char* pk_ring = ctab + 256 * Digits<WB>::entry;
     const int pk_bytes = 4 * p.unit_bytes;
     __shared__ uint64_t full[kStages], empty[kStages], pk_full[kMaxPk], pk_empty[kMaxPk], tm_full[2], tm_empty[2];
-    __shared__ float2 sc_s[2][2][kChannels];   // per-channel scales of the current tile and the next, a copy per token half
+    // Per-channel scales of the current tile and its neighbours. Both token halves write a tile's (the same values); a half that
+    // has finished tile i + 2 knows the other to be past tile i, whose buffer tile i + 3 takes.
+    __shared__ float2 sc_s[3][kChannels];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
 
@@ -257,7 +270,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         };
         if (group < units) fetch();
         bool ok = true;
-        int slot = group, s = group;   // n_pk >= 2
+        int slot = group, s = group;   // n_pk is even: a slot belongs to one group
         uint32_t pk_par = 0, st_par = 1;   // st_par: parity of the stage's previous release (the first round passes at once)
         for (int u = group; u < units; u += 2) {
             uint32_t cc[GPB];
@@ -334,8 +347,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         if (h2 < p.tt)
         for (int i = 0; i < my_tiles; ++i, tile += gridDim.x) {
             const int ch0 = (tile % p.tiles_x) * kChannels, tok = ((tile / p.tiles_x) * p.tt + h2) * kTokens + quarter * 32 + lane;
-            float2* sc = sc_s[h2][i & 1];
-            // every warp of a token half writes the same values; the readers of this buffer's previous use are two tiles behind
+            float2* sc = sc_s[i % 3];
             if (p.y) {
                 for (int c = lane; c < 64; c += 32) sc[c] = ch0 + c < p.n_out ? *reinterpret_cast<const float2*>(p.sc + (size_t)(ch0 + c) * 2) : make_float2(0.f, 0.f);
             }
@@ -427,10 +439,11 @@ static int sm_count() {
 }
 template <int WB, int GPB>
 static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& x_map, const CUtensorMap& packed_map, cudaStream_t st) {
-    const size_t fixed = 1024 + (size_t)kStages * kStageBytes + kLut8Bytes + 256 * Digits<WB>::entry, pk = (size_t)4 * g.unit_bytes;
-    p.n_pk = (int)((224 * 1024 - fixed) / pk);
-    if (p.n_pk > kMaxPk) p.n_pk = kMaxPk;
-    const size_t smem = fixed + p.n_pk * pk;
+    constexpr int kUnitBytes = kCodeBytesPerUnit + 64 * GPB + (WB == 4 ? kWordsPerBlock : 0), kSlots = ring_slots(kUnitBytes, Digits<WB>::entry);
+    static_assert(kSlots >= kDecGroups && kSlots % kDecGroups == 0, "a slot must belong to one decoding group");
+    if (g.unit_bytes != kUnitBytes) return cudaErrorInvalidValue;
+    p.n_pk = kSlots;
+    const size_t smem = fixed_bytes(Digits<WB>::entry) + (size_t)kSlots * 4 * kUnitBytes;
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_i8tc_kernel<WB, GPB>, smem, smem_attr)) return e;
     cudaLaunchConfig_t cfg = {};

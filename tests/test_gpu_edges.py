@@ -253,11 +253,11 @@ def test_activation_quantizer_edges(goq, m, k, abits, dtype):
 
 @pytest.mark.parametrize("n,k,g,b,m", [(1, 32, 32, 3, 1), (16, 32, 32, 2, 127), (63, 96, 32, 4, 128), (64, 128, 64, 3, 129), (65, 192, 64, 4, 255),
                                        (130, 320, 64, 2, 256), (200, 1024, 128, 3, 257), (72, 416, 32, 3, 300), (8, 1024, 128, 4, 700),
-                                       (4800, 128, 64, 3, 600), (192, 3072, 64, 3, 40000 // 64)])
+                                       (4800, 128, 64, 3, 600), (192, 3072, 64, 3, 40000 // 64), (640, 3072, 32, 3, 4200), (192, 768, 32, 2, 1500)])
 @pytest.mark.parametrize("out", ["f32", "bf16"])
 def test_int8_tensor_core_gemm_edges(goq, n, k, g, b, m, out):
     """The int8 layer on the tensor cores: channel and token tiles that do not fill, one and two token halves a tile, fewer and more tiles
-    than SMs, every bit width and group, coefficients over the whole byte (-128 and 0 among them): accumulators bit-exact, outputs
+    than SMs, every bit width and group, many rounds of the record ring with the largest records, coefficients over the whole byte (-128 and 0 among them): accumulators bit-exact, outputs
     those accumulators give in fp32 (2^-22 of the two terms' magnitudes), bf16 within its rounding."""
     from tests.gpu_util import dev, pack_weights
     rng = np.random.default_rng(n + k + m)
