@@ -349,7 +349,10 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             const int ch0 = (tile % p.tiles_x) * kChannels, tok = ((tile / p.tiles_x) * p.tt + h2) * kTokens + quarter * 32 + lane;
             float2* sc = sc_s[i % 3];
             if (p.y) {
-                for (int c = lane; c < 64; c += 32) sc[c] = ch0 + c < p.n_out ? *reinterpret_cast<const float2*>(p.sc + (size_t)(ch0 + c) * 2) : make_float2(0.f, 0.f);
+                for (int c = lane; c < 64; c += 32) {
+                    const float* src = p.sc + (size_t)(ch0 + c) * 2;   // 4-byte aligned is all that the caller promises
+                    sc[c] = ch0 + c < p.n_out ? make_float2(src[0], src[1]) : make_float2(0.f, 0.f);
+                }
             }
             __syncwarp();
             const float sxk = (p.sx && tok < p.m ? p.sx[tok] : 1.f) * kInvScale;

@@ -284,6 +284,32 @@ def test_int8_tensor_core_gemm_edges(goq, n, k, g, b, m, out):
     assert np.all(np.abs(yh - t[0] - t[1]) <= bound)
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(65, 192, 64, 3, 129), (64, 128, 32, 4, 5), (40, 64, 16, 2, 33)])
+def test_int8_layer_takes_scales_at_any_float_address(goq, n, k, g, b, m):
+    """Scale and output arrays that begin one float behind an aligned address, as slices of larger arrays do: same accumulators and
+    outputs as at an aligned one, from goq_gemm and from the requantising entry point."""
+    from tests.gpu_util import dev, pack_weights
+    rng = np.random.default_rng(n)
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    cq = dev(rng.integers(-127, 128, size=(n, k // g, 2)).astype(np.int8))
+    x = dev(rng.integers(-127, 128, size=(m, k)).astype(np.int8))
+    sx, sc = rng.uniform(0.5, 2, size=m).astype(np.float32), rng.uniform(-1, 1, size=(n, 2)).astype(np.float32)
+    got = []
+    for shift in (0, 1):
+        zeros = np.zeros((m, n), dtype=np.float32)
+        y, h = _unaligned(zeros, shift), _unaligned(zeros, shift)
+        acc = _unaligned(np.zeros((2, m, n), dtype=np.int32), shift)
+        amax, sy = _unaligned(np.zeros(m, dtype=np.float32), shift), _unaligned(np.zeros(m, dtype=np.float32), shift)
+        yq = _unaligned(np.zeros((m, n), dtype=np.int8), shift)
+        sxd, scd = _unaligned(sx, shift), _unaligned(sc, shift)
+        goq.gemm(d, packed, x, m, goq.I8, y=y, y_dtype=goq.F32, sx=sxd, cq=cq, sc=scd, acc=acc)
+        goq.gemm_i8_requant(d, packed, x, m, sxd, cq, scd, h, amax, yq, sy)
+        torch.cuda.synchronize()
+        got.append([t.cpu().numpy().copy() for t in (y, acc, h, amax, yq, sy)])
+    assert got[0][1].any() and all(np.array_equal(a, c) for a, c in zip(*got))
+
+
 @pytest.mark.parametrize("k,n,inner,m,g,b", [(256, 64, 512, 1, 64, 3), (1024, 256, 2816, 4, 128, 3), (128, 128, 256, 3, 32, 2), (4096, 1024, 11008, 4, 128, 3),
                                              (2048, 2048, 4096, 7, 128, 3), (512, 128, 1408, 2, 128, 2)])
 def test_chain_shares_staged_activations(goq, k, n, inner, m, g, b):
