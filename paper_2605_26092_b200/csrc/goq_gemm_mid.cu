@@ -502,7 +502,8 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_mid_kernel<WB, TWO, GL>, p, map, pmap)) return e;
-    if (p.units % pl.grid == 0 && (p.units / pl.grid) % g.k_blocks == 0) return cudaSuccess;   // whole tiles only
+    // whole tiles only: one k-block a tile, or every range a whole number of tiles
+    if (g.k_blocks == 1 || (p.units % pl.grid == 0 && (p.units / pl.grid) % g.k_blocks == 0)) return cudaSuccess;
     const FinishParams f = {p.partial, p.inv_scale, y, y_dtype, g.n_out, m, pl.n_cols, pl.tiles_x, g.k_blocks, pl.units, pl.grid};
     cfg.gridDim = dim3(pl.tiles_x * pl.t_tiles, (pl.n_cols + kFinishTokens - 1) / kFinishTokens);
     cfg.blockDim = dim3(kFinishThreads);

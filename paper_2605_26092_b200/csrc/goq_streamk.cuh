@@ -78,16 +78,17 @@ static __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const Fin
     // that CTA's first)
     const int c_lo = (int)((((long long)tile * p.k_blocks + 1) * p.n_ctas - 1) / p.units);
     const int c_hi = (int)((((long long)(tile + 1) * p.k_blocks) * p.n_ctas - 1) / p.units);
-    if (c_lo == c_hi) return;   // one CTA had the whole tile and has stored it
     const int slot = range_begin(c_lo, p.units, p.n_ctas) == tile * p.k_blocks ? 0 : 1;
     const int tok0 = (tile / p.tiles_x) * p.n_cols, cols = min(p.n_cols, p.m - tok0);
     const int col = blockIdx.y * kFinishTokens + (threadIdx.x >> 5);
-    if (col >= cols) return;
     const int col2 = min(col + kFinishTokens / 2, cols - 1);
     const size_t park = (size_t)p.n_cols * kTileN, stride = 2 * park;
     const float* lo = p.partial + ((size_t)c_lo * 2 + slot) * park + ch;
     const float* rest = p.partial + (size_t)(c_lo + 1) * stride + ch;
+    // Every CTA waits, also one that finds nothing to add: what follows on the stream is ordered behind this grid alone, and a grid of
+    // CTAs that return at once would be complete while the kernel before it still runs.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (c_lo == c_hi || col >= cols) return;   // one CTA had the whole tile and has stored it; no such token
     float4 f0 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col * kTileN));
     float4 f1 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col2 * kTileN));
     const float s0 = __ldcg(p.scale + tok0 + col), s1 = __ldcg(p.scale + tok0 + col2);

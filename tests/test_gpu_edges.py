@@ -130,6 +130,36 @@ def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
     check_parity(out[0].astype(np.float64), y_ref, 2e-5 if exact else 5e-4, 1e-4 if exact else 2e-3)
 
 
+@pytest.mark.parametrize("n,k,g,m", [(20000, 128, 128, 64), (20000, 64, 64, 200), (3000, 256, 128, 40), (1024, 2048, 128, 250)])
+def test_mid_batch_gemm_back_to_back_on_one_scratch_buffer(goq, n, k, g, m):
+    """Calls that follow one another without a wait in between: the second overwrites the fp16 activations and the parked parts of the
+    first, and a copy on the same stream reads each output. One k-block (no tile is shared, nothing to add behind the kernel) with
+    more units than SMs, and shapes with shared tiles. Every output as from a call of its own, bit for bit."""
+    from tests.gpu_util import dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, 3, seed=n + k)
+    d, packed = pack_weights(n, k, g, 3, codes, meta, coef)
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+    xs = [dev(si.bf16_activations(m, k, seed=s)) for s in range(4)]
+    y = torch.empty((m, n), dtype=torch.float32, device="cuda")
+    alone = []
+    prev = goq.set_gemv_variant(4)
+    try:
+        for x in xs:
+            goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+            torch.cuda.synchronize()
+            alone.append(y.clone())
+        for _ in range(10):
+            got = []
+            for x in xs:
+                goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+                got.append(y.clone())
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, c) for a, c in zip(got, alone))
+    finally:
+        goq.set_gemv_variant(prev)
+    assert goq.workspace_status(ws) == goq.OK
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
