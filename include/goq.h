@@ -142,7 +142,7 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
  *      to fp16 (normwise output error about 1.5e-4 to 2.5e-4). The coefficients of every output channel are scaled by a
  *      power of two taken from the channel's largest |c1|, |c2| before that rounding and the output is scaled back, so
  *      the result does not depend on the magnitude of the weights; inside one channel, coefficients more than 2^13
- *      below the channel's largest lose precision to fp16's range. Weights are fetched early, as in goq_gemv.
+ *      below the channel's largest lose precision to fp16's range.
  *  x_dtype GOQ_I8 (Eq. 4 with integer X~ and c~; left shifts x~ << (emax-e), exact int32):
  *      x    [m][k_in] int8         sx [m] fp32 per-token scale
  *      cq   [n_out][k_in/group][2] int8 integer coefficients,  sc [n_out][2] fp32 their per-channel scales
@@ -150,8 +150,8 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
  *      y    out, optional: [m][n_out] = sx[m] * 2^-emax * (sc[n][0]*ACC_1 + sc[n][1]*ACC_2)
  *    At least one of acc, y must be given. Returns GOQ_ERR_OVERFLOW_BOUND if k_in*127*127*2^emax >= 2^31 (W3: k_in up
  *    to 16642; W4, emax = 7: k_in up to 1040). Groups of 16 run on the packed-dot-product kernel, larger ones on the int8
- *    tensor cores. Needs no scratch; if ws is given, a give-up of a bounded wait is reported in its status word. Weights are
- *    fetched early, as in goq_gemv. */
+ *    tensor cores. Needs no scratch; if ws is given, a give-up of a bounded wait is reported in its status word.
+ *  Stream order: every argument, the packed weights among them, is read and written in plain stream order. */
 goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int m, int x_dtype,
                     const float* sx, const int8_t* cq, const float* sc, void* y, int y_dtype,
                     int32_t* acc, void* ws, size_t ws_bytes, void* stream);

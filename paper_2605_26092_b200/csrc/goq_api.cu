@@ -146,7 +146,7 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         if (variant == 3) return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
     }
     if (variant == 0 && goq::gemv_mma_supported(g, batch))
-        return from_cuda(goq::launch_gemv_mma(g, packed, x_bf16, batch, y, y_dtype, (cudaStream_t)stream));
+        return from_cuda(goq::launch_gemv_mma(g, packed, x_bf16, batch, y, y_dtype, true, (cudaStream_t)stream));
     bool use_mma = goq::linear_mma_supported(g);
     if (variant == 1) use_mma = false;
     if (variant == 2 && !use_mma) return GOQ_ERR_UNSUPPORTED;
@@ -191,7 +191,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
             for (int t0 = 0; t0 < m; t0 += 16) {
                 const int nb = (m - t0 < 16) ? (m - t0) : 16;
                 cudaError_t e = goq::launch_gemv_mma(g, packed, (const uint16_t*)x + (size_t)t0 * g.k_in, nb,
-                                                     (uint8_t*)y + (size_t)t0 * g.n_out * ybytes, y_dtype, (cudaStream_t)stream);
+                                                     (uint8_t*)y + (size_t)t0 * g.n_out * ybytes, y_dtype, false, (cudaStream_t)stream);
                 if (e != cudaSuccess) return from_cuda(e);
             }
             return GOQ_OK;

@@ -133,7 +133,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     const int my_tiles = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, units = my_tiles * p.k_blocks;
 
-    // packed records of the CTA's tiles, k-block by k-block; the ring is filled before anything else
+    // packed records of the CTA's tiles, k-block by k-block
     struct { int tile, kb, slot, round, issued; } pk = {(int)blockIdx.x, 0, 0, 0, 0};
     auto pk_issue = [&]() {
         mbar_expect_tx(&pk_full[pk.slot], (uint32_t)pk_bytes);   // (rows past the last tile arrive as zeros)
@@ -145,7 +145,6 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     if (warp == kPkWarp && lane == 0) {
         for (int i = 0; i < kMaxPk; ++i) { mbar_init(&pk_full[i], 1); mbar_init(&pk_empty[i], 8); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        while (pk.issued < units && pk.round == 0) pk_issue();
     }
     if (tid == 0) {
         abort_flag = 0;
@@ -180,14 +179,14 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the packed weights, like everything else, only after earlier kernels
     const uint32_t tmem_base = tmem_slot;
 
     if (warp == kPkWarp) {
         if (lane == 0) {
             bool ok = true;
             while (pk.issued < units && ok) {
-                ok = mbar_wait(&pk_empty[pk.slot], (pk.round - 1) & 1, &abort_flag);
+                if (pk.round > 0) ok = mbar_wait(&pk_empty[pk.slot], (pk.round - 1) & 1, &abort_flag);
                 if (ok) pk_issue();
             }
             if (!ok || abort_flag)

@@ -379,8 +379,10 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f16_kernel(const uint16_t* 
                                                                 const uint8_t* __restrict__ packed, int unit_bytes, int k_blocks,
                                                                 int groups_per_block, uint32_t* __restrict__ row_scale,
                                                                 float* __restrict__ row_inv) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the GEMM's CTAs may set themselves up meanwhile
-    asm volatile("griddepcontrol.wait;" ::: "memory");                // (launched as a dependent itself: what precedes it is complete)
+    // Launched as a dependent itself. It lets its own dependents in only when everything before it is complete: the GEMM's CTAs may then
+    // read the packed weights at once, in stream order, and set themselves up beside this pass.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if ((int)blockIdx.x >= m_total) {
         __shared__ uint32_t part_max[kPrepThreads / 16][16];
         const int T = (int)blockIdx.x - m_total, r = threadIdx.x & 15, part = threadIdx.x >> 4;

@@ -10,7 +10,7 @@
 // than 40 KB of activations every fragment then came from L2 (4096 x 4096, 8 tokens: 13.9 us). A tile's k-blocks are split
 // over the warps of a CTA and, where the tiles are fewer than the chip wants, over the CTAs of a cluster; sums are added in warp
 // order, then in rank order through distributed shared memory: deterministic, and no scratch.
-// The launch is a programmatic dependent: tables and first records are fetched while the kernel before still runs.
+// The launch is a programmatic dependent: tables and, in goq_gemv, first records are fetched while the kernel before still runs.
 // Bound: instruction issue of the decode (about 280 a record) and, with one or two CTAs a SM, the last wave. 128 registers and 16 warps a
 // SM beat 80 and 24 (spills). Measured, W3 g128: 256 x 256 2.3 us (streaming kernel 5.8), 4096 x 4096 6.4 us at 8 tokens and 8.2
 // at 16 (13.9, 15.5), 8192 x 8192 21.7 and 27.3 (30.0, 36.8); W4 26.3 at 8 tokens (the earlier fragment kernel 34.4).
@@ -28,6 +28,7 @@ struct Params {
     const uint16_t* x;
     void* y;
     int unit_bytes, meta_off, y_dtype, n_out, k_in, k_blocks, m, cluster;
+    int early;   // records may be read before the kernels ahead on the stream are complete
 };
 
 // weights of a record as a lane holds them: 8 micro-block words, (W4) their records, the coefficient pairs of rows g and g + 8
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) gemv_mma_kernel(const Param
     const uint8_t* unit = p.packed + unit_offset(T, kb0 + warp, p.k_blocks, p.unit_bytes);
     const size_t step = (size_t)n_warps * p.unit_bytes;
 
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     Record<WB, GPB> next;
     int bk = kb0 + warp;
     if (bk < kb1) next.load(unit, p.meta_off);
@@ -245,11 +247,11 @@ static cudaError_t launch(const Geometry& g, Params& p, cudaStream_t st) {
 
 bool gemv_mma_supported(const Geometry& g, int m) { return g.group >= 32 && m <= 16 && g.n_tiles < (1 << 27); }
 
-cudaError_t launch_gemv_mma(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, cudaStream_t st) {
+cudaError_t launch_gemv_mma(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, bool early, cudaStream_t st) {
     gmma::Params p;
     p.packed = (const uint8_t*)packed; p.x = (const uint16_t*)x; p.y = y;
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.y_dtype = y_dtype; p.n_out = g.n_out; p.k_in = g.k_in;
-    p.k_blocks = g.k_blocks; p.m = m;
+    p.k_blocks = g.k_blocks; p.m = m; p.early = early ? 1 : 0;
 #define GOQ_GMMA_NT(WB_, NT_) \
     (g.group == 32 ? gmma::launch<WB_, NT_, 1>(g, p, st) : g.group == 64 ? gmma::launch<WB_, NT_, 2>(g, p, st) : gmma::launch<WB_, NT_, 4>(g, p, st))
 #define GOQ_GMMA(WB_) (m <= 8 ? GOQ_GMMA_NT(WB_, 1) : GOQ_GMMA_NT(WB_, 2))

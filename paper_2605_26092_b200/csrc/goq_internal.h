@@ -37,8 +37,9 @@ cudaError_t launch_linear_mma(const Geometry& g, const void* packed, const void*
 bool linear_mma_supported(const Geometry& g);
 
 // Decode GEMV on bf16 fragments straight from global memory (group >= 32, wbits 2..4, m <= 16); no scratch (goq_gemv_mma.cu).
+// early: the first weights may be read before earlier kernels of the stream are complete.
 bool gemv_mma_supported(const Geometry& g, int m);
-cudaError_t launch_gemv_mma(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, cudaStream_t st);
+cudaError_t launch_gemv_mma(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, bool early, cudaStream_t st);
 
 // Decode GEMV, streaming kernel (group >= 32, wbits <= 3, m <= 16). `ws` holds gemv_stream_workspace(g)
 // bytes whose tile counters are zero on entry (goq_workspace_init) and are left zero on return.
