@@ -234,11 +234,12 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
                             umma_i8(tmem_base + h * 256, ad + h * (kABytes >> 4) + 2 * ks, bd + 2 * ks, (kb > 0 || ks > 0) ? 1u : 0u);
+                        // the stage first: once the last tile's epilogue has its accumulators no arrival is outstanding
+                        if (h == p.tt - 1) umma_commit(&empty[s]);
                         if (kb == p.k_blocks - 1) umma_commit(&tm_full[h]);
                     }
                 }
                 if (!ok) break;
-                if (leader) umma_commit(&empty[s]);
                 __syncwarp();
                 s = s_next; par = par_next;
             }
@@ -364,6 +365,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
 #pragma unroll 1
             for (int c0 = 0; c0 < 64; c0 += 8) {
                 int h[8], l[8], a1[8], a2[8];
+                __syncwarp();   // lanes without a token skip the stores: the warp reads tensor memory as one
                 tmem_ld8(ta + c0, h); tmem_ld8(ta + 64 + c0, l);
                 tmem_ld8(ta + 128 + c0, a1); tmem_ld8(ta + 192 + c0, a2);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");

@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         const uint32_t taddr = tmem_base + (uint32_t)(q & 1) * 256u + ((uint32_t)(quarter * 32) << 16);
         for (int c0 = first; c0 < cols; c0 += step) {
             float v[16];
+            __syncwarp();   // lanes without a channel skip the stores: the warp reads tensor memory as one
             tmem_sum16(taddr + c0, p.na, 256u / (uint32_t)p.na, v);
             if (!whole) {
 #pragma unroll

@@ -289,6 +289,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
             for (int cb = 0; cb < n_cb && ok; ++cb) {
                 uint32_t v[32];
                 const int col0 = col_half * 256 + cb * 32;
+                __syncwarp();   // the stores before may have diverged: the warp reads tensor memory as one
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)col0, v);
                 float* st = reinterpret_cast<float*>(b_tiles) + (col_half * 2 + (cb & 1)) * (32 * kTileN);
                 const float irs = row_i[q * 32 + lane];   // this lane's channel: undo the coefficient scale (a power of two)
