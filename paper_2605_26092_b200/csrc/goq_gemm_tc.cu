@@ -368,7 +368,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap x_map) {
 
 // ---- activation pre-pass: bf16 -> scaled fp16, one CTA per token ------------------------------------
 // xh[tok][k] = fp16(x[tok][k] * 2^s), inv_scale[tok] = 2^-s, s chosen from the exponent field of the token's largest
-// magnitude (an all-zero token gets the largest scale, harmlessly; inf / nan stay inf / nan).
+// magnitude (an all-zero token gets the largest scale, harmlessly). Finite elements never reach fp16's top; inf / nan stay inf / nan and
+// make the token's outputs that.
 constexpr int kPrepThreads = 256;
 constexpr int kPrepHold = 6;   // 16-byte vectors a thread keeps: rows up to 12288
 // Blocks beyond the tokens compute the per-channel scales of the weight operand, one 16-row tile each: w_hat is

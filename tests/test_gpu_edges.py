@@ -160,6 +160,28 @@ def test_mid_batch_gemm_back_to_back_on_one_scratch_buffer(goq, n, k, g, m):
     assert goq.workspace_status(ws) == goq.OK
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(300, 512, 128, 3, 16), (300, 512, 128, 3, 17), (129, 256, 64, 4, 32), (200, 384, 16, 2, 20), (300, 512, 128, 3, 100),
+                                       (256, 136, 8, 4, 60), (128, 1024, 128, 3, 700)])
+def test_gemm_non_finite_activations_stay_with_their_token(goq, n, k, g, b, m):
+    """A token with an infinite element and one with a NaN: every output of theirs is non-finite (an infinity times a weight is one, times
+    the zero state NaN); the other tokens' outputs do not change by a bit."""
+    from tests.gpu_util import pack_weights, run_gemm_bf16
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    clean = run_gemm_bf16(d, packed, xb)
+    bad = xb.copy()
+    bad[1, 5], bad[m - 1, k - 1], bad[m // 2, k // 2] = 0x7F80, 0xFF80, 0x7FC0   # +inf, -inf, NaN
+    got = run_gemm_bf16(d, packed, bad)
+    hit = sorted({1, m // 2, m - 1})
+    rest = [t for t in range(m) if t not in hit]
+    assert np.isfinite(clean).all() and not np.isfinite(got[hit]).any()
+    assert np.isnan(got[m // 2]).all()
+    assert np.array_equal(got[rest], clean[rest])
+    yh = run_gemm_bf16(d, packed, bad, goq.BF16)
+    assert not np.isfinite(yh[hit]).any() and np.isfinite(yh[rest]).all()
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
