@@ -150,7 +150,8 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
  *      y    out, optional: [m][n_out] = sx[m] * 2^-emax * (sc[n][0]*ACC_1 + sc[n][1]*ACC_2)
  *    At least one of acc, y must be given. Returns GOQ_ERR_OVERFLOW_BOUND if k_in*127*127*2^emax >= 2^31 (W3: k_in up
  *    to 16642; W4, emax = 7: k_in up to 1040). Groups of 16 run on the packed-dot-product kernel, larger ones on the int8
- *    tensor cores. Needs no scratch; if ws is given, a give-up of a bounded wait is reported in its status word.
+ *    tensor cores. Needs no scratch; if ws is given, a give-up of a bounded wait is reported in its status
+ *    word (without one it cannot be seen: acc and y are then partly unwritten).
  *  Stream order: every argument, the packed weights among them, is read and written in plain stream order. */
 goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int m, int x_dtype,
                     const float* sx, const int8_t* cq, const float* sc, void* y, int y_dtype,
@@ -171,7 +172,8 @@ goq_status goq_quantize_activations(const void* x, int x_dtype, int m, int k, in
  * largest |y| recorded by the GEMM's epilogue, and - when yq, sy are given - y requantised to the next layer's int8
  * activations with goq_quantize_activations' arithmetic (one more kernel that reads y once).
  *   x, sx, cq, sc as in goq_gemm;  y out [m][n_out] fp32;  amax out [m] fp32 (cleared by the call);
- *   yq out [m][n_out] int8 and sy out [m] fp32, both or neither. */
+ *   yq out [m][n_out] int8 and sy out [m] fp32, both or neither.
+ * If a bounded wait on the device gives up, every element of amax (and of sy) is NaN. */
 goq_status goq_gemm_i8_requant(const goq_desc* desc, const void* packed, const int8_t* x, int m, const float* sx,
                                const int8_t* cq, const float* sc, float* y, float* amax, int8_t* yq, float* sy, void* stream);
 
@@ -307,7 +309,8 @@ int goq_last_cuda_error(void);
  * 5 = integer-operand kernel of one linear (goq_gemv). Process-wide. Returns the previous value. */
 int goq_set_gemv_variant(int variant);
 
-/* Bound, in polls, of every device-side wait of goq_gemv_sequence (tests only; 0 restores the kernel's own bound).
+/* Bound, in polls, of every device-side wait of goq_gemv_sequence, of goq_gemv's integer-operand kernel and of the integer layer on the
+ * tensor cores (tests only; 0 restores the kernels' own bounds).
  * With a bound of a few polls a dependent chain gives up at once: the call returns GOQ_OK (it only enqueues), the
  * status word then reads GOQ_ERR_TIMEOUT, the context stays usable. Process-wide. Returns the previous value. */
 int goq_set_wait_limit(int polls);

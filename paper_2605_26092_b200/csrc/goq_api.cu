@@ -225,7 +225,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (goq_status s = check_arch()) return s;
         int* status = (ws && aligned(ws, 256) && ws_bytes >= goq::kWsStatusBytes) ? (int*)ws : nullptr;   // needs no scratch; reports there if it may
         return from_cuda(goq::launch_gemm_a8(g, packed, (const int8_t*)x, m, sx, cq, sc, y, y_dtype, acc, nullptr, status,
-                                             (cudaStream_t)stream));
+                                             g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
     }
     return GOQ_ERR_INVALID_ARG;
 }
@@ -244,7 +244,8 @@ goq_status goq_gemm_i8_requant(const goq_desc* desc, const void* packed, const i
     if (goq_status s = check_arch()) return s;
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaError_t e = cudaMemsetAsync(amax, 0, (size_t)m * sizeof(float), st)) return from_cuda(e);
-    if (cudaError_t e = goq::launch_gemm_a8(g, packed, x, m, sx, cq, sc, y, GOQ_F32, nullptr, amax, nullptr, st)) return from_cuda(e);
+    if (cudaError_t e = goq::launch_gemm_a8(g, packed, x, m, sx, cq, sc, y, GOQ_F32, nullptr, amax, nullptr,
+                                               g_wait_limit.load(std::memory_order_relaxed), st)) return from_cuda(e);
     if (yq) return from_cuda(goq::launch_quantize_act(y, GOQ_F32, m, g.n_out, 8, amax, yq, sy, st));
     return GOQ_OK;
 }

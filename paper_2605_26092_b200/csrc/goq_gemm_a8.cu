@@ -161,9 +161,9 @@ gemm_a8_dp4a_kernel(const uint8_t* __restrict__ packed, int unit_bytes, const in
 
 cudaError_t launch_gemm_a8(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx,
                            const int8_t* cq, const float* sc, void* y, int y_dtype, int32_t* acc, float* amax, int* status,
-                           cudaStream_t st) {
+                           int spin_limit, cudaStream_t st) {
     auto* words = (const uint8_t*)packed;
-    if (gemm_i8tc_supported(g, m)) return launch_gemm_i8tc(g, packed, x, m, sx, cq, sc, y, y_dtype, acc, amax, status, st);
+    if (gemm_i8tc_supported(g, m)) return launch_gemm_i8tc(g, packed, x, m, sx, cq, sc, y, y_dtype, acc, amax, status, spin_limit, st);
     dim3 grid(g.n_tiles, (m + kA8Tokens - 1) / kA8Tokens), block(kA8Tokens);
 #define GOQ_A8_DP4A(WB_)                                                                                                    \
     gemm_a8_dp4a_kernel<WB_><<<grid, block, 0, st>>>(words, g.unit_bytes, x, sx, cq, sc, y, y_dtype, acc, amax, g.n_out, g.k_in, \

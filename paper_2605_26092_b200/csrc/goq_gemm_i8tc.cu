@@ -19,8 +19,8 @@
 // copy per 64 channels x 128 k), 9 activation tiles (TMA), 10 MMA issue, 11-26 decode: two groups of eight alternate k-blocks, warp (e, v)
 // of a group takes rows 8 v .. of record e. Bound: shared-memory bandwidth (per 64 x 256 x 128: operand reads of the MMAs ~770 clocks, digit
 // stores, lookups and copies ~900). With 128 x 128 tiles the second part was twice that and the kernel ran at its sum (98 %).
-// Every mbarrier wait is bounded; a CTA that gives up leaves its outputs unwritten and reports GOQ_ERR_TIMEOUT where it is given a
-// status word.
+// Every mbarrier wait is bounded; a CTA that gives up leaves its outputs unwritten, reports GOQ_ERR_TIMEOUT where it is given a
+// status word, and makes every token's largest magnitude NaN where those are recorded (the caller without scratch sees that).
 #include "goq_tc_core.cuh"
 #include "goq_internal.h"
 
@@ -46,6 +46,7 @@ struct Params {
     int* status;
     int unit_bytes, meta_off, k_blocks, groups_in, n_out, m, y_dtype, tiles_x, tiles, n_pk;
     int tt;   // M = 128 operands per tile: 1 or 2
+    int spin;   // bound of every wait, in polls
 };
 
 // kind::i8: s8 x s8 -> s32, both K-major, M = 128, N = 256
@@ -186,12 +187,9 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         if (lane == 0) {
             bool ok = true;
             while (pk.issued < units && ok) {
-                if (pk.round > 0) ok = mbar_wait(&pk_empty[pk.slot], (pk.round - 1) & 1, &abort_flag);
+                if (pk.round > 0) ok = mbar_wait(&pk_empty[pk.slot], (pk.round - 1) & 1, &abort_flag, p.spin);
                 if (ok) pk_issue();
             }
-            if (!ok || abort_flag)
-                for (int i = pk.issued > p.n_pk ? pk.issued - p.n_pk : 0; i < pk.issued; ++i)
-                    for (int it = 0; it < kSpin && !mbar_try(&pk_full[i % p.n_pk], (uint32_t)(i / p.n_pk) & 1u); ++it) { }
         }
     } else if (warp == kXWarp) {
         if (lane == 0) {
@@ -200,14 +198,12 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x)
                 for (int kb = 0; kb < p.k_blocks; ++kb, ++u) {
                     const int s = u % kStages;
-                    if (u >= kStages) ok = mbar_wait(&empty[s], ((u / kStages) - 1) & 1, &abort_flag);
+                    if (u >= kStages) ok = mbar_wait(&empty[s], ((u / kStages) - 1) & 1, &abort_flag, p.spin);
                     if (!ok) break;
                     mbar_expect_tx(&full[s], (uint32_t)(p.tt * kABytes));
                     for (int i = 0; i < p.tt; ++i)
                         tma_load_2d(stages + s * kStageBytes + kBBytes + i * kABytes, &x_map, kb * kBlockK, ((tile / p.tiles_x) * p.tt + i) * kTokens, &full[s]);
                 }
-            if (!ok || abort_flag)   // as in the mid-batch kernel: a millisecond, which no copy takes
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);
         }
     } else if (warp == kMmaWarp) {
         const uint64_t bdesc0 = smem_desc_sw128(s32(stages)), adesc0 = smem_desc_sw128(s32(stages + kBBytes));
@@ -217,7 +213,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         uint32_t par = 0;
         for (int i = 0; i < my_tiles && ok; ++i) {
             for (int kb = 0; kb < p.k_blocks; ++kb) {
-                if (!ready) ok = mbar_wait(&full[s], par, &abort_flag);
+                if (!ready) ok = mbar_wait(&full[s], par, &abort_flag, p.spin);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 const int s_next = s + 1 == kStages ? 0 : s + 1;
@@ -226,7 +222,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
                 const uint64_t ad = adesc0 + (uint32_t)(s * (kStageBytes >> 4)), bd = bdesc0 + (uint32_t)(s * (kStageBytes >> 4));
                 for (int h = 0; h < p.tt; ++h) {   // 128 tokens each
                     if (kb == 0 && i > 0) {
-                        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_empty[h], (i - 1) & 1, &abort_flag));
+                        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_empty[h], (i - 1) & 1, &abort_flag, p.spin));
                         if (!ok) break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -277,7 +273,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
 #pragma unroll
             for (int jj = 0; jj < GPB; ++jj) cc[jj] = next_c[jj];
             if (u + 2 < units) fetch();
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&pk_full[slot], pk_par, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&pk_full[slot], pk_par, &abort_flag, p.spin));
             if (!ok) break;
             const uint32_t unit = after_wait(s32(pk_ring) + slot * pk_bytes + e * p.unit_bytes);
             const uint4 wv = lds128(unit + v * 512 + lane * 16);
@@ -286,7 +282,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             const bool odd = flip != 0;
             const uint32_t w[4] = {odd ? wv.z : wv.x, odd ? wv.w : wv.y, odd ? wv.x : wv.z, odd ? wv.y : wv.w};
             if constexpr (WB == 4) mv = odd ? __funnelshift_l(mv, mv, 16) : mv;
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], st_par, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], st_par, &abort_flag, p.spin));
             if (!ok) break;
             const uint32_t at = s32(stages) + (uint32_t)(s * kStageBytes);
 #pragma unroll
@@ -356,7 +352,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
             }
             __syncwarp();
             const float sxk = (p.sx && tok < p.m ? p.sx[tok] : 1.f) * kInvScale;
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[h2], i & 1, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[h2], i & 1, &abort_flag, p.spin));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + h2 * 256;
@@ -426,11 +422,19 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
         }
     }
     __syncthreads();
+    if (abort_flag) {
+        // Copies and MMAs in flight must land before shared and tensor memory go away. Their barriers may count arrivals that never come,
+        // so this waits a time that none of them takes (a millisecond).
+        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+        if (tid == 0 && p.status) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
+        if (p.amax)   // NaN is the largest of the non-negative floats' bit patterns: it stays, and the quantizer behind passes it on
+            for (int tok = tid; tok < p.m; tok += kThreads) atomicMax(reinterpret_cast<int*>(p.amax) + tok, 0x7FC00000);
+        __syncthreads();
+    }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem_dealloc<512>(tmem_base);
     }
-    if (tid == 0 && abort_flag && p.status) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
 
 static int sm_count() {
@@ -468,7 +472,7 @@ static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& x_map
 bool gemm_i8tc_supported(const Geometry& g, int m) { return g.group >= 32 && g.k_in % 16 == 0 && tc::packed_map_supported(g) && m >= 1; }
 
 cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx, const int8_t* cq, const float* sc,
-                             void* y, int y_dtype, int32_t* acc, float* amax, int* status, cudaStream_t st) {
+                             void* y, int y_dtype, int32_t* acc, float* amax, int* status, int spin_limit, cudaStream_t st) {
     CUtensorMap xm, pm;
     if (cudaError_t e = tc::encode_i8_map(&xm, x, g.k_in, m, i8tc::kTokens)) return e;
     if (cudaError_t e = tc::encode_packed_map(&pm, packed, g, 4)) return e;
@@ -482,6 +486,7 @@ cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t
     p.tt = p.tiles_x * ((half_tiles + 1) / 2) >= i8tc::sm_count() ? 2 : 1;
     p.tiles = p.tiles_x * ((half_tiles + p.tt - 1) / p.tt);
     p.status = status;
+    p.spin = spin_limit > 0 ? spin_limit : tc::kSpin;
 #define GOQ_I8TC(WB_)                                                                                                       \
     (g.groups_per_block == 1 ? i8tc::launch<WB_, 1>(g, p, xm, pm, st) : g.groups_per_block == 2 ? i8tc::launch<WB_, 2>(g, p, xm, pm, st) \
                                                                                                : i8tc::launch<WB_, 4>(g, p, xm, pm, st))

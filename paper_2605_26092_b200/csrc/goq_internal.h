@@ -100,15 +100,16 @@ cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x
                             bool exact, cudaStream_t st);
 
 // Integer-activation layer.
-// amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch).
+// amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch); NaN after a
+// give-up. spin_limit > 0 replaces the bound of every device-side wait (tests).
 cudaError_t launch_gemm_a8(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx,
                            const int8_t* cq, const float* sc, void* y, int y_dtype, int32_t* acc, float* amax, int* status,
-                           cudaStream_t st);
+                           int spin_limit, cudaStream_t st);
 
 // The same on tcgen05 (goq_gemm_i8tc.cu), group >= 32, any wbits.
 bool gemm_i8tc_supported(const Geometry& g, int m);
 cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t* x, int m, const float* sx, const int8_t* cq, const float* sc,
-                             void* y, int y_dtype, int32_t* acc, float* amax, int* status, cudaStream_t st);
+                             void* y, int y_dtype, int32_t* acc, float* amax, int* status, int spin_limit, cudaStream_t st);
 
 // The steps before the inner product (goq_quant.cu).
 cudaError_t launch_quantize_geo(const Geometry& g, const float* w, uint8_t* codes, uint8_t* meta, uint16_t* coef, cudaStream_t st);

@@ -38,8 +38,8 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
         : "=r"(ok) : "r"(s32(b)), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-    for (int it = 0; it < kSpin; ++it) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, int limit = kSpin) {
+    for (int it = 0; it < limit; ++it) {
         if (mbar_try(b, parity)) return true;
         if ((it & 63) == 63 && *abort_flag) return false;
     }

@@ -202,7 +202,8 @@ def set_gemv_variant(variant: int) -> int:
 
 
 def set_wait_limit(polls: int) -> int:
-    """goq_set_wait_limit: bound of the device-side waits of goq_gemv_sequence (tests only; 0 = the kernel's own)."""
+    """goq_set_wait_limit: bound of the device-side waits of the decode chain, the integer-operand decode kernel and the integer layer
+    (tests only; 0 = the kernels' own)."""
     return lib().goq_set_wait_limit(polls)
 
 

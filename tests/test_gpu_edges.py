@@ -362,6 +362,41 @@ def test_int8_layer_takes_scales_at_any_float_address(goq, n, k, g, b, m):
     assert got[0][1].any() and all(np.array_equal(a, c) for a, c in zip(*got))
 
 
+def test_int8_layer_reports_a_wait_that_runs_out(goq):
+    """With one poll a wait the epilogue of 128 k-blocks runs out of it: the status word of goq_gemm reads GOQ_ERR_TIMEOUT, and the
+    requantising entry point, which has no scratch, returns NaN magnitudes and scales. The next calls are right again."""
+    from tests.gpu_util import dev, pack_weights
+    rng = np.random.default_rng(1)
+    n, k, g, b, m = 256, 16384, 128, 3, 300
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=1)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    cq = dev(rng.integers(-127, 128, size=(n, k // g, 2)).astype(np.int8))
+    x = dev(rng.integers(-127, 128, size=(m, k)).astype(np.int8))
+    sx, sc = torch.rand(m, device="cuda") + 0.5, torch.rand((n, 2), device="cuda") + 0.1
+    ws = torch.zeros(1024, dtype=torch.uint8, device="cuda")
+
+    def call():
+        y, h = torch.zeros((m, n), device="cuda"), torch.zeros((m, n), device="cuda")
+        amax, sy, yq = torch.zeros(m, device="cuda"), torch.zeros(m, device="cuda"), torch.zeros((m, n), dtype=torch.int8, device="cuda")
+        goq.gemm(d, packed, x, m, goq.I8, y=y, y_dtype=goq.F32, sx=sx, cq=cq, sc=sc, ws=ws)
+        goq.gemm_i8_requant(d, packed, x, m, sx, cq, sc, h, amax, yq, sy)
+        torch.cuda.synchronize()
+        return y, h, amax, sy, yq
+    good = call()
+    assert goq.workspace_status(ws) == goq.OK and torch.isfinite(good[2]).all() and torch.equal(good[0], good[1])
+    goq.set_wait_limit(1)
+    try:
+        cut = call()
+    finally:
+        goq.set_wait_limit(0)
+    assert goq.workspace_status(ws) == goq.ERR_TIMEOUT
+    assert torch.isnan(cut[2]).all() and torch.isnan(cut[3]).all()
+    goq.workspace_init(ws)
+    again = call()
+    assert goq.workspace_status(ws) == goq.OK
+    assert all(torch.equal(a, c) for a, c in zip(good, again))
+
+
 @pytest.mark.parametrize("k,n,inner,m,g,b", [(256, 64, 512, 1, 64, 3), (1024, 256, 2816, 4, 128, 3), (128, 128, 256, 3, 32, 2), (4096, 1024, 11008, 4, 128, 3),
                                              (2048, 2048, 4096, 7, 128, 3), (512, 128, 1408, 2, 128, 2)])
 def test_chain_shares_staged_activations(goq, k, n, inner, m, g, b):
