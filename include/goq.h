@@ -83,7 +83,9 @@ size_t goq_algorithmic_bytes(const goq_desc* desc);
 /* Scratch bytes goq_gemv / goq_gemm need for `m` activation rows (may be 0). Every kernel keeps its counters in
  * the same leading area and leaves them zero, and nothing else in the buffer is carried from one call to the
  * next: one buffer of the largest size, initialised once, can serve calls for different layers, ops and m, as
- * long as those calls cannot overlap on the GPU. */
+ * long as those calls cannot overlap on the GPU. For one layer and GOQ_OP_GEMM the size never falls as m grows: a buffer
+ * for the largest m serves every smaller one, on the same kernels. (goq_gemm with less than this may take another kernel
+ * that the buffer suffices for, of the same stated accuracy, or return GOQ_ERR_WORKSPACE.) */
 size_t goq_workspace_bytes(const goq_desc* desc, int op, int m);
 
 /* Zero-fill a scratch buffer (asynchronous on `stream`). A scratch buffer must be initialised once

@@ -536,6 +536,15 @@ size_t gemm_mid_workspace(const Geometry& g, int m, bool exact) {
     mid::Plan p;
     return mid::make_plan(g, m, exact && !g.k1, &p) ? p.total : 0;
 }
+size_t gemm_mid_workspace_upto(const Geometry& g, int m) {
+    if (!(g.k_in % 8 == 0 && tc::packed_map_supported(g))) return 0;
+    // the offsets of make_plan; token tiles no wider than 256 or the call, and no more CTAs than units (more token tiles than one per
+    // 256 rows only where the units fill the SMs anyway)
+    const long long units = (long long)((m + 255) / 256) * ((g.n_pad + mid::kTileN - 1) / mid::kTileN) * g.k_blocks;
+    const size_t grid = units < mid::sm_count() ? (size_t)units : (size_t)mid::sm_count(), cols = m < 256 ? (m + 15) & ~15 : 256;
+    const size_t xh_off = kWsScratchOff + mid::align256((size_t)(m + 16) * sizeof(float));
+    return mid::align256(xh_off + (size_t)m * g.k_in * 2) + grid * 2 * cols * mid::kTileN * sizeof(float);
+}
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws, bool exact,
                             cudaStream_t st) {
     const bool two = exact && !g.k1;   // single-basis weights: c1 b1 alone is exact already

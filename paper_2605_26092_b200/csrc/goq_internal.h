@@ -96,6 +96,7 @@ cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x_
 bool gemm_mid_supported(const Geometry& g, int m, bool exact);
 float gemm_mid_us(const Geometry& g, int m);   // estimated time
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact);
+size_t gemm_mid_workspace_upto(const Geometry& g, int m);   // enough for every call of up to m rows, either form
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
                             bool exact, cudaStream_t st);
 

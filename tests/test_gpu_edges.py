@@ -182,6 +182,22 @@ def test_gemm_non_finite_activations_stay_with_their_token(goq, n, k, g, b, m):
     assert not np.isfinite(yh[hit]).any() and np.isfinite(yh[rest]).all()
 
 
+@pytest.mark.parametrize("n,k,g,b,largest,ms", [(4096, 4096, 128, 3, 257, (17, 100, 256)), (1024, 2048, 16, 3, 300, (20, 32, 200, 256)),
+                                                (2048, 1024, 64, 4, 2048, (18, 33, 255, 700))])
+def test_gemm_on_a_buffer_for_a_larger_batch(goq, n, k, g, b, largest, ms):
+    """A scratch buffer sized for a larger batch: the same kernel, so the same bits, as with a buffer of the call's own size."""
+    from tests.gpu_util import dev, pack_weights, run_gemm_bf16
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    ws = goq.new_workspace(d, goq.OP_GEMM, largest)
+    for m in ms:
+        xb = si.bf16_activations(m, k, seed=m)
+        y = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+        goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), run_gemm_bf16(d, packed, xb))
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])

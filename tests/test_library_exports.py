@@ -49,6 +49,18 @@ def test_size_queries(goq):
         assert goq.packed_bytes(bad) == 0 and goq.algorithmic_bytes(bad) == 0
 
 
+def test_gemm_scratch_never_falls_as_the_batch_grows(goq):
+    """A buffer sized for the largest batch holds what every smaller batch asks for."""
+    for n, k in ((8192, 8192), (4096, 4096), (1024, 8192), (16000, 512), (256, 256), (20000, 128), (37, 136), (2000, 11008)):
+        for g, b in ((128, 3), (128, 4), (32, 2), (16, 3), (8, 3), (8, 4)):
+            if k % g:
+                continue
+            d = goq.desc(n, k, g, b)
+            ms = list(range(1, 70)) + list(range(120, 140)) + list(range(250, 310)) + list(range(500, 1100, 7)) + [1279, 1280, 1281, 2048, 4096, 5000]
+            sizes = [goq.workspace_bytes(d, goq.OP_GEMM, m) for m in ms]
+            assert sizes == sorted(sizes), (n, k, g, b)
+
+
 def test_status_strings(goq):
     seen = {goq.status_string(s) for s in range(9)}
     assert len(seen) == 9 and "ok" in seen
