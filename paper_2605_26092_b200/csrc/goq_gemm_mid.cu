@@ -44,7 +44,7 @@ struct Params {
     const float* inv_scale;   // [m] 2^-s of each token
     int* status;
     float* partial;           // [CTA][2][n_cols][128]
-    int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m, y_dtype, group_log2, gpb;
+    int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m, y_dtype, group_log2;
     int n_cols;               // tokens per tile (MMA N): a multiple of 16, at most 256
     int tiles_x;              // channel tiles
     int units;                // token tiles x channel tiles x k-blocks
@@ -81,6 +81,22 @@ __device__ __forceinline__ uint32_t coef_max(const uint8_t* pair) {
     const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(pair));
     return max(w & 0x7FFFu, (w >> 16) & 0x7FFFu);
 }
+// largest magnitude of a channel's pairs first, first + step, .. below n (pair i: macro-block i & (gpb - 1) of record i >> gpb_log2).
+// BATCH loads in flight whatever n is (past the end the last pair again): left to the compiler, the remainder of an unrolled loop is
+// one load after another, and with narrow groups and few k-blocks that was most of the kernel's time (W3, 28672 x 896 in groups of 8
+// at 512 tokens 153 us).
+template <int BATCH>
+__device__ __forceinline__ uint32_t coef_max_of(const uint8_t* src, int first, int step, int n, int gpb_log2, int unit_bytes) {
+    uint32_t mx = 0;
+    for (int i0 = first; i0 < n; i0 += BATCH * step) {
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int i = min(i0 + u * step, n - 1);
+            mx = max(mx, coef_max(src + (size_t)(i >> gpb_log2) * unit_bytes + (i & ((1 << gpb_log2) - 1)) * 64));
+        }
+    }
+    return mx;
+}
 
 __device__ __forceinline__ __half2 u2h(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 __device__ __forceinline__ uint32_t h2u(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
@@ -110,6 +126,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
     const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     const int G = gridDim.x, cta = blockIdx.x;
     const int u0 = range_begin(cta, p.units, G), u1 = range_begin(cta + 1, p.units, G);
+    const int gpb_log2 = GL == 7 ? 0 : 7 - p.group_log2;   // macro-blocks per k-block
 
     // Packed records: unit by unit of the range, the eight records of a unit with one 2-D copy (a copy a record, issued by one
     // thread, took ~1700 clocks a unit and was what bound this kernel). The ring is filled before anything else.
@@ -142,12 +159,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         const int row = tid & (kTileN - 1), sub = tid >> 7, T = (part.tile % p.tiles_x) * 8 + (row >> 4);
         if (sub < 5 && T < p.n_tiles) {
             const uint8_t* src = p.packed + unit_offset(T, part.kb, p.k_blocks, p.unit_bytes) + kCodeBytesPerUnit + (row & 15) * 4;
-            uint32_t mx = 0;
-            for (int jj = 0; jj < p.gpb; ++jj) {
-#pragma unroll 8
-                for (int k = sub; k < part.n; k += 5) mx = max(mx, coef_max(src + (size_t)k * p.unit_bytes + jj * 64));
-            }
-            atomicMax(&row_max[row], mx);
+            atomicMax(&row_max[row], coef_max_of<8>(src, sub, 5, part.n << gpb_log2, gpb_log2, p.unit_bytes));
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -368,13 +380,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
             const Part part = part_at(u, u1, p.k_blocks);
             const int T = (part.tile % p.tiles_x) * 8 + 2 * warp + (lane >> 4);
             uint32_t mx = 0;
-            if (T < p.n_tiles) {
-                const uint8_t* src = p.packed + unit_offset(T, part.kb, p.k_blocks, p.unit_bytes) + kCodeBytesPerUnit + (lane & 15) * 4;
-                for (int jj = 0; jj < p.gpb; ++jj) {
-#pragma unroll 8
-                    for (int k = 0; k < part.n; ++k) mx = max(mx, coef_max(src + (size_t)k * p.unit_bytes + jj * 64));
-                }
-            }
+            if (T < p.n_tiles)
+                mx = coef_max_of<16>(p.packed + unit_offset(T, part.kb, p.k_blocks, p.unit_bytes) + kCodeBytesPerUnit + (lane & 15) * 4, 0, 1,
+                                     part.n << gpb_log2, gpb_log2, p.unit_bytes);
             return publish(mx, q);
         };
         float inv_row = publish(row_max[warp * 32 + lane], 0);
@@ -481,7 +489,7 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     p.status = (int*)ws;
     p.partial = (float*)(ws + pl.partial_off);
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.k_blocks = g.k_blocks; p.n_tiles = g.n_tiles; p.n_out = g.n_out;
-    p.m = m; p.y_dtype = y_dtype; p.gpb = g.groups_per_block;
+    p.m = m; p.y_dtype = y_dtype;
     int lg = 3;
     while ((1 << lg) < g.group) ++lg;
     p.group_log2 = lg;
