@@ -482,8 +482,9 @@ cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t
     p.m = m; p.y_dtype = y_dtype;
     p.tiles_x = (g.n_pad + i8tc::kChannels - 1) / i8tc::kChannels;
     const int half_tiles = (m + i8tc::kTokens - 1) / i8tc::kTokens;
-    // 256 tokens a tile halve the decode; 128 where that would leave SMs without a tile
-    p.tt = p.tiles_x * ((half_tiles + 1) / 2) >= i8tc::sm_count() ? 2 : 1;
+    // 256 tokens a tile halve the decode; 128 where that would leave SMs without a tile, or where there are no more (the second half's
+    // MMAs would be padding: 16000 x 512 at 64 tokens 11.9 us)
+    p.tt = half_tiles > 1 && p.tiles_x * ((half_tiles + 1) / 2) >= i8tc::sm_count() ? 2 : 1;
     p.tiles = p.tiles_x * ((half_tiles + p.tt - 1) / p.tt);
     p.status = status;
     p.spin = spin_limit > 0 ? spin_limit : tc::kSpin;
