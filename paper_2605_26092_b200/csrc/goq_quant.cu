@@ -427,8 +427,8 @@ struct Scale {
     double s, qmax;
     float inv;    // 0: always divide
     __device__ __forceinline__ Scale(double amax, double q) : s(amax == 0.0 ? 1.0 : amax / q), qmax(q) {
-        const double r = q / amax;
-        inv = (r > 1e-36 && r < 1e36) ? (float)r : 0.f;
+        const float r = (float)q / (float)amax;   // (the maximum is an fp32 number: one rounding, as a float64 quotient's would be)
+        inv = (r > 1e-36f && r < 1e36f) ? r : 0.f;
     }
     __device__ __forceinline__ int exact(double x) const {
         const double q = rint(x / s);   // round half to even
