@@ -241,6 +241,7 @@ solve_ref_kernel(const float* __restrict__ w, const uint8_t* __restrict__ codes,
     const float* xj = xc + (size_t)j * G;
 
     if constexpr (DIRECT) {   // operand = the observations: fragment (block of 8 observations, 4 channels), element (channel, observation)
+#pragma unroll 4
         for (int i = threadIdx.x; i < ((m + 7) / 8) * 8 * G; i += kRefWarps * 32) {
             const int o = i / G, k = i - o * G;
             frag[((o >> 3) * (2 * NB) + (k >> 2)) * 32 + (o & 7) * 4 + (k & 3)] = o < m ? (double)xj[(size_t)o * k_in + k] : 0.0;
@@ -258,8 +259,9 @@ solve_ref_kernel(const float* __restrict__ w, const uint8_t* __restrict__ codes,
         for (int b = 0; b < kAcc; ++b) acc_a[b][0] = acc_a[b][1] = acc_b[b][0] = acc_b[b][1] = 0.0;
         for (int o0 = 0; o0 < m; o0 += kRefChunk) {
             __syncthreads();
-            for (int i = threadIdx.x; i < kRefChunk * G; i += kRefWarps * 32) {
-                const int o = i / G, k = i - o * G;
+#pragma unroll
+            for (int q = 0; q < (kRefChunk * G) / (kRefWarps * 32); ++q) {   // all of a thread's loads in flight
+                const int i = (int)threadIdx.x + q * (kRefWarps * 32), o = i / G, k = i - o * G;
                 stage[o * kStride + k] = (o0 + o < m) ? xj[(size_t)(o0 + o) * k_in + k] : 0.f;
             }
             __syncthreads();
@@ -335,9 +337,19 @@ solve_ref_kernel(const float* __restrict__ w, const uint8_t* __restrict__ codes,
                 for (int e = 0; e < 8; ++e) dst[e] = 0u;
             }
         }
-        for (int i = lane; i < 8 * G; i += 32) {
-            const int r = i / G, k = i - r * G, row = rt * 8 + r;
-            vw[r * kStride + k] = row < n_out ? w[(size_t)row * k_in + (size_t)j * G + k] : 0.f;
+#pragma unroll
+        for (int q0 = 0; q0 < 2 * NB; q0 += 8) {   // up to eight loads of a lane in flight (one after another they were most of a small solve)
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8 && q0 + q < 2 * NB; ++q) {
+                const int i = lane + (q0 + q) * 32, r = i / G, k = i - r * G, row = rt * 8 + r;
+                v[q] = row < n_out ? w[(size_t)row * k_in + (size_t)j * G + k] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 8 && q0 + q < 2 * NB; ++q) {
+                const int i = lane + (q0 + q) * 32, r = i / G;
+                vw[r * kStride + (i - r * G)] = v[q];
+            }
         }
         __syncwarp();
         double g11 = 0, g12 = 0, g22 = 0, r1 = 0, r2 = 0;
@@ -556,7 +568,8 @@ static cudaError_t launch_ref(const Geometry& g, const float* w, const uint8_t* 
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 148;
     // Row chunks per column: every CTA forms its column's G again, so few chunks save work and many fill the chip. Take the
-    // split whose waves cost least in float64 tensor clocks (4 per m8n8k4 and SM, a row tile's loads and epilogue about 400).
+    // split whose waves cost least in float64 tensor clocks (4 per m8n8k4 and SM, a row tile's loads and epilogue about 400). Row
+    // tiles go in rounds of 16 warps; a CTA with fewer is bound by one warp's chain of products instead, about four tiles' clocks.
     const int cols = g.k_in / g.group, tiles = (g.n_out + 7) / 8, slots = sms;
     const double form = direct ? 500.0 : 4.0 * (NB * (NB + 1) / 2) * ((m + 63) / 64 * 16) + 1500.0;
     const double tile = 12.0 * (direct ? (m + 7) / 8 * 2 * NB : NB * (NB + 1)) + 400.0;
@@ -564,7 +577,9 @@ static cudaError_t launch_ref(const Geometry& g, const float* w, const uint8_t* 
     double best_cost = 0.0;
     for (int c = 1; c <= tiles && c <= 65535 && c <= 4 * slots; ++c) {
         const double waves = (double)(((long long)cols * c + slots - 1) / slots);
-        const double cost = waves * (form + ((tiles + c - 1) / c + quant::kRefWarps - 1) / quant::kRefWarps * quant::kRefWarps * tile);
+        const int per = (tiles + c - 1) / c;
+        const int paid = per >= quant::kRefWarps ? (per + quant::kRefWarps - 1) / quant::kRefWarps * quant::kRefWarps : (per > 4 ? per : 4);
+        const double cost = waves * (form + paid * tile);
         if (c == 1 || cost < best_cost) { best = c; best_cost = cost; }
     }
     kernel<<<dim3(cols, best), quant::kRefWarps * 32, smem, st>>>(w, codes, meta, x_calib, m, lambda, coef, c_out, g.n_out, g.k_in);
