@@ -223,7 +223,10 @@ static int sm_count() {
 
 template <int WB, int NT, int CPG>
 static cudaError_t launch(const Geometry& g, Params& p, cudaStream_t st) {
-    const int warps = g.k_blocks < kMaxWarps ? (g.k_blocks < 4 ? 4 : g.k_blocks) : kMaxWarps;
+    int warps = g.k_blocks < kMaxWarps ? (g.k_blocks < 4 ? 4 : g.k_blocks) : kMaxWarps;
+    // Few k-blocks and many tiles: what a CTA costs beside its records (table, start, sums) counts, and half the warps mean twice the CTAs
+    // in flight and two records a warp
+    if (g.k_blocks <= kMaxWarps && g.n_tiles > 4 * sm_count()) warps = 4;
     // A cluster per tile only while there are fewer CTAs than SMs and every warp keeps a record (1024 x 4096: 3.7 us, without 6.0; a
     // second CTA per SM by the same means costs more than it gives: 4096 x 4096 6.3 -> 9 us)
     int cluster = 1;
