@@ -139,9 +139,9 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
 /* goq_gemm - the same layer for m activation rows.
  *  x_dtype GOQ_BF16: x [m][k_in] bf16; y out [m][n_out] (GOQ_BF16 or GOQ_F32); sx, cq, sc, acc unused (NULL).
  *      ws: goq_workspace_bytes(desc, GOQ_OP_GEMM, m) bytes, 256-byte aligned, initialised once with
- *      goq_workspace_init. Up to 32 rows results carry fp32 accuracy. From 33 rows on the kernels keep an fp16 copy of
- *      x (each row scaled by a power of two, undone in the output) in ws, so the size grows with m * k_in, and round c1*b1 + c2*b2 once
- *      to fp16 (normwise output error about 1.5e-4 to 2.5e-4). The coefficients of every output channel are scaled by a
+ *      goq_workspace_init. Up to 32 rows results carry fp32 accuracy, whatever the group. The kernels for more than a
+ *      few rows keep an fp16 copy of x (each row scaled by a power of two, undone in the output) in ws, so the size grows with m * k_in;
+ *      from 33 rows on they round c1*b1 + c2*b2 once to fp16 (normwise output error about 1.5e-4 to 2.5e-4). The coefficients of every output channel are scaled by a
  *      power of two taken from the channel's largest |c1|, |c2| before that rounding and the output is scaled back, so
  *      the result does not depend on the magnitude of the weights; inside one channel, coefficients more than 2^13
  *      below the channel's largest lose precision to fp16's range.

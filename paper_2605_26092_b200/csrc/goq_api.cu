@@ -178,8 +178,10 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         // Above 256 tokens it decodes the weights once per 256 tokens, but spreads any number of tiles evenly; the two kernels'
         // estimates decide. Measured, us, this kernel / prefill kernel: 1024 x 8192 W4 at 777 tokens 35 / 102, at 4096 107 / 137;
         // 4096 x 4096 at 1024 51 / 56, at 1280 65 / 59; 11008 x 4096 at 512 67 / 69, at 1280 137 / 125; 16000 x 512 at 512 38 / 24.
-        const bool mid_wanted = variant == 4 || (variant == 0 && m > 16 && (m <= kGemmMidMaxTokens || !goq::gemm_tc_supported(g) ||
-                                                                            goq::gemm_mid_us(g, m) <= goq::gemm_tc_us(g, m)));
+        // Groups of 8 and 16 have no other tensor-core kernel that keeps fp32 accuracy: up to 32 rows they take this one from the first on.
+        const bool narrow = !goq::gemv_mma_supported(g, 16);
+        const bool mid_wanted = variant == 4 || (variant == 0 && (m > 16 || narrow) && (m <= kGemmMidMaxTokens || !goq::gemm_tc_supported(g) ||
+                                                                                        goq::gemm_mid_us(g, m) <= goq::gemm_tc_us(g, m)));
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
             return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
         if (variant == 4) return GOQ_ERR_UNSUPPORTED;
@@ -202,11 +204,13 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (goq::gemm_tc_supported(g) && variant != 2) {
             if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
             if (ws_bytes < goq::gemm_tc_workspace(g, m)) return GOQ_ERR_WORKSPACE;
-            return from_cuda(goq::launch_gemm_tc(g, packed, x, m, y, y_dtype, ws, (cudaStream_t)stream));
         }
+        // (up to 32 rows of a narrow group in less scratch than documented: the scalar kernel, slow but of the stated accuracy)
+        if (goq::gemm_tc_supported(g) && variant != 2 && !(variant == 0 && exact && narrow))
+            return from_cuda(goq::launch_gemm_tc(g, packed, x, m, y, y_dtype, ws, (cudaStream_t)stream));
         if (goq::linear_mma_supported(g))
             return from_cuda(goq::launch_linear_mma(g, packed, x, m, y, y_dtype, (cudaStream_t)stream));
-        // remaining configurations (macro-blocks narrower than 32): the scalar kernel, 16 tokens at a time
+        // what is left of the groups narrower than 32: the scalar kernel, 16 tokens at a time
         const size_t ybytes = (y_dtype == GOQ_F32) ? 4 : 2;
         for (int t0 = 0; t0 < m; t0 += 16) {
             const int nb = (m - t0 < 16) ? (m - t0) : 16;

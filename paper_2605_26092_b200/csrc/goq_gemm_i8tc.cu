@@ -15,7 +15,7 @@
 // record; its pair signs negate bytes. For B = 16 both digits are chosen non-zero, so a byte's negation is (~q) + 1 without a
 // carry into the next byte; for B = 192 the addition masks the top bits.
 //
-// Roles (27 warps, persistent CTAs): 0-7 epilogue (a thread is a token: ACC or y, eight channels a store), 8 packed records (one 2-D TMA
+// Roles (27 warps, persistent CTAs): 0-7 epilogue (a thread is a token: ACC or y, eight channels a store), 8 packed records (one TMA
 // copy per 64 channels x 128 k), 9 activation tiles (TMA), 10 MMA issue, 11-26 decode: two groups of eight alternate k-blocks, warp (e, v)
 // of a group takes rows 8 v .. of record e. Bound: shared-memory bandwidth (per 64 x 256 x 128: operand reads of the MMAs ~770 clocks, digit
 // stores, lookups and copies ~900). With 128 x 128 tiles the second part was twice that and the kernel ran at its sum (98 %).
@@ -138,7 +138,7 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     struct { int tile, kb, slot, round, issued; } pk = {(int)blockIdx.x, 0, 0, 0, 0};
     auto pk_issue = [&]() {
         mbar_expect_tx(&pk_full[pk.slot], (uint32_t)pk_bytes);   // (rows past the last tile arrive as zeros)
-        tma_load_2d(pk_ring + pk.slot * pk_bytes, &packed_map, pk.kb * (p.unit_bytes >> 3), (pk.tile % p.tiles_x) * 4, &pk_full[pk.slot]);
+        tma_load_3d(pk_ring + pk.slot * pk_bytes, &packed_map, 0, pk.kb, (pk.tile % p.tiles_x) * 4, &pk_full[pk.slot]);   // (groups of 32 or more: one piece a record)
         if (++pk.kb == p.k_blocks) { pk.kb = 0; pk.tile += (int)gridDim.x; }
         ++pk.issued;
         if (++pk.slot == p.n_pk) { pk.slot = 0; ++pk.round; }

@@ -11,7 +11,7 @@
 // warps.
 //
 // Roles (23 warps). Warps 0-3: coefficient scales ahead of each tile, then the epilogue (tensor memory -> y or the parked part).
-// Warp 4: packed records into a ring (one 2-D TMA copy per unit). Warp 5: activation tiles (2-D TMA, 128-byte swizzle). Warp 6:
+// Warp 4: packed records into a ring (one TMA copy per unit). Warp 5: activation tiles (2-D TMA, 128-byte swizzle). Warp 6:
 // tcgen05.mma issue. Warps 7-22: two groups of eight decode alternate k-blocks, warp e of a group record e, and write fp16
 // operand tiles of 64 k. The accumulator is double-buffered in tensor memory, so a tile's epilogue overlaps the next tile.
 //
@@ -50,6 +50,7 @@ struct Params {
     int units;                // token tiles x channel tiles x k-blocks
     int na;                   // accumulators of a part (1, 2, 4; TWO: 8), 256 / na tensor-memory columns apart: short sums
     int n_stages, n_pk;       // ring depths: operand stages (64 k), packed k-blocks
+    int pk_pieces;            // pieces of a record in its tensor map
 };
 
 // 16 accumulator columns of this warp's 32 lanes
@@ -128,13 +129,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
     const int u0 = range_begin(cta, p.units, G), u1 = range_begin(cta + 1, p.units, G);
     const int gpb_log2 = GL == 7 ? 0 : 7 - p.group_log2;   // macro-blocks per k-block
 
-    // Packed records: unit by unit of the range, the eight records of a unit with one 2-D copy (a copy a record, issued by one
+    // Packed records: unit by unit of the range, the eight records of a unit with one tiled copy (a copy a record, issued by one
     // thread, took ~1700 clocks a unit and was what bound this kernel). The ring is filled before anything else.
     struct PkState { int u, tile, kb, slot, round, issued; } pk = {u0, 0, -1, 0, 0, 0};
     auto pk_issue = [&]() {   // next unit into its slot (which must be free)
         if (pk.kb < 0) { pk.tile = pk.u / p.k_blocks; pk.kb = pk.u - pk.tile * p.k_blocks; }
         mbar_expect_tx(&pk_full[pk.slot], (uint32_t)pk_bytes);   // (rows past the last tile arrive as zeros)
-        tma_load_2d(pk_ring + pk.slot * pk_bytes, &packed_map, pk.kb * (p.unit_bytes >> 3), (pk.tile % p.tiles_x) * 8, &pk_full[pk.slot]);
+        tma_load_3d(pk_ring + pk.slot * pk_bytes, &packed_map, 0, pk.kb * p.pk_pieces, (pk.tile % p.tiles_x) * 8, &pk_full[pk.slot]);
         if (++pk.kb == p.k_blocks) { pk.kb = 0; ++pk.tile; }
         ++pk.u; ++pk.issued;
         if (++pk.slot == p.n_pk) { pk.slot = 0; ++pk.round; }
@@ -495,7 +496,7 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     p.group_log2 = lg;
     p.n_cols = pl.n_cols;
     p.na = TWO ? 8 : (pl.n_cols <= 64 ? 4 : pl.n_cols <= 128 ? 2 : 1);
-    p.tiles_x = pl.tiles_x; p.units = pl.units; p.n_stages = pl.n_stages; p.n_pk = pl.n_pk;
+    p.tiles_x = pl.tiles_x; p.units = pl.units; p.n_stages = pl.n_stages; p.n_pk = pl.n_pk; p.pk_pieces = packed_pieces(g);
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_mid_kernel<WB, TWO, GL>, pl.smem, smem_attr)) return e;
     // programmatic dependent of the pre-pass: tables, rings, coefficient scan and decode run ahead; only the activations' TMA

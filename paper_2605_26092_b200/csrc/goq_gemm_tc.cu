@@ -503,16 +503,17 @@ cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int 
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
 }
 bool packed_map_supported(const Geometry& g) {
-    return g.unit_bytes / 8 <= 256 && (unsigned long long)g.k_blocks * g.unit_bytes / 8 < (1ull << 31);
+    return (unsigned long long)g.k_blocks * g.unit_bytes / 8 < (1ull << 31);
 }
 cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g, int row_tiles) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return cudaErrorNotSupported;
-    const cuuint64_t dims[2] = {(cuuint64_t)g.k_blocks * g.unit_bytes / 8, (cuuint64_t)g.n_tiles};
-    const cuuint64_t strides[1] = {(cuuint64_t)g.k_blocks * g.unit_bytes};
-    const cuuint32_t box[2] = {(cuuint32_t)g.unit_bytes / 8, (cuuint32_t)row_tiles};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<void*>(packed), dims, strides, box, estr,
+    const int pieces = packed_pieces(g), piece = g.unit_bytes / pieces;   // bytes of a piece: a multiple of 16
+    const cuuint64_t dims[3] = {(cuuint64_t)piece / 8, (cuuint64_t)g.k_blocks * pieces, (cuuint64_t)g.n_tiles};
+    const cuuint64_t strides[2] = {(cuuint64_t)piece, (cuuint64_t)g.k_blocks * g.unit_bytes};
+    const cuuint32_t box[3] = {(cuuint32_t)piece / 8, (cuuint32_t)pieces, (cuuint32_t)row_tiles};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void*>(packed), dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;

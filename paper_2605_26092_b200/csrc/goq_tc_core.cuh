@@ -55,6 +55,11 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(s32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(s32(bar)) : "memory");
 }
+// ... 3-D: packed records, {c0 = 8-byte element of a piece, c1 = piece of the row of records, c2 = row tile}
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, uint64_t* bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(s32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(s32(bar)) : "memory");
+}
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     uint32_t d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
@@ -245,7 +250,9 @@ __device__ __forceinline__ void fill_lut(unsigned char* lut, int tid, int n_thre
 // host side, defined in goq_gemm_tc.cu
 cudaError_t encode_x_map(CUtensorMap* map, void* xh, int k_in, int m, int rows);
 cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int rows);
-// packed records as boxes of one k-block x `row_tiles` row tiles (8-byte elements; rows past the end read as zeros)
+// packed records as boxes of one k-block x `row_tiles` row tiles (8-byte elements; rows past the end read as zeros). A record is one
+// piece, or two where it has more elements than a box row may (W4 in groups of 8: 288).
+inline int packed_pieces(const Geometry& g) { return g.unit_bytes / 8 > 256 ? 2 : 1; }
 bool packed_map_supported(const Geometry& g);
 cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g, int row_tiles);
 cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st);

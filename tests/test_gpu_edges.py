@@ -102,7 +102,7 @@ def test_ref_solve_edges(goq, n, k, g, b, m):
 
 @pytest.mark.parametrize("n,k,g,b,m", [
     (1, 8, 8, 3, 17), (129, 136, 8, 3, 33), (127, 256, 16, 4, 32), (128, 128, 128, 3, 64),
-    (4000, 384, 128, 3, 65), (257, 1152, 64, 3, 256), (300, 640, 128, 4, 257), (1000, 4096, 32, 3, 511),
+    (4000, 384, 128, 3, 65), (250, 512, 8, 4, 200), (257, 1152, 64, 3, 256), (300, 640, 128, 4, 257), (1000, 4096, 32, 3, 511),
     (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 20), (1100, 2304, 128, 3, 200)])
 def test_mid_batch_gemm_edges(goq, n, k, g, b, m):
     """The kernel between decode and prefill: channel tiles and token tiles that do not fill, one unit in all, one tile shared by
@@ -180,6 +180,33 @@ def test_gemm_non_finite_activations_stay_with_their_token(goq, n, k, g, b, m):
     assert np.array_equal(got[rest], clean[rest])
     yh = run_gemm_bf16(d, packed, bad, goq.BF16)
     assert not np.isfinite(yh[hit]).any() and np.isfinite(yh[rest]).all()
+
+
+@pytest.mark.parametrize("n,k,g,b", [(200, 384, 16, 3), (130, 136, 8, 3), (257, 512, 8, 4), (64, 1024, 16, 4), (1, 8, 8, 4), (300, 256, 32, 4)])
+def test_gemm_up_to_32_rows_is_fp32_accurate_in_every_group(goq, n, k, g, b):
+    """Automatic dispatch at 1, 16, 17 and 32 rows, narrow groups and the largest records (W4 in groups of 8: two pieces a copy) among
+    them, also in a buffer sized for one row: 2e-5 as for every fp32-accumulating kernel; a single output, which may be small by
+    cancellation, within 2^-20 of its terms' magnitudes (fp32 sums of exact products)."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    w = O.decode_b1(codes, b) * np.repeat(coef[..., 0].astype(np.float64), g, 1) + O.decode_b2(codes, meta, b) * np.repeat(coef[..., 1].astype(np.float64), g, 1)
+    for m, sized_for in ((1, 1), (16, 16), (17, 17), (32, 32), (32, 1)):
+        xb = si.bf16_activations(m, k, seed=m)
+        x = si.bf16_bits_to_f64(xb)
+        y_ref = O.linear_f64(codes, meta, coef, x, g, b)
+        y = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+        try:
+            goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=goq.new_workspace(d, goq.OP_GEMM, sized_for))
+        except goq.GoqError as e:   # less scratch than documented may be refused
+            assert sized_for < m and e.status == goq.ERR_WORKSPACE
+            continue
+        torch.cuda.synchronize()
+        got = y.cpu().numpy().astype(np.float64)
+        if n > 1:
+            check_parity(got, y_ref, 2e-5, 1e-4)
+        else:
+            assert (np.abs(got - y_ref) <= 2.0 ** -20 * np.abs(x) @ np.abs(w).T).all()
 
 
 @pytest.mark.parametrize("n,k,g,b,largest,ms", [(4096, 4096, 128, 3, 257, (17, 100, 256)), (1024, 2048, 16, 3, 300, (20, 32, 200, 256)),
