@@ -12,8 +12,7 @@ namespace {
 std::atomic<int> g_gemv_variant{0};
 std::atomic<int> g_wait_limit{0};   // 0: the kernels' own bound on device-side waits
 constexpr int kGemmExactMaxTokens = 32;     // goq_gemm: fp32-accurate results up to here
-constexpr int kGemmMidMaxTokens = 256;
-constexpr int kGemmViaGemvMaxTokens = 32;   // above: the tcgen05 GEMM (split-K) is faster than 16-token GEMV launches
+constexpr int kGemmMidMaxTokens = 256;      // ... one token tile of the mid-batch kernel
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
@@ -169,24 +168,34 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (!y) return GOQ_ERR_INVALID_ARG;
         if (goq_status s = check_arch()) return s;
         const int variant = g_gemv_variant.load(std::memory_order_relaxed);
-        // More tokens than one streaming GEMV takes, fewer than fill the prefill kernel's 128 x 512 tiles: the tensor-core kernel
-        // that splits the packed records evenly over the SMs. Up to 32 tokens with both bases as exact operands (fp32 accuracy),
-        // above with w_hat rounded once to fp16. Measured, W3 g128, us (this kernel / streaming launches or prefill kernel):
-        // 8192 x 8192: 43 / 72 at 32 tokens, 43 / 92 at 64, 65 / 95 at 256, 92 / 121 at 512; 4096 x 4096: 23 / 31, 27 / 52,
-        // 44 / 53, 50 / 67; 1024 x 8192: 20 / 23, 27 / 75, 70 / 75, 57 / 118.
-        const bool exact = m <= kGemmExactMaxTokens;
-        // Above 256 tokens it decodes the weights once per 256 tokens, but spreads any number of tiles evenly; the two kernels'
-        // estimates decide. Measured, us, this kernel / prefill kernel: 1024 x 8192 W4 at 777 tokens 35 / 102, at 4096 107 / 137;
-        // 4096 x 4096 at 1024 51 / 56, at 1280 65 / 59; 11008 x 4096 at 512 67 / 69, at 1280 137 / 125; 16000 x 512 at 512 38 / 24.
-        // Groups of 8 and 16 have no other tensor-core kernel that keeps fp32 accuracy: up to 32 rows they take this one from the first on.
-        const bool narrow = !goq::gemv_mma_supported(g, 16);
-        const bool mid_wanted = variant == 4 || (variant == 0 && (m > 16 || narrow) && (m <= kGemmMidMaxTokens || !goq::gemm_tc_supported(g) ||
-                                                                                        goq::gemm_mid_us(g, m) <= goq::gemm_tc_us(g, m)));
+        // Three kernels: the decode GEMV (16 tokens a launch), the mid-batch kernel (an even split of the packed records over the SMs; up to
+        // 32 tokens with both bases as exact operands, above with w_hat rounded once to fp16) and the prefill kernel (128 x 512 tiles).
+        //   Up to 32 tokens: groups of 8 and 16 have only the mid-batch kernel that keeps fp32 accuracy. Others take two decode launches
+        //   unless the linear is large or wide (units = 16-row tiles x k-blocks). Measured at 17 tokens, W3 g128, us, mid-batch over decode:
+        //   4096 x 4096 1.22, 8192 x 2048 0.99, 11008 x 2048 0.91, 4096 x 8192 0.96, 2048 x 11008 1.05, 16000 x 512 1.11, 28672 x 512 0.88.
+        //   33 to 256 tokens: mid-batch (0.25 to 0.95 of the prefill kernel's time), except where the channel tiles fill most of one wave of
+        //   the prefill kernel and the few k-blocks are soon decoded: at 256 tokens, mid-batch over prefill, 16000 x 256 1.23, x 512
+        //   1.25, x 896 1.10, x 2048 1.00; 11008 x 512 1.06; 8192 x 512 (64 tiles, two splits of K) 0.88.
+        //   Above: it decodes the weights once per 256 tokens, but spreads any number of tiles evenly; the two kernels' estimates decide
+        //   (the prefill kernel's is the surer one, hence the margin). us, mid-batch / prefill: 1024 x 8192 W4 at 777 tokens 35 / 102;
+        //   4096 x 4096 at 1024 52 / 54; 11008 x 4096 at 512 69 / 65; 16000 x 512 at 512 40 / 23.
+        const bool exact = m <= kGemmExactMaxTokens, narrow = !goq::gemv_mma_supported(g, 16);
+        bool mid_wanted = variant == 4;
+        if (variant == 0) {
+            if (exact) {
+                mid_wanted = narrow || (m > 16 && (g.n_units >= 12000 || (g.n_tiles >= 500 && g.n_units >= 8000) || g.n_tiles >= 1700));
+            } else if (m <= kGemmMidMaxTokens) {
+                const int wide_tiles = (g.n_tiles + 7) / 8, sms = goq::gemm_mid_ctas();
+                mid_wanted = !(goq::gemm_tc_supported(g) && 2 * wide_tiles > sms && wide_tiles <= sms && g.k_blocks >= 2 && g.k_blocks < 8);
+            } else {
+                mid_wanted = !goq::gemm_tc_supported(g) || goq::gemm_mid_us(g, m) <= 0.95f * goq::gemm_tc_us(g, m);
+            }
+        }
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
             return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
         if (variant == 4) return GOQ_ERR_UNSUPPORTED;
-        // What the mid-batch kernel does not take up to 32 tokens: the decode GEMV, 16 tokens per launch
-        if (m <= kGemmViaGemvMaxTokens && variant == 0 && goq::gemv_mma_supported(g, 16)) {
+        // the decode GEMV, 16 tokens per launch
+        if (exact && variant == 0 && goq::gemv_mma_supported(g, 16)) {
             if (goq::gemv_stream_supported(g)) {
                 if (!ws || !aligned(ws, 256)) return ws ? GOQ_ERR_ALIGNMENT : GOQ_ERR_WORKSPACE;
                 if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;

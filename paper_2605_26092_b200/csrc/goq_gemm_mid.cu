@@ -533,14 +533,16 @@ bool gemm_mid_supported(const Geometry& g, int m, bool exact) {
     return g.k_in % 8 == 0 && tc::packed_map_supported(g) && mid::make_plan(g, m, exact && !g.k1, &p);
 }
 // Estimated time of a call: a unit's decode plus a share that grows with its tokens, or the drain of its tile by four warps where
-// the tile has few k-blocks, and 14 us for the pre-pass, the start and the shared tiles. (W3, us a unit: 0.75 at 64 tokens, 1.4 at
-// 256; 0.15 more at W4; 16 us for the drain of 256 tokens.)
+// the tile has few k-blocks, and 14 us for the pre-pass, the start and the shared tiles. (W3 g128, us a unit: 0.75 at 64 tokens, 1.4
+// at 256; 0.15 more at W4, and more in narrow groups; 18 us for the drain of 256 tokens.)
 float gemm_mid_us(const Geometry& g, int m) {
     mid::Plan p;
     if (!mid::make_plan(g, m, false, &p)) return 1e30f;
-    const float unit = 0.55f + 0.0032f * (float)p.n_cols + (g.wbits == 4 ? 0.15f : 0.f), drain = 0.0625f * (float)p.n_cols / (float)g.k_blocks;
+    const float unit = 0.55f + 0.0032f * (float)p.n_cols + (g.wbits == 4 ? 0.15f : 0.f) + (g.group == 128 ? 0.f : g.group >= 32 ? 0.05f : g.group == 16 ? 0.1f : 0.3f);
+    const float drain = 0.07f * (float)p.n_cols / (float)g.k_blocks;
     return 14.f + (float)((p.units + p.grid - 1) / p.grid) * (unit > drain ? unit : drain);
 }
+int gemm_mid_ctas() { return mid::sm_count(); }
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact) {
     mid::Plan p;
     return mid::make_plan(g, m, exact && !g.k1, &p) ? p.total : 0;

@@ -94,7 +94,8 @@ cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x_
 // The same layer for a few to a few hundred tokens (goq_gemm_mid.cu), any group, wbits 2..4. exact: the two bases as separate
 // operands without rounding (fp32 accuracy), else w_hat rounded once to fp16. `ws` holds gemm_mid_workspace bytes.
 bool gemm_mid_supported(const Geometry& g, int m, bool exact);
-float gemm_mid_us(const Geometry& g, int m);   // estimated time
+float gemm_mid_us(const Geometry& g, int m);   // estimated time, more than 256 tokens
+int gemm_mid_ctas();                           // CTAs of a full grid: one per SM
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact);
 size_t gemm_mid_workspace_upto(const Geometry& g, int m);   // enough for every call of up to m rows, either form
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,

@@ -182,6 +182,24 @@ def test_gemm_non_finite_activations_stay_with_their_token(goq, n, k, g, b, m):
     assert not np.isfinite(yh[hit]).any() and np.isfinite(yh[rest]).all()
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(9472, 256, 64, 3, 200), (9473, 256, 64, 3, 256), (18944, 768, 128, 4, 33), (18945, 256, 128, 3, 100), (9600, 128, 128, 3, 64),
+                                       (9600, 1024, 128, 2, 64), (7984, 2048, 128, 3, 20), (8000, 2048, 128, 3, 20), (27200, 96, 32, 4, 32),
+                                       (9500, 512, 8, 4, 150), (4096, 1024, 16, 3, 1200), (4096, 1024, 16, 3, 520)])
+def test_gemm_either_side_of_the_dispatch_lines(goq, n, k, g, b, m):
+    """Automatic dispatch next to its lines (148 SMs): channel tiles that half fill, fill and overfill one wave, one and eight k-blocks; up
+    to 32 tokens the units and tiles where the mid-batch kernel takes over from the decode launches; above 256 either estimate.
+    Sampled channels of every token: 2e-5 up to 32 tokens, w_hat rounded once to fp16 5e-4 above."""
+    from tests.gpu_util import check_parity, pack_weights, run_gemm_bf16
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    rows = np.unique(np.concatenate([si.sample_rows(n, 200, seed=2), np.arange(n - 20, n)]))
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b, rows=rows)
+    y = run_gemm_bf16(d, packed, xb)
+    assert np.isfinite(y).all()
+    check_parity(y[:, rows], y_ref, 2e-5 if m <= 32 else 5e-4, 1e-4 if m <= 32 else 2e-3)
+
+
 @pytest.mark.parametrize("n,k,g,b", [(200, 384, 16, 3), (130, 136, 8, 3), (257, 512, 8, 4), (64, 1024, 16, 4), (1, 8, 8, 4), (300, 256, 32, 4)])
 def test_gemm_up_to_32_rows_is_fp32_accurate_in_every_group(goq, n, k, g, b):
     """Automatic dispatch at 1, 16, 17 and 32 rows, narrow groups and the largest records (W4 in groups of 8: two pieces a copy) among
