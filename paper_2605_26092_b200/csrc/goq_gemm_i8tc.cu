@@ -230,12 +230,11 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
                             umma_i8(tmem_base + h * 256, ad + h * (kABytes >> 4) + 2 * ks, bd + 2 * ks, (kb > 0 || ks > 0) ? 1u : 0u);
-                        // the stage first: once the last tile's epilogue has its accumulators no arrival is outstanding
-                        if (h == p.tt - 1) umma_commit(&empty[s]);
                         if (kb == p.k_blocks - 1) umma_commit(&tm_full[h]);
                     }
                 }
                 if (!ok) break;
+                if (leader) umma_commit(&empty[s]);   // (the last one arrives with the accumulators', a tile's epilogue before the CTA leaves)
                 __syncwarp();
                 s = s_next; par = par_next;
             }
