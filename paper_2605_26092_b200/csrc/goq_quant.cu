@@ -17,17 +17,6 @@ namespace quant {
 constexpr int kWarps = 8;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
-    return v;
-}
-
 // value of code c on the b-bit asymmetric lattice (Section 3.2): (-1)^sign 2^-e, the smallest positive bin being zero
 __device__ __forceinline__ double lattice_value(int c, int wbits) {
     const int emax = (1 << (wbits - 1)) - 1, sg = c >> (wbits - 1), e = c & emax;
@@ -431,9 +420,8 @@ solve_ref_kernel(const float* __restrict__ w, const uint8_t* __restrict__ codes,
 // made only where it can matter: x * (q_max / max|x|) in fp32 is within 127 * 3 * 2^-24 < 1e-4 of x / s_x, so any quotient further
 // than that from a half rounds the same way; the others, and everything that is not finite, take the division.
 // Measured, 12608 x 768 fp32: 17.9 us (a division per element, two passes: 39.5); 12608 x 3072 with the maxima given: 43.4 us (88.6).
-template <typename T> __device__ __forceinline__ double load_act(const T* p);
-template <> __device__ __forceinline__ double load_act<float>(const float* p) { return (double)*p; }
-template <> __device__ __forceinline__ double load_act<uint16_t>(const uint16_t* p) { return (double)bf16_to_f32(*p); }
+__device__ __forceinline__ float load_act(const float* p) { return *p; }
+__device__ __forceinline__ float load_act(const uint16_t* p) { return bf16_to_f32(*p); }
 
 struct Scale {
     double s, qmax;
@@ -512,21 +500,23 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 quantize_act_kernel(const T* __restrict__ x, int k, const float* __restrict__ amax_in, int8_t* __restrict__ xq, float* __restrict__ sx,
                     double qmax) {
-    __shared__ double red[8];
+    __shared__ float red[8];
     const int tok = blockIdx.x, tid = threadIdx.x;
     const T* row = x + (size_t)tok * k;
-    double a = 0.0;
+    float a = 0.f;
     if (amax_in) {
-        a = (double)amax_in[tok];
+        a = amax_in[tok];
     } else {
-        for (int i = tid; i < k; i += 256) a = fmax(a, fabs(load_act<T>(row + i)));
-        a = warp_max(a);
+        for (int i = tid; i < k; i += 256) a = fmaxf(a, fabsf(load_act(row + i)));
+#pragma unroll
+        for (int o = 16; o; o >>= 1) a = fmaxf(a, __shfl_xor_sync(kFull, a, o));
         if ((tid & 31) == 0) red[tid >> 5] = a;
         __syncthreads();
-        for (int i = 0; i < 8; ++i) a = fmax(a, red[i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a = fmaxf(a, red[i]);
     }
-    const Scale sc(a, qmax);
-    for (int i = tid; i < k; i += 256) xq[(size_t)tok * k + i] = (int8_t)sc((float)load_act<T>(row + i));
+    const Scale sc((double)a, qmax);
+    for (int i = tid; i < k; i += 256) xq[(size_t)tok * k + i] = (int8_t)sc(load_act(row + i));
     if (tid == 0) sx[tok] = (float)sc.s;
 }
 
