@@ -436,8 +436,8 @@ def run_cuda(args):
         if int(goq.workspace_status(ws_seq)) != 0:
             raise RuntimeError("sequence kernel reported a device-side timeout")
     else:
-        kernel_name = {2: "linear_mma_kernel<3,1>", 1: "gemv_scalar_kernel"}.get(
-            args.gemv_variant, "gemv_stream_kernel<3,1,4,true>")
+        kernel_name = {3: "gemv_stream_kernel<3,1,4,true>", 2: "linear_mma_kernel<3,1>", 1: "gemv_scalar_kernel"}.get(
+            args.gemv_variant, "gemv_one_kernel<3,4,false>")
         launch_desc = "one CUDA graph of %d goq_gemv nodes per step" % n_lin
         # one ncu capture of the 4096x4096 launch read 8.96 MB of DRAM for 8.39 MB of algorithmic bytes;
         # the packed image grows in proportion to n*k, so the ratio is applied to the average launch
@@ -751,7 +751,7 @@ def run_extras(torch, goq, stack, layers, tf_peak, ws):
 
 
 NCU_TRAFFIC_RATIO = 8.96 / 8.39
-NCU_TRAFFIC_RATIO_SEQ = (215.8 + 4.4) / 202.9   # ncu: 215.2 MB read + 4.2 MB written for the 202.9 MB (algorithmic) of a 14-linear launch
+NCU_TRAFFIC_RATIO_SEQ = (215.7 + 5.3) / 202.9   # ncu: 215.7 MB read + 5.3 MB written for the 202.9 MB (algorithmic) of a 14-linear launch
 
 
 def run_probe_steady(args):
@@ -837,7 +837,7 @@ def main():
     ap.add_argument("--launch", choices=("sequence", "graph"), default="sequence",
                     help="how a step is issued: one goq_gemv_sequence call, or a CUDA graph of per-linear goq_gemv launches")
     ap.add_argument("--gemv-variant", type=int, default=0,
-                    help="force a kernel variant (goq_set_gemv_variant): 0 automatic, 3 streaming, 4 tcgen05 tensor-memory GEMV, ...")
+                    help="force a kernel variant (goq_set_gemv_variant): 0 automatic, 1 scalar, 2 fragment, 3 streaming")
     ap.add_argument("--traffic-bytes", type=float, default=None,
                     help="dram bytes per launch of the dominant kernel from an ncu capture (reported as-is)")
     ap.add_argument("--probe", choices=("steady", "gemm"), default=None, help="run one small case only (for profiler captures)")

@@ -138,8 +138,11 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         if (ws_bytes < goq::gemv_stream_workspace(g)) return GOQ_ERR_WORKSPACE;
         if (!goq::stream_hash_is_bijective()) return GOQ_ERR_UNSUPPORTED;
         // Up to 4 tokens on a large linear: integer operands, half the decode's instructions; below, the fragment kernel's shorter
-        // start and end count for more. Measured, us, integer / fragment, at 1 token: 4096 units (1024 x 8192) 5.2 / 4.9,
-        // 8192 (4096 x 4096) 6.1 / 6.3; at 4 tokens: 6.2 / 4.9, 7.3 / 6.3, 22016 (11008 x 4096) 13.2 / 15.4.
+        // start and end count for more. Measured, W3 g128, integer over fragment at 1 / 2 / 3 / 4 tokens: 4096 units (1024 x 8192) 1.03 / 1.07 /
+        // 1.16 / 1.20, (8192 x 1024) 0.99 / 0.99 / 0.98 / 0.99; 8192 (4096 x 4096) 0.95 / 1.01 / 1.06 / 1.09, (2048 x 8192) 0.91 / 0.98 / 1.10 /
+        // 1.16, (8192 x 2048) 0.80 / 0.82 / 0.85 / 0.86; 22016 (11008 x 4096) 0.75 / 0.77 / 0.78 / 0.80, (4096 x 11008) 0.77 / 0.84 / 0.93 / 0.97.
+        // W2 and groups of 32 lie within 0.03 of these; single-basis weights, whose integer decode is shorter still, 0.1 to 0.25 below, so
+        // that for them the line could lie lower. Between 8192 and 12000 units at 2 to 4 tokens it depends on the width: narrow ones lose.
         const bool one = goq::gemv_one_supported(g, batch) && (variant == 5 || (variant == 0 && g.n_units > (batch == 1 ? 6000u : 12000u)));
         if (variant == 5 && !one) return GOQ_ERR_UNSUPPORTED;
         if (one)

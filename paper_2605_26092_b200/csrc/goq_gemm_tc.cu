@@ -4,7 +4,7 @@
 //   y[m,n] = sum_k x[m,k] * w_hat[n,k],   w_hat[n,k] = c1[n,j] b1[n,k] + c2[n,j] b2[n,k]   (Section 3.1)
 // Each CTA computes a tile of 128 output channels x up to 512 tokens (two halves of at most 256). Per 64-wide k-chunk
 //   - a producer thread bulk-copies the packed unit records of the 128 rows (cp.async.bulk, 8 records per
-//     128 k) and loads the 512 x 64 bf16 activation tile with two 2-D TMA copies (128-byte swizzle);
+//     128 k) and loads the 512 x 64 fp16 activation tile with two 2-D TMA copies (128-byte swizzle);
 //   - eight expander warps decode the records (same byte-table decode and record lookup as the GEMV:
 //     b1 from the code bytes, b2 = byte-permuted b1 with pair signs, Section 3.3), form
 //     w_hat = c1*b1 + c2*b2 with one half2 multiply and one half2 fma (a single rounding to fp16: the products
@@ -33,7 +33,7 @@ namespace tc {
 
 constexpr int kTileN = 128;     // output channels per CTA (MMA M)
 constexpr int kTileM = 512;     // tokens per CTA (two MMA N = 256 halves)
-constexpr int kChunkK = 64;     // k per pipeline stage: 128 bytes of bf16 = one swizzle row
+constexpr int kChunkK = 64;     // k per pipeline stage: 128 bytes of fp16 = one swizzle row
 constexpr int kStages = 2;
 constexpr int kExpanders = 8;   // expander warps; each owns one 16-row unit record per k-block
 constexpr int kThreads = (2 + kExpanders) * 32;
@@ -551,7 +551,8 @@ static int sm_count_cached() {
 // makes the waves over the SMs clearly shorter (a call with few channel tiles leaves SMs idle): a CTA takes, for each k-block,
 // the weights' decode plus a share that grows with its tokens (4096 x 4096 W3, us a k-block: 1.1 at 128 tokens, 1.3 at 256, 1.6 at
 // 512), and about 8 us to start and to drain. 2000 x 11008 at 2048 tokens: 8 tiles 142 us, 4 tiles 176. Where every SM has work
-// anyway more tiles only decode more (4096 x 4096 at 4096 tokens: 9 tiles 153 us, 8 tiles 141), hence the margin of 8 %.
+// anyway more tiles only decode more (4096 x 4096 at 4096 tokens: 9 tiles 153 us, 8 tiles 141; the estimates differ by 2.3 %), hence
+// the margin of 2.5 %.
 static float wave_us(int k_blocks, int tokens) { return 8.f + (float)k_blocks * (0.95f + 0.00135f * (float)tokens); }
 struct TokenTiles { int n, half, n_full, n_tail; float us; };   // tiles of 2 * half tokens; n_full CTAs take whole tiles, n_tail tiles go as halves
 static TokenTiles token_tiles(const Geometry& g, int m) {

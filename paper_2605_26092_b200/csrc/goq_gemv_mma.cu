@@ -12,7 +12,7 @@
 // order, then in rank order through distributed shared memory: deterministic, and no scratch.
 // The launch is a programmatic dependent: tables and, in goq_gemv, first records are fetched while the kernel before still runs.
 // Bound: instruction issue of the decode (about 280 a record) and, with one or two CTAs a SM, the last wave. 128 registers and 16 warps a
-// SM beat 80 and 24 (spills). Measured, W3 g128: 256 x 256 2.3 us (streaming kernel 5.8), 4096 x 4096 6.4 us at 8 tokens and 8.2
+// SM beat 80 and 24 (spills). Measured, W3 g128: 256 x 256 1.5 us in a graph (streaming kernel 5.8), 4096 x 4096 6.4 us at 8 tokens and 8.2
 // at 16 (13.9, 15.5), 8192 x 8192 21.7 and 27.3 (30.0, 36.8); W4 26.3 at 8 tokens (the earlier fragment kernel 34.4).
 #include <cooperative_groups.h>
 #include "goq_stream_core.cuh"

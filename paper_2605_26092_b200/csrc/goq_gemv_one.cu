@@ -8,8 +8,9 @@
 //
 // Tiles shared by several CTAs: every CTA but the one that holds the tile's end posts its part (at most one per CTA) in the
 // zero-kept counter area, a word a value: zero means "not there yet" and a sum of +0 is posted as -0. The finisher polls the words it
-// needs and zeroes them again: no fence, no counter, no launch number. It waits on lower-numbered CTAs only, which are dispatched
-// before it. Every wait is bounded (abort flag, GOQ_ERR_TIMEOUT in the status word).
+// needs and zeroes them again: no fence, no counter, no launch number. It waits on lower-numbered CTAs only. That these run is not a
+// guarantee of an ordinary launch: it relies on CTAs being dispatched in the order of their numbers, one per SM, as they are in practice;
+// were they not, the wait would run out and be reported. Every wait is bounded (abort flag, GOQ_ERR_TIMEOUT in the status word).
 // Bound: instruction issue of the decode (see goq_gemv_chain.cu) plus ~4 us of start, conversion and hand-over latency.
 #include "goq_int_core.cuh"
 #include "goq_internal.h"

@@ -82,7 +82,7 @@ bool gemv_one_supported(const Geometry& g, int m);
 cudaError_t launch_gemv_one(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
                             int spin_limit, cudaStream_t st);
 
-// Prefill GEMM on tcgen05 tensor cores (wbits <= 3). `ws` holds gemm_tc_workspace(g, m) bytes: status word and
+// Prefill GEMM on tcgen05 tensor cores (any wbits and group whose records fit the ring). `ws` holds gemm_tc_workspace(g, m) bytes: status word and
 // (split-K) tile counters in the common areas, then the per-token scales, the fp16 copy of the m x k_in activations
 // and the split-K partial tiles.
 bool gemm_tc_supported(const Geometry& g);
