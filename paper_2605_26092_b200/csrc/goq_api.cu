@@ -195,7 +195,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
             }
         }
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
-            return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, (cudaStream_t)stream));
+            return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
         if (variant == 4) return GOQ_ERR_UNSUPPORTED;
         // the decode GEMV, 16 tokens per launch
         if (exact && variant == 0 && goq::gemv_mma_supported(g, 16)) {

@@ -422,13 +422,10 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     }
     __syncthreads();
     if (abort_flag) {
-        // Copies and MMAs in flight must land before shared and tensor memory go away. Their barriers may count arrivals that never come,
-        // so this waits a time that none of them takes (a millisecond).
-        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+        settle_after_give_up();
         if (tid == 0 && p.status) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
         if (p.amax)   // NaN is the largest of the non-negative floats' bit patterns: it stays, and the quantizer behind passes it on
             for (int tok = tid; tok < p.m; tok += kThreads) atomicMax(reinterpret_cast<int*>(p.amax) + tok, 0x7FC00000);
-        __syncthreads();
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -21,8 +21,8 @@
 //   TWO = true:  two operands, c1 b1 and c2 b2, each exact in fp16 (a power of two times an fp16 number): no rounding before the
 //                fp32 sums. For the calls whose results carry fp32 accuracy (few tokens).
 //
-// Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, runs out its control flow, frees its tensor memory
-// and records GOQ_ERR_TIMEOUT in the status word.
+// Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, runs out its control flow, waits for what it has in flight,
+// frees its tensor memory and records GOQ_ERR_TIMEOUT in the status word.
 #include "goq_streamk.cuh"
 #include "goq_internal.h"
 
@@ -51,6 +51,7 @@ struct Params {
     int na;                   // accumulators of a part (1, 2, 4; TWO: 8), 256 / na tensor-memory columns apart: short sums
     int n_stages, n_pk;       // ring depths: operand stages (64 k), packed k-blocks
     int pk_pieces;            // pieces of a record in its tensor map
+    int spin;                 // bound of the waits for a finished accumulator, in polls (of all of them it cost 2 %)
 };
 
 // 16 accumulator columns of this warp's 32 lanes
@@ -213,9 +214,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
                 ok = mbar_wait(&pk_empty[pk.slot], (pk.round - 1) & 1, &abort_flag);
                 if (ok) pk_issue();
             }
-            if (!ok || abort_flag)   // copies already issued must land before the CTA's shared memory goes away (bounded waits)
-                for (int i = pk.issued > p.n_pk ? pk.issued - p.n_pk : 0; i < pk.issued; ++i)
-                    for (int it = 0; it < kSpin && !mbar_try(&pk_full[i % p.n_pk], (uint32_t)(i / p.n_pk) & 1u); ++it) { }
         }
     } else if (warp == kXWarp) {
         // ------------------------------ activation tiles ------------------------------
@@ -235,10 +233,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
                 }
                 u += part.n;
             }
-            // After a give-up the copies in flight must land before the CTA's shared memory goes away. Their barriers count the
-            // decoders' arrivals too and may never complete, so this waits a time no copy takes (a millisecond).
-            if (!ok || abort_flag)
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------ MMA issue ------------------------------
@@ -395,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
             const bool last_part = u + part.n >= u1;
             const float inv_next = last_part ? inv_row : scan(u + part.n, q + 1);
             if (last_part) break;   // drained by all warps, below
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[q & 1], (q >> 1) & 1, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[q & 1], (q >> 1) & 1, &abort_flag, p.spin));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             drain(part, q, warp, 0, 16, inv_row);
@@ -414,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
     const Part last = part_at(max(u0, last_tile * p.k_blocks), u1, p.k_blocks);
     {
         const int quarter = warp & 3, rank = warp >> 2, peers = (kThreads / 32 - quarter + 3) / 4;
-        bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[q_last & 1], (q_last >> 1) & 1, &abort_flag));
+        bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tm_full[q_last & 1], (q_last >> 1) & 1, &abort_flag, p.spin));
         if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t scale = row_s[q_last & 1][quarter * 32 + lane] >> 26;   // exponent field of the fp16 power of two
@@ -423,11 +417,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
         }
     }
     __syncthreads();
+    if (abort_flag) {
+        settle_after_give_up();
+        if (tid == 0) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
+    }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem_dealloc<kTmemCols>(tmem_base);
     }
-    if (tid == 0 && abort_flag) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
 
 // ---- host side ------------------------------------------------------------------------------------
@@ -479,7 +476,7 @@ static bool make_plan(const Geometry& g, int m, bool two, Plan* p) {
 }
 
 template <int WB, bool TWO, int GL>
-static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, cudaStream_t st) {
+static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
     CUtensorMap map, pmap;
     if (cudaError_t e = encode_packed_map(&pmap, packed, g, 8)) return e;
     if (cudaError_t e = encode_x_map(&map, ws + pl.xh_off, g.k_in, m, pl.n_cols)) return e;
@@ -497,6 +494,7 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
     p.n_cols = pl.n_cols;
     p.na = TWO ? 8 : (pl.n_cols <= 64 ? 4 : pl.n_cols <= 128 ? 2 : 1);
     p.tiles_x = pl.tiles_x; p.units = pl.units; p.n_stages = pl.n_stages; p.n_pk = pl.n_pk; p.pk_pieces = packed_pieces(g);
+    p.spin = spin_limit > 0 ? spin_limit : kSpin;
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_mid_kernel<WB, TWO, GL>, pl.smem, smem_attr)) return e;
     // programmatic dependent of the pre-pass: tables, rings, coefficient scan and decode run ahead; only the activations' TMA
@@ -522,8 +520,9 @@ static cudaError_t launch_gl(const Geometry& g, const Plan& pl, const void* pack
 }
 
 template <int WB, bool TWO>
-static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, cudaStream_t st) {
-    return g.group == 128 ? launch_gl<WB, TWO, 7>(g, pl, packed, m, y, y_dtype, ws, st) : launch_gl<WB, TWO, 0>(g, pl, packed, m, y, y_dtype, ws, st);
+static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
+    return g.group == 128 ? launch_gl<WB, TWO, 7>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st)
+                          : launch_gl<WB, TWO, 0>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st);
 }
 
 }  // namespace mid
@@ -557,13 +556,14 @@ size_t gemm_mid_workspace_upto(const Geometry& g, int m) {
     return mid::align256(xh_off + (size_t)m * g.k_in * 2) + grid * 2 * cols * mid::kTileN * sizeof(float);
 }
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws, bool exact,
-                            cudaStream_t st) {
+                            int spin_limit, cudaStream_t st) {
     const bool two = exact && !g.k1;   // single-basis weights: c1 b1 alone is exact already
     mid::Plan p;
     if (!mid::make_plan(g, m, two, &p)) return cudaErrorInvalidValue;
     uint8_t* b = (uint8_t*)ws;
     if (cudaError_t e = tc::launch_x_to_f16(x, g.k_in, m, (uint16_t*)(b + p.xh_off), (float*)(b + p.inv_off), st)) return e;
-#define GOQ_MID(WB_) (two ? mid::launch<WB_, true>(g, p, packed, m, y, y_dtype, b, st) : mid::launch<WB_, false>(g, p, packed, m, y, y_dtype, b, st))
+#define GOQ_MID(WB_) \
+    (two ? mid::launch<WB_, true>(g, p, packed, m, y, y_dtype, b, spin_limit, st) : mid::launch<WB_, false>(g, p, packed, m, y, y_dtype, b, spin_limit, st))
     return g.wbits == 4 ? GOQ_MID(4) : g.wbits == 3 ? GOQ_MID(3) : GOQ_MID(2);
 #undef GOQ_MID
 }

@@ -99,7 +99,7 @@ int gemm_mid_ctas();                           // CTAs of a full grid: one per S
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact);
 size_t gemm_mid_workspace_upto(const Geometry& g, int m);   // enough for every call of up to m rows, either form
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
-                            bool exact, cudaStream_t st);
+                            bool exact, int spin_limit, cudaStream_t st);
 
 // Integer-activation layer.
 // amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch); NaN after a

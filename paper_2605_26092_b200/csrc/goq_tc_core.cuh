@@ -46,6 +46,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
     *abort_flag = 1;
     return false;
 }
+// Copies and MMAs in flight must land before a CTA that has given up lets go of its shared and tensor memory. Their barriers may count
+// arrivals that never come, so this waits a time that none of them takes (a millisecond). Every thread calls it, behind the last barrier.
+__device__ __forceinline__ void settle_after_give_up() {
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    __syncthreads();
+}
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(s32(dst)),
                  "l"(src), "r"(bytes), "r"(s32(bar)) : "memory");

@@ -243,6 +243,36 @@ def test_gemm_on_a_buffer_for_a_larger_batch(goq, n, k, g, b, largest, ms):
         assert np.array_equal(y.cpu().numpy().astype(np.float64), run_gemm_bf16(d, packed, xb))
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(4000, 8192, 128, 3, 200), (4000, 8192, 128, 3, 20)])
+def test_mid_batch_gemm_reports_a_wait_that_runs_out(goq, n, k, g, b, m):
+    """With one poll for the accumulator the mid-batch kernel gives up, either operand form: the status word reads GOQ_ERR_TIMEOUT, the
+    context stays usable, and on a fresh scratch buffer the next call is right again."""
+    from tests.gpu_util import dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    x = dev(si.bf16_activations(m, k, seed=m))
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+
+    def call():
+        y = torch.zeros((m, n), dtype=torch.float32, device="cuda")
+        goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+        return y, goq.workspace_status(ws)
+    prev = goq.set_gemv_variant(4)
+    try:
+        good, status = call()
+        assert status == goq.OK
+        goq.set_wait_limit(1)
+        assert call()[1] == goq.ERR_TIMEOUT
+        goq.set_wait_limit(0)
+        goq.workspace_init(ws)
+        again, status = call()
+        assert status == goq.OK and torch.equal(good, again)
+    finally:
+        goq.set_wait_limit(0)
+        goq.set_gemv_variant(prev)
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
