@@ -248,6 +248,46 @@ def test_small_batches_integer_operand_form(goq, g, b, form):
         assert err <= TIGHT, err
 
 
+@pytest.mark.parametrize("g,b,batch,widths", [
+    (128, 3, 1, (16, 1, 40)),            # fewer records than SMs, one-tile and one-row linears
+    (128, 3, 4, (1030, 129, 256, 64)),   # ragged widths, a range over three linears
+    (64, 2, 6, (2432, 2432)),            # two column groups, several stages a range
+    (32, 3, 3, (700,) * 9),
+])
+def test_linears_that_read_the_same_activations_form_one_range(goq, form, g, b, batch, widths):
+    """Linears side by side on one input (q, k, v; gate, up), outputs of either type, then linears that read the middle one's bf16 output: ordered
+    by data flow (two of them: a span that waits) and, the last, by a flag. Every item against the oracle on the bits that it read."""
+    from tests.gpu_util import dev, check_bf16_output
+    k, mid = 384, len(widths) // 2
+    n_mid = widths[mid] // 128 * 128 if widths[mid] >= 128 else 0
+    first = [_layer(goq, n, k, g, b, seed=70 + i) for i, n in enumerate(widths)]
+    x0 = si.bf16_activations(batch, k, seed=3)
+    xd = dev(x0)
+    out = [torch.zeros((batch, n), dtype=torch.float32 if i == 0 and i != mid else torch.bfloat16, device="cuda") for i, n in enumerate(widths)]
+    items = [(L["d"], L["packed"], xd, batch, y, goq.F32 if y.dtype == torch.float32 else goq.BF16, False) for L, y in zip(first, out)]
+    checks = [(L, xd, y) for L, y in zip(first, out)]
+    if n_mid and widths[mid] % g == 0:   # the whole output feeds the next ones
+        for i, n in enumerate((200, 33, 48)):
+            L, y = _layer(goq, n, widths[mid], g, b, seed=90 + i), torch.zeros((batch, n), dtype=torch.bfloat16, device="cuda")
+            items.append((L["d"], L["packed"], out[mid], batch, y, goq.BF16, i == 2))
+            checks.append((L, out[mid], y))
+    seq, ws = goq.make_sequence(items), _ws(goq, len(items))
+    for _ in range(2):
+        for _, _, y in checks:
+            y.fill_(float("nan"))
+        goq.gemv_sequence(seq, ws)
+        torch.cuda.synchronize()
+        assert goq.workspace_status(ws) == goq.OK
+        for i, (L, x, y) in enumerate(checks):
+            bits = x0 if x is xd else x.view(torch.int16).cpu().numpy().view(np.uint16)
+            y_ref = O.linear_f64(L["codes"], L["meta"], L["coef"], si.bf16_bits_to_f64(bits), g, b)
+            got = y.float().cpu().numpy().astype(np.float64)
+            if y.dtype == torch.float32:
+                assert O.normwise_rel_err(got, y_ref) <= TIGHT, i
+            else:
+                check_bf16_output(got, y_ref, 1e-4, "item %d" % i)
+
+
 @pytest.mark.parametrize("shapes", [
     [(64, 4224, 4), (48, 11008, 3), (300, 256, 1)],      # batch <= 4: integer form unless bf16 operands are forced
     [(32, 4096, 8), (500, 2304, 7), (40, 128, 2)],       # batch up to 8: bf16 operands
