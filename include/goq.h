@@ -192,7 +192,9 @@ goq_status goq_quantize_geo(const goq_desc* desc, const float* w, uint8_t* codes
 /* goq_solve_ref - REF-mode coefficients (Section 3.4, Eq. 3): per row and macro-block, with X_q the calibration inputs
  * restricted to the macro-block's channels, A = [X_q b1, X_q b2], Y = X_q w:  c* = (A^T A + lambda I)^-1 A^T Y.
  *   w [n_out][k_in] fp32; codes, meta as produced by goq_quantize_geo; x_calib [m][k_in] fp32 (m observations);
- *   lambda >= 0 (the paper uses 1e-4);  coef_f16 out [n_out][k_in/group][2];  c_f64 optional out, the unrounded pairs. */
+ *   lambda >= 0 (the paper uses 1e-4);  coef_f16 out [n_out][k_in/group][2];  c_f64 optional out, the unrounded pairs.
+ *   Float64 throughout (sums of the Gram matrix's products in 64-bit fixed point on the tensor cores: no less accurate). If a bounded wait on the device
+ *   gives up, the pairs it would have given are NaN. */
 goq_status goq_solve_ref(const goq_desc* desc, const float* w, const uint8_t* codes, const uint8_t* meta,
                          const float* x_calib, int m, double lambda, uint16_t* coef_f16, double* c_f64, void* stream);
 
@@ -311,8 +313,8 @@ int goq_last_cuda_error(void);
  * 5 = integer-operand kernel of one linear (goq_gemv). Process-wide. Returns the previous value. */
 int goq_set_gemv_variant(int variant);
 
-/* Bound, in polls, of every device-side wait of goq_gemv_sequence, of goq_gemv's integer-operand kernel and of the integer layer on the
- * tensor cores, and of goq_gemm's mid-batch kernel's waits for a finished accumulator (tests only; 0 restores the kernels' own bounds).
+/* Bound, in polls, of every device-side wait of goq_gemv_sequence, of goq_gemv's integer-operand kernel, of the integer layer on the
+ * tensor cores and of goq_solve_ref, and of goq_gemm's mid-batch kernel's waits for a finished accumulator (tests only; 0 restores the kernels' own bounds).
  * With a bound of a few polls a dependent chain gives up at once: the call returns GOQ_OK (it only enqueues), the
  * status word then reads GOQ_ERR_TIMEOUT, the context stays usable. Process-wide. Returns the previous value. */
 int goq_set_wait_limit(int polls);

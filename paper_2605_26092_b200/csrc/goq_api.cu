@@ -295,6 +295,9 @@ goq_status goq_solve_ref(const goq_desc* desc, const float* w, const uint8_t* co
     if (g.k1) return GOQ_ERR_UNSUPPORTED;
     if (!aligned(w, 4) || !aligned(x_calib, 4) || !aligned(coef_f16, 2) || !aligned(c_f64, 8)) return GOQ_ERR_ALIGNMENT;
     if (goq_status s = check_arch()) return s;
+    if (goq::solve_ref_tc_supported(g, w, x_calib, m))
+        return from_cuda(goq::launch_solve_ref_tc(g, w, codes, meta, x_calib, m, lambda, coef_f16, c_f64,
+                                              g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
     return from_cuda(goq::launch_solve_ref(g, w, codes, meta, x_calib, m, lambda, coef_f16, c_f64, (cudaStream_t)stream));
 }
 

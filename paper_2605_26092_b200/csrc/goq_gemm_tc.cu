@@ -495,6 +495,18 @@ cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int 
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
 }
+// fp32 matrix [rows][cols] as boxes of `bc` columns (16: 64 bytes, 64-byte swizzle) x `br` rows
+cudaError_t encode_f32_map(CUtensorMap* map, const float* w, int cols, int rows, int bc, int br) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)bc, (cuuint32_t)br};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(w), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidTexture;
+}
 bool packed_map_supported(const Geometry& g) {
     return (unsigned long long)g.k_blocks * g.unit_bytes / 8 < (1ull << 31);
 }

@@ -117,6 +117,11 @@ cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t
 cudaError_t launch_quantize_geo(const Geometry& g, const float* w, uint8_t* codes, uint8_t* meta, uint16_t* coef, cudaStream_t st);
 cudaError_t launch_solve_ref(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib,
                              int m, double lambda, uint16_t* coef, double* c_out, cudaStream_t st);
+// The same on int8 tensor cores (goq_ref_tc.cu): groups of 32 and more, more observations than half a group, aligned inputs. Without a status
+// word: a give-up of a bounded wait leaves NaN coefficients.
+bool solve_ref_tc_supported(const Geometry& g, const float* w, const float* x_calib, int m);
+cudaError_t launch_solve_ref_tc(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib, int m,
+                                double lambda, uint16_t* coef, double* c_out, int spin_limit, cudaStream_t st);
 cudaError_t launch_quantize_act(const void* x, int x_dtype, int m, int k, int abits, const float* amax, int8_t* xq, float* sx,
                                 cudaStream_t st);
 

@@ -256,6 +256,7 @@ __device__ __forceinline__ void fill_lut(unsigned char* lut, int tid, int n_thre
 // host side, defined in goq_gemm_tc.cu
 cudaError_t encode_x_map(CUtensorMap* map, void* xh, int k_in, int m, int rows);
 cudaError_t encode_i8_map(CUtensorMap* map, const void* x, int k_in, int m, int rows);
+cudaError_t encode_f32_map(CUtensorMap* map, const float* w, int cols, int rows, int bc, int br);
 // packed records as boxes of one k-block x `row_tiles` row tiles (8-byte elements; rows past the end read as zeros). A record is one
 // piece, or two where it has more elements than a box row may (W4 in groups of 8: 288).
 inline int packed_pieces(const Geometry& g) { return g.unit_bytes / 8 > 256 ? 2 : 1; }

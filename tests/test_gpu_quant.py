@@ -225,3 +225,98 @@ def test_ref_solve_matches_oracle(goq, n, k, g, b, m):
     # REF differs from GEO (the calibration covariance is not the identity) but stays a small correction of it
     _, _, c_geo = _objective(w.astype(np.float64), codes, meta, g, b)
     assert not np.allclose(got, c_geo, rtol=1e-3)
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [
+    (1, 128, 128, 3, 65),      # one row, one column, the fewest observations that form a Gram matrix
+    (127, 256, 128, 3, 128),   # a tile short of a row; whole chunks of observations
+    (129, 384, 128, 2, 129),   # a tile and a row
+    (700, 256, 128, 4, 70),    # W4: a positive 2^emax is no int8; several CTAs a column
+    (1100, 128, 128, 3, 300),  # nine tiles over eight CTAs
+    (260, 320, 64, 3, 33), (130, 192, 64, 4, 200), (40, 96, 32, 2, 17), (513, 64, 32, 4, 64), (1500, 32, 32, 3, 1000),
+])
+def test_ref_solve_digits_match_oracle(goq, n, k, g, b, m):
+    """The Gram matrix as byte digits: pairs equal to the oracle's float64 solution (numpy's observations one by one) within 1e-9, as above, also with
+    channels 1000 times the others' magnitude (every row of the matrix has a scale of its own). Rows beyond a sample are compared
+    with the same rows solved alone."""
+    from tests.gpu_util import dev
+    w = si.gaussian_weights(n, k, seed=n + m).astype(np.float32)
+    codes, meta, _ = O.quantize_geo(w, g, b)
+    x = si.f32_activations(m, k, seed=m).astype(np.float32)
+    x[:, ::37] *= np.float32(1000.0)
+
+    def solve(rows):
+        d = goq.desc(len(rows), k, g, b)
+        coef = torch.zeros((len(rows), k // g, 2), dtype=torch.int16, device="cuda")
+        c64 = torch.zeros((len(rows), k // g, 2), dtype=torch.float64, device="cuda")
+        goq.solve_ref(d, dev(w[rows]), dev(codes[rows]), dev(meta[rows]), torch.from_numpy(x).cuda(), m, 1e-4, coef, c64)
+        torch.cuda.synchronize()
+        got = c64.cpu().numpy()
+        assert np.array_equal(coef.cpu().numpy().view(np.uint16), got.astype(np.float16).view(np.uint16))
+        return got
+    got = solve(np.arange(n))
+    rows = np.unique(np.concatenate([np.arange(min(n, 40)), np.arange(max(0, n - 40), n)]))
+    assert np.allclose(got[rows], O.solve_ref(w[rows], codes[rows], meta[rows], x, g, b, lam=1e-4), rtol=1e-9, atol=1e-12)
+    for lo in range(0, n, 500):
+        part = np.arange(lo, min(n, lo + 500))
+        assert np.array_equal(solve(part), got[part])
+
+
+def test_ref_solve_non_finite_inputs_and_unaligned_buffers(goq):
+    """A NaN observation makes its column's pairs NaN and no other's; codes, weights and observations at any element's address are taken."""
+    from tests.gpu_util import dev
+    n, k, g, b, m = 140, 256, 128, 3, 100
+    w = si.gaussian_weights(n, k, seed=5).astype(np.float32)
+    codes, meta, _ = O.quantize_geo(w, g, b)
+    x = si.f32_activations(m, k, seed=6).astype(np.float32)
+    d = goq.desc(n, k, g, b)
+
+    def solve(xd, wd, cd):
+        coef = torch.zeros((n, k // g, 2), dtype=torch.int16, device="cuda")
+        c64 = torch.zeros((n, k // g, 2), dtype=torch.float64, device="cuda")
+        goq.solve_ref(d, wd, cd, dev(meta), xd, m, 1e-4, coef, c64)
+        torch.cuda.synchronize()
+        return c64.cpu().numpy()
+
+    def off(a, by):   # the same array `by` elements behind an aligned address
+        t = dev(a)
+        buf = torch.empty(t.numel() + by, dtype=t.dtype, device="cuda")
+        buf[by:] = t.reshape(-1)
+        return buf[by:]
+    c_ref = O.solve_ref(w, codes, meta, x, g, b, lam=1e-4)
+    for by_x, by_w, by_c in ((0, 0, 0), (0, 0, 1), (0, 0, 4), (1, 0, 0), (0, 3, 0)):
+        assert np.allclose(solve(off(x, by_x), off(w, by_w), off(codes, by_c)), c_ref, rtol=1e-9, atol=1e-12)
+    for bad in (np.nan, np.inf):
+        xb = x.copy()
+        xb[7, 130] = bad
+        got = solve(dev(xb), dev(w), dev(codes))
+        assert np.isnan(got[:, 1]).all() and np.allclose(got[:, 0], c_ref[:, 0], rtol=1e-9, atol=1e-12)
+
+
+def test_ref_solve_that_gives_up_leaves_nan(goq):
+    """goq_solve_ref has no scratch: a bounded wait that runs out shows as NaN coefficients, and the next call is whole again."""
+    from tests.gpu_util import dev
+    n, k, g, b, m = 600, 256, 128, 3, 100
+    w = si.gaussian_weights(n, k, seed=5).astype(np.float32)
+    codes, meta, _ = O.quantize_geo(w, g, b)
+    x = si.f32_activations(m, k, seed=6).astype(np.float32)
+    d = goq.desc(n, k, g, b)
+    args = (dev(w), dev(codes), dev(meta), torch.from_numpy(x).cuda())
+    c64 = torch.zeros((n, k // g, 2), dtype=torch.float64, device="cuda")
+    coef = torch.zeros((n, k // g, 2), dtype=torch.int16, device="cuda")
+    goq.solve_ref(d, *args, m, 1e-4, coef, c64)
+    torch.cuda.synchronize()
+    want = c64.cpu().numpy()
+    goq.set_wait_limit(1)
+    try:
+        goq.solve_ref(d, *args, m, 1e-4, coef, c64)
+        torch.cuda.synchronize()
+    finally:
+        goq.set_wait_limit(0)
+    got = c64.cpu().numpy()
+    whole = np.isfinite(got).all(axis=2)
+    assert np.array_equal(got[whole], want[whole])   # a column whose waits all held
+    assert not whole.all()
+    goq.solve_ref(d, *args, m, 1e-4, coef, c64)
+    torch.cuda.synchronize()
+    assert np.array_equal(c64.cpu().numpy(), want)
