@@ -33,6 +33,22 @@ goq_status check_arch() {
     return ok ? GOQ_OK : GOQ_ERR_ARCH;
 }
 
+// Estimated times of the other kernels for a few tokens, us (W3 g128, W4; the kernels in e4m3 operands have gemm_f8_us). One decode launch of up to
+// 16 tokens: measured 5.2 for 2048 x 2048, 8.2 4096 x 4096, 19.1 11008 x 4096, 27.4 8192 x 8192, 83 28672 x 8192 at 16 tokens, 22 and 66 for the last two at 8.
+float decode_us(const Geometry& g, int m) {
+    return 4.f + (float)g.n_units * ((m > 8 ? 7.0e-4f : 5.5e-4f) + (g.wbits == 4 ? 1.0e-4f : 0.f));
+}
+// The mid-batch kernel up to 256 tokens: 34.6 for 8192 x 8192, 21 4096 x 4096, 18.5 2048 x 2048, 23 1024 x 8192 at 64 tokens, 39.5 and 23 for the first two at 128.
+float mid_us(const Geometry& g, int m, bool exact) {
+    const int tiles = (g.n_tiles + 7) / 8, units = tiles * g.k_blocks, sms = goq::gemm_mid_ctas(), grid = units < sms ? units : sms;
+    const float unit = (exact ? 0.8f : 0.55f + 0.0032f * (float)m) + (g.wbits == 4 ? 0.08f : 0.f) + (g.group < 128 ? 0.03f : 0.f);
+    return 13.f + 0.4f * (float)grid / (float)tiles + unit * (float)((units + grid - 1) / grid);
+}
+// goq_gemv on the kernel in e4m3 operands: above 4 tokens (or W4, which has no integer form), large linears only; W2 and W3 where a call needs scratch anyway
+bool gemv_takes_f8(const Geometry& g, int m) {
+    return (g.wbits == 4 || (m > 4 && goq::gemv_stream_supported(g))) && goq::gemm_f8_supported(g, m) && goq::gemm_f8_us(g, m) <= 0.97f * decode_us(g, m);
+}
+
 std::atomic<int> g_last_cuda_error{0};
 goq_status from_cuda(cudaError_t e) { return goq::status_from_cuda(e); }
 
@@ -83,6 +99,10 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
     if (op == GOQ_OP_GEMV && m <= 16) {
         size_t need = 0;
         if (goq::gemv_stream_supported(g)) need = goq::gemv_stream_workspace(g);
+        if (gemv_takes_f8(g, m)) {   // (with less the call takes another kernel)
+            const size_t f8 = goq::gemm_f8_workspace(g, m);
+            if (f8 > need) need = f8;
+        }
         return need;
     }
     if (op == GOQ_OP_GEMM) {
@@ -96,6 +116,7 @@ size_t goq_workspace_bytes(const goq_desc* desc, int op, int m) {
         }
         if (goq::gemv_stream_supported(g)) cover(goq::gemv_stream_workspace(g));
         cover(goq::gemm_mid_workspace_upto(g, m));
+        cover(goq::gemm_f8_workspace_upto(g, m < kGemmMidMaxTokens ? m : kGemmMidMaxTokens));
         return need;
     }
     return 0;
@@ -150,6 +171,11 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
                                                   (cudaStream_t)stream));
         if (variant == 3) return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
     }
+    // Large linears above 4 tokens (W4: any number): both bases as e4m3 operands of the tensor cores, half the decode's instructions, for a pre-pass and a
+    // summing kernel around it. us, fragment kernel / this: W3 28672 x 8192 66 / 54 at 8 tokens, 83 / 55 at 16; 8192 x 8192 22.0 / 22.8 and 27.4 / 23.2;
+    // W4 26.7 / 23.9 at 8 tokens; 4096 x 4096 at 16 tokens 8.2 / 13.4.
+    if (variant == 0 && gemv_takes_f8(g, batch) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_f8_workspace(g, batch))
+        return from_cuda(goq::launch_gemm_f8(g, packed, x_bf16, batch, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
     if (variant == 0 && goq::gemv_mma_supported(g, batch))
         return from_cuda(goq::launch_gemv_mma(g, packed, x_bf16, batch, y, y_dtype, true, (cudaStream_t)stream));
     bool use_mma = goq::linear_mma_supported(g);
@@ -171,7 +197,8 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (!y) return GOQ_ERR_INVALID_ARG;
         if (goq_status s = check_arch()) return s;
         const int variant = g_gemv_variant.load(std::memory_order_relaxed);
-        // Three kernels: the decode GEMV (16 tokens a launch), the mid-batch kernel (an even split of the packed records over the SMs; up to
+        // Four kernels: the decode GEMV (16 tokens a launch), the kernel in e4m3 operands (a few tokens to about 128, fp32 accuracy, no rounding of
+        // weights), the mid-batch kernel (an even split of the packed records over the SMs; up to
         // 32 tokens with both bases as exact operands, above with w_hat rounded once to fp16) and the prefill kernel (128 x 512 tiles).
         //   Up to 32 tokens: groups of 8 and 16 have only the mid-batch kernel that keeps fp32 accuracy. Others take two decode launches
         //   unless the linear is large or wide (units = 16-row tiles x k-blocks). Measured at 17 tokens, W3 g128, us, mid-batch over decode:
@@ -183,7 +210,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         //   (the prefill kernel's is the surer one, hence the margin). us, mid-batch / prefill: 1024 x 8192 W4 at 777 tokens 35 / 102;
         //   4096 x 4096 at 1024 52 / 54; 11008 x 4096 at 512 69 / 65; 16000 x 512 at 512 40 / 23.
         const bool exact = m <= kGemmExactMaxTokens, narrow = !goq::gemv_mma_supported(g, 16);
-        bool mid_wanted = variant == 4;
+        bool mid_wanted = variant == 4, f8_wanted = variant == 6;
         if (variant == 0) {
             if (exact) {
                 mid_wanted = narrow || (m > 16 && (g.n_units >= 12000 || (g.n_tiles >= 500 && g.n_units >= 8000) || g.n_tiles >= 1700));
@@ -193,10 +220,20 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
             } else {
                 mid_wanted = !goq::gemm_tc_supported(g) || goq::gemm_mid_us(g, m) <= 0.95f * goq::gemm_tc_us(g, m);
             }
+            //   Up to 256 tokens, groups of 32 and more: e4m3 operands where the estimates say so. us, the others / e4m3: at 32 tokens 4096 x 4096 17.4 / 14.6,
+            //   28672 x 8192 98 / 61, 2048 x 2048 10.9 / 12.3, 1024 x 8192 13.6 / 15.2; at 64 2048 x 2048 18.5 / 13.6, 28672 x 8192 90 / 78, in groups of
+            //   64 8192 x 8192 36 / 42, 4096 x 4096 21.6 / 19.6; at 128 (two token tiles) 2048 x 2048 20 / 14.8, 8192 x 8192 39.7 / 50.6.
+            if (m <= 16) f8_wanted = !narrow && gemv_takes_f8(g, m);
+            else if (m <= kGemmMidMaxTokens && goq::gemm_f8_supported(g, m)) {
+                const int second = m - 16;   // (up to 32 tokens: of the second decode launch)
+                f8_wanted = goq::gemm_f8_us(g, m) <= 0.97f * (exact && !mid_wanted ? decode_us(g, 16) + decode_us(g, second) : mid_us(g, m, exact));
+            }
         }
+        if (f8_wanted && goq::gemm_f8_supported(g, m) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_f8_workspace(g, m))
+            return from_cuda(goq::launch_gemm_f8(g, packed, x, m, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
         if (mid_wanted && goq::gemm_mid_supported(g, m, exact) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_mid_workspace(g, m, exact))
             return from_cuda(goq::launch_gemm_mid(g, packed, x, m, y, y_dtype, ws, exact, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
-        if (variant == 4) return GOQ_ERR_UNSUPPORTED;
+        if (variant == 4 || variant == 6) return GOQ_ERR_UNSUPPORTED;
         // the decode GEMV, 16 tokens per launch
         if (exact && variant == 0 && goq::gemv_mma_supported(g, 16)) {
             if (goq::gemv_stream_supported(g)) {

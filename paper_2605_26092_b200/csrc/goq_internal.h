@@ -101,6 +101,13 @@ size_t gemm_mid_workspace_upto(const Geometry& g, int m);   // enough for every 
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
                             bool exact, int spin_limit, cudaStream_t st);
 
+// The same layer for a few tokens up to about 128 (goq_gemm_f8.cu): both bases as exact e4m3 operands, activations as two e4m3 slices; group >= 32.
+bool gemm_f8_supported(const Geometry& g, int m);
+float gemm_f8_us(const Geometry& g, int m);   // estimated time
+size_t gemm_f8_workspace(const Geometry& g, int m);
+size_t gemm_f8_workspace_upto(const Geometry& g, int m);
+cudaError_t launch_gemm_f8(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws, int spin_limit, cudaStream_t st);
+
 // Integer-activation layer.
 // amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch); NaN after a
 // give-up. spin_limit > 0 replaces the bound of every device-side wait (tests).

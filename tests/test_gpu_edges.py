@@ -273,6 +273,96 @@ def test_mid_batch_gemm_reports_a_wait_that_runs_out(goq, n, k, g, b, m):
         goq.set_gemv_variant(prev)
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [
+    (1, 32, 32, 3, 1), (129, 160, 32, 4, 33), (127, 256, 64, 2, 48), (128, 128, 128, 3, 16), (4000, 384, 128, 3, 17), (300, 640, 128, 4, 64),
+    (1000, 4096, 32, 3, 65), (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 128), (19200, 128, 128, 3, 24), (257, 1152, 64, 4, 129), (1100, 2304, 128, 3, 200)])
+def test_e4m3_operand_gemm_edges(goq, n, k, g, b, m):
+    """Both bases and two slices of the activations as e4m3 numbers: channel and token tiles that do not fill, every bit width and number of macro-blocks a
+    k-block, one unit in all, one tile shared by many SMs, tiles an SM has whole; tokens of tiny and huge magnitude, of zeros, and with one element 2^14
+    times the others (exact: 2^-15). Twice, bit for bit, two calls back to back. Bounds as for every fp32-accumulating kernel."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    x = si.bf16_bits_to_f64(si.bf16_activations(m, k, seed=m))
+    x[0, k // 2] *= 2.0 ** 14
+    if m > 3:
+        x[1] *= 2.0 ** -100
+        x[2] *= 2.0 ** 100
+        x[3] = 0.0
+    xb = si.f32_to_bf16_bits(x.astype(np.float32))
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b)
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+    prev = goq.set_gemv_variant(6)
+    try:
+        out = [torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda") for _ in range(2)]
+        y16 = torch.full((m, n), float("nan"), dtype=torch.bfloat16, device="cuda")
+        for y in out:
+            goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y16, y_dtype=goq.BF16, ws=ws)
+        torch.cuda.synchronize()
+        assert goq.workspace_status(ws) == goq.OK
+    finally:
+        goq.set_gemv_variant(prev)
+    assert torch.equal(out[0], out[1]) and torch.equal(y16, out[0].to(torch.bfloat16))
+    got = out[0].cpu().numpy().astype(np.float64)
+    scale = np.ones((m, 1))
+    if m > 3:
+        scale[1], scale[2] = 2.0 ** 100, 2.0 ** -100   # tokens of one magnitude again, for the element-wise bound
+        assert not got[3].any()
+    check_parity(got * scale, y_ref * scale, 2e-5, 1e-4)
+
+
+@pytest.mark.parametrize("n,k,g,b,m", [(8192, 4096, 128, 4, 4), (12000, 4096, 128, 3, 16), (9000, 8192, 64, 2, 9), (4000, 4096, 128, 3, 30), (16000, 512, 64, 4, 17),
+                                       (4096, 4096, 64, 3, 64), (2048, 2048, 128, 3, 128), (8192, 2048, 128, 3, 128)])
+def test_calls_either_side_of_the_lines_of_the_e4m3_kernel(goq, n, k, g, b, m):
+    """Automatic dispatch next to the lines of that kernel, through goq_gemm and (up to 16 tokens) goq_gemv, with a buffer of the documented size and, for
+    goq_gemv at W4, with none. Sampled channels; 2e-5 up to 32 tokens, 5e-4 (w_hat rounded once to fp16) above."""
+    from tests.gpu_util import check_parity, dev, pack_weights, run_gemm_bf16, run_gemv
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    rows = np.unique(np.concatenate([si.sample_rows(n, 200, seed=2), np.arange(n - 20, n)]))
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b, rows=rows)
+    tol = (2e-5, 1e-4) if m <= 32 else (5e-4, 2e-3)
+    check_parity(run_gemm_bf16(d, packed, xb)[:, rows], y_ref, *tol)
+    if m <= 16:
+        check_parity(run_gemv(d, packed, xb)[:, rows], y_ref, *tol)
+        if b == 4:
+            y = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+            goq.gemv(d, packed, dev(xb), m, y, goq.F32)
+            torch.cuda.synchronize()
+            check_parity(y.cpu().numpy().astype(np.float64)[:, rows], y_ref, *tol)
+
+
+def test_e4m3_operand_gemm_reports_a_wait_that_runs_out(goq):
+    """With one poll a wait the kernel gives up: the status word reads GOQ_ERR_TIMEOUT, and on a fresh scratch buffer the next call is right again."""
+    from tests.gpu_util import dev, pack_weights
+    n, k, g, b, m = 4000, 8192, 128, 3, 40
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    x = dev(si.bf16_activations(m, k, seed=m))
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+
+    def call():
+        y = torch.zeros((m, n), dtype=torch.float32, device="cuda")
+        goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+        return y, goq.workspace_status(ws)
+    prev = goq.set_gemv_variant(6)
+    try:
+        good, status = call()
+        assert status == goq.OK
+        goq.set_wait_limit(1)
+        assert call()[1] == goq.ERR_TIMEOUT
+        goq.set_wait_limit(0)
+        goq.workspace_init(ws)
+        again, status = call()
+        assert status == goq.OK and torch.equal(good, again)
+    finally:
+        goq.set_wait_limit(0)
+        goq.set_gemv_variant(prev)
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
