@@ -1,4 +1,5 @@
-// Prefill GEMM (float activations, many tokens) on the 5th-generation tensor cores.
+// Prefill GEMM (float activations, many tokens) on the 5th-generation tensor cores: the pre-pass of every such call, and the kernel for up to 256 tokens and
+// for the formats that goq_gemm_pair.cu does not hold.
 //
 // Eq. 4 of the paper with the coefficients folded into the weight operand:
 //   y[m,n] = sum_k x[m,k] * w_hat[n,k],   w_hat[n,k] = c1[n,j] b1[n,k] + c2[n,j] b2[n,k]   (Section 3.1)
@@ -525,8 +526,8 @@ cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geomet
 }
 // The activation pre-pass (and, with `row_tiles` blocks more, the channel scales) as a programmatic dependent of what precedes it:
 // its launch overlaps the tail of that kernel.
-static cudaError_t launch_pre_pass(const void* x, int k_in, int m, int row_tiles, uint16_t* xh, float* inv_scale, const void* packed,
-                                   int unit_bytes, int k_blocks, int gpb, uint32_t* row_scale, float* row_inv, cudaStream_t st) {
+cudaError_t launch_pre_pass(const void* x, int k_in, int m, int row_tiles, uint16_t* xh, float* inv_scale, const void* packed,
+                            int unit_bytes, int k_blocks, int gpb, uint32_t* row_scale, float* row_inv, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m + row_tiles);
     cfg.blockDim = dim3(kPrepThreads);
@@ -595,6 +596,10 @@ static size_t smem_bytes(const Geometry& g) {
            (size_t)2 * kExpanders * g.unit_bytes + 16 * sizeof(uint64_t);
 }
 
+// More than 256 tokens: pairs of SMs wherever their four stages fit (all but groups of 8, and W4 in groups of 16). Faster at every shape measured
+// (goq_gemm_pair.cu), 2048 x 2048 at 2048 tokens 34 -> 30 us, 4096 x 4096 at 300 52 -> 44, 16000 x 512 at 512 23.1 -> 22.7.
+static bool takes_pairs(const Geometry& g, int m) { return gemm_pair_supported(g, m); }
+
 template <int WB>
 static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, int* status,
                              float* inv_scale, uint32_t* row_scale, float* row_inv, uint16_t* xh, int* tile_counter, float* partial,
@@ -602,6 +607,7 @@ static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* 
     if (g.k_in % 8 != 0) return cudaErrorInvalidValue;
     if (cudaError_t e = launch_pre_pass(x, g.k_in, m, g.n_tiles, xh, inv_scale, packed, g.unit_bytes, g.k_blocks, g.groups_per_block,
                                         row_scale, row_inv, st)) return e;
+    if (takes_pairs(g, m)) return launch_gemm_pair(g, packed, xh, inv_scale, row_scale, row_inv, m, y, y_dtype, status, st);
     CUtensorMap map;
     const TokenTiles tt = token_tiles(g, m);
     if (cudaError_t e = encode_x_map(&map, xh, g.k_in, m, tt.half)) return e;
@@ -674,7 +680,7 @@ TcScratch tc_scratch(const Geometry& g, int m) {
 }
 }  // namespace
 // estimated time of a call of more than 256 tokens (pre-pass and launch 9 us)
-float gemm_tc_us(const Geometry& g, int m) { return 9.f + tc::token_tiles(g, m).us; }
+float gemm_tc_us(const Geometry& g, int m) { return tc::takes_pairs(g, m) ? gemm_pair_us(g, m) : 9.f + tc::token_tiles(g, m).us; }
 size_t gemm_tc_workspace(const Geometry& g, int m) { return tc_scratch(g, m).total; }
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws,
                            cudaStream_t st) {

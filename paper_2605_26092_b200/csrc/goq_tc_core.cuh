@@ -207,7 +207,8 @@ __device__ __forceinline__ uint32_t hfma2(uint32_t a, uint32_t b, uint32_t c) {
 // nibbles are full (the sign is bit 3), the record comes from the unit's byte plane (`record`) and the table is filled
 // in record order; the high byte is taken from a positive or a negative table per weight, chosen by a byte mask that
 // prmt's sign-replicate mode makes of the sign bits (top bit of each byte of w: odd weights; of w << 4: even weights).
-template <int WB>
+// ADD: the table lies at any 1 KiB boundary (one more addition a word).
+template <int WB, bool ADD = false>
 __device__ __forceinline__ void expand_bases(uint32_t w, uint32_t record, uint32_t lut_lane, uint32_t (&R)[4], uint32_t (&Q)[4]) {
     const uint32_t m = w & 0x77777777u, mh = m >> 16;
     uint32_t ha, hb, slot_off;
@@ -222,7 +223,7 @@ __device__ __forceinline__ void expand_bases(uint32_t w, uint32_t record, uint32
         hb = (prmt(PotBytes4::PH0, PotBytes4::PH1, mh) & ~mb) | (prmt(PotBytes4::NH0, PotBytes4::NH1, mh) & mb);
         slot_off = (record & 63u) << 7;
     }
-    const uint4 e = lds128(slot_off | lut_lane);  // table is 8 KiB aligned, lut_lane selects the copy
+    const uint4 e = lds128(ADD ? slot_off + lut_lane : slot_off | lut_lane);  // table is 8 KiB aligned, lut_lane selects the copy
     const uint32_t qa = prmt(ha, hb, e.x) ^ e.z, qb = prmt(ha, hb, e.y) ^ e.w;   // b2: permuted, pair signs applied
     // bytes {0, h[2q], 0, h[2q+1]}: weights 2q, 2q+1 as one f16x2 word
     R[0] = prmt(ha, 0u, 0x1404u); R[1] = prmt(ha, 0u, 0x3424u); R[2] = prmt(hb, 0u, 0x1404u); R[3] = prmt(hb, 0u, 0x3424u);
@@ -230,10 +231,10 @@ __device__ __forceinline__ void expand_bases(uint32_t w, uint32_t record, uint32
 }
 // w_hat = c1*b1 + c2*b2 in fp16. c1, c2: the coefficient in both halves of a register. c1*b1 is a power-of-two scaling (exact)
 // and the fused multiply-add rounds once: the same value as fp32 arithmetic rounded to fp16.
-template <int WB>
+template <int WB, bool ADD = false>
 __device__ __forceinline__ void expand_what(uint32_t w, uint32_t record, uint32_t lut_lane, uint32_t c1, uint32_t c2, uint32_t (&out)[4]) {
     uint32_t R[4], Q[4];
-    expand_bases<WB>(w, record, lut_lane, R, Q);
+    expand_bases<WB, ADD>(w, record, lut_lane, R, Q);
 #pragma unroll
     for (int q = 0; q < 4; ++q) out[q] = hfma2(c2, Q[q], hmul2(c1, R[q]));
 }
@@ -263,6 +264,9 @@ inline int packed_pieces(const Geometry& g) { return g.unit_bytes / 8 > 256 ? 2 
 bool packed_map_supported(const Geometry& g);
 cudaError_t encode_packed_map(CUtensorMap* map, const void* packed, const Geometry& g, int row_tiles);
 cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float* inv_scale, cudaStream_t st);
+// ... and, with `row_tiles` CTAs more, the channel scales
+cudaError_t launch_pre_pass(const void* x, int k_in, int m, int row_tiles, uint16_t* xh, float* inv_scale, const void* packed,
+                            int unit_bytes, int k_blocks, int gpb, uint32_t* row_scale, float* row_inv, cudaStream_t st);
 
 }  // namespace tc
 }  // namespace goq

@@ -363,6 +363,38 @@ def test_e4m3_operand_gemm_reports_a_wait_that_runs_out(goq):
         goq.set_gemv_variant(prev)
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [
+    (40, 64, 32, 3, 257),        # one channel tile: the pair's second CTA has none; one k-block, half of it padding
+    (300, 640, 64, 4, 300),      # three tiles, W4
+    (260, 256, 16, 2, 1000),     # token tiles that do not fill, narrow groups
+    (19000, 128, 128, 3, 513),   # one more pair of tiles than pairs of SMs: the last ones as token halves
+    (9600, 512, 128, 3, 600),    # full and half tiles in one launch
+    (512, 2176, 128, 2, 4100),
+    (4096, 4096, 128, 3, 2048)])  # every pair busy: records, stages and hops at full rate
+def test_prefill_gemm_on_pairs_of_sms_edges(goq, n, k, g, b, m):
+    """More than 256 tokens: channel tiles, token tiles and k that do not fill a pair, twice back to back, bit for bit. w_hat rounded once to fp16: 5e-4."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    xb = si.bf16_activations(m, k, seed=m)
+    rows = np.unique(np.concatenate([si.sample_rows(n, min(n, 150), seed=2), np.arange(n - 20, n)]))
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b, rows=rows)
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+    out = [torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda") for _ in range(2)]
+    y16 = torch.full((m, n), float("nan"), dtype=torch.bfloat16, device="cuda")
+    prev = goq.set_gemv_variant(3)   # the prefill kernels whatever the estimates
+    try:
+        for y in out:
+            goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        goq.gemm(d, packed, dev(xb), m, goq.BF16, y=y16, y_dtype=goq.BF16, ws=ws)
+        torch.cuda.synchronize()
+    finally:
+        goq.set_gemv_variant(prev)
+    assert goq.workspace_status(ws) == goq.OK
+    assert torch.equal(out[0], out[1]) and torch.equal(y16, out[0].to(torch.bfloat16))
+    check_parity(out[0].cpu().numpy().astype(np.float64)[:, rows], y_ref, 5e-4, 2e-3)
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
