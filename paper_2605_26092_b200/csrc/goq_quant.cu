@@ -27,15 +27,16 @@ __device__ __forceinline__ double lattice_value(int c, int wbits) {
 // ---- GEO quantizer -----------------------------------------------------------------------------------------
 // A lane owns a whole micro-block (8 weights), so all four pair patterns stay inside the thread; the LPG = group / 8 lanes
 // of a macro-block share its sums. Everything is flat: macro-blocks do not straddle rows, so lane l of a warp takes
-// micro-block base + l whatever the shape. Bound: the float64 pipe (about 110 operations per micro-block) and the memory
-// system, near each other. What keeps float64 work down without changing one result:
-//   - codes need no division (rtn_codes);
+// micro-block base + l whatever the shape. Bound: instruction issue, with the float64 pipe (about 85 operations per
+// micro-block) and the memory system near behind. What keeps float64 work down without changing one result:
+//   - codes need no division (rtn_codes), the two quotients share one reciprocal (quotient), ||b1||^2 is summed in integers (norm_units);
 //   - every product has a power of two as a factor, hence is exact; ||b2||^2 = ||b1||^2 (b2 is a signed permutation
 //     of b1), <w, b2> is the sum of the chosen patterns' |d|;
 // Sums are added in a fixed order: elements 0..3 and 4..7 of a micro-block apart, each over the lanes from the farthest
 // partner down, then the halves.
-// Measured, 11008 x 4096 W3 g128: 92 us (one lane per four weights, with a float64 quotient per weight and a warp-wide float64
-// reduction for every sum: 438 us). 62 registers and 32 warps an SM: latency, not a pipe, is what is left (float64 pipe ~30 %).
+// Measured, 11008 x 4096 W3 g128: 84 us (two float64 divisions, ||b1||^2 in float64 and the sums of |d| as two halves: 92; one lane per four weights, with a
+// float64 quotient per weight and a warp-wide float64 reduction for every sum: 438). 62 registers and 32 warps an SM, issue slots ~70 % busy: the number
+// of instructions counts. Not kept: the next micro-block's loads in flight (24 warps 89 us, 32 warps with spills 98), 32-byte loads (88).
 template <int LPG>
 __device__ __forceinline__ double group_sum2(double p0, double p1) {
     if constexpr (LPG == 1) {
@@ -48,6 +49,29 @@ __device__ __forceinline__ double group_sum2(double p0, double p1) {
         for (int o = o0 / 2; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
         return v + __shfl_xor_sync(kFull, v, o0);
     }
+}
+
+// a / b rounded to nearest, as a division would, given r = 1/b to about 2^-42. b = ||b1||^2 is an integer of at most 21 bits times a power of two. Then
+//   q = a r is off by at most 2^11 ulp, so a - q b fits 53 bits and the fma gives it exactly, and the corrected quotient is off by 2^-31 ulp before its one
+//   rounding; a / b itself is never a midpoint of two doubles (54-bit odd times b has more bits than a) and at least 2^-22 ulp away from one.
+// No underflow: a is a multiple of 2^-156. An infinite a stays what it is.
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+    const double q = a * r;
+    return fabs(q) <= 1.7976931348623157e308 ? fma(fma(-q, b, a), r, q) : q;
+}
+// sum over a micro-block of (b1 2^emax)^2: the magnitudes as bytes
+template <int WB>
+__device__ __forceinline__ uint32_t norm_units(uint32_t code) {
+    // W3 codes 0..7: 8 4 2 0 8 4 2 1;  W2 codes 0..3: 2 0 2 1;  W4 by e: 128 64 32 16 8 4 2 and 0 (the zero; -2^-7, code 15, is counted apart)
+    constexpr uint32_t t0 = WB == 3 ? 0x00020408u : WB == 2 ? 0x01020002u : 0x10204080u, t1 = WB == 3 ? 0x01020408u : WB == 2 ? 0u : 0x00020408u;
+    const uint32_t sel = WB == 4 ? code & 0x77777777u : code;
+    const uint32_t a = __byte_perm(t0, t1, sel), b = __byte_perm(t0, t1, sel >> 16);
+    uint32_t n = __dp4a(a, a, __dp4a(b, b, 0u));
+    if constexpr (WB == 4) {
+        const uint32_t two = code & (code >> 1);
+        n += __popc(two & (two >> 2) & 0x11111111u);
+    }
+    return n;
 }
 
 // Codes of a micro-block, a nibble each: nearest lattice state in linear distance, exact ties to the state of smaller
@@ -138,18 +162,18 @@ quantize_geo_kernel(const float* __restrict__ w, uint8_t* __restrict__ codes, ui
 #pragma unroll
     for (int o = LPG / 2; o; o >>= 1) s = fmaxf(s, __shfl_xor_sync(kFull, s, o));
     const uint32_t code = rtn_codes<WB>(wf, midpoints<WB>(s));
-    double x[8], p[2] = {0.0, 0.0}, n2 = 0.0;
+    double x[8], p[2] = {0.0, 0.0};
     code_values<WB>(code, x);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        p[i >> 2] = fma((double)wf[i], x[i], p[i >> 2]);   // exact product
-        n2 = fma(x[i], x[i], n2);
-    }
-    float nb = (float)n2;   // ||b1||^2: a multiple of 2^(-2 emax), at most 128, so exact in fp32 whatever the order
+    for (int i = 0; i < 8; ++i) p[i >> 2] = fma((double)wf[i], x[i], p[i >> 2]);   // exact product
+    uint32_t nu = norm_units<WB>(code);
 #pragma unroll
-    for (int o = LPG / 2; o; o >>= 1) nb += __shfl_xor_sync(kFull, nb, o);
+    for (int o = LPG / 2; o; o >>= 1) nu += __shfl_xor_sync(kFull, nu, o);
+    const float nb = (float)nu * (1.0f / (float)(1 << (2 * Midpoints<WB>::emax)));   // ||b1||^2: at most 128 and 21 bits, exact
+    double rb = (double)__fdividef(1.0f, nb);
+    rb = fma(fma(-rb, (double)nb, 1.0), rb, rb);   // one Newton step: 2^-21 -> 2^-42
     // zero-norm bypass: an all-zero block keeps c1 = c2 = 0
-    const double c1 = nb == 0.f ? 0.0 : group_sum2<LPG>(p[0], p[1]) / (double)nb;
+    const double c1 = nb == 0.f ? 0.0 : quotient(group_sum2<LPG>(p[0], p[1]), (double)nb, rb);
     double c2 = 0.0;
     uint32_t rec = 0;
     if constexpr (!K1) {
@@ -177,8 +201,10 @@ quantize_geo_kernel(const float* __restrict__ w, uint8_t* __restrict__ codes, ui
             if (a > best) { best = a; rec = f; }
         }
         // step 3 and Eq. 2: with eta = sgn d, <w, b2> of the micro-block is the chosen pattern's sum |d| (<b1, b2> = 0)
-        const double wb2 = group_sum2<LPG>(best, 0.0);
-        c2 = nb == 0.f ? 0.0 : wb2 / (double)nb;
+        double wb2 = best;
+#pragma unroll
+        for (int o = LPG / 2; o; o >>= 1) wb2 += __shfl_xor_sync(kFull, wb2, o);
+        c2 = nb == 0.f ? 0.0 : quotient(wb2, (double)nb, rb);
         if (nb == 0.f) rec = 0;   // s_norm = 0 iff b1 = 0: the largest weight never rounds to zero
     }
     if (!on) return;

@@ -203,6 +203,32 @@ def test_geo_quantizer_single_basis_layout(goq):
     assert np.array_equal(coef.cpu().numpy().view(np.uint16), f_o.view(np.uint16))
 
 
+@pytest.mark.parametrize("b", [2, 3, 4])
+@pytest.mark.parametrize("g", [8, 16, 128])
+def test_geo_first_coefficient_is_the_rounded_quotient(goq, g, b):
+    """c1 = <w, b1> / ||b1||^2 (Eq. 2) bit for bit. Weights are integers / 1024, so both sums are exact whatever their order; blocks from a single large
+    weight to all at the smallest negative state, whose norms run over their whole range."""
+    rng = np.random.default_rng(g + b)
+    n, k = 64, 1024
+    w = rng.integers(-1000, 1001, size=(n, k)).astype(np.float32) / 1024
+    w *= (rng.random((n, k)) < np.linspace(0.01, 1.0, n)[:, None])
+    w[1] = 0.0
+    w[2] = 1.0
+    w[3] = -2.0 ** -(2 ** (b - 1) - 1); w[3, ::g] = -1.0
+    d = goq.desc(n, k, g, b)
+    codes = torch.empty((n, k), dtype=torch.uint8, device="cuda")
+    meta = torch.empty((n, k // 8), dtype=torch.uint8, device="cuda")
+    coef = torch.zeros((n, k // g, 2), dtype=torch.int16, device="cuda")
+    goq.quantize_geo(d, torch.from_numpy(w).cuda(), codes, meta, coef)
+    torch.cuda.synchronize()
+    codes_o, _, _ = O.quantize_geo(w, g, b)
+    assert np.array_equal(codes.cpu().numpy(), codes_o)
+    b1 = O.lattice_values(b)[codes_o].reshape(n, k // g, g)
+    norm = (b1 * b1).sum(-1)
+    c1 = np.divide((w.astype(np.float64).reshape(b1.shape) * b1).sum(-1), norm, out=np.zeros_like(norm), where=norm > 0)
+    assert np.array_equal(coef.cpu().numpy().view(np.uint16)[..., 0], c1.astype(np.float16).view(np.uint16))
+
+
 # --------------------------------------------------------------------------------------------- REF solve
 @pytest.mark.parametrize("n,k,g,b,m", [(40, 512, 128, 3, 100), (17, 256, 64, 2, 33), (24, 128, 32, 4, 7)])
 def test_ref_solve_matches_oracle(goq, n, k, g, b, m):
