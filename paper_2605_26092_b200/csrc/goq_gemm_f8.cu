@@ -97,6 +97,8 @@ __device__ __forceinline__ void fma2(float& a0, float& a1, float b0, float b1, f
         : "=f"(a0), "=f"(a1) : "f"(b0), "f"(b1), "f"(c), "f"(d0), "f"(d1));
 }
 // Waits for three barriers. A wait takes a trip through the shared-memory pipe even where it holds already: the three are probed at once.
+// Every lane of the warp polls the same barriers and leaves with the same answer: what follows are warp-wide (.aligned) tcgen05 instructions and loop state in
+// uniform registers, so a barrier per lane or one lane that polls for the others has no place here.
 __device__ __forceinline__ bool wait_all(uint64_t* a, uint32_t pa, uint64_t* b, uint32_t pb, uint64_t* c, uint32_t pc, volatile int* abort_flag, int limit) {
     const bool ra = mbar_test(a, pa), rb = mbar_test(b, pb), rc = mbar_test(c, pc);
     return (ra || mbar_wait(a, pa, abort_flag, limit)) && (rb || mbar_wait(b, pb, abort_flag, limit)) && (rc || mbar_wait(c, pc, abort_flag, limit));

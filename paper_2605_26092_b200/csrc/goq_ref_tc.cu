@@ -536,7 +536,10 @@ static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& w_map
     const int cols = g.k_in / G;
     double best = 0.0;
     for (int c = 1; c <= 8 && c <= p.tiles; c *= 2) {
-        const double waves = (double)(((long long)cols * c + sms - 1) / sms);
+        // clusters that were seen to run at once (a cluster lies in one group of SMs): 12 of eight CTAs did, 16 took two waves (1024 x 512 in groups of 32 at 32
+        // observations 18 us; 512 rows, as clusters of four, 9.6)
+        const int at_once = c == 8 ? sms / 12 : c == 4 ? sms * 8 / 37 : sms / c;
+        const double waves = (double)((cols + at_once - 1) / at_once);
         const double cost = waves * (4.0 * Gram<G>::kBlocks / c * ((p.m + 3) / 4) + 8000.0 + (c > 1 ? 2500.0 : 0.0) + (double)((p.tiles + c - 1) / c) * (40.0 * G + 800.0));
         if (c == 1 || cost < best) { best = cost; p.c = c; }
     }
@@ -561,7 +564,16 @@ static cudaError_t launch_group(const Geometry& g, Params& p, const CUtensorMap&
 
 bool solve_ref_tc_supported(const Geometry& g, const float* w, const float* x_calib, int m) {
     // Half as many observations as a group has channels: the observations one by one are as cheap and need no Gram matrix.
-    return g.group >= 32 && 2 * m > g.group && ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x_calib)) & 15u) == 0;
+    if (g.group < 32 || 2 * m <= g.group || ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x_calib)) & 15u) != 0) return false;
+    // Few columns and few observations: solve_ref_kernel splits a column's rows over more CTAs than a cluster has, and G is cheap for either. Where the line
+    // lies was measured at 592 sizes (512 to 8192 wide and high, 32 to 512 observations); us, solve_ref_kernel / this:
+    const int cols = g.k_in / g.group, n = g.n_out, tiles = (n + reftc::kRows - 1) / reftc::kRows;
+    // 600 x 768 at 100 observations 11.3 / 13.0, 1281 x 768 15.0 / 15.5, 512 x 1024 at 32 9.4 / 10.6, 64 x 4096 at 100 9.6 / 10.3; 512 x 1536 at 128 and 4096 x 1024 faster here
+    if (g.group == 32) return cols > 24 && (m > 128 || (n > 128 && (cols > 32 || m > 32)));
+    // 1500 x 512 W4 at 128 19.5 / 24.9, 6000 x 512 W4 45.1 / 46.5, 1281 x 640 at 100 19.2 / 21.5; 3000 x 640 41.3 / 26.0, 1281 x 768 at 200 28.4 / 24.9
+    if (g.group == 64) return cols > 16 || m > 128 || (n > 2048 && g.wbits < 4);
+    // in groups of 128 only where a cluster's CTAs get uneven shares or a few columns have many tiles: 600 x 640 at 100 35.2 / 36.9, 1500 x 512 W4 40.6 / 46.1, 8192 x 512 92 / 93
+    return m > 128 || !((cols <= 6 && tiles > 4 && tiles < 8) || (cols <= 4 && tiles > 8));
 }
 cudaError_t launch_solve_ref_tc(const Geometry& g, const float* w, const uint8_t* codes, const uint8_t* meta, const float* x_calib, int m,
                                 double lambda, uint16_t* coef, double* c_out, int spin_limit, cudaStream_t st) {

@@ -257,14 +257,16 @@ def test_ref_solve_matches_oracle(goq, n, k, g, b, m):
     (1, 128, 128, 3, 65),      # one row, one column, the fewest observations that form a Gram matrix
     (127, 256, 128, 3, 128),   # a tile short of a row; whole chunks of observations
     (129, 384, 128, 2, 129),   # a tile and a row
-    (700, 256, 128, 4, 70),    # W4: a positive 2^emax is no int8; several CTAs a column
+    (700, 896, 128, 4, 70),    # W4: a positive 2^emax is no int8; several CTAs a column
     (1100, 128, 128, 3, 300),  # nine tiles over eight CTAs
-    (260, 320, 64, 3, 33), (130, 192, 64, 4, 200), (40, 96, 32, 2, 17), (513, 64, 32, 4, 64), (1500, 32, 32, 3, 1000),
+    (260, 1088, 64, 3, 33), (130, 192, 64, 4, 200), (40, 800, 32, 2, 129), (513, 832, 32, 4, 130), (1500, 800, 32, 3, 1000),
+    # (every size and every part of it on the side of the digits; narrower ones run in solve_ref_kernel, above)
 ])
 def test_ref_solve_digits_match_oracle(goq, n, k, g, b, m):
-    """The Gram matrix as byte digits: pairs equal to the oracle's float64 solution (numpy's observations one by one) within 1e-9, as above, also with
-    channels 1000 times the others' magnitude (every row of the matrix has a scale of its own). Rows beyond a sample are compared
-    with the same rows solved alone."""
+    """The Gram matrix as byte digits: pairs equal to the oracle's float64 solution (numpy's observations one by one), also with channels 1000 times the
+    others' magnitude (every row of the matrix has a scale of its own). Bound: the entries of the 2 x 2 system are sums of m g rounded products, and its
+    condition (at most (trace)^2 / det) carries their error to the pair: sqrt(m g) eps cond of the pair's larger coefficient (against long double the
+    oracle itself is off by up to 10 eps cond). Rows beyond a sample are compared with the same rows solved alone."""
     from tests.gpu_util import dev
     w = si.gaussian_weights(n, k, seed=n + m).astype(np.float32)
     codes, meta, _ = O.quantize_geo(w, g, b)
@@ -282,7 +284,14 @@ def test_ref_solve_digits_match_oracle(goq, n, k, g, b, m):
         return got
     got = solve(np.arange(n))
     rows = np.unique(np.concatenate([np.arange(min(n, 40)), np.arange(max(0, n - 40), n)]))
-    assert np.allclose(got[rows], O.solve_ref(w[rows], codes[rows], meta[rows], x, g, b, lam=1e-4), rtol=1e-9, atol=1e-12)
+    want = O.solve_ref(w[rows], codes[rows], meta[rows], x, g, b, lam=1e-4)
+    b1, b2 = O.decode_b1(codes[rows], b), O.decode_b2(codes[rows], meta[rows], b)
+    for j in range(k // g):
+        s = slice(j * g, (j + 1) * g)
+        a1, a2 = x[:, s].astype(np.float64) @ b1[:, s].T, x[:, s].astype(np.float64) @ b2[:, s].T
+        p, q, t = (a1 * a1).sum(0) + 1e-4, (a2 * a2).sum(0) + 1e-4, (a1 * a2).sum(0)
+        bound = np.sqrt(m * g) * 2.3e-16 * (p + q) ** 2 / (p * q - t * t) * np.abs(want[:, j]).max(-1)
+        assert (np.abs(got[rows, j] - want[:, j]).max(-1) <= bound).all()
     for lo in range(0, n, 500):
         part = np.arange(lo, min(n, lo + 500))
         assert np.array_equal(solve(part), got[part])
@@ -322,7 +331,7 @@ def test_ref_solve_non_finite_inputs_and_unaligned_buffers(goq):
 def test_ref_solve_that_gives_up_leaves_nan(goq):
     """goq_solve_ref has no scratch: a bounded wait that runs out shows as NaN coefficients, and the next call is whole again."""
     from tests.gpu_util import dev
-    n, k, g, b, m = 600, 256, 128, 3, 100
+    n, k, g, b, m = 600, 256, 128, 3, 130
     w = si.gaussian_weights(n, k, seed=5).astype(np.float32)
     codes, meta, _ = O.quantize_geo(w, g, b)
     x = si.f32_activations(m, k, seed=6).astype(np.float32)
