@@ -206,25 +206,36 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                 bool tokv[NG];
 #pragma unroll
                 for (int cg = 0; cg < NG; ++cg) tokv[cg] = cg * 4 + tok0 < it.m;
+                // what the stores need of the linear a tile belongs to: read again only where a tile is another linear's
+                int li = -1, t0 = 0, lin_n = 0, lin_tiles = 0;
+                bool y32 = false, tagw = false;
+                void* lin_y = nullptr;
+                auto take = [&](int l) {
+                    const Item& lin = p.item[l];
+                    li = l; t0 = lin.t0; lin_n = lin.n_out; lin_tiles = lin.n_tiles; lin_y = lin.y;
+                    y32 = lin.y_dtype == GOQ_F32; tagw = lin.tag_out && (lane & 4) == 0;
+                };
+                take(i);
                 for (int q = 0; q < wk.P; ++q) {
                     const unsigned sq = seq + (unsigned)q;
                     const int rs = (int)(sq % kTileSlots);
                     const int T = walk_tile_of_part(wk, q);
-                    int li = i;   // the linear this tile belongs to
-                    for (int s = 1; s < it.span && T >= p.item[i + s].t0; ++s) li = i + s;
-                    const Item& lin = p.item[li];
-                    const int Tl = T - lin.t0;
-                    const size_t tstride4 = (size_t)4 * (lin.n_tiles * 8), ystride4 = (size_t)4 * lin.n_out;
-                    const bool y32 = lin.y_dtype == GOQ_F32, tagw = lin.tag_out && (lane & 4) == 0;
+                    if (it.span > 1) {
+                        int l = i;
+                        for (int s = 1; s < it.span && T >= p.item[i + s].t0; ++s) l = i + s;
+                        if (l != li) take(l);
+                    }
+                    const int Tl = T - t0;
+                    const size_t tstride4 = (size_t)4 * (lin_tiles * 8), ystride4 = (size_t)4 * lin_n;
                     const unsigned r_lo = (unsigned)T * kb, r_hi = r_lo + kb;
                     const bool whole = r_lo >= wk.a && r_hi <= wk.b;   // every record of the tile is this CTA's
                     const bool finisher = r_hi <= wk.b;                  // this CTA holds the tile's end
                     uint2* post = p.parts + (((size_t)i * G + cta) * 2 + (T == wk.Ta ? 0 : 1)) * kPartWords + lane;
-                    uint2* tgp = p.tags + (size_t)li * kTagWords + (size_t)tok0 * (lin.n_tiles * 8) + Tl * 8 + (lane >> 3);
-                    const size_t yoff = (size_t)tok0 * lin.n_out + Tl * 16 + (lane >> 2);
+                    uint2* tgp = p.tags + (size_t)li * kTagWords + (size_t)tok0 * (lin_tiles * 8) + Tl * 8 + (lane >> 3);
+                    const size_t yoff = (size_t)tok0 * lin_n + Tl * 16 + (lane >> 2);
                     bool rowv[2];
-                    rowv[0] = Tl * 16 + (lane >> 2) < lin.n_out;
-                    rowv[1] = Tl * 16 + (lane >> 2) + 8 < lin.n_out;
+                    rowv[0] = Tl * 16 + (lane >> 2) < lin_n;
+                    rowv[1] = Tl * 16 + (lane >> 2) + 8 < lin_n;
                     const float* rall = red + (size_t)rs * kNW * (NG * 64) + lane;
                     // A tile this CTA finishes for others: their parts were posted early (every CTA starts with the tile that is
                     // open at the end of its range), so they are fetched now, before this CTA's own sums are ready - nearest CTA
@@ -334,8 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                             for (int hh = 0; hh < 2; ++hh)
                                 if (rowv[hh] && tokv[cg]) {
                                     const size_t o = yoff + cg * ystride4 + hh * 8;
-                                    if (y32) reinterpret_cast<float*>(lin.y)[o] = out[cg][hh];
-                                    else reinterpret_cast<uint16_t*>(lin.y)[o] = (uint16_t)(pair[cg][hh] & 0xFFFFu);   // the bits the copy carries
+                                    if (y32) reinterpret_cast<float*>(lin_y)[o] = out[cg][hh];
+                                    else reinterpret_cast<uint16_t*>(lin_y)[o] = (uint16_t)(pair[cg][hh] & 0xFFFFu);   // the bits the copy carries
                                 }
                     }
                 }
