@@ -53,17 +53,14 @@ struct Item {
     const uint16_t* x;
     void* y;
     unsigned long long kb_magic;             // ceil(2^32 / k_blocks): record number -> tile by multiply and shift (exact while units * k_blocks < 2^32)
-    // Neighbouring linears that read the same activations form a span: their records are numbered one after another and split over the CTAs as
-    // one range. The span's first item holds its length and totals; every item its first tile inside the span.
-    int span, t0;
-    unsigned int units;                      // (first item) tiles of the span * k_blocks
+    unsigned int units;                      // n_tiles * k_blocks
     int n_tiles, k_blocks, k_in, n_out, m, y_dtype, depends;
     int xsrc;                                // earlier item whose output this item's x lies in (read from that item's tagged copy), or -1
     unsigned int xoff;                       // first 64-bit word of x inside that copy
     int tag_out;                             // a later item reads this item's output: keep the tagged copy
     int xid;                                 // items that read the same activations have the same number: staged once for all of them
-    int x_shared;                            // another span has this number too: stage every k-block, not just this CTA's
-    unsigned int uq, ur;                     // (first item) units / G and units % G for the launch's G CTAs (the kernel never divides)
+    int x_shared;                            // another item has this number too: stage every k-block, not just this CTA's
+    unsigned int uq, ur;                     // units / G and units % G for the launch's G CTAs (the kernel never divides)
 };
 struct Params {
     Item item[kSeqMaxItems];
@@ -126,25 +123,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
         if (lane == 0) {
             int slot = 0, round = 0, issued = 0;
             bool ok = true;
-            for (int i = 0; i < p.n_items && ok; i += p.item[i].span) {
+            for (int i = 0; i < p.n_items && ok; ++i) {
                 const Item& it = p.item[i];
                 const Walk wk = make_walk(it, cta, p.g_magic);
-                // n records of the span from number rho on: one copy for each linear they lie in
-                auto copy_run = [&](unsigned char* dst, unsigned rho, unsigned n, uint64_t* bar) {
-                    int s = 0;
-                    unsigned rec0 = 0;   // number of the linear's first record
-                    while (n) {
-                        unsigned next = it.units;
-                        for (; s + 1 < it.span; ++s) {
-                            next = (unsigned)p.item[i + s + 1].t0 * (unsigned)it.k_blocks;
-                            if (rho < next) break;
-                            rec0 = next; next = it.units;
-                        }
-                        const unsigned c = min(n, next - rho);
-                        bulk_copy_g2s(dst, p.item[i + s].packed + (size_t)(rho - rec0) * p.unit_bytes, c * (unsigned)p.unit_bytes, bar);
-                        dst += (size_t)c * p.unit_bytes; rho += c; n -= c;
-                    }
-                };
                 for (unsigned j0 = 0; j0 < wk.L; j0 += kStageRecs) {
                     if (round > 0 && !wait_bar(&empty_bar[slot], (round - 1) & 1, &abort_flag, spin)) { ok = false; break; }
                     const unsigned n = min((unsigned)kStageRecs, wk.L - j0);
@@ -152,8 +133,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                     mbar_arrive_expect_tx(&full_bar[slot], n * (unsigned)p.unit_bytes);
                     // positions j0 .. j0+n-1 of the walk: one run of records, or two if the stage straddles the turn of the walk
                     const unsigned n1 = (j0 < wk.L1) ? min(n, wk.L1 - j0) : 0u;
-                    if (n1) copy_run(dst, walk_record(wk, j0), n1, &full_bar[slot]);
-                    if (n > n1) copy_run(dst + (size_t)n1 * p.unit_bytes, walk_record(wk, j0 + n1), n - n1, &full_bar[slot]);
+                    if (n1) bulk_copy_g2s(dst, it.packed + (size_t)walk_record(wk, j0) * p.unit_bytes, n1 * (unsigned)p.unit_bytes, &full_bar[slot]);
+                    if (n > n1)
+                        bulk_copy_g2s(dst + (size_t)n1 * p.unit_bytes, it.packed + (size_t)walk_record(wk, j0 + n1) * p.unit_bytes,
+                                      (n - n1) * (unsigned)p.unit_bytes, &full_bar[slot]);
                     if (++slot == p.n_stages) { slot = 0; ++round; }
                     ++issued;
                 }
@@ -182,14 +165,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
         // nobody changes the count before every CTA has finished the last linear; the tag is the count scrambled (and odd,
         // hence non-zero), so that neither zero-filled scratch nor small integers left by other kernels pass for it
         const unsigned epoch = *p.epoch, tag = ((epoch + 1u) * 0x9E3779B1u) | 1u;
-        for (int i = 0, before = 0; i < p.n_items && ok; before = i, i += p.item[i].span) {   // before: first item of the previous span
+        for (int i = 0; i < p.n_items && ok; ++i) {
             const Item& it = p.item[i];
             const Walk wk = make_walk(it, cta, p.g_magic);
             if (wk.L) {
                 if (it.depends && i > 0) {
                     if (lane == 0) {
                         int spins = 0;
-                        while (abort_flag == 0 && ld_acquire_gpu(&p.done[before]) < G)
+                        while (abort_flag == 0 && ld_acquire_gpu(&p.done[i - 1]) < G)
                             if (++spins > kGlobalSpin || spins > spin) { abort_flag = 1; break; }
                         if (abort_flag == 0) mbar_arrive(dep_bar);
                     }
@@ -203,39 +186,25 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                 const unsigned uq = it.uq, ur = it.ur;   // range boundaries step by uq (+1) from CTA to CTA
                 const unsigned rem_a = (unsigned)cta * ur - (unsigned)G * mul_shift32((unsigned)cta * ur, p.g_magic);
                 const int tok0 = lane & 3;
+                const size_t tstride4 = (size_t)4 * (it.n_tiles * 8), ystride4 = (size_t)4 * it.n_out;
+                const bool y32 = it.y_dtype == GOQ_F32;
                 bool tokv[NG];
 #pragma unroll
                 for (int cg = 0; cg < NG; ++cg) tokv[cg] = cg * 4 + tok0 < it.m;
-                // what the stores need of the linear a tile belongs to: read again only where a tile is another linear's
-                int li = -1, t0 = 0, lin_n = 0, lin_tiles = 0;
-                bool y32 = false, tagw = false;
-                void* lin_y = nullptr;
-                auto take = [&](int l) {
-                    const Item& lin = p.item[l];
-                    li = l; t0 = lin.t0; lin_n = lin.n_out; lin_tiles = lin.n_tiles; lin_y = lin.y;
-                    y32 = lin.y_dtype == GOQ_F32; tagw = lin.tag_out && (lane & 4) == 0;
-                };
-                take(i);
+                const bool tagw = it.tag_out && (lane & 4) == 0;
                 for (int q = 0; q < wk.P; ++q) {
                     const unsigned sq = seq + (unsigned)q;
                     const int rs = (int)(sq % kTileSlots);
                     const int T = walk_tile_of_part(wk, q);
-                    if (it.span > 1) {
-                        int l = i;
-                        for (int s = 1; s < it.span && T >= p.item[i + s].t0; ++s) l = i + s;
-                        if (l != li) take(l);
-                    }
-                    const int Tl = T - t0;
-                    const size_t tstride4 = (size_t)4 * (lin_tiles * 8), ystride4 = (size_t)4 * lin_n;
                     const unsigned r_lo = (unsigned)T * kb, r_hi = r_lo + kb;
                     const bool whole = r_lo >= wk.a && r_hi <= wk.b;   // every record of the tile is this CTA's
                     const bool finisher = r_hi <= wk.b;                  // this CTA holds the tile's end
                     uint2* post = p.parts + (((size_t)i * G + cta) * 2 + (T == wk.Ta ? 0 : 1)) * kPartWords + lane;
-                    uint2* tgp = p.tags + (size_t)li * kTagWords + (size_t)tok0 * (lin_tiles * 8) + Tl * 8 + (lane >> 3);
-                    const size_t yoff = (size_t)tok0 * lin_n + Tl * 16 + (lane >> 2);
+                    uint2* tgp = p.tags + (size_t)i * kTagWords + (size_t)tok0 * (it.n_tiles * 8) + T * 8 + (lane >> 3);
+                    const size_t yoff = (size_t)tok0 * it.n_out + T * 16 + (lane >> 2);
                     bool rowv[2];
-                    rowv[0] = Tl * 16 + (lane >> 2) < lin_n;
-                    rowv[1] = Tl * 16 + (lane >> 2) + 8 < lin_n;
+                    rowv[0] = T * 16 + (lane >> 2) < it.n_out;
+                    rowv[1] = T * 16 + (lane >> 2) + 8 < it.n_out;
                     const float* rall = red + (size_t)rs * kNW * (NG * 64) + lane;
                     // A tile this CTA finishes for others: their parts were posted early (every CTA starts with the tile that is
                     // open at the end of its range), so they are fetched now, before this CTA's own sums are ready - nearest CTA
@@ -345,8 +314,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
                             for (int hh = 0; hh < 2; ++hh)
                                 if (rowv[hh] && tokv[cg]) {
                                     const size_t o = yoff + cg * ystride4 + hh * 8;
-                                    if (y32) reinterpret_cast<float*>(lin_y)[o] = out[cg][hh];
-                                    else reinterpret_cast<uint16_t*>(lin_y)[o] = (uint16_t)(pair[cg][hh] & 0xFFFFu);   // the bits the copy carries
+                                    if (y32) reinterpret_cast<float*>(it.y)[o] = out[cg][hh];
+                                    else reinterpret_cast<uint16_t*>(it.y)[o] = (uint16_t)(pair[cg][hh] & 0xFFFFu);   // the bits the copy carries
                                 }
                     }
                 }
@@ -357,9 +326,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
             // next linear waits for the counter (a release costs the warp the round trip of all its stores).
             __syncwarp();
             if (lane == 0) {
-                const int next = i + it.span;
-                if (next < p.n_items) {
-                    if (p.item[next].depends) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&p.done[i]) : "memory");
+                if (i < p.n_items - 1) {
+                    if (p.item[i + 1].depends) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(&p.done[i]) : "memory");
                 } else {   // the CTA that completes the last linear last leaves the counters zero for the next call
                     const int prev = atomic_add_acq_rel_gpu(&p.done[i], 1);
                     if (prev == G - 1) {
@@ -387,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
     bool alive = true;
     int staged = -1;                  // number of the activations in the buffer in use
 
-    for (int i = 0; i < p.n_items && alive; i += p.item[i].span) {
+    for (int i = 0; i < p.n_items && alive; ++i) {
         const Item& it = p.item[i];
         const Walk wk = make_walk(it, cta, p.g_magic);
         if (wk.L == 0) continue;   // nothing of this linear belongs to this CTA (the control warp reports it finished)
@@ -790,7 +758,6 @@ cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, i
         it.y = calls[i].y;
         it.kb_magic = ((1ull << 32) + (unsigned)g.k_blocks - 1) / (unsigned)g.k_blocks;
         it.units = (unsigned)g.n_units;
-        it.span = 1; it.t0 = 0;
         it.n_tiles = g.n_tiles;
         it.k_blocks = g.k_blocks;
         it.k_in = g.k_in;
@@ -799,6 +766,8 @@ cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, i
         it.y_dtype = calls[i].y_dtype;
         it.depends = calls[i].depends;
         it.xsrc = -1; it.xoff = 0; it.tag_out = 0;
+        it.uq = it.units / (unsigned)G;
+        it.ur = it.units % (unsigned)G;
         if (calls[i].m > m_max) m_max = calls[i].m;
         k1 = k1 && g.k1;
         const size_t b = chain_xbuf_bytes(calls[i].m, g.k_pad);
@@ -820,25 +789,15 @@ cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, i
             }
         }
     }
-    // Neighbouring items that read the same activations (same address, shape and source, no barrier between) share their staging and, as far as
-    // the record arithmetic reaches, form a span: one range of records for each CTA, with one tail stage and one set of shared tiles where
-    // every linear had its own (LLaMA-2-7B layers with q, k, v and gate, up apart: 32 layers, 1 token, 1554 -> 1449 us; 4 layers, 4 tokens, 239 -> 225).
-    for (int j = 0, head = 0; j < n; ++j) {
-        chain::Item &a = p.item[j], &b = p.item[j > 0 ? j - 1 : 0], &h = p.item[head];
+    // Neighbouring items that read the same activations share their staging: same address, shape and source, no barrier between.
+    for (int j = 0; j < n; ++j) {
+        chain::Item &a = p.item[j], &b = p.item[j > 0 ? j - 1 : 0];
         a.xid = j; a.x_shared = 0;
-        const bool same = j > 0 && !a.depends && a.x == b.x && a.k_in == b.k_in && a.m == b.m && a.xsrc == b.xsrc && a.xoff == b.xoff;
-        if (same) a.xid = b.xid;
-        const unsigned tiles = j > 0 ? (unsigned)(b.t0 + b.n_tiles) : 0u;   // of the span so far
-        if (same && ((unsigned long long)h.units + a.units) * (unsigned)a.k_blocks < (1ull << 32) && tiles + (unsigned)a.n_tiles <= (1u << 21)) {
-            a.t0 = (int)tiles;
-            h.units += a.units;
-            ++h.span;
-        } else {
-            if (same) a.x_shared = h.x_shared = 1;
-            head = j;
+        if (j > 0 && !a.depends && a.x == b.x && a.k_in == b.k_in && a.m == b.m && a.xsrc == b.xsrc && a.xoff == b.xoff) {
+            a.xid = b.xid;
+            a.x_shared = b.x_shared = 1;
         }
     }
-    for (int j = 0; j < n; j += p.item[j].span) { p.item[j].uq = p.item[j].units / (unsigned)G; p.item[j].ur = p.item[j].units % (unsigned)G; }
     const int cpg = group / 32;
 #define GOQ_CHAIN(WB_, NG_, K1_)                                                                             \
     (cpg == 1 ? launch_chain_cfg<WB_, 1, NG_, K1_>(p, x_need, st) : cpg == 2 ? launch_chain_cfg<WB_, 2, NG_, K1_>(p, x_need, st) \

@@ -250,13 +250,13 @@ def test_small_batches_integer_operand_form(goq, g, b, form):
 
 @pytest.mark.parametrize("g,b,batch,widths", [
     (128, 3, 1, (16, 1, 40)),            # fewer records than SMs, one-tile and one-row linears
-    (128, 3, 4, (1030, 129, 256, 64)),   # ragged widths, a range over three linears
+    (128, 3, 4, (1030, 129, 256, 64)),   # ragged widths
     (64, 2, 6, (2432, 2432)),            # two column groups, several stages a range
     (32, 3, 3, (700,) * 9),
 ])
-def test_linears_that_read_the_same_activations_form_one_range(goq, form, g, b, batch, widths):
+def test_linears_that_read_the_same_activations_stand_side_by_side(goq, form, g, b, batch, widths):
     """Linears side by side on one input (q, k, v; gate, up), outputs of either type, then linears that read the middle one's bf16 output: ordered
-    by data flow (two of them: a span that waits) and, the last, by a flag. Every item against the oracle on the bits that it read."""
+    by data flow and, the last, by a flag. Every item against the oracle on the bits that it read."""
     from tests.gpu_util import dev, check_bf16_output
     k, mid = 384, len(widths) // 2
     n_mid = widths[mid] // 128 * 128 if widths[mid] >= 128 else 0
@@ -286,6 +286,29 @@ def test_linears_that_read_the_same_activations_form_one_range(goq, form, g, b, 
                 assert O.normwise_rel_err(got, y_ref) <= TIGHT, i
             else:
                 check_bf16_output(got, y_ref, 1e-4, "item %d" % i)
+
+
+@pytest.mark.parametrize("n,kv,k,inner,batch,g,b", [(256, 256, 256, 640, 1, 128, 3), (2048, 512, 2048, 5504, 4, 64, 3), (1024, 1024, 1024, 2736, 2, 32, 2),
+                                                     (384, 130, 384, 1000, 6, 32, 3)])
+def test_a_linear_gives_the_same_bits_whatever_stands_beside_it(goq, form, n, kv, k, inner, batch, g, b):
+    """q, k and v on one input, gate and up on another's output: which SM adds which records of a linear, hence the order of its fp32 sums, is the linear's
+    own affair. Every output of the chain equals, bit for bit, the same linear in a call of its own on the bits that it read."""
+    from tests.gpu_util import dev
+    xd = dev(si.bf16_activations(batch, k, seed=9))
+    shapes = [(n, k), (kv, k), (kv, k), (inner, n), (inner, n), (100, n)]
+    layers = [_layer(goq, a, c, g, b, seed=60 + i) for i, (a, c) in enumerate(shapes)]
+    out = [torch.zeros((batch, L["n"]), dtype=torch.bfloat16 if i == 0 or i == 3 else torch.float32, device="cuda") for i, L in enumerate(layers)]
+    reads = [xd, xd, xd] + [out[0]] * 3
+    items = [(L["d"], L["packed"], x, batch, y, goq.F32 if y.dtype == torch.float32 else goq.BF16, False) for L, x, y in zip(layers, reads, out)]
+    ws = _ws(goq, len(items))
+    goq.gemv_sequence(goq.make_sequence(items), ws)
+    torch.cuda.synchronize()
+    assert goq.workspace_status(ws) == goq.OK
+    for i, (L, x, y) in enumerate(zip(layers, reads, out)):
+        alone = torch.zeros_like(y)
+        goq.gemv_sequence(goq.make_sequence([(L["d"], L["packed"], x, batch, alone, goq.F32 if y.dtype == torch.float32 else goq.BF16, False)]), ws)
+        torch.cuda.synchronize()
+        assert torch.equal(y, alone), i
 
 
 @pytest.mark.parametrize("shapes", [
