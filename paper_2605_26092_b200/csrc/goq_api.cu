@@ -38,11 +38,13 @@ goq_status check_arch() {
 float decode_us(const Geometry& g, int m) {
     return 4.f + (float)g.n_units * ((m > 8 ? 7.0e-4f : 5.5e-4f) + (g.wbits == 4 ? 1.0e-4f : 0.f));
 }
-// The mid-batch kernel up to 256 tokens: 34.6 for 8192 x 8192, 21 4096 x 4096, 18.5 2048 x 2048, 23 1024 x 8192 at 64 tokens, 39.5 and 23 for the first two at 128.
+// The mid-batch kernel up to 256 tokens: 34.6 for 8192 x 8192, 21 4096 x 4096, 18.5 2048 x 2048, 23 1024 x 8192 at 64 tokens, 39.5 and 23 for the first two at 128;
+// with at most one unit for every SM 10.2 for 1024 x 512, 13.2 1024 x 2048, 15.9 512 x 4096 at 40.
 float mid_us(const Geometry& g, int m, bool exact) {
     const int tiles = (g.n_tiles + 7) / 8, units = tiles * g.k_blocks, sms = goq::gemm_mid_ctas(), grid = units < sms ? units : sms;
     const float unit = (exact ? 0.8f : 0.55f + 0.0032f * (float)m) + (g.wbits == 4 ? 0.08f : 0.f) + (g.group < 128 ? 0.03f : 0.f);
-    return 13.f + 0.4f * (float)grid / (float)tiles + unit * (float)((units + grid - 1) / grid);
+    const float parts = (float)grid / (float)tiles;
+    return units <= sms ? 9.5f + 0.17f * parts + unit : 13.f + 0.4f * parts + unit * (float)((units + grid - 1) / grid);
 }
 // goq_gemv on the kernel in e4m3 operands: above 4 tokens (or W4, which has no integer form), large linears only; W2 and W3 where a call needs scratch anyway
 bool gemv_takes_f8(const Geometry& g, int m) {
@@ -172,8 +174,8 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
         if (variant == 3) return from_cuda(goq::launch_gemv_stream(g, packed, x_bf16, batch, y, y_dtype, ws, (cudaStream_t)stream));
     }
     // Large linears above 4 tokens (W4: any number): both bases as e4m3 operands of the tensor cores, half the decode's instructions, for a pre-pass and a
-    // summing kernel around it. us, fragment kernel / this: W3 28672 x 8192 66 / 54 at 8 tokens, 83 / 55 at 16; 8192 x 8192 22.0 / 22.8 and 27.4 / 23.2;
-    // W4 26.7 / 23.9 at 8 tokens; 4096 x 4096 at 16 tokens 8.2 / 13.4.
+    // summing kernel around it. us, fragment kernel / this: W3 28672 x 8192 66 / 55 at 8 tokens, 83 / 60 at 16; 8192 x 8192 22.0 / 23.0 and 27.4 / 25.0;
+    // W4 25.6 / 24.3 at 8 tokens; 4096 x 4096 at 16 tokens 8.1 / 14.2.
     if (variant == 0 && gemv_takes_f8(g, batch) && ws && aligned(ws, 256) && ws_bytes >= goq::gemm_f8_workspace(g, batch))
         return from_cuda(goq::launch_gemm_f8(g, packed, x_bf16, batch, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
     if (variant == 0 && goq::gemv_mma_supported(g, batch))
@@ -198,7 +200,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         if (goq_status s = check_arch()) return s;
         const int variant = g_gemv_variant.load(std::memory_order_relaxed);
         // Four kernels: the decode GEMV (16 tokens a launch), the kernel in e4m3 operands (a few tokens to about 128, fp32 accuracy, no rounding of
-        // weights), the mid-batch kernel (an even split of the packed records over the SMs; up to
+        // weights or activations), the mid-batch kernel (an even split of the packed records over the SMs; up to
         // 32 tokens with both bases as exact operands, above with w_hat rounded once to fp16) and the prefill kernel (128 x 512 tiles).
         //   Up to 32 tokens: groups of 8 and 16 have only the mid-batch kernel that keeps fp32 accuracy. Others take two decode launches
         //   unless the linear is large or wide (units = 16-row tiles x k-blocks). Measured at 17 tokens, W3 g128, us, mid-batch over decode:
@@ -220,9 +222,9 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
             } else {
                 mid_wanted = !goq::gemm_tc_supported(g) || goq::gemm_mid_us(g, m) <= 0.95f * goq::gemm_tc_us(g, m);
             }
-            //   Up to 256 tokens, groups of 32 and more: e4m3 operands where the estimates say so. us, the others / e4m3: at 32 tokens 4096 x 4096 17.4 / 14.6,
-            //   28672 x 8192 98 / 61, 2048 x 2048 10.9 / 12.3, 1024 x 8192 13.6 / 15.2; at 64 2048 x 2048 18.5 / 13.6, 28672 x 8192 90 / 78, in groups of
-            //   64 8192 x 8192 36 / 42, 4096 x 4096 21.6 / 19.6; at 128 (two token tiles) 2048 x 2048 20 / 14.8, 8192 x 8192 39.7 / 50.6.
+            //   Up to 256 tokens, groups of 32 and more: e4m3 operands where the estimates say so. us, the others / e4m3: at 32 tokens 4096 x 4096 17.4 / 16.1,
+            //   28672 x 8192 98 / 77, 2048 x 2048 9.9 / 11.4, 1024 x 8192 13.6 / 15.5, in groups of 64 8192 x 8192 38 / 41; at 64 (two token tiles) 2048 x 4096
+            //   18.4 / 16.0, 2048 x 8192 22.5 / 21.6; at 128 1024 x 3072 20.5 / 15.0, 2048 x 4096 19.9 / 21.1, 7200 x 512 16.2 / 16.4.
             if (m <= 16) f8_wanted = !narrow && gemv_takes_f8(g, m);
             else if (m <= kGemmMidMaxTokens && goq::gemm_f8_supported(g, m)) {
                 const int second = m - 16;   // (up to 32 tokens: of the second decode launch)

@@ -4,22 +4,27 @@
 //
 // The inner sums have PoT operands only, and a PoT state is an e4m3 number: one byte a weight, found by the byte permutes of the decode alone
 // (b1: a table lookup per four weights; b2: the same bytes routed by the exchange record, sign bits flipped), with no coefficient in the inner
-// loop. The activations are two e4m3 slices, hi + 2^-5 lo: each keeps four significant bits, so a bf16 number is exact down to 2^-15 of its
-// token's largest magnitude (every token is scaled by a power of two) and off by at most 2^-23 of it below. Products are exact, sums fp32; the
-// coefficients multiply the group sums in fp32 as they are read back. The fp16 form (w_hat = c1 b1 + c2 b2 rounded once, goq_gemm_mid.cu)
-// has 19 operations on the integer pipe and 8 on the other per 8 weights; this has 13, and no rounding of the weights.
+// loop. The activations are two e4m3 slices, hi + 2^-5 lo, of four significant bits each, which hold a bf16 number exactly if it is at least 2^-14 of its
+// token's largest magnitude (every token is scaled by a power of two). What is smaller goes, times 2^15, into two slices of its own, as if it were another
+// token; a macro-block's two sums are added as they are read back, and the coefficients multiply them in fp32. Exact down to 2^-29 of the largest. A token
+// with anything below that, or with an infinity or a NaN, is marked by the pre-pass, and its outputs are computed from the bf16 elements themselves by the
+// summing kernel. So products are exact whatever the activations, and sums are fp32. (With one pair of slices an element 2^13 times the others left errors of
+// 8e-4 in the channels whose code is zero there.) The fp16 form (w_hat = c1 b1 + c2 b2 rounded once, goq_gemm_mid.cu) has 19 operations on the integer pipe
+// and 8 on the other per 8 weights; this has 13, and no rounding of the weights.
 //
-// Work split: units of 128 channels x one 128-wide k-block spread evenly over the SMs, as in goq_streamk.cuh; a token tile is 16 to 64 tokens.
+// Work split: units of 128 channels x one 128-wide k-block spread evenly over the SMs, as in goq_streamk.cuh; a token tile is 16 to 64 rows of activations, two
+// rows a token ("tokens" of a tile or column below are these rows).
 // Roles: four warps (eight above 32 tokens) read the group sums back (a thread is a channel) and hold y in registers until the part ends, sixteen
 // decode (two groups of eight alternate k-blocks; warp = one 16-row record), one each packed records (TMA), activations (TMA) and MMA issue. The decoded
 // operand goes straight to tensor memory (tcgen05.st 16x256b: its element map is the packed words' ownership), so that shared memory serves
 // only the packed records, the record table and the activations. Tensor memory: four operand stages of 64 columns, and a ring of group sums
 // (2 x tokens columns a basis) in the other half.
-// Bound: the chain of waits between decode, MMA and read-back; no pipe is above 40 % (integer 40 %, issue 51 % at 16 tokens; tensor 33 % at 64).
-// Measured, W3 g128, us, goq_gemm before (mid-batch kernel or decode launches) -> this: 28672 x 8192 at 17 / 32 / 64 tokens 97 / 98 / 90 -> 60 / 61 / 78; 8192 x 8192
-// 37 / 37 / 34.6 -> 25 / 25 / 31; 4096 x 4096 16 / 17 / 21 -> 14.5 / 14.6 / 17; W4 28672 x 8192 at 32 tokens 98 -> 65. As goq_gemv (gemv_mma_kernel before): 28672 x 8192
-// at 16 tokens 83 -> 55, W4 at 4 to 8 tokens 81 -> 59. A unit takes 0.46 us at 16 tokens, 0.70 at 64. Normwise error 5e-8 to 1.1e-7 (w_hat rounded to fp16: 2.1e-4).
-// Not kept: three decoding groups (28672 x 8192 at 16 tokens 55.2 -> 56.5), records copied one by one (71.5) or four k-blocks at a time (55.6).
+// Bound: the chain of waits between decode, MMA and read-back; no pipe is above 40 % (profiles/gemm_f8_8192x8192_m8.md).
+// Measured, W3 g128, us, goq_gemm otherwise (mid-batch kernel or decode launches) -> this: 28672 x 8192 at 24 / 32 tokens 97 / 98 -> 71 / 77; 8192 x 8192 36 / 37 -> 28 / 30.5;
+// 4096 x 4096 16 / 17 -> 15.3 / 16.1; 2048 x 4096 at 64 18.4 -> 16.0; W4 28672 x 8192 at 32 tokens 98 -> 83. As goq_gemv (gemv_mma_kernel otherwise): 28672 x 8192 at 8 / 16
+// tokens 66 / 83 -> 55 / 60, W4 at 1 to 8 tokens 81 -> 59. A unit takes 0.46 us with 16 rows, 0.54 with 32, 0.70 with 64. Normwise error 5.1e-8 to 1.0e-7, no larger than the
+// fragment kernel's at any of 60 sizes (w_hat rounded to fp16: 2.1e-4).
+// Not kept: three decoding groups (28672 x 8192 at 16 rows 55.2 -> 56.5), records copied one by one (71.5) or four k-blocks at a time (55.6).
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, runs out its control flow, waits for what it has in flight,
 // frees its tensor memory and records GOQ_ERR_TIMEOUT in the status word.
 #include "goq_streamk.cuh"
@@ -37,7 +42,10 @@ template <int NB8> struct Roles {
     static constexpr int kDrain = kPair ? 4 : 8, kDec0 = kDrain, kPk = kDec0 + 16, kX = kPk + 1, kMma = kPk + 2, kThreads = (kPk + 3) * 32;
 };
 constexpr int kStages = 4, kMaxX = 8, kMaxPk = 8, kMaxSums = 8, kCoefSlots = 8;
-constexpr int kMaxTokens = 64;             // of a tile
+constexpr int kMaxTokens = 64;             // rows of a tile: two a token, its larger and its smaller elements
+constexpr float kSmall = 1.f / 32768.f;    // what undoes the smaller elements' factor
+// Rows of activations: four tokens' larger elements, the same tokens' smaller ones, the next four's larger ones, ...
+__host__ __device__ constexpr int rows_of(int m) { return (m + 3) / 4 * 8; }
 
 struct Params {
     const uint8_t* packed;
@@ -45,8 +53,9 @@ struct Params {
     const float* inv_scale;   // [m] 2^-s of each token
     int* status;
     float* partial;           // [CTA][2][tokens][128]
-    int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m, y_dtype;
+    int unit_bytes, meta_off, k_blocks, n_tiles, n_out, m, rows, y_dtype;   // rows: of activations
     int tiles_x, units, n_x, n_pk;   // channel tiles; units; ring depths: activation tiles, packed units
+    int run;    // units added up in one chain: about sqrt(k-blocks / macro-blocks of one), where its roundings and those of the sum over the runs are as large
     int spin;
 };
 
@@ -197,7 +206,7 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
                 const int tok0 = (tile / p.tiles_x) * kTok;
                 mbar_expect_tx(&x_full[s], kXBytes);   // (rows past the end arrive as zeros; tokens past the last read the other slice: columns of their own)
                 tma_load_2d(x_tiles + s * kXBytes, &x_map, kb * kBlockK, tok0, &x_full[s]);
-                tma_load_2d(x_tiles + s * kXBytes + kTok * 128, &x_map, kb * kBlockK, p.m + tok0, &x_full[s]);
+                tma_load_2d(x_tiles + s * kXBytes + kTok * 128, &x_map, kb * kBlockK, p.rows + tok0, &x_full[s]);
                 if (++s == p.n_x) { s = 0; ++round; }
                 if (++kb == p.k_blocks) { kb = 0; ++tile; }
             }
@@ -291,21 +300,23 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
         }
     } else {
         // ------------------------------ group sums -> y ------------------------------
-        // Warp (h, quarter): channels 32 quarter + lane, tokens kMine h .. of the tile
+        // Warp (h, quarter): channels 32 quarter + lane, rows kMine h .. of the tile: kMine / 2 tokens
         constexpr int kMine = kTok * 4 / kDrainWarps;
         const int quarter = warp & 3, h = warp >> 2, row = quarter * 32 + lane;
         const uint32_t taddr = tmem_sums + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * kMine), coef_a = s32(coef) + (uint32_t)row * 4;
         const Output out = {p.y, p.y_dtype, p.n_out};
-        constexpr size_t kPark = (size_t)kTok * kTileN;
+        constexpr size_t kPark = (size_t)(kTok / 2) * kTileN;
         asm volatile("griddepcontrol.wait;" ::: "memory");   // outputs, parked parts and the token scales: only after earlier kernels
         bool ok = true;
         int d = 0, cs = 0, q = 0;
         uint32_t d_par = 0;
         for (int u = u0; u < u1 && ok; ++q) {
             const Part part = part_at(u, u1, p.k_blocks);
-            float acc[kMine];
+            // sums of a run of units, and of the runs before: one chain of fp32 additions over a part doubled the error (28672 x 8192: 1.8e-7, in runs 8.5e-8)
+            float acc[kMine / 2], tot[kMine / 2];
 #pragma unroll
-            for (int i = 0; i < kMine; ++i) acc[i] = 0.f;
+            for (int i = 0; i < kMine / 2; ++i) acc[i] = tot[i] = 0.f;
+            int run = 0;
             for (int k = 0; k < part.n && ok; ++k) {
 #pragma unroll
                 for (int j = 0; j < kSteps; ++j) {
@@ -316,7 +327,7 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
                     const float2 c = __half22float2(*reinterpret_cast<const __half2*>(&pair));
                     const uint32_t at = taddr + (uint32_t)(d * kStepCols);
                     __syncwarp();   // stores and arrivals may have diverged: the warp reads tensor memory as one
-                    // 32 columns at a time: eight tokens of both bases, or sixteen of one (24 tokens: eight). Nothing but the wait follows a load
+                    // 32 columns at a time: eight rows of both bases, or sixteen of one (24 rows: eight). Nothing but the wait follows a load
                     // that is on its way: its registers are not the compiler's to move or use until then.
                     constexpr int kPer = kBases == 2 || kMine % 16 != 0 ? 8 : 16, kLoads = kBases * kPer / 8;
 #pragma unroll
@@ -329,16 +340,26 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
                         }
                         if constexpr (kLoads == 2) tmem_ld_wait(v[0], v[1], v[2], v[3]);
                         else tmem_ld_wait(v[0], v[1]);
+                        float both[4] = {0.f, 0.f, 0.f, 0.f};   // (both bases at once: c1 S1 + c2 S2 is one addition)
 #pragma unroll
                         for (int i = 0; i < kLoads; ++i) {
                             const float cc = kBases == 2 ? (i ? c.y : c.x) : ((j & 1) ? c.y : c.x);
-                            float* to = acc + b + (kBases == 2 ? 0 : i * 8);
+                            float* to = acc + (b + (kBases == 2 ? 0 : i * 8)) / 2;
+                            float f[8];   // hi + 2^-5 lo of four tokens' larger elements, and of their smaller ones
 #pragma unroll
-                            for (int e = 0; e < 8; e += 2) {
-                                float s0, s1;
-                                fma2(s0, s1, __uint_as_float(v[2 * i + 1][e]), __uint_as_float(v[2 * i + 1][e + 1]), 0.03125f, __uint_as_float(v[2 * i][e]),
+                            for (int e = 0; e < 8; e += 2)
+                                fma2(f[e], f[e + 1], __uint_as_float(v[2 * i + 1][e]), __uint_as_float(v[2 * i + 1][e + 1]), 0.03125f, __uint_as_float(v[2 * i][e]),
                                      __uint_as_float(v[2 * i][e + 1]));
-                                fma2(to[e], to[e + 1], s0, s1, cc, to[e], to[e + 1]);
+#pragma unroll
+                            for (int e = 0; e < 4; e += 2) {
+                                float s0, s1;
+                                fma2(s0, s1, f[4 + e], f[5 + e], kSmall, f[e], f[e + 1]);
+                                if constexpr (kBases == 2) {
+                                    fma2(both[e], both[e + 1], s0, s1, cc, both[e], both[e + 1]);
+                                    if (i == 1) { to[e] += both[e]; to[e + 1] += both[e + 1]; }
+                                } else {
+                                    fma2(to[e], to[e + 1], s0, s1, cc, to[e], to[e + 1]);
+                                }
                             }
                         }
                     }
@@ -348,25 +369,30 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
                     if (++d == kSums) { d = 0; d_par ^= 1u; }
                 }
                 cs = (cs + 1) & (kCoefSlots - 1);
+                if (++run == p.run || k + 1 == part.n) {
+                    run = 0;
+#pragma unroll
+                    for (int i = 0; i < kMine / 2; ++i) { tot[i] += acc[i]; acc[i] = 0.f; }
+                }
             }
             if (!ok) break;
-            const int t0 = (part.tile / p.tiles_x) * kTok, first = h * kMine, cols = min(kTok, p.m - t0);
+            const int t0 = (part.tile / p.tiles_x) * (kTok / 2), first = h * (kMine / 2), cols = min(kTok / 2, p.m - t0);
             const int ch = (part.tile % p.tiles_x) * kTileN + row;
             if (part.n < p.k_blocks) {
                 float* park = p.partial + ((size_t)cta * 2 + (q == 0 ? 0 : 1)) * kPark + row;
 #pragma unroll
-                for (int i = 0; i < kMine; ++i)
-                    if (first + i < cols) __stcg(park + (size_t)(first + i) * kTileN, acc[i]);
+                for (int i = 0; i < kMine / 2; ++i)
+                    if (first + i < cols) __stcg(park + (size_t)(first + i) * kTileN, tot[i]);
             } else {
 #pragma unroll
-                for (int b = 0; b < kMine / 8; ++b) {   // (eight factors at once; the array ends 16 behind the last token)
-                    const int c0 = first + b * 8;
+                for (int b = 0; b < kMine / 8; ++b) {   // (four factors at once; the array ends 16 behind the last token)
+                    const int c0 = first + b * 4;
                     if (c0 >= cols) break;
-                    const float4 s0 = __ldcg(reinterpret_cast<const float4*>(p.inv_scale + t0 + c0)), s1 = __ldcg(reinterpret_cast<const float4*>(p.inv_scale + t0 + c0) + 1);
-                    const float sc[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+                    const float4 s0 = __ldcg(reinterpret_cast<const float4*>(p.inv_scale + t0 + c0));
+                    const float sc[4] = {s0.x, s0.y, s0.z, s0.w};
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (c0 + i < cols && ch < p.n_out) out.store1(t0 + c0 + i, ch, acc[b * 8 + i] * sc[i]);
+                    for (int i = 0; i < 4; ++i)
+                        if (c0 + i < cols && ch < p.n_out) out.store1(t0 + c0 + i, ch, tot[b * 4 + i] * sc[i]);
                 }
             }
             u += part.n;
@@ -383,9 +409,9 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
     }
 }
 
-// ---- activation pre-pass: bf16 -> two e4m3 slices, one CTA per token ------------------------------------
-// x 2^s with the token's largest magnitude in [2^7, 2^8): hi = e4m3(x 2^s), lo = e4m3((x 2^s - hi) 2^5); zeros past k_in. A token with an
-// infinite or NaN element gets NaN slices there (e4m3 has no infinity), which make its outputs (and no other token's) NaN.
+// ---- activation pre-pass: bf16 -> e4m3 slices, one CTA per token ------------------------------------
+// v = x 2^s with the token's largest magnitude in [2^7, 2^8). Its first row holds the elements of 2^-7 and more (hi = e4m3(v), lo = e4m3((v - hi) 2^5): exact),
+// its second one, four rows on, the others, times 2^15; zeros past k_in. A token with an element that these do not give back, an infinity and a NaN among them, is marked.
 constexpr int kPrepThreads = 256;
 constexpr int kPrepHold = 6;   // 16-byte vectors a thread keeps: rows up to 12288
 __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {   // a in the low byte
@@ -399,13 +425,14 @@ __device__ __forceinline__ float2 from_e4m3x2(uint32_t v) {
     return __half22float2(*reinterpret_cast<__half2*>(&h));
 }
 __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* __restrict__ x, int k_in, int k_pad, uint8_t* __restrict__ x8,
-                                                               float* __restrict__ inv_scale, int m) {
+                                                               float* __restrict__ inv_scale, int* __restrict__ inexact, int m) {
     // its own dependents only when everything before it is complete: they read the packed weights at once, in stream order
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tok = blockIdx.x, tid = threadIdx.x;
     const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)tok * k_in);
-    uint8_t *hi_out = x8 + (size_t)tok * k_pad, *lo_out = x8 + ((size_t)m + tok) * k_pad;
+    const int first_row = (tok >> 2) * 8 + (tok & 3);
+    uint8_t *hi_out = x8 + (size_t)first_row * k_pad, *lo_out = x8 + (size_t)(rows_of(m) + first_row) * k_pad;
     const int n_vec = k_in / 8, n_pad = k_pad / 8;
     __shared__ uint32_t warp_max[kPrepThreads / 32];
     uint32_t amax = 0;
@@ -432,27 +459,119 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
     int sfield = 261 - (int)(amax >> 7);   // exponent field of 2^s
     sfield = sfield < 1 ? 1 : (sfield > 253 ? 253 : sfield);
     const float mult = __uint_as_float((uint32_t)sfield << 23);
+    bool lost = false;
     auto convert = [&](int i, const uint4& v) {
         const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
-        uint32_t hi[2] = {0u, 0u}, lo[2] = {0u, 0u};
+        uint32_t hi[2][2] = {{0u, 0u}, {0u, 0u}}, lo[2][2] = {{0u, 0u}, {0u, 0u}};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float a = __uint_as_float(in32[j] << 16) * mult, b = __uint_as_float(in32[j] & 0xFFFF0000u) * mult;
-            uint32_t h = e4m3x2(a, b);
-            if ((in32[j] & 0x7F80u) == 0x7F80u) h |= 0x7Fu;             // inf and NaN: NaN (the conversion would saturate)
-            if ((in32[j] & 0x7F800000u) == 0x7F800000u) h |= 0x7F00u;
-            const float2 back = from_e4m3x2(h);
-            hi[j >> 1] |= h << (16 * (j & 1));
-            lo[j >> 1] |= e4m3x2((a - back.x) * 32.f, (b - back.y) * 32.f) << (16 * (j & 1));   // the differences are exact
+            const bool big_a = !(fabsf(a) < 0.0078125f), big_b = !(fabsf(b) < 0.0078125f);
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                const float pa = big_a == (part == 0) ? (part ? a * 32768.f : a) : 0.f, pb = big_b == (part == 0) ? (part ? b * 32768.f : b) : 0.f;
+                const uint32_t h = e4m3x2(pa, pb);
+                const float2 back = from_e4m3x2(h);
+                const float ra = pa - back.x, rb = pb - back.y;   // exact
+                const uint32_t l = e4m3x2(ra * 32.f, rb * 32.f);
+                const float2 rest = from_e4m3x2(l);
+                lost = lost || !(rest.x == ra * 32.f) || !(rest.y == rb * 32.f);   // (the conversions saturate; inf - inf and NaN equal nothing)
+                hi[part][j >> 1] |= h << (16 * (j & 1));
+                lo[part][j >> 1] |= l << (16 * (j & 1));
+            }
         }
-        *reinterpret_cast<uint2*>(hi_out + (size_t)i * 8) = make_uint2(hi[0], hi[1]);
-        *reinterpret_cast<uint2*>(lo_out + (size_t)i * 8) = make_uint2(lo[0], lo[1]);
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            *reinterpret_cast<uint2*>(hi_out + (size_t)(4 * part) * k_pad + (size_t)i * 8) = make_uint2(hi[part][0], hi[part][1]);
+            *reinterpret_cast<uint2*>(lo_out + (size_t)(4 * part) * k_pad + (size_t)i * 8) = make_uint2(lo[part][0], lo[part][1]);
+        }
     };
 #pragma unroll
     for (int h = 0; h < kPrepHold; ++h)
         if (tid + h * kPrepThreads < n_pad) convert(tid + h * kPrepThreads, held[h]);
     for (int i = tid + kPrepHold * kPrepThreads; i < n_pad; i += kPrepThreads) convert(i, i < n_vec ? __ldg(&row[i]) : make_uint4(0u, 0u, 0u, 0u));
-    if (tid == 0) inv_scale[tok] = __uint_as_float((uint32_t)(254 - sfield) << 23);
+    lost = __syncthreads_or(lost) != 0;
+    if (tid == 0) {
+        inv_scale[tok] = __uint_as_float((uint32_t)(254 - sfield) << 23);
+        inexact[tok] = lost;
+    }
+}
+
+// ---- sums of shared tiles, and the marked tokens ------------------------------------------------
+struct ExactParams {
+    const uint8_t* packed;
+    const uint16_t* x;
+    const int* inexact;
+    int unit_bytes, meta_off, k_in, n_tiles, groups_per_block;
+};
+template <int WB>
+__device__ __forceinline__ float pot_value(uint32_t code) {   // zero times an infinity is to be NaN: a value, not a skipped term
+    constexpr uint32_t emax = (1u << (WB - 1)) - 1u;
+    const uint32_t e = code & emax, sign = (code >> (WB - 1)) & 1u;
+    return code == emax ? 0.f : __uint_as_float(((127u - e) << 23) | (sign << 31));
+}
+// A warp: 16 channels of one token by fp32 multiply-adds (Eq. 4 as it stands). Lane (g, t) owns whole micro-blocks of rows g and g + 8. About a microsecond a
+// k-block; only for marked tokens.
+template <int WB>
+__device__ __noinline__ void exact_outputs(const FinishParams& p, const ExactParams& e, int T, int tok) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    constexpr uint32_t kMask = WB <= 3 ? 0x77777777u : 0xFFFFFFFFu;
+    const int chunks = 4 / e.groups_per_block;   // 32-wide ones of a macro-block
+    float acc[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f}, s2[2] = {0.f, 0.f};
+    for (int bk = 0; bk < p.k_blocks; ++bk) {
+        const uint8_t* unit = e.packed + unit_offset(T, bk, p.k_blocks, e.unit_bytes);
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+            const int k0 = bk * kBlockK + c * 32 + t * 8;
+            const uint4 xv = k0 < e.k_in ? __ldg(reinterpret_cast<const uint4*>(e.x + (size_t)tok * e.k_in + k0)) : make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t xr[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int at = v * 128 + lane * 4 + c;
+                const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(unit) + at);
+                const uint32_t record = WB <= 3 ? gather_meta(w) : (uint32_t)(__ldg(unit + e.meta_off + at) & 63u);
+                const uint32_t b1 = w & kMask, b2 = xor_permute_nibbles(b1, (int)(record & 3u) + 1), flips = flip_mask(record);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float xi = __uint_as_float((i & 1) ? (xr[i >> 1] & 0xFFFF0000u) : (xr[i >> 1] << 16));
+                    s1[v] = fmaf(xi, pot_value<WB>((b1 >> (4 * i)) & 15u), s1[v]);
+                    const float q = pot_value<WB>((b2 >> (4 * i)) & 15u);
+                    s2[v] = fmaf(xi, ((flips >> i) & 1u) ? -q : q, s2[v]);
+                }
+            }
+            if ((c + 1) % chunks == 0) {
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const uint32_t pair = __ldg(reinterpret_cast<const uint32_t*>(unit + kCodeBytesPerUnit) + (c / chunks) * kTileRows + v * 8 + g);
+                    const float2 cf = __half22float2(*reinterpret_cast<const __half2*>(&pair));
+                    acc[v] += cf.x * s1[v] + cf.y * s2[v];
+                    s1[v] = s2[v] = 0.f;
+                }
+            }
+        }
+    }
+    const Output out = {p.y, p.y_dtype, p.n_out};
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        float a = acc[v];
+        a += __shfl_xor_sync(0xFFFFFFFFu, a, 1);
+        a += __shfl_xor_sync(0xFFFFFFFFu, a, 2);
+        const int ch = T * kTileRows + v * 8 + g;
+        if (t == 0 && ch < p.n_out) out.store1(tok, ch, a);
+    }
+}
+template <int WB>
+__global__ void __launch_bounds__(kFinishThreads) finish_f8_kernel(const __grid_constant__ FinishParams p, const __grid_constant__ ExactParams e) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int tile = blockIdx.x, tok0 = (tile / p.tiles_x) * p.n_cols + blockIdx.y * kFinishTokens;
+    const int n = min(min(kFinishTokens, p.n_cols - (int)blockIdx.y * kFinishTokens), p.m - tok0);
+    uint32_t marked = 0u;
+    finish_tile(p, [&] { marked = __ballot_sync(0xFFFFFFFFu, (int)(threadIdx.x & 31) < n && __ldcg(e.inexact + tok0 + (threadIdx.x & 31)) != 0); });
+    if (marked == 0u) return;
+    __syncthreads();   // over what was stored above
+    const int T = (tile % p.tiles_x) * (kTileN / kTileRows) + (int)(threadIdx.x >> 5);
+    if (T >= e.n_tiles) return;
+    for (; marked; marked &= marked - 1u) exact_outputs<WB>(p, e, T, tok0 + __ffs((int)marked) - 1);
 }
 
 // ---- host side ------------------------------------------------------------------------------------
@@ -467,12 +586,13 @@ static int sm_count() {
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct Plan {
-    int tokens, t_tiles, tiles_x, units, grid, n_x, n_pk;   // tokens: of a tile
-    size_t smem, inv_off, x8_off, partial_off, total;
+    int tokens, t_tiles, tiles_x, units, grid, n_x, n_pk;   // tokens: rows of a tile
+    size_t smem, inv_off, mark_off, x8_off, partial_off, total;
 };
 static bool make_plan(const Geometry& g, int m, Plan* p) {
-    p->t_tiles = (m + kMaxTokens - 1) / kMaxTokens;
-    p->tokens = ((m + p->t_tiles - 1) / p->t_tiles + 15) & ~15;   // equal token tiles
+    const int rows = rows_of(m);
+    p->t_tiles = (rows + kMaxTokens - 1) / kMaxTokens;
+    p->tokens = ((rows + p->t_tiles - 1) / p->t_tiles + 15) & ~15;   // equal token tiles
     p->tiles_x = (g.n_pad + kTileN - 1) / kTileN;
     const long long units = (long long)p->t_tiles * p->tiles_x * g.k_blocks;
     if (units >= (1ll << 30)) return false;
@@ -486,17 +606,18 @@ static bool make_plan(const Geometry& g, int m, Plan* p) {
     if (p->n_pk < 2) return false;
     p->smem = 8192 + kLutBytes + (size_t)kCoefSlots * g.groups_per_block * kTileN * 4 + p->n_x * x + p->n_pk * pk;
     p->inv_off = kWsScratchOff;
-    p->x8_off = p->inv_off + align256((size_t)(m + 16) * sizeof(float));
-    p->partial_off = align256(p->x8_off + (size_t)2 * m * g.k_pad);
-    p->total = p->partial_off + (size_t)p->grid * 2 * p->tokens * kTileN * sizeof(float);
+    p->mark_off = p->inv_off + align256((size_t)(m + 16) * sizeof(float));
+    p->x8_off = p->mark_off + align256((size_t)m * sizeof(int));
+    p->partial_off = align256(p->x8_off + (size_t)2 * rows * g.k_pad);
+    p->total = p->partial_off + (size_t)p->grid * p->tokens * kTileN * sizeof(float);   // (two parts a CTA, two rows a token)
     return true;
 }
 
 template <int WB, int GPB, int NB8>
-static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
+static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed, const void* x, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
     CUtensorMap map, pmap;
     if (cudaError_t e = encode_packed_map(&pmap, packed, g, 8)) return e;
-    if (cudaError_t e = encode_i8_map(&map, ws + pl.x8_off, g.k_pad, 2 * m, pl.tokens)) return e;
+    if (cudaError_t e = encode_i8_map(&map, ws + pl.x8_off, g.k_pad, 2 * rows_of(m), pl.tokens)) return e;
     Params p;
     p.packed = (const uint8_t*)packed;
     p.y = y;
@@ -504,7 +625,9 @@ static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed,
     p.status = (int*)ws;
     p.partial = (float*)(ws + pl.partial_off);
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.k_blocks = g.k_blocks; p.n_tiles = g.n_tiles; p.n_out = g.n_out;
-    p.m = m; p.y_dtype = y_dtype; p.tiles_x = pl.tiles_x; p.units = pl.units; p.n_x = pl.n_x; p.n_pk = pl.n_pk;
+    p.m = m; p.rows = rows_of(m); p.y_dtype = y_dtype; p.tiles_x = pl.tiles_x; p.units = pl.units; p.n_x = pl.n_x; p.n_pk = pl.n_pk;
+    p.run = 1;
+    while (p.run * (p.run + 1) * g.groups_per_block <= g.k_blocks) ++p.run;
     p.spin = spin_limit > 0 ? spin_limit : kSpin;
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(gemm_f8_kernel<WB, GPB, NB8>, pl.smem, smem_attr)) return e;
@@ -519,21 +642,20 @@ static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_f8_kernel<WB, GPB, NB8>, p, map, pmap)) return e;
-    // whole tiles only: one k-block a tile, or every range a whole number of tiles
-    if (g.k_blocks == 1 || (p.units % pl.grid == 0 && (p.units / pl.grid) % g.k_blocks == 0)) return cudaSuccess;
-    const FinishParams f = {p.partial, p.inv_scale, y, y_dtype, g.n_out, m, pl.tokens, pl.tiles_x, g.k_blocks, pl.units, pl.grid};
-    cfg.gridDim = dim3(pl.tiles_x * pl.t_tiles, (pl.tokens + kFinishTokens - 1) / kFinishTokens);
+    const FinishParams f = {p.partial, p.inv_scale, y, y_dtype, g.n_out, m, pl.tokens / 2, pl.tiles_x, g.k_blocks, pl.units, pl.grid};
+    const ExactParams e = {(const uint8_t*)packed, (const uint16_t*)x, (const int*)(ws + pl.mark_off), g.unit_bytes, g.meta_off, g.k_in, g.n_tiles, g.groups_per_block};
+    cfg.gridDim = dim3(pl.tiles_x * pl.t_tiles, (pl.tokens / 2 + kFinishTokens - 1) / kFinishTokens);
     cfg.blockDim = dim3(kFinishThreads);
     cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, finish_kernel, f);
+    return cudaLaunchKernelEx(&cfg, finish_f8_kernel<WB>, f, e);
 }
 template <int WB, int GPB>
-static cudaError_t launch_tokens(const Geometry& g, const Plan& pl, const void* packed, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
+static cudaError_t launch_tokens(const Geometry& g, const Plan& pl, const void* packed, const void* x, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {
     switch (pl.tokens / 16) {
-        case 1: return launch<WB, GPB, 1>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st);
-        case 2: return launch<WB, GPB, 2>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st);
-        case 3: return launch<WB, GPB, 3>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st);
-        default: return launch<WB, GPB, 4>(g, pl, packed, m, y, y_dtype, ws, spin_limit, st);
+        case 1: return launch<WB, GPB, 1>(g, pl, packed, x, m, y, y_dtype, ws, spin_limit, st);
+        case 2: return launch<WB, GPB, 2>(g, pl, packed, x, m, y, y_dtype, ws, spin_limit, st);
+        case 3: return launch<WB, GPB, 3>(g, pl, packed, x, m, y, y_dtype, ws, spin_limit, st);
+        default: return launch<WB, GPB, 4>(g, pl, packed, x, m, y, y_dtype, ws, spin_limit, st);
     }
 }
 
@@ -548,7 +670,7 @@ size_t gemm_f8_workspace(const Geometry& g, int m) {
     return f8::make_plan(g, m, &p) ? p.total : 0;
 }
 // Estimated time: waves of units, a unit by its tokens and the steps its sums are read back in, and pre-pass, start and the sum of shared tiles
-// (us; within 8 % of the measured times at 2048 x 2048 .. 28672 x 8192, 16000 x 512 and 1024 x 8192, 8 to 128 tokens).
+// (us; within 10 % of the measured times from 4096 x 4096 to 28672 x 8192, 1 to 32 tokens; up to 19 % above them where an SM has a few units, 8 % below at k = 28672).
 float gemm_f8_us(const Geometry& g, int m) {
     f8::Plan p;
     if (!f8::make_plan(g, m, &p)) return 1e30f;
@@ -558,9 +680,11 @@ float gemm_f8_us(const Geometry& g, int m) {
 }
 size_t gemm_f8_workspace_upto(const Geometry& g, int m) {   // enough for every call of up to m rows
     if (!gemm_f8_supported(g, 1)) return 0;
-    const long long units = (long long)((m + f8::kMaxTokens - 1) / f8::kMaxTokens) * ((g.n_pad + f8::kTileN - 1) / f8::kTileN) * g.k_blocks;
-    const size_t grid = units < f8::sm_count() ? (size_t)units : (size_t)f8::sm_count(), tokens = m < f8::kMaxTokens ? (m + 15) & ~15 : f8::kMaxTokens;
-    return f8::align256(kWsScratchOff + f8::align256((size_t)(m + 16) * sizeof(float)) + (size_t)2 * m * g.k_pad) + grid * 2 * tokens * f8::kTileN * sizeof(float);
+    const int rows = f8::rows_of(m);
+    const long long units = (long long)((rows + f8::kMaxTokens - 1) / f8::kMaxTokens) * ((g.n_pad + f8::kTileN - 1) / f8::kTileN) * g.k_blocks;
+    const size_t grid = units < f8::sm_count() ? (size_t)units : (size_t)f8::sm_count(), tokens = rows < f8::kMaxTokens ? (rows + 15) & ~15 : f8::kMaxTokens;
+    return f8::align256(kWsScratchOff + f8::align256((size_t)(m + 16) * sizeof(float)) + f8::align256((size_t)m * sizeof(int)) + (size_t)2 * rows * g.k_pad) +
+           grid * tokens * f8::kTileN * sizeof(float);
 }
 cudaError_t launch_gemm_f8(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws, int spin_limit, cudaStream_t st) {
     f8::Plan p;
@@ -575,11 +699,12 @@ cudaError_t launch_gemm_f8(const Geometry& g, const void* packed, const void* x,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaError_t e = cudaLaunchKernelEx(&cfg, f8::x_to_f8_kernel, (const uint16_t*)x, g.k_in, g.k_pad, b + p.x8_off, (float*)(b + p.inv_off), m)) return e;
+    if (cudaError_t e = cudaLaunchKernelEx(&cfg, f8::x_to_f8_kernel, (const uint16_t*)x, g.k_in, g.k_pad, b + p.x8_off, (float*)(b + p.inv_off),
+                                           (int*)(b + p.mark_off), m)) return e;
 #define GOQ_F8(WB_)                                                                                                       \
-    (g.groups_per_block == 1 ? f8::launch_tokens<WB_, 1>(g, p, packed, m, y, y_dtype, b, spin_limit, st)                  \
-     : g.groups_per_block == 2 ? f8::launch_tokens<WB_, 2>(g, p, packed, m, y, y_dtype, b, spin_limit, st)                \
-                               : f8::launch_tokens<WB_, 4>(g, p, packed, m, y, y_dtype, b, spin_limit, st))
+    (g.groups_per_block == 1 ? f8::launch_tokens<WB_, 1>(g, p, packed, x, m, y, y_dtype, b, spin_limit, st)                  \
+     : g.groups_per_block == 2 ? f8::launch_tokens<WB_, 2>(g, p, packed, x, m, y, y_dtype, b, spin_limit, st)                \
+                               : f8::launch_tokens<WB_, 4>(g, p, packed, x, m, y, y_dtype, b, spin_limit, st))
     return g.wbits == 4 ? GOQ_F8(4) : g.wbits == 3 ? GOQ_F8(3) : GOQ_F8(2);
 #undef GOQ_F8
 }

@@ -107,7 +107,7 @@ size_t gemm_mid_workspace_upto(const Geometry& g, int m);   // enough for every 
 cudaError_t launch_gemm_mid(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws,
                             bool exact, int spin_limit, cudaStream_t st);
 
-// The same layer for a few tokens up to about 128 (goq_gemm_f8.cu): both bases as exact e4m3 operands, activations as two e4m3 slices; group >= 32.
+// The same layer for a few tokens up to about 128 (goq_gemm_f8.cu): both bases and the activations as exact e4m3 operands; group >= 32.
 bool gemm_f8_supported(const Geometry& g, int m);
 float gemm_f8_us(const Geometry& g, int m);   // estimated time
 size_t gemm_f8_workspace(const Geometry& g, int m);

@@ -334,6 +334,42 @@ def test_calls_either_side_of_the_lines_of_the_e4m3_kernel(goq, n, k, g, b, m):
             check_parity(y.cpu().numpy().astype(np.float64)[:, rows], y_ref, *tol)
 
 
+@pytest.mark.parametrize("n,k,g,b,m,variant", [(16384, 4096, 128, 4, 4, 0), (12000, 4096, 128, 3, 16, 0), (28672, 2048, 64, 2, 11, 0), (300, 640, 32, 3, 24, 6), (130, 128, 128, 2, 40, 6),
+                                               (8192, 4096, 128, 3, 32, 0)])
+def test_small_elements_beside_a_large_one_and_non_finite_ones_in_e4m3_operands(goq, n, k, g, b, m, variant):
+    """One element of a token 2^13 .. 2^40 times the others, and channels whose states are zero there: to them the token is an ordinary one, and their
+    outputs are held to their own magnitude, by the bounds of every fp32-accumulating kernel. An infinite or NaN element gives what Eq. 4 gives: infinite or
+    NaN channel by channel. Through goq_gemm and (up to 16 tokens) goq_gemv; every other token is that of a call without these elements, bit for bit."""
+    from tests.gpu_util import check_parity, pack_weights, run_gemm_bf16, run_gemv
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    at, blind = k // 2 + 3, np.arange(0, n, 3)   # channels that do not see the micro-block of that element
+    mb = at // 8 * 8
+    codes[blind, mb:mb + 8] = (1 << (b - 1)) - 1
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    plain = si.bf16_activations(m, k, seed=m)
+    x = si.bf16_bits_to_f64(plain)
+    powers = [2.0 ** e for e in (13, 16, 22, 28, 40)][:m - 2]
+    for tok, f in enumerate(powers):
+        x[tok, at] = f * 1.5
+    xb = si.f32_to_bf16_bits(x.astype(np.float32))
+    xb[m - 2, at] = 0x7F80 if m % 2 else 0xFF80
+    xb[m - 1, at] = 0x7FC0
+    rows = np.unique(np.concatenate([blind[si.sample_rows(len(blind), min(len(blind), 150), seed=2)], si.sample_rows(n, min(n, 150), seed=3), np.arange(n - 20, n)]))
+    with np.errstate(invalid="ignore"):
+        y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b, rows=rows)
+    unseen = np.isin(rows, blind)
+    for run in (run_gemm_bf16, run_gemv)[:2 if m <= 16 and variant == 0 else 1]:
+        all_y, base = run(d, packed, xb, variant=variant), run(d, packed, plain, variant=variant)
+        y = all_y[:, rows]
+        for tok in range(len(powers)):
+            check_parity(y[tok, unseen], y_ref[tok, unseen], 2e-5, 1e-4, "2^%g" % np.log2(powers[tok]))
+        check_parity(y[:m - 2], y_ref[:m - 2], 2e-5, 1e-4)
+        for tok in (m - 2, m - 1):
+            assert np.array_equal(np.isnan(y[tok]), np.isnan(y_ref[tok])) and np.array_equal(np.isposinf(y[tok]), np.isposinf(y_ref[tok]))
+            assert np.array_equal(np.isneginf(y[tok]), np.isneginf(y_ref[tok]))
+        assert np.array_equal(all_y[len(powers):m - 2], base[len(powers):m - 2])
+
+
 def test_e4m3_operand_gemm_reports_a_wait_that_runs_out(goq):
     """With one poll a wait the kernel gives up: the status word reads GOQ_ERR_TIMEOUT, and on a fresh scratch buffer the next call is right again."""
     from tests.gpu_util import dev, pack_weights
