@@ -195,8 +195,8 @@ goq_status goq_quantize_geo(const goq_desc* desc, const float* w, uint8_t* codes
  * restricted to the macro-block's channels, A = [X_q b1, X_q b2], Y = X_q w:  c* = (A^T A + lambda I)^-1 A^T Y.
  *   w [n_out][k_in] fp32; codes, meta as produced by goq_quantize_geo; x_calib [m][k_in] fp32 (m observations);
  *   lambda >= 0 (the paper uses 1e-4);  coef_f16 out [n_out][k_in/group][2];  c_f64 optional out, the unrounded pairs.
- *   Float64 throughout (sums of the Gram matrix's products in 64-bit fixed point on the tensor cores: no less accurate). If a bounded wait on the device
- *   gives up, the pairs it would have given are NaN. */
+ *   Float64 throughout (sums of the Gram matrix's products in 64-bit fixed point on the tensor cores where a macro-block's channels are of magnitudes
+ *   so alike that this is no less accurate). If a bounded wait on the device gives up, the pairs it would have given are NaN. */
 goq_status goq_solve_ref(const goq_desc* desc, const float* w, const uint8_t* codes, const uint8_t* meta,
                          const float* x_calib, int m, double lambda, uint16_t* coef_f16, double* c_f64, void* stream);
 

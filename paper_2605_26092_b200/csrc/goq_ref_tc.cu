@@ -6,8 +6,11 @@
 // b1 and b2 are small integers times 2^-emax. So V_b needs no float64 products: every row k of G is written as 64-bit fixed point against its
 // largest element, |G_kl| 2^s_k < 2^62, and cut into eight signed byte digits; the digits times b_b are tcgen05 kind::i8 MMAs, exact in int32.
 // Recombining the eight sums and the five products with b1, b2, w is all the float64 that is left: 8 operations per element and vector
-// instead of 1.5 g. Rounding a G_kl to 2^-63 of its row's largest element is 2^9 below a float64 product of the largest element, so the
-// result is no further from the exact one than float64 sums are (the entries of G itself are float64 sums, as in solve_ref_kernel).
+// instead of 1.5 g. A G_kl is rounded to 2^-63 of its row's largest element. While that is at most 2^10 times the row's diagonal element, the rounding is at
+// most 2^-53 G_kk, no more than that of a float64 product with a state of 1, and the result is no further from the exact one than float64 sums are (the
+// entries of G itself are float64 sums, as in solve_ref_kernel). Where one channel is so much larger than another that a row goes beyond (some 10^4 times),
+// rows of W with zero states there would see the rounding of elements that they multiply by zero (2^20 times: 6e-14): such a column is solved in float64 from
+// G as it is (solve_wide), its digits unused. 4096 x 4096, 256 observations, every column so: 106 -> 317 us (solve_ref_kernel 324).
 //
 // A column belongs to a cluster of `C` CTAs: each forms 1 / C of the lower triangle of G (float64 tensor pipe), takes the others'
 // blocks through distributed shared memory, cuts all of G into digits, and solves its share of the 128-row tiles. Roles: warps 0-15 add up V_1 and V_2
@@ -15,14 +18,15 @@
 // (N = 256: 32 x 8 digits); V_1 and V_2 have half of tensor memory each, so one is read while the other is computed.
 // Bound: instruction issue of the recombination (about 35 instructions an element and vector; issue 46 %, integer pipe 28 %, float64 15 %, int8 MMAs
 // 14 %), 17.6 K clocks a tile of 128 rows x 128, and 35 K clocks at the start (G 19 K, its exchange 7 K, digits 8 K).
-// Measured, W3, in groups of 128: 4096 x 4096 with 256 observations 332 -> 108 us (solve_ref_kernel before), 8192 x 8192 with 512 1230 -> 364, 512 x 512
-// with 128 38 -> 31; groups of 64: 207 -> 95; of 32: 208 -> 110. Not kept: V in passes of 8 elements with two passes a warp in tensor memory (134 us: a
+// Measured, W3, in groups of 128: 4096 x 4096 with 256 observations 324 -> 104 us (solve_ref_kernel before), 8192 x 8192 with 512 1227 -> 355, 512 x 512
+// with 128 37 -> 29; groups of 64: 205 -> 92; of 32, W4: 201 -> 107. Not kept: V in passes of 8 elements with two passes a warp in tensor memory (134 us: a
 // wait costs more than the overlap gives); eight recombining warps (134); operands and w set up while G is formed (111).
 // Error against long double (2-norm, relative) 1.7e-16 where the float64 products had 2.7e-16, 3.3e-12 against 3.7e-12 where the observations' mean is 100
 // times their deviation.
 // Every mbarrier wait is bounded; a CTA that gives up writes NaN for its rows.
 #include "goq_tc_core.cuh"
 #include "goq_internal.h"
+#include "goq_ref_rows.cuh"
 #include <type_traits>
 
 namespace goq {
@@ -58,6 +62,7 @@ template <int WB, int G> struct Smem {
     static constexpr size_t kForm = (Gram<G>::kStageBytes > Gram<G>::kDigitBytes ? Gram<G>::kStageBytes : Gram<G>::kDigitBytes) + kTri;
     static constexpr size_t kTriOff = (kRun > kForm ? kRun : kForm) - kTri;
     static constexpr size_t kBytes = (kRun > kForm ? kRun : kForm) + 1024;
+    static_assert(quant::RefSmem<G / 8>::kFrags * 32 * sizeof(double) <= kTriOff && quant::RefSmem<G / 8>::kBytes + 1024 <= kBytes, "solve_wide");
 };
 
 struct Params {
@@ -76,9 +81,6 @@ __device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t adesc, uint64_
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool on) {   // off: zeros
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
@@ -124,6 +126,27 @@ __device__ __forceinline__ double combine(const uint32_t* u, double c) {
     return fma(h, c32, l * c);
 }
 
+// The CTA's rows in float64, as solve_ref_kernel has them. H = the lower triangle of G and half its diagonal goes as operand fragments to the start of `room`; the
+// triangle's own room is used again behind. A call of its own: its registers are not the other roles'.
+template <int WB, int G>
+__device__ __noinline__ void solve_wide(const float* w, const uint8_t* codes, const uint8_t* meta, double lambda, uint16_t* coef, double* c_out, int n_out, int k_in,
+                                        unsigned char* base, int j, int rt_lo, int rt_hi) {
+    constexpr int NB = G / 8;
+    const double* tri = reinterpret_cast<const double*>(base + Smem<WB, G>::kTriOff);
+    double* room = reinterpret_cast<double*>(base);
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31, lr = lane >> 2, lc = lane & 3;
+    for (int ib = warp; ib < NB; ib += kThreads / 32)
+        for (int s = 0; s < 2 * (ib + 1); ++s) {
+            const int l = (s & 1) * 4 + lc;
+            const double g = tri[(ib * (ib + 1) / 2 + (s >> 1)) * kBlkStride + lr * kBlkRow + l];
+            room[(ib * (ib + 1) + s) * 32 + lane] = s >> 1 < ib || l < lr ? g : l == lr ? 0.5 * g : 0.0;
+        }
+    __syncthreads();
+    if (warp < quant::kRefWarps)
+        quant::solve_rows<WB, NB, false>(room, reinterpret_cast<float*>(room + quant::RefSmem<NB>::kFrags * 32), w, codes, meta, 0, lambda, coef, c_out, n_out, k_in, j, rt_lo,
+                                         rt_hi);
+}
+
 template <int WB, int G>
 __global__ void __launch_bounds__(kThreads, 1)
 solve_ref_tc_kernel(const Params p, const __grid_constant__ CUtensorMap w_map) {
@@ -142,12 +165,13 @@ solve_ref_tc_kernel(const Params p, const __grid_constant__ CUtensorMap w_map) {
     __shared__ uint2 flip_bytes[64];      // 0xFF where b2 takes the opposite sign
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
+    __shared__ int wide;   // wide: a row of G has an element more than 2^10 times its diagonal one
 
     const int tid = threadIdx.x, warp = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31, lr = lane >> 2, lc = lane & 3;
     const int j = (int)blockIdx.x / p.c, rank = (int)blockIdx.x - j * p.c, nj = p.k_in / G;
 
     if (tid == 0) {
-        abort_flag = 0;
+        abort_flag = 0; wide = 0;
         for (int i = 0; i < 2; ++i) {
             mbar_init(&a_full[i], kDecWarps); mbar_init(&a_empty[i], kEpiWarps);
             mbar_init(&tm_full[i], 1); mbar_init(&tm_empty[i], kEpiWarps / 2);
@@ -219,7 +243,7 @@ solve_ref_tc_kernel(const Params p, const __grid_constant__ CUtensorMap w_map) {
                     const float* xs = x0 + s * 4 * kStride;
 #pragma unroll
                     for (int i = 0; i < kMax; ++i)
-                        if (i < n) dmma(acc[i], (double)xs[at_a[i]], (double)xs[at_b[i]]);
+                        if (i < n) quant::dmma(acc[i], (double)xs[at_a[i]], (double)xs[at_b[i]]);
                 }
             }
             __syncthreads();
@@ -282,6 +306,7 @@ solve_ref_tc_kernel(const Params p, const __grid_constant__ CUtensorMap w_map) {
         }
         const int e = big == 0.0 ? 61 : (int)((__double2hiint(big) >> 20) & 2047) - 1023;   // (sums of squares of fp32 numbers: never subnormal)
         const double up = pow2(61 - e);   // |G_kl| 2^(61 - e) < 2^62
+        if (big > 1024.0 * tri[(kb * (kb + 1) / 2 + kb) * kBlkStride + (k & 7) * (kBlkRow + 1)] && !bad) wide = 1;
         if (q == 0) scale[k] = bad ? __longlong_as_double(0x7FF8000000000000ll) : pow2(e - 61 - 2 * emax);
         const uint32_t row0 = s32(base) + (uint32_t)k * (kDigits * 128);
 #pragma unroll
@@ -309,6 +334,15 @@ solve_ref_tc_kernel(const Params p, const __grid_constant__ CUtensorMap w_map) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_slot;
+    if (wide) {   // (all CTAs of the cluster have the same G and find the same)
+        solve_wide<WB, G>(p.w, p.codes, p.meta, p.lambda, p.coef, p.c_out, p.n_out, p.k_in, base, j, t_lo * (kRows / 8),
+                          min(t_hi * (kRows / 8), (p.n_out + 7) / 8));
+        if (warp == kMmaWarp) {
+            __syncwarp();
+            tmem_dealloc<512>(tmem_base);
+        }
+        return;
+    }
     const uint32_t a_base = s32(base + SM::kA), w_base = s32(base + SM::kW);
 
     if (warp == kWWarp) {

@@ -297,6 +297,42 @@ def test_ref_solve_digits_match_oracle(goq, n, k, g, b, m):
         assert np.array_equal(solve(part), got[part])
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(300, 384, 128, 3, 130), (129, 256, 128, 4, 256), (140, 1280, 64, 3, 100), (200, 1152, 32, 2, 130), (1030, 128, 128, 2, 70)])
+@pytest.mark.parametrize("power", [12, 20, 30, 40])
+def test_ref_solve_channels_far_above_the_others(goq, n, k, g, b, m, power):
+    """A channel 2^12 .. 2^40 times the others in some columns. Every second row has zero states and weights at its micro-block and does not see it: its pairs
+    are as exact as if it were not there. Bound as above, and with the rounding of A^T Y, whose terms reach |A| |Y|: a weight may see the channel where the
+    states do not."""
+    from tests.gpu_util import dev
+    w = si.gaussian_weights(n, k, seed=n + m).astype(np.float32)
+    codes, meta, _ = O.quantize_geo(w, g, b)
+    x = si.f32_activations(m, k, seed=m).astype(np.float32)
+    for j in range(0, k // g, 2):
+        mb = j * g + g // 2
+        x[:, mb + 3] *= np.float32(2.0 ** power)
+        codes[::2, mb:mb + 8] = (1 << (b - 1)) - 1
+        w[::2, mb:mb + 8] = 0.0
+    d = goq.desc(n, k, g, b)
+    coef = torch.zeros((n, k // g, 2), dtype=torch.int16, device="cuda")
+    c64 = torch.zeros((n, k // g, 2), dtype=torch.float64, device="cuda")
+    goq.solve_ref(d, dev(w), dev(codes), dev(meta), torch.from_numpy(x).cuda(), m, 1e-4, coef, c64)
+    torch.cuda.synchronize()
+    got = c64.cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(min(n, 60)), np.arange(n - 40, n)]))
+    if power > 20:
+        rows = rows[rows % 2 == 0]   # to float64 the channel makes b1's and b2's columns of the others parallel
+    assert np.array_equal(coef.cpu().numpy().view(np.uint16)[rows], got[rows].astype(np.float16).view(np.uint16))
+    want = O.solve_ref(w[rows], codes[rows], meta[rows], x, g, b, lam=1e-4)
+    b1, b2 = O.decode_b1(codes[rows], b), O.decode_b2(codes[rows], meta[rows], b)
+    for j in range(k // g):
+        s = slice(j * g, (j + 1) * g)
+        a1, a2 = x[:, s].astype(np.float64) @ b1[:, s].T, x[:, s].astype(np.float64) @ b2[:, s].T
+        p, q, t = (a1 * a1).sum(0) + 1e-4, (a2 * a2).sum(0) + 1e-4, (a1 * a2).sum(0)
+        size, y = np.abs(want[:, j]).max(-1), x[:, s].astype(np.float64) @ w[rows][:, s].astype(np.float64).T
+        bound = np.sqrt(m * g) * 2.3e-16 * (p + q) / np.maximum(p * q - t * t, 1e-300) * ((p + q) * size + np.sqrt(p + q) * np.linalg.norm(y, axis=0))
+        assert (bound[rows % 2 == 0] < size[rows % 2 == 0]).all() and (np.abs(got[rows, j] - want[:, j]).max(-1) <= bound).all(), j
+
+
 def test_ref_solve_non_finite_inputs_and_unaligned_buffers(goq):
     """A NaN observation makes its column's pairs NaN and no other's; codes, weights and observations at any element's address are taken."""
     from tests.gpu_util import dev
