@@ -575,14 +575,6 @@ __global__ void __launch_bounds__(kFinishThreads) finish_f8_kernel(const __grid_
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-static int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-    }
-    return n;
-}
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct Plan {
@@ -682,7 +674,7 @@ size_t gemm_f8_workspace_upto(const Geometry& g, int m) {   // enough for every 
     if (!gemm_f8_supported(g, 1)) return 0;
     const int rows = f8::rows_of(m);
     const long long units = (long long)((rows + f8::kMaxTokens - 1) / f8::kMaxTokens) * ((g.n_pad + f8::kTileN - 1) / f8::kTileN) * g.k_blocks;
-    const size_t grid = units < f8::sm_count() ? (size_t)units : (size_t)f8::sm_count(), tokens = rows < f8::kMaxTokens ? (rows + 15) & ~15 : f8::kMaxTokens;
+    const size_t grid = units < sm_count() ? (size_t)units : (size_t)sm_count(), tokens = rows < f8::kMaxTokens ? (rows + 15) & ~15 : f8::kMaxTokens;
     return f8::align256(kWsScratchOff + f8::align256((size_t)(m + 16) * sizeof(float)) + f8::align256((size_t)m * sizeof(int)) + (size_t)2 * rows * g.k_pad) +
            grid * tokens * f8::kTileN * sizeof(float);
 }

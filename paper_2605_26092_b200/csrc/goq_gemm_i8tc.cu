@@ -433,14 +433,6 @@ gemm_i8tc_kernel(const Params p, const __grid_constant__ CUtensorMap x_map, cons
     }
 }
 
-static int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-    }
-    return n;
-}
 template <int WB, int GPB>
 static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& x_map, const CUtensorMap& packed_map, cudaStream_t st) {
     constexpr int kUnitBytes = kCodeBytesPerUnit + 64 * GPB + (WB == 4 ? kWordsPerBlock : 0), kSlots = ring_slots(kUnitBytes, Digits<WB>::entry);
@@ -480,7 +472,7 @@ cudaError_t launch_gemm_i8tc(const Geometry& g, const void* packed, const int8_t
     const int half_tiles = (m + i8tc::kTokens - 1) / i8tc::kTokens;
     // 256 tokens a tile halve the decode; 128 where that would leave SMs without a tile, or where there are no more (the second half's
     // MMAs would be padding: 16000 x 512 at 64 tokens 11.9 us)
-    p.tt = half_tiles > 1 && p.tiles_x * ((half_tiles + 1) / 2) >= i8tc::sm_count() ? 2 : 1;
+    p.tt = half_tiles > 1 && p.tiles_x * ((half_tiles + 1) / 2) >= sm_count() ? 2 : 1;
     p.tiles = p.tiles_x * ((half_tiles + p.tt - 1) / p.tt);
     p.status = status;
     p.spin = spin_limit > 0 ? spin_limit : tc::kSpin;

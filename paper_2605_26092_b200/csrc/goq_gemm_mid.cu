@@ -428,15 +428,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mid_kernel(const Params p, c
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-static int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-            n = 148;
-    }
-    return n;
-}
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct Plan {
@@ -541,7 +532,7 @@ float gemm_mid_us(const Geometry& g, int m) {
     const float drain = 0.07f * (float)p.n_cols / (float)g.k_blocks;
     return 14.f + (float)((p.units + p.grid - 1) / p.grid) * (unit > drain ? unit : drain);
 }
-int gemm_mid_ctas() { return mid::sm_count(); }
+int gemm_mid_ctas() { return sm_count(); }
 size_t gemm_mid_workspace(const Geometry& g, int m, bool exact) {
     mid::Plan p;
     return mid::make_plan(g, m, exact && !g.k1, &p) ? p.total : 0;
@@ -551,7 +542,7 @@ size_t gemm_mid_workspace_upto(const Geometry& g, int m) {
     // the offsets of make_plan; token tiles no wider than 256 or the call, and no more CTAs than units (more token tiles than one per
     // 256 rows only where the units fill the SMs anyway)
     const long long units = (long long)((m + 255) / 256) * ((g.n_pad + mid::kTileN - 1) / mid::kTileN) * g.k_blocks;
-    const size_t grid = units < mid::sm_count() ? (size_t)units : (size_t)mid::sm_count(), cols = m < 256 ? (m + 15) & ~15 : 256;
+    const size_t grid = units < sm_count() ? (size_t)units : (size_t)sm_count(), cols = m < 256 ? (m + 15) & ~15 : 256;
     const size_t xh_off = kWsScratchOff + mid::align256((size_t)(m + 16) * sizeof(float));
     return mid::align256(xh_off + (size_t)m * g.k_in * 2) + grid * 2 * cols * mid::kTileN * sizeof(float);
 }

@@ -353,21 +353,12 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-static int pair_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        n /= 2;
-    }
-    return n;
-}
 static size_t smem_for(const Geometry& g) { return 1024 + (size_t)kStages * kStageBytes + kLutBytes + (size_t)2 * kExpanders * g.unit_bytes; }
 // Token tiles of a call, equally wide, as in goq_gemm_tc.cu, over pairs of SMs
 static float wave_us(int k_blocks, int tokens) { return 8.f + (float)k_blocks * (0.75f + 0.00085f * (float)tokens); }
 struct TokenTiles { int n, half, n_full, n_tail; float us; };
 static TokenTiles token_tiles(const Geometry& g, int m) {
-    const int pairs = pair_count(), pairs_x = (g.n_pad + 2 * kTileN - 1) / (2 * kTileN);
+    const int pairs = sm_count() / 2, pairs_x = (g.n_pad + 2 * kTileN - 1) / (2 * kTileN);
     TokenTiles best = {};
     const int n0 = (m + 511) / 512;
     for (int n = n0; n <= n0 + 4; ++n) {

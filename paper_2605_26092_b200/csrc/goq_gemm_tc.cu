@@ -544,15 +544,6 @@ cudaError_t launch_x_to_f16(const void* x, int k_in, int m, uint16_t* xh, float*
     return launch_pre_pass(x, k_in, m, 0, xh, inv_scale, nullptr, 0, 0, 0, nullptr, nullptr, st);
 }
 
-static int sm_count_cached() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-            n = 148;
-    }
-    return n;
-}
 // Token tiles of a call, equally wide (600 tokens: 2 of 320, not 512 and 88). More of them than 512 tokens each allow where that
 // makes the waves over the SMs clearly shorter (a call with few channel tiles leaves SMs idle): a CTA takes, for each k-block,
 // the weights' decode plus a share that grows with its tokens (4096 x 4096 W3, us a k-block: 1.1 at 128 tokens, 1.3 at 256, 1.6 at
@@ -562,7 +553,7 @@ static int sm_count_cached() {
 static float wave_us(int k_blocks, int tokens) { return 8.f + (float)k_blocks * (0.95f + 0.00135f * (float)tokens); }
 struct TokenTiles { int n, half, n_full, n_tail; float us; };   // tiles of 2 * half tokens; n_full CTAs take whole tiles, n_tail tiles go as halves
 static TokenTiles token_tiles(const Geometry& g, int m) {
-    const int sms = sm_count_cached(), tiles_x = (g.n_pad + kTileN - 1) / kTileN;
+    const int sms = sm_count(), tiles_x = (g.n_pad + kTileN - 1) / kTileN;
     TokenTiles best = {};
     if (m <= 256) { best.n = 1; best.half = (m + 15) & ~15; best.n_tail = tiles_x; return best; }
     const int n0 = (m + kTileM - 1) / kTileM;
@@ -583,7 +574,7 @@ static TokenTiles token_tiles(const Geometry& g, int m) {
 static int split_factor(const Geometry& g, int m) {
     if (m > 256) return 1;
     const int tiles_x = (g.n_pad + kTileN - 1) / kTileN;
-    int s = sm_count_cached() / tiles_x;
+    int s = sm_count() / tiles_x;
     if (s > 4) s = 4;
     if (s > g.k_blocks / 4) s = g.k_blocks / 4;
     if (s < 2) return 1;

@@ -622,13 +622,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_chain_kernel(const __grid_co
 // ---- host side -------------------------------------------------------------------------------------
 namespace goq {
 
-static int chain_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 148;
-    return n > 0 ? n : 148;
-}
-
 static constexpr size_t kChainSmemMax = 226 * 1024;   // the opt-in limit is 227 KiB per CTA, static shared variables included
 
 static size_t chain_fixed_smem(int ng) {
@@ -654,7 +647,7 @@ size_t gemv_seq_zeroed_prefix(int n_items) {
     return z > kWsScratchOff ? z : kWsScratchOff;
 }
 static size_t chain_parts_bytes(int n_items) {
-    return (size_t)(n_items > 0 ? n_items : 0) * (size_t)chain_sm_count() * 2 * chain::kPartWords * sizeof(uint2);
+    return (size_t)(n_items > 0 ? n_items : 0) * (size_t)sm_count() * 2 * chain::kPartWords * sizeof(uint2);
 }
 size_t gemv_seq_workspace(int n_items) {
     // a single linear feeds nobody: no tagged copies
@@ -679,7 +672,7 @@ static cudaError_t launch_chain_cfg(chain::Params& p, size_t x_need, cudaStream_
     static SmemAttrCache smem_attr;
     if (cudaError_t e = ensure_dynamic_smem(kernel, smem, smem_attr)) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(chain_sm_count());   // every CTA must be resident: the completion counters are waited on
+    cfg.gridDim = dim3(sm_count());   // every CTA must be resident: the completion counters are waited on
     cfg.blockDim = dim3(chain::kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -745,7 +738,7 @@ cudaError_t launch_gemv_seq(const SeqCall* calls, int n, int wbits, int group, i
     p.epoch = (unsigned*)(wsb + 4);
     p.parts = (uint2*)(wsb + gemv_seq_zeroed_prefix(n));
     p.tags = (uint2*)(wsb + gemv_seq_zeroed_prefix(n) + chain_parts_bytes(n));
-    const int G = chain_sm_count();   // the grid
+    const int G = sm_count();   // the grid
     p.g_magic = ((1ull << 32) + (unsigned)G - 1) / (unsigned)G;
     int m_max = 1;
     bool k1 = true;

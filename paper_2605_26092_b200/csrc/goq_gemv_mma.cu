@@ -211,16 +211,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) gemv_mma_kernel(const Param
     for (int o2 = o + blockDim.x; o2 < 32 * NT * 4; o2 += blockDim.x) store(o2, red[0][o2]);
 }
 
-static int sm_count() {
-    static int cached[64];
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (dev >= 0 && dev < 64 && cached[dev]) return cached[dev];
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    if (dev >= 0 && dev < 64) cached[dev] = n;
-    return n;
-}
-
 template <int WB, int NT, int CPG>
 static cudaError_t launch(const Geometry& g, Params& p, cudaStream_t st) {
     int warps = g.k_blocks < kMaxWarps ? (g.k_blocks < 4 ? 4 : g.k_blocks) : kMaxWarps;

@@ -320,16 +320,6 @@ __global__ void __launch_bounds__(kOneThreads, 1) gemv_one_kernel(const __grid_c
     if (lane == 0 && abort_flag) atomicExch(p.status, (int)GOQ_ERR_TIMEOUT);
 }
 
-static int one_sm_count() {
-    int dev = 0, n = 0;
-    static int cached[64];
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (dev >= 0 && dev < 64 && cached[dev]) return cached[dev];
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    if (dev >= 0 && dev < 64) cached[dev] = n;
-    return n;
-}
-
 static constexpr size_t kOneSmemMax = 226 * 1024;   // the opt-in limit is 227 KiB per CTA, static shared variables included
 static size_t one_fixed_smem(const Geometry& g, int m) {
     return 8192 /* alignment slack */ + (size_t)kLutBytes + (size_t)kTileSlots * kNW * 64 * sizeof(float) +
@@ -365,7 +355,7 @@ static cudaError_t launch_one_cfg(const Geometry& g, One& p, int grid, cudaStrea
 
 bool gemv_one_supported(const Geometry& g, int m) {
     return m <= 4 && gemv_seq_supported(g, m) && chain::one_fixed_smem(g, m) + (size_t)2 * chain::kStageRecs * g.unit_bytes <= chain::kOneSmemMax &&
-           (size_t)chain::one_sm_count() * chain::kPostWords * sizeof(uint32_t) <= kWsCounterBytes;
+           (size_t)sm_count() * chain::kPostWords * sizeof(uint32_t) <= kWsCounterBytes;
 }
 
 cudaError_t launch_gemv_one(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws, int spin_limit,
@@ -377,7 +367,7 @@ cudaError_t launch_gemv_one(const Geometry& g, const void* packed, const void* x
     p.status = (int*)ws;
     p.posts = (uint32_t*)((uint8_t*)ws + kWsStatusBytes);
     p.units = (unsigned)g.n_units;
-    const int sms = chain::one_sm_count(), grid = p.units < (unsigned)sms ? (int)p.units : sms;
+    const int sms = sm_count(), grid = p.units < (unsigned)sms ? (int)p.units : sms;
     p.kb_magic = ((1ull << 32) + (unsigned)g.k_blocks - 1) / (unsigned)g.k_blocks;
     p.g_magic = ((1ull << 32) + (unsigned)grid - 1) / (unsigned)grid;
     p.m_magic = ((1ull << 32) + (unsigned)m - 1) / (unsigned)m;

@@ -374,19 +374,6 @@ bool stream_hash_is_bijective() {
     return ok;
 }
 
-static int sm_count() {
-    static int cached[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) dev = 0;
-    if (cached[dev] == 0) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cached[dev] = n > 0 ? n : 148;
-    }
-    return cached[dev];
-}
-
 bool g_stream_pdl = true;  // programmatic dependent launch on the streaming kernel
 int g_stream_grid_per_sm = 0;  // 0: as many CTAs per SM as fit; 1: leave room for the next kernel's CTAs
 

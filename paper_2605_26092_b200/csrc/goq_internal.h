@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include "goq_common.cuh"
+#include "goq_device.h"
 
 namespace goq {
 

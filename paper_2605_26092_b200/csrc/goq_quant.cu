@@ -450,8 +450,7 @@ static cudaError_t launch_ref(const Geometry& g, const float* w, const uint8_t* 
     const size_t smem = quant::RefSmem<NB>::kBytes;
     static SmemAttrCache cache[2];
     if (cudaError_t e = ensure_dynamic_smem(kernel, smem, cache[direct ? 1 : 0])) return e;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 148;
+    const int sms = sm_count();
     // Row chunks per column: every CTA forms its column's G again, so few chunks save work and many fill the chip. Take the
     // split whose waves cost least in float64 tensor clocks (4 per m8n8k4 and SM, a row tile's loads and epilogue about 400). Row
     // tiles go in rounds of 16 warps; a CTA with fewer is bound by one warp's chain of products instead, about four tiles' clocks.

@@ -563,8 +563,7 @@ static cudaError_t launch(const Geometry& g, Params& p, const CUtensorMap& w_map
     static_assert(smem + sizeof(double) * (G + 7 * kRows) + 64 * 8 + 256 <= 227 * 1024, "shared memory");
     static SmemAttrCache cache;
     if (cudaError_t e = ensure_dynamic_smem(solve_ref_tc_kernel<WB, G>, smem, cache)) return e;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 148;
+    const int sms = sm_count();
     // CTAs of a column: the split whose waves cost least, in clocks: forming G (16 per product and scheduler), its exchange and digits, and the
     // tiles of the CTA that has most
     const int cols = g.k_in / G;
