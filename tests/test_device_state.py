@@ -58,6 +58,35 @@ int main() {
 """)
 
 
+def test_shared_memory_limit_never_falls_below_what_is_noted(tmp_path):
+    """A call of 200000 bytes is held up between setting the limit and noting it; one of 100000 on another thread sets it meanwhile, if it is let. Whatever is
+    noted as set then is: a later call of 200000 finds the limit there or sets it again. Per device."""
+    _run(tmp_path, r"""
+static std::atomic<int> limit[2];
+extern "C" cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int v) {
+    if (v == 200000) { limit[device] = v; pause_ms(100); }
+    else { pause_ms(30); limit[device] = v; }
+    return cudaSuccess;
+}
+static void kernel() {}
+int main() {
+    goq::SmemAttrCache cache;
+    std::vector<std::thread> t;
+    for (int i = 0; i < 4; ++i) t.emplace_back([&, i] { device = i >> 1; goq::ensure_dynamic_smem(kernel, (i & 1) ? 100000 : 200000, cache); });
+    for (auto& x : t) x.join();
+    int wrong = 0;
+    for (device = 0; device < 2; ++device) {
+        goq::ensure_dynamic_smem(kernel, 200000, cache);
+        wrong += limit[device] != 200000;
+        goq::ensure_dynamic_smem(kernel, 100000, cache);
+        wrong += limit[device] != 200000;
+    }
+    std::printf("limits %d %d\n", limit[0].load(), limit[1].load());
+    return wrong;
+}
+""")
+
+
 def test_one_place_asks_for_the_number_of_sms():
     """Every launcher plans with goq_device.h's count: no copy with a cache of its own (one was halved in place by whoever came first, some kept the first
     device's number for all)."""
