@@ -316,7 +316,8 @@ int goq_last_cuda_error(void);
 int goq_set_gemv_variant(int variant);
 
 /* Bound, in polls, of every device-side wait of goq_gemv_sequence, of goq_gemv's integer-operand kernel, of the integer layer on the
- * tensor cores and of goq_solve_ref and of goq_gemm's e4m3-operand kernel, and of its mid-batch kernel's waits for a finished accumulator (tests only; 0 restores the kernels' own bounds).
+ * tensor cores, of goq_solve_ref and of goq_gemm's e4m3-operand kernel and its prefill kernel on pairs of SMs, and of its mid-batch kernel's waits for a
+ * finished accumulator (tests only; 0 restores the kernels' own bounds).
  * With a bound of a few polls a dependent chain gives up at once: the call returns GOQ_OK (it only enqueues), the
  * status word then reads GOQ_ERR_TIMEOUT, the context stays usable. Process-wide. Returns the previous value. */
 int goq_set_wait_limit(int polls);

@@ -258,7 +258,7 @@ goq_status goq_gemm(const goq_desc* desc, const void* packed, const void* x, int
         }
         // (up to 32 rows of a narrow group in less scratch than documented: the scalar kernel, slow but of the stated accuracy)
         if (goq::gemm_tc_supported(g) && variant != 2 && !(variant == 0 && exact && narrow))
-            return from_cuda(goq::launch_gemm_tc(g, packed, x, m, y, y_dtype, ws, (cudaStream_t)stream));
+            return from_cuda(goq::launch_gemm_tc(g, packed, x, m, y, y_dtype, ws, g_wait_limit.load(std::memory_order_relaxed), (cudaStream_t)stream));
         if (goq::linear_mma_supported(g))
             return from_cuda(goq::launch_linear_mma(g, packed, x, m, y, y_dtype, (cudaStream_t)stream));
         // what is left of the groups narrower than 32: the scalar kernel, 16 tokens at a time

@@ -42,6 +42,7 @@ struct Params {
     int pairs_x;    // pairs of channel tiles
     int n_full;     // pairs [0, n_full) take whole tiles (2 * half tokens); the rest take the last tiles as token halves
     int half;       // tokens of a half tile (MMA N): a multiple of 32, at most 256
+    int spin;       // polls of a wait
 };
 
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
@@ -72,8 +73,8 @@ __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
 }
 // Wait without suspending: a thread that try_wait has put to sleep is woken late when the phase is completed from the other CTA or by a commit.
 template <int SLEEP>
-__device__ __forceinline__ bool poll(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-    for (int it = 0; it < kSpin; ++it) {
+__device__ __forceinline__ bool poll(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int limit) {
+    for (int it = 0; it < limit; ++it) {
         if (mbar_test(bar, parity)) return true;
         if ((it & 63) == 63 && *abort_flag) return false;
         if constexpr (SLEEP > 0) __nanosleep(SLEEP);
@@ -156,7 +157,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
             bool ok = true;
             int s = 0, round = 0;
             for (int chunk = 0; chunk < n_chunks; ++chunk) {
-                if (round > 0) ok = poll<0>(&empty[s], (round - 1) & 1, &abort_flag);
+                if (round > 0) ok = poll<0>(&empty[s], (round - 1) & 1, &abort_flag, p.spin);
                 if (!ok) break;
                 unsigned char* b = stages + s * kStageBytes + kABytes;
                 if (rank == 0) mbar_expect_tx(&full_b[s], (uint32_t)(n_half * p.half) * 128u);   // both CTAs' bytes
@@ -171,7 +172,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
         const int n_rec = min(kExpanders, max(0, p.n_tiles - T0));
         for (int kb = 0; 2 * kb < n_chunks; ++kb) {
             const int ps = kb & 1;
-            if (kb >= 2 && !__all_sync(0xFFFFFFFFu, mbar_wait(&pk_empty[ps], ((kb >> 1) - 1) & 1, &abort_flag))) break;
+            if (kb >= 2 && !__all_sync(0xFFFFFFFFu, mbar_wait(&pk_empty[ps], ((kb >> 1) - 1) & 1, &abort_flag, p.spin))) break;
             if (lane == 0) mbar_expect_tx(&pk_full[ps], (uint32_t)(n_rec * p.unit_bytes));
             __syncwarp();
             if (lane < n_rec)
@@ -191,7 +192,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
             uint32_t par = 0;
             for (int chunk = 0; chunk < n_chunks; ++chunk) {
                 if (!__all_sync(0xFFFFFFFFu, ready)) {
-                    ok = poll<0>(&full_b[s], par, &abort_flag) && poll<0>(&full_a[s], par, &abort_flag) && poll<0>(&peer_a[s], par, &abort_flag);
+                    ok = poll<0>(&full_b[s], par, &abort_flag, p.spin) && poll<0>(&full_a[s], par, &abort_flag, p.spin) && poll<0>(&peer_a[s], par, &abort_flag, p.spin);
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
                 }
@@ -221,7 +222,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
             int s = 0;
             uint32_t par = 0;
             for (int chunk = 0; chunk < n_chunks; ++chunk) {
-                if (!poll<0>(&full_a[s], par, &abort_flag)) break;
+                if (!poll<0>(&full_a[s], par, &abort_flag, p.spin)) break;
                 arrive_cluster(map_rank(s32(&peer_a[s]), 0));
                 if (++s == kStages) { s = 0; par ^= 1u; }
             }
@@ -238,7 +239,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
         uint32_t par = 1;   // parity of the stage's previous release (the first round passes at once)
         for (int kb = 0; 2 * kb < n_chunks && ok; ++kb) {
             const int ps = kb & 1;
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&pk_full[ps], (kb >> 1) & 1, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&pk_full[ps], (kb >> 1) & 1, &abort_flag, p.spin));
             if (!ok) break;
             const uint32_t unit = after_wait(s32(pk_ring) + ps * pk_bytes + e * p.unit_bytes);
             uint2 wv0 = make_uint2(kZeroWord, kZeroWord), wv1 = wv0;   // its two words of rows g and g + 8
@@ -253,7 +254,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
                     cf[cc][0] = lds32(at); cf[cc][1] = lds32(at + 32);
                 }
             }
-            ok = __all_sync(0xFFFFFFFFu, poll<20>(&empty[s], par, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, poll<20>(&empty[s], par, &abort_flag, p.spin));
             if (!ok) break;
             const uint32_t a_tile = s32(stages + s * kStageBytes);
 #pragma unroll
@@ -280,7 +281,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
         }
         // ---- epilogue: tensor memory -> registers -> shared memory (transposed) -> y ----
         if (n_chunks == 0) ok = false;
-        if (ok) ok = mbar_wait(&tmem_full, 0, &abort_flag);
+        if (ok) ok = mbar_wait(&tmem_full, 0, &abort_flag, p.spin);
         ok = __all_sync(0xFFFFFFFFu, ok);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int set = (warp - kExp0) >> 2, col_half = set & 1;   // four warps: every second 32 tokens of a half
@@ -306,7 +307,7 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
                 // bounded rendezvous of the half's four warps (a named barrier could not give up)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&epi_bar[set]);
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[set], it & 1, &abort_flag));
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(&epi_bar[set], it & 1, &abort_flag, p.spin));
                 if (!ok) break;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -404,9 +405,10 @@ static cudaError_t launch(const Geometry& g, const Params& p0, const void* xh, i
 bool gemm_pair_supported(const Geometry& g, int m) { return m > 256 && g.k_in % 8 == 0 && tc2::smem_for(g) + 2048 <= 227 * 1024; }
 float gemm_pair_us(const Geometry& g, int m) { return 9.f + tc2::token_tiles(g, m).us; }
 cudaError_t launch_gemm_pair(const Geometry& g, const void* packed, const void* xh, const float* inv_scale, const uint32_t* row_scale, const float* row_inv,
-                             int m, void* y, int y_dtype, int* status, cudaStream_t st) {
+                             int m, void* y, int y_dtype, int* status, int spin_limit, cudaStream_t st) {
     tc2::Params p;
     p.packed = (const uint8_t*)packed; p.y = y; p.inv_scale = inv_scale; p.row_scale = row_scale; p.row_inv = row_inv; p.status = status;
+    p.spin = spin_limit > 0 ? spin_limit : tc::kSpin;
     p.unit_bytes = g.unit_bytes; p.meta_off = g.meta_off; p.k_blocks = g.k_blocks; p.n_tiles = g.n_tiles; p.n_out = g.n_out; p.m = m; p.y_dtype = y_dtype;
     int lg = 3;
     while ((1 << lg) < g.group) ++lg;

@@ -594,11 +594,11 @@ static bool takes_pairs(const Geometry& g, int m) { return gemm_pair_supported(g
 template <int WB>
 static cudaError_t launch_wb(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, int* status,
                              float* inv_scale, uint32_t* row_scale, float* row_inv, uint16_t* xh, int* tile_counter, float* partial,
-                             cudaStream_t st) {
+                             int spin_limit, cudaStream_t st) {
     if (g.k_in % 8 != 0) return cudaErrorInvalidValue;
     if (cudaError_t e = launch_pre_pass(x, g.k_in, m, g.n_tiles, xh, inv_scale, packed, g.unit_bytes, g.k_blocks, g.groups_per_block,
                                         row_scale, row_inv, st)) return e;
-    if (takes_pairs(g, m)) return launch_gemm_pair(g, packed, xh, inv_scale, row_scale, row_inv, m, y, y_dtype, status, st);
+    if (takes_pairs(g, m)) return launch_gemm_pair(g, packed, xh, inv_scale, row_scale, row_inv, m, y, y_dtype, status, spin_limit, st);
     CUtensorMap map;
     const TokenTiles tt = token_tiles(g, m);
     if (cudaError_t e = encode_x_map(&map, xh, g.k_in, m, tt.half)) return e;
@@ -674,7 +674,7 @@ TcScratch tc_scratch(const Geometry& g, int m) {
 float gemm_tc_us(const Geometry& g, int m) { return tc::takes_pairs(g, m) ? gemm_pair_us(g, m) : 9.f + tc::token_tiles(g, m).us; }
 size_t gemm_tc_workspace(const Geometry& g, int m) { return tc_scratch(g, m).total; }
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, void* ws,
-                           cudaStream_t st) {
+                           int spin_limit, cudaStream_t st) {
     int* status = (int*)ws;
     const TcScratch t = tc_scratch(g, m);
     uint8_t* b = (uint8_t*)ws;
@@ -684,8 +684,8 @@ cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x,
     uint16_t* xh = (uint16_t*)(b + t.xh_off);
     int* counters = (int*)(b + kWsStatusBytes);   // at most sm_count / 2 tiles when the split is on
     float* partial = (float*)(b + t.partial_off);
-    if (g.wbits == 4) return tc::launch_wb<4>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, st);
-    return g.wbits == 3 ? tc::launch_wb<3>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, st)
-                        : tc::launch_wb<2>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, st);
+    if (g.wbits == 4) return tc::launch_wb<4>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, spin_limit, st);
+    return g.wbits == 3 ? tc::launch_wb<3>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, spin_limit, st)
+                        : tc::launch_wb<2>(g, packed, x, m, y, y_dtype, status, inv_scale, rs, ri, xh, counters, partial, spin_limit, st);
 }
 }  // namespace goq

@@ -75,13 +75,13 @@ bool gemm_tc_supported(const Geometry& g);
 size_t gemm_tc_workspace(const Geometry& g, int m);
 float gemm_tc_us(const Geometry& g, int m);   // estimated time, more than 256 tokens
 cudaError_t launch_gemm_tc(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype,
-                           void* ws, cudaStream_t st);
+                           void* ws, int spin_limit, cudaStream_t st);
 
 // Its main kernel on pairs of SMs, more than 256 tokens (goq_gemm_pair.cu): xh, inv_scale, row_scale, row_inv as the pre-pass leaves them.
 bool gemm_pair_supported(const Geometry& g, int m);
 float gemm_pair_us(const Geometry& g, int m);   // estimated time, pre-pass included
 cudaError_t launch_gemm_pair(const Geometry& g, const void* packed, const void* xh, const float* inv_scale, const uint32_t* row_scale, const float* row_inv,
-                             int m, void* y, int y_dtype, int* status, cudaStream_t st);
+                             int m, void* y, int y_dtype, int* status, int spin_limit, cudaStream_t st);
 
 // The same layer for a few to a few hundred tokens (goq_gemm_mid.cu), any group, wbits 2..4. exact: the two bases as separate
 // operands without rounding (fp32 accuracy), else w_hat rounded once to fp16. `ws` holds gemm_mid_workspace bytes.

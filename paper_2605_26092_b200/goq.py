@@ -202,8 +202,8 @@ def set_gemv_variant(variant: int) -> int:
 
 
 def set_wait_limit(polls: int) -> int:
-    """goq_set_wait_limit: bound of the device-side waits of the decode chain, the integer-operand decode kernel, the integer layer and
-    (accumulator waits) the mid-batch kernel (tests only; 0 = the kernels' own)."""
+    """goq_set_wait_limit: bound of the device-side waits of the decode chain, the integer-operand decode kernel, the integer layer, the REF solve, the
+    e4m3-operand kernel, the prefill kernel on pairs of SMs and (accumulator waits) the mid-batch kernel (tests only; 0 = the kernels' own)."""
     return lib().goq_set_wait_limit(polls)
 
 

@@ -431,6 +431,36 @@ def test_prefill_gemm_on_pairs_of_sms_edges(goq, n, k, g, b, m):
     check_parity(out[0].cpu().numpy().astype(np.float64)[:, rows], y_ref, 5e-4, 2e-3)
 
 
+@pytest.mark.parametrize("n,k,g,b,m", [(4000, 2048, 128, 3, 600), (300, 128, 64, 4, 300)])   # many chunks; as many as there are stages or fewer
+def test_prefill_gemm_on_pairs_of_sms_reports_a_wait_that_runs_out(goq, n, k, g, b, m):
+    """With one poll a wait either CTA of a pair gives up by itself and both end: the status word reads GOQ_ERR_TIMEOUT, and on a fresh scratch buffer the next
+    call is right again."""
+    from tests.gpu_util import dev, pack_weights
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k)
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    x = dev(si.bf16_activations(m, k, seed=m))
+    ws = goq.new_workspace(d, goq.OP_GEMM, m)
+
+    def call():
+        y = torch.zeros((m, n), dtype=torch.float32, device="cuda")
+        goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+        return y, goq.workspace_status(ws)
+    prev = goq.set_gemv_variant(3)
+    try:
+        good, status = call()
+        assert status == goq.OK
+        goq.set_wait_limit(1)
+        assert call()[1] == goq.ERR_TIMEOUT
+        goq.set_wait_limit(0)
+        goq.workspace_init(ws)
+        again, status = call()
+        assert status == goq.OK and torch.equal(good, again)
+    finally:
+        goq.set_wait_limit(0)
+        goq.set_gemv_variant(prev)
+
+
 @pytest.mark.parametrize("variant,n,k,g,b,m", [
     (3, 1, 8, 8, 3, 257), (3, 130, 256, 64, 2, 513), (3, 33, 136, 8, 3, 600), (3, 384, 384, 32, 4, 1025), (3, 9600, 128, 128, 3, 1024),
     (3, 9500, 64, 64, 3, 1030), (4, 20000, 256, 128, 3, 300), (4, 5000, 128, 32, 4, 1025), (0, 4100, 256, 64, 3, 700)])
