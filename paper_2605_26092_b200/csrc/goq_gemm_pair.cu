@@ -11,8 +11,8 @@
 // "stage is free" comes back to both by one multicast commit. Four stages of 48 KB (A 16, B 32) hold more than these hops.
 // Bound: MMA rate at the clock the power limit leaves, and for few tokens the round of expanders and hops (~1 us a k-block). Measured, W3 g128, us, pre-pass
 // included, goq_gemm_tc.cu -> this: 4096 x 4096 at 512 / 1024 / 2048 tokens 53 / 59 / 70 -> 50 / 56 / 60; 11008 x 4096 at 1024 / 2048 116 / 188 -> 95 / 158;
-// 4096 x 11008 at 2048 193 -> 154 to 164; 8192 x 8192 at 2048 274 -> 211 to 239; 28672 x 8192 at 512 258 -> 198. What it took: the passed-on arrival without a
-// cluster-scope release (with one, 78 us for the first at 2048; eight warps arriving across, 95), a warp that issues as one (from one lane's registers eight
+// 4096 x 11008 at 2048 193 -> 154 to 164; 8192 x 8192 at 2048 274 -> 211 to 239; 28672 x 8192 at 512 258 -> 198. What it took: one thread's arrival across with a
+// release restricted to shared memory (arrive_cluster; eight warps arriving across 95 us for the first at 2048), a warp that issues as one (from one lane's registers eight
 // MMAs took 830 clocks: 61 at 1024 tokens, now 56), sixteen expander warps, and a warp of its own for the records.
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag (its partner's waits run out too), skips the remaining work, waits for what it has
 // in flight, frees its tensor memory and records GOQ_ERR_TIMEOUT in the status word.
@@ -68,14 +68,26 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
+// What crosses from CTA to CTA by generic writes is a weight tile: written and fenced for the tensor cores by its expanders, whose arrivals one thread of their CTA
+// waits for; that thread's release of cluster scope and the issuing warp's acquire order the tile before the MMA. The fences are restricted to shared memory: a
+// release that orders every kind of memory took 0.7 us a chunk (4096 x 4096 at 2048 tokens 58 -> 72 us, by two such threads in turn 62; restricted 58).
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;\n\tmbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void acquire_cluster() { asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory"); }
+// mbar_test of a phase that the other CTA completes; acquire_cluster() behind it
+__device__ __forceinline__ bool test_cluster(uint64_t* b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(s32(b)), "r"(parity) : "memory");
+    return ok != 0;
 }
 // Wait without suspending: a thread that try_wait has put to sleep is woken late when the phase is completed from the other CTA or by a commit.
-template <int SLEEP>
+template <int SLEEP, bool PEER = false>
 __device__ __forceinline__ bool poll(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int limit) {
     for (int it = 0; it < limit; ++it) {
-        if (mbar_test(bar, parity)) return true;
+        if (PEER ? test_cluster(bar, parity) : mbar_test(bar, parity)) return true;
         if ((it & 63) == 63 && *abort_flag) return false;
         if constexpr (SLEEP > 0) __nanosleep(SLEEP);
     }
@@ -192,14 +204,15 @@ gemm_pair_kernel(const Params p, const __grid_constant__ CUtensorMap x_map) {
             uint32_t par = 0;
             for (int chunk = 0; chunk < n_chunks; ++chunk) {
                 if (!__all_sync(0xFFFFFFFFu, ready)) {
-                    ok = poll<0>(&full_b[s], par, &abort_flag, p.spin) && poll<0>(&full_a[s], par, &abort_flag, p.spin) && poll<0>(&peer_a[s], par, &abort_flag, p.spin);
+                    ok = poll<0>(&full_b[s], par, &abort_flag, p.spin) && poll<0>(&full_a[s], par, &abort_flag, p.spin) && poll<0, true>(&peer_a[s], par, &abort_flag, p.spin);
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
                 }
+                acquire_cluster();
                 const int next = s + 1 == kStages ? 0 : s + 1;
                 const uint32_t par_next = next == 0 ? par ^ 1u : par;
                 {
-                    const bool rb = mbar_test(&full_b[next], par_next), ra = mbar_test(&full_a[next], par_next), rp = mbar_test(&peer_a[next], par_next);
+                    const bool rb = mbar_test(&full_b[next], par_next), ra = mbar_test(&full_a[next], par_next), rp = test_cluster(&peer_a[next], par_next);
                     ready = rb && ra && rp;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

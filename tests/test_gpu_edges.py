@@ -431,6 +431,34 @@ def test_prefill_gemm_on_pairs_of_sms_edges(goq, n, k, g, b, m):
     check_parity(out[0].cpu().numpy().astype(np.float64)[:, rows], y_ref, 5e-4, 2e-3)
 
 
+def test_prefill_gemm_on_pairs_of_sms_reads_no_tile_of_the_call_before(goq):
+    """Every pair busy, two sets of weights and activations in turn on one scratch buffer: a weight tile that an MMA read before the other CTA's part of it was in
+    place would carry the other call's weights. Every call repeats its first result bit for bit."""
+    from tests.gpu_util import check_parity, dev, pack_weights
+    n, k, g, b, m = 4096, 2048, 128, 3, 1536
+    calls, rows = [], si.sample_rows(n, 100, seed=2)
+    for seed in (1, 2):
+        codes, meta, coef = si.random_quantized(n, k, g, b, seed=seed)
+        d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+        xb = si.bf16_activations(m, k, seed=seed)
+        calls.append((d, packed, dev(xb), O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b, rows=rows)))
+    ws = goq.new_workspace(calls[0][0], goq.OP_GEMM, m)
+    prev = goq.set_gemv_variant(3)
+    try:
+        out = [torch.zeros((m, n), dtype=torch.float32, device="cuda") for _ in range(24)]
+        for i, y in enumerate(out):
+            d, packed, x, _ = calls[i % 2]
+            goq.gemm(d, packed, x, m, goq.BF16, y=y, y_dtype=goq.F32, ws=ws)
+        torch.cuda.synchronize()
+    finally:
+        goq.set_gemv_variant(prev)
+    assert goq.workspace_status(ws) == goq.OK
+    for i, y in enumerate(out):
+        assert torch.equal(y, out[i % 2]), i
+    for i in range(2):
+        check_parity(out[i].cpu().numpy().astype(np.float64)[:, rows], calls[i][3], 5e-4, 2e-3)
+
+
 @pytest.mark.parametrize("n,k,g,b,m", [(4000, 2048, 128, 3, 600), (300, 128, 64, 4, 300)])   # many chunks; as many as there are stages or fewer
 def test_prefill_gemm_on_pairs_of_sms_reports_a_wait_that_runs_out(goq, n, k, g, b, m):
     """With one poll a wait either CTA of a pair gives up by itself and both end: the status word reads GOQ_ERR_TIMEOUT, and on a fresh scratch buffer the next
