@@ -19,7 +19,8 @@
 // operand goes straight to tensor memory (tcgen05.st 16x256b: its element map is the packed words' ownership), so that shared memory serves
 // only the packed records, the record table and the activations. Tensor memory: four operand stages of 64 columns, and a ring of group sums
 // (2 x tokens columns a basis) in the other half.
-// Bound: the chain of waits between decode, MMA and read-back; no pipe is above 40 % (profiles/gemm_f8_8192x8192_m8.md).
+// Bound: the chain of waits between decode, MMA and read-back; no pipe is above 41 % (integer 41, 39 and 35 % at 16, 32 and 64 rows, tensor
+// 11, 21 and 34 %, issue 55 to 60 %).
 // Measured, W3 g128, us, goq_gemm otherwise (mid-batch kernel or decode launches) -> this: 28672 x 8192 at 24 / 32 tokens 97 / 98 -> 71 / 77; 8192 x 8192 36 / 37 -> 28 / 30.5;
 // 4096 x 4096 16 / 17 -> 15.3 / 16.1; 2048 x 4096 at 64 18.4 -> 16.0; W4 28672 x 8192 at 32 tokens 98 -> 83. As goq_gemv (gemv_mma_kernel otherwise): 28672 x 8192 at 8 / 16
 // tokens 66 / 83 -> 55 / 60, W4 at 1 to 8 tokens 81 -> 59. A unit takes 0.46 us with 16 rows, 0.54 with 32, 0.70 with 64. Normwise error 5.1e-8 to 1.0e-7, no larger than the
@@ -94,11 +95,6 @@ __device__ __forceinline__ uint32_t lds32v(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
-}
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
 }
 // (a0, a1) = (b0, b1) * (c0, c1) + (d0, d1)
 __device__ __forceinline__ void fma2(float& a0, float& a1, float b0, float b1, float c, float d0, float d1) {

@@ -102,11 +102,6 @@ __device__ __forceinline__ uint32_t coef_max_of(const uint8_t* src, int first, i
 
 __device__ __forceinline__ __half2 u2h(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 __device__ __forceinline__ uint32_t h2u(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
-}
 
 // GL: log2 of the group size where it is known at compile time (7: one coefficient pair per row and record), else 0
 template <int WB, bool TWO, int GL>
