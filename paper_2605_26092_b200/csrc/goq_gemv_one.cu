@@ -3,8 +3,9 @@
 //
 // A single linear of 8-24 MB is 2-8 us of work, so what surrounds it counts: a cooperative launch cannot overlap the kernel before
 // it, and its 17 KB of parameters for up to 256 linears are copied on every call. This kernel takes 150 bytes of parameters and is a
-// programmatic dependent of the kernel before it: the ring of packed records fills, tables and barriers are set up while
-// that one still runs; activations, outputs and scratch are touched after griddepcontrol.wait.
+// programmatic dependent of the kernel before it: on an SM that has room, the ring of packed records fills, tables and barriers are set up while
+// that one still runs; activations, outputs and scratch are touched after griddepcontrol.wait. (Behind a call of its own kind a CTA, 576 threads of 88
+// registers, finds room only where that call's CTA has ended.)
 //
 // Tiles shared by several CTAs: every CTA but the one that holds the tile's end posts its part (at most one per CTA) in the
 // zero-kept counter area, a word a value: zero means "not there yet" and a sum of +0 is posted as -0. The finisher polls the words it

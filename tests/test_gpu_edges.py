@@ -277,9 +277,10 @@ def test_mid_batch_gemm_reports_a_wait_that_runs_out(goq, n, k, g, b, m):
     (1, 32, 32, 3, 1), (129, 160, 32, 4, 33), (127, 256, 64, 2, 48), (128, 128, 128, 3, 16), (4000, 384, 128, 3, 17), (300, 640, 128, 4, 64),
     (1000, 4096, 32, 3, 65), (130, 8192, 128, 2, 40), (2400, 256, 64, 3, 128), (19200, 128, 128, 3, 24), (257, 1152, 64, 4, 129), (1100, 2304, 128, 3, 200)])
 def test_e4m3_operand_gemm_edges(goq, n, k, g, b, m):
-    """Both bases and two slices of the activations as e4m3 numbers: channel and token tiles that do not fill, every bit width and number of macro-blocks a
+    """Both bases and the activations as e4m3 numbers: channel and token tiles that do not fill, every bit width and number of macro-blocks a
     k-block, one unit in all, one tile shared by many SMs, tiles an SM has whole; tokens of tiny and huge magnitude, of zeros, and with one element 2^14
-    times the others (exact: 2^-15). Twice, bit for bit, two calls back to back. Bounds as for every fp32-accumulating kernel."""
+    times the others (what such an element leaves of the others: the next test but one). Twice, bit for bit, two calls back to back. Bounds as for every
+    fp32-accumulating kernel."""
     from tests.gpu_util import check_parity, dev, pack_weights
     codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
     d, packed = pack_weights(n, k, g, b, codes, meta, coef)
@@ -368,6 +369,28 @@ def test_small_elements_beside_a_large_one_and_non_finite_ones_in_e4m3_operands(
             assert np.array_equal(np.isnan(y[tok]), np.isnan(y_ref[tok])) and np.array_equal(np.isposinf(y[tok]), np.isposinf(y_ref[tok]))
             assert np.array_equal(np.isneginf(y[tok]), np.isneginf(y_ref[tok]))
         assert np.array_equal(all_y[len(powers):m - 2], base[len(powers):m - 2])
+
+
+@pytest.mark.parametrize("variant,n,k,g,b,m", [(0, 144, 512, 64, 3, 200), (4, 300, 640, 16, 4, 70), (3, 260, 512, 128, 3, 400), (3, 130, 256, 8, 2, 300)])
+def test_small_elements_beside_a_large_one_in_fp16_operands(goq, variant, n, k, g, b, m):
+    """The kernels with an fp16 copy of the activations: one element of a token 2^13 .. 2^24 times the others, channels whose states are zero there, held to
+    their own magnitude. fp16 holds 2^-28 of a token's largest element with bf16's eight bits; w_hat rounded once: 5e-4."""
+    from tests.gpu_util import check_parity, pack_weights, run_gemm_bf16
+    codes, meta, coef = si.random_quantized(n, k, g, b, seed=n + k + m)
+    at, blind = k // 2 + 3, np.arange(0, n, 3)
+    mb = at // 8 * 8
+    codes[blind, mb:mb + 8] = (1 << (b - 1)) - 1
+    d, packed = pack_weights(n, k, g, b, codes, meta, coef)
+    x = si.bf16_bits_to_f64(si.bf16_activations(m, k, seed=m))
+    powers = (13, 16, 20, 24)
+    for tok, e in enumerate(powers):
+        x[tok, at] = 1.5 * 2.0 ** e
+    xb = si.f32_to_bf16_bits(x.astype(np.float32))
+    y_ref = O.linear_f64(codes, meta, coef, si.bf16_bits_to_f64(xb), g, b)
+    y = run_gemm_bf16(d, packed, xb, variant=variant)
+    for tok, e in enumerate(powers):
+        check_parity(y[tok, blind], y_ref[tok, blind], 5e-4, 2e-3, "2^%d" % e)
+    check_parity(y, y_ref, 5e-4, 2e-3)
 
 
 def test_e4m3_operand_gemm_reports_a_wait_that_runs_out(goq):
