@@ -129,7 +129,7 @@ goq_status goq_unpack(const goq_desc* desc, const void* packed, uint8_t* codes_b
  * Each PoT term is applied to the activation as an exponent shift (a bf16 operand of the tensor core);
  * sums are fp32. Large linears (W2, W3) at up to 4 tokens take goq_gemv_sequence's arithmetic
  * (integer operands: same rounding and saturation of non-finite activations as stated there); above that (W4: at any
- * batch) those whose ws is of the documented size take goq_gemm's e4m3 operands: products exact there too, sums fp32.
+ * batch) those whose ws is of the documented size take goq_gemm's e4m3 operands, as stated there: fp32 accuracy too.
  * Stream order: the kernels start fetching `packed` before earlier work on the stream has
  * finished (programmatic dependent launch), so the packed weights must not be written by work that
  * is still in flight on the stream when the call is issued (synchronise after goq_pack, or put
@@ -141,8 +141,9 @@ goq_status goq_gemv(const goq_desc* desc, const void* packed, const void* x_bf16
  *  x_dtype GOQ_BF16: x [m][k_in] bf16; y out [m][n_out] (GOQ_BF16 or GOQ_F32); sx, cq, sc, acc unused (NULL).
  *      ws: goq_workspace_bytes(desc, GOQ_OP_GEMM, m) bytes, 256-byte aligned, initialised once with
  *      goq_workspace_init. Up to 32 rows results carry fp32 accuracy, whatever the group. Many calls of up to about 128 rows, groups
- *      of 32 and more, do too: PoT states as e4m3 numbers, x as e4m3 slices in ws that hold its elements exactly (rows that they do not hold, with elements below
- *      2^-29 of the row's largest, infinities or NaN, are computed from x itself, more slowly). The other kernels for more than a few rows keep an fp16 copy of x (each row scaled by a power of two, undone in the output) in ws, so the size grows with m * k_in;
+ *      of 32 and more, do too: PoT states as e4m3 numbers, x as e4m3 slices in ws that hold its elements exactly down to
+ *      2^-29 of the row's largest and are off by at most 2^-37 of it below (rows where those are more than one in 1024 of the elements above 2^-14, or that
+ *      have infinities or NaN, are computed from x itself, more slowly). The other kernels for more than a few rows keep an fp16 copy of x (each row scaled by a power of two, undone in the output) in ws, so the size grows with m * k_in;
  *      from 33 rows on those round c1*b1 + c2*b2 once to fp16 (normwise output error about 1.5e-4 to 2.5e-4). The coefficients of every output channel are scaled by a
  *      power of two taken from the channel's largest |c1|, |c2| before that rounding and the output is scaled back, so
  *      the result does not depend on the magnitude of the weights; inside one channel, coefficients more than 2^13

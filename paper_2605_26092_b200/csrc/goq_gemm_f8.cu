@@ -6,9 +6,10 @@
 // (b1: a table lookup per four weights; b2: the same bytes routed by the exchange record, sign bits flipped), with no coefficient in the inner
 // loop. The activations are two e4m3 slices, hi + 2^-5 lo, of four significant bits each, which hold a bf16 number exactly if it is at least 2^-14 of its
 // token's largest magnitude (every token is scaled by a power of two). What is smaller goes, times 2^15, into two slices of its own, as if it were another
-// token; a macro-block's two sums are added as they are read back, and the coefficients multiply them in fp32. Exact down to 2^-29 of the largest. A token
-// with anything below that, or with an infinity or a NaN, is marked by the pre-pass, and its outputs are computed from the bf16 elements themselves by the
-// summing kernel. So products are exact whatever the activations, and sums are fp32. (With one pair of slices an element 2^13 times the others left errors of
+// token; a macro-block's two sums are added as they are read back, and the coefficients multiply them in fp32. Exact down to 2^-29 of the largest, and below
+// that off by at most 2^-37 of it: for a few elements of an ordinary token (0.5 to 0.9 % of the tokens that silu(gate) up makes have one) that is nothing to
+// any sum. A token with more of them, or with an infinity or a NaN, is marked by the pre-pass, and its outputs are computed from the bf16 elements themselves
+// by the summing kernel (goq_gemm_f8_finish.cu). (With one pair of slices an element 2^13 times the others left errors of
 // 8e-4 in the channels whose code is zero there.) The fp16 form (w_hat = c1 b1 + c2 b2 rounded once, goq_gemm_mid.cu) has 19 operations on the integer pipe
 // and 8 on the other per 8 weights; this has 13, and no rounding of the weights.
 //
@@ -407,7 +408,9 @@ __global__ void __launch_bounds__(Roles<NB8>::kThreads, 1) gemm_f8_kernel(const 
 
 // ---- activation pre-pass: bf16 -> e4m3 slices, one CTA per token ------------------------------------
 // v = x 2^s with the token's largest magnitude in [2^7, 2^8). Its first row holds the elements of 2^-7 and more (hi = e4m3(v), lo = e4m3((v - hi) 2^5): exact),
-// its second one, four rows on, the others, times 2^15; zeros past k_in. A token with an element that these do not give back, an infinity and a NaN among them, is marked.
+// its second one, four rows on, the others, times 2^15; zeros past k_in. What these do not give back is below 2^-22 and off by at most 2^-30. Where at most one
+// element in 1024 of the first row's number is such a one, the error is below 2^-28 of what a channel sees of the first row (2^-30 / 2^-7 / sqrt(1024) at the
+// worst, under fp32's own roundings). Else, and with an infinity or a NaN, the token is marked.
 constexpr int kPrepThreads = 256;
 constexpr int kPrepHold = 6;   // 16-byte vectors a thread keeps: rows up to 12288
 __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {   // a in the low byte
@@ -431,6 +434,7 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
     uint8_t *hi_out = x8 + (size_t)first_row * k_pad, *lo_out = x8 + (size_t)(rows_of(m) + first_row) * k_pad;
     const int n_vec = k_in / 8, n_pad = k_pad / 8;
     __shared__ uint32_t warp_max[kPrepThreads / 32];
+    __shared__ int2 warp_count[kPrepThreads / 32];
     uint32_t amax = 0;
     auto largest = [&](const uint4& v) {
         const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
@@ -455,7 +459,7 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
     int sfield = 261 - (int)(amax >> 7);   // exponent field of 2^s
     sfield = sfield < 1 ? 1 : (sfield > 253 ? 253 : sfield);
     const float mult = __uint_as_float((uint32_t)sfield << 23);
-    bool lost = false;
+    int lost = 0, large = 0;   // elements that the slices do not hold; elements of the first row
     auto convert = [&](int i, const uint4& v) {
         const uint32_t in32[4] = {v.x, v.y, v.z, v.w};
         uint32_t hi[2][2] = {{0u, 0u}, {0u, 0u}}, lo[2][2] = {{0u, 0u}, {0u, 0u}};
@@ -463,6 +467,7 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
         for (int j = 0; j < 4; ++j) {
             const float a = __uint_as_float(in32[j] << 16) * mult, b = __uint_as_float(in32[j] & 0xFFFF0000u) * mult;
             const bool big_a = !(fabsf(a) < 0.0078125f), big_b = !(fabsf(b) < 0.0078125f);
+            large += (int)big_a + (int)big_b;
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 const float pa = big_a == (part == 0) ? (part ? a * 32768.f : a) : 0.f, pb = big_b == (part == 0) ? (part ? b * 32768.f : b) : 0.f;
@@ -471,7 +476,7 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
                 const float ra = pa - back.x, rb = pb - back.y;   // exact
                 const uint32_t l = e4m3x2(ra * 32.f, rb * 32.f);
                 const float2 rest = from_e4m3x2(l);
-                lost = lost || !(rest.x == ra * 32.f) || !(rest.y == rb * 32.f);   // (the conversions saturate; inf - inf and NaN equal nothing)
+                lost += (int)!(rest.x == ra * 32.f) + (int)!(rest.y == rb * 32.f);
                 hi[part][j >> 1] |= h << (16 * (j & 1));
                 lo[part][j >> 1] |= l << (16 * (j & 1));
             }
@@ -486,88 +491,16 @@ __global__ void __launch_bounds__(kPrepThreads) x_to_f8_kernel(const uint16_t* _
     for (int h = 0; h < kPrepHold; ++h)
         if (tid + h * kPrepThreads < n_pad) convert(tid + h * kPrepThreads, held[h]);
     for (int i = tid + kPrepHold * kPrepThreads; i < n_pad; i += kPrepThreads) convert(i, i < n_vec ? __ldg(&row[i]) : make_uint4(0u, 0u, 0u, 0u));
-    lost = __syncthreads_or(lost) != 0;
+    lost = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)lost);
+    large = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)large);
+    if ((tid & 31) == 0) warp_count[tid >> 5] = make_int2(lost, large);
+    __syncthreads();
     if (tid == 0) {
+        int2 n = make_int2(0, 0);
+        for (int w = 0; w < kPrepThreads / 32; ++w) { n.x += warp_count[w].x; n.y += warp_count[w].y; }
         inv_scale[tok] = __uint_as_float((uint32_t)(254 - sfield) << 23);
-        inexact[tok] = lost;
+        inexact[tok] = amax >= 0x7F80u || n.x > n.y / 1024;
     }
-}
-
-// ---- sums of shared tiles, and the marked tokens ------------------------------------------------
-struct ExactParams {
-    const uint8_t* packed;
-    const uint16_t* x;
-    const int* inexact;
-    int unit_bytes, meta_off, k_in, n_tiles, groups_per_block;
-};
-template <int WB>
-__device__ __forceinline__ float pot_value(uint32_t code) {   // zero times an infinity is to be NaN: a value, not a skipped term
-    constexpr uint32_t emax = (1u << (WB - 1)) - 1u;
-    const uint32_t e = code & emax, sign = (code >> (WB - 1)) & 1u;
-    return code == emax ? 0.f : __uint_as_float(((127u - e) << 23) | (sign << 31));
-}
-// A warp: 16 channels of one token by fp32 multiply-adds (Eq. 4 as it stands). Lane (g, t) owns whole micro-blocks of rows g and g + 8. About a microsecond a
-// k-block; only for marked tokens.
-template <int WB>
-__device__ __noinline__ void exact_outputs(const FinishParams& p, const ExactParams& e, int T, int tok) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    constexpr uint32_t kMask = WB <= 3 ? 0x77777777u : 0xFFFFFFFFu;
-    const int chunks = 4 / e.groups_per_block;   // 32-wide ones of a macro-block
-    float acc[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f}, s2[2] = {0.f, 0.f};
-    for (int bk = 0; bk < p.k_blocks; ++bk) {
-        const uint8_t* unit = e.packed + unit_offset(T, bk, p.k_blocks, e.unit_bytes);
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-            const int k0 = bk * kBlockK + c * 32 + t * 8;
-            const uint4 xv = k0 < e.k_in ? __ldg(reinterpret_cast<const uint4*>(e.x + (size_t)tok * e.k_in + k0)) : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t xr[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int at = v * 128 + lane * 4 + c;
-                const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(unit) + at);
-                const uint32_t record = WB <= 3 ? gather_meta(w) : (uint32_t)(__ldg(unit + e.meta_off + at) & 63u);
-                const uint32_t b1 = w & kMask, b2 = xor_permute_nibbles(b1, (int)(record & 3u) + 1), flips = flip_mask(record);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float xi = __uint_as_float((i & 1) ? (xr[i >> 1] & 0xFFFF0000u) : (xr[i >> 1] << 16));
-                    s1[v] = fmaf(xi, pot_value<WB>((b1 >> (4 * i)) & 15u), s1[v]);
-                    const float q = pot_value<WB>((b2 >> (4 * i)) & 15u);
-                    s2[v] = fmaf(xi, ((flips >> i) & 1u) ? -q : q, s2[v]);
-                }
-            }
-            if ((c + 1) % chunks == 0) {
-#pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    const uint32_t pair = __ldg(reinterpret_cast<const uint32_t*>(unit + kCodeBytesPerUnit) + (c / chunks) * kTileRows + v * 8 + g);
-                    const float2 cf = __half22float2(*reinterpret_cast<const __half2*>(&pair));
-                    acc[v] += cf.x * s1[v] + cf.y * s2[v];
-                    s1[v] = s2[v] = 0.f;
-                }
-            }
-        }
-    }
-    const Output out = {p.y, p.y_dtype, p.n_out};
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        float a = acc[v];
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, 1);
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, 2);
-        const int ch = T * kTileRows + v * 8 + g;
-        if (t == 0 && ch < p.n_out) out.store1(tok, ch, a);
-    }
-}
-template <int WB>
-__global__ void __launch_bounds__(kFinishThreads) finish_f8_kernel(const __grid_constant__ FinishParams p, const __grid_constant__ ExactParams e) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int tile = blockIdx.x, tok0 = (tile / p.tiles_x) * p.n_cols + blockIdx.y * kFinishTokens;
-    const int n = min(min(kFinishTokens, p.n_cols - (int)blockIdx.y * kFinishTokens), p.m - tok0);
-    uint32_t marked = 0u;
-    finish_tile(p, [&] { marked = __ballot_sync(0xFFFFFFFFu, (int)(threadIdx.x & 31) < n && __ldcg(e.inexact + tok0 + (threadIdx.x & 31)) != 0); });
-    if (marked == 0u) return;
-    __syncthreads();   // over what was stored above
-    const int T = (tile % p.tiles_x) * (kTileN / kTileRows) + (int)(threadIdx.x >> 5);
-    if (T >= e.n_tiles) return;
-    for (; marked; marked &= marked - 1u) exact_outputs<WB>(p, e, T, tok0 + __ffs((int)marked) - 1);
 }
 
 // ---- host side ------------------------------------------------------------------------------------
@@ -630,12 +563,7 @@ static cudaError_t launch(const Geometry& g, const Plan& pl, const void* packed,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_f8_kernel<WB, GPB, NB8>, p, map, pmap)) return e;
-    const FinishParams f = {p.partial, p.inv_scale, y, y_dtype, g.n_out, m, pl.tokens / 2, pl.tiles_x, g.k_blocks, pl.units, pl.grid};
-    const ExactParams e = {(const uint8_t*)packed, (const uint16_t*)x, (const int*)(ws + pl.mark_off), g.unit_bytes, g.meta_off, g.k_in, g.n_tiles, g.groups_per_block};
-    cfg.gridDim = dim3(pl.tiles_x * pl.t_tiles, (pl.tokens / 2 + kFinishTokens - 1) / kFinishTokens);
-    cfg.blockDim = dim3(kFinishThreads);
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, finish_f8_kernel<WB>, f, e);
+    return launch_f8_finish(g, packed, x, m, y, y_dtype, p.partial, p.inv_scale, (const int*)(ws + pl.mark_off), pl.tokens / 2, pl.tiles_x, pl.t_tiles, pl.units, pl.grid, st);
 }
 template <int WB, int GPB>
 static cudaError_t launch_tokens(const Geometry& g, const Plan& pl, const void* packed, const void* x, int m, void* y, int y_dtype, uint8_t* ws, int spin_limit, cudaStream_t st) {

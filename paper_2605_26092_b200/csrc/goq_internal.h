@@ -100,6 +100,10 @@ size_t gemm_f8_workspace(const Geometry& g, int m);
 size_t gemm_f8_workspace_upto(const Geometry& g, int m);
 cudaError_t launch_gemm_f8(const Geometry& g, const void* packed, const void* x_bf16, int m, void* y, int y_dtype, void* ws, int spin_limit, cudaStream_t st);
 
+// ... its summing kernel, which also computes the tokens of which the pre-pass has left a mark (goq_gemm_f8_finish.cu). tile_tokens: of a token tile
+cudaError_t launch_f8_finish(const Geometry& g, const void* packed, const void* x, int m, void* y, int y_dtype, const float* partial, const float* inv_scale,
+                             const int* marks, int tile_tokens, int tiles_x, int t_tiles, int units, int n_ctas, cudaStream_t st);
+
 // Integer-activation layer.
 // amax (optional, with y): per-token largest |y|, combined into the array with an integer max (zero it before the launch); NaN after a
 // give-up. spin_limit > 0 replaces the bound of every device-side wait (tests).

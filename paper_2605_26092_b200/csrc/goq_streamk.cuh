@@ -70,7 +70,8 @@ struct FinishParams {
 };
 constexpr int kFinishThreads = 256, kFinishTokens = 16;   // of a CTA: 16 tokens of a tile, two tokens x four channels a thread
 
-// grid: (channel tiles x token tiles, token slices). Bound by the parts' way through L2. `after_wait`: called once the kernels before are complete.
+// grid: (channel tiles x token tiles, token slices). Bound by the parts' way through L2. `after_wait`: called once the kernels before are complete;
+// gives the slice's tokens whose sums are not wanted, a bit each.
 template <class F>
 __device__ __forceinline__ void finish_tile(const FinishParams& p, F&& after_wait) {
     const int tile = blockIdx.x, ch = (threadIdx.x & 31) * 4;
@@ -88,7 +89,7 @@ __device__ __forceinline__ void finish_tile(const FinishParams& p, F&& after_wai
     // Every CTA waits, also one that finds nothing to add: what follows on the stream is ordered behind this grid alone, and a grid of
     // CTAs that return at once would be complete while the kernel before it still runs.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    after_wait();
+    const uint32_t skip = after_wait();
     if (c_lo == c_hi || col >= cols) return;   // one CTA had the whole tile and has stored it; no such token
     float4 f0 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col * kTileN));
     float4 f1 = __ldcg(reinterpret_cast<const float4*>(lo + (size_t)col2 * kTileN));
@@ -102,12 +103,13 @@ __device__ __forceinline__ void finish_tile(const FinishParams& p, F&& after_wai
     }
     const Output out = {p.y, p.y_dtype, p.n_out};
     const int ch0 = (tile % p.tiles_x) * kTileN + ch;
-    out.store4(tok0 + col, ch0, make_float4(f0.x * s0, f0.y * s0, f0.z * s0, f0.w * s0));
-    if (col + kFinishTokens / 2 < cols) out.store4(tok0 + col2, ch0, make_float4(f1.x * s1, f1.y * s1, f1.z * s1, f1.w * s1));
+    const int bit = threadIdx.x >> 5;
+    if (!((skip >> bit) & 1u)) out.store4(tok0 + col, ch0, make_float4(f0.x * s0, f0.y * s0, f0.z * s0, f0.w * s0));
+    if (col + kFinishTokens / 2 < cols && !((skip >> (bit + kFinishTokens / 2)) & 1u)) out.store4(tok0 + col2, ch0, make_float4(f1.x * s1, f1.y * s1, f1.z * s1, f1.w * s1));
 }
 static __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const FinishParams p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    finish_tile(p, [] {});
+    finish_tile(p, [] { return 0u; });
 }
 
 }  // namespace streamk

@@ -393,6 +393,27 @@ def test_small_elements_beside_a_large_one_in_fp16_operands(goq, variant, n, k, 
     check_parity(y, y_ref, 5e-4, 2e-3)
 
 
+@pytest.mark.parametrize("n,k,g,m", [(16384, 4096, 128, 4), (9000, 8192, 128, 16)])
+def test_tokens_that_e4m3_operands_do_not_hold_are_the_fragment_kernels(goq, n, k, g, m):
+    """W4: a token whose elements span 2^28 is computed from its bf16 elements, bit for bit as goq_gemv without scratch (the fragment kernel) has it; one with
+    a few tiny elements among ordinary ones keeps to its slices (within fp32 sums of the other, not the same bits)."""
+    from tests.gpu_util import dev, pack_weights, run_gemv
+    codes, meta, coef = si.random_quantized(n, k, g, 4, seed=n + k)
+    d, packed = pack_weights(n, k, g, 4, codes, meta, coef)
+    x = si.bf16_bits_to_f64(si.bf16_activations(m, k, seed=m))
+    x[1, 5] = 2.0 ** 28
+    x[2, 7:10] = 1e-12
+    xb = si.f32_to_bf16_bits(x.astype(np.float32))
+    y = run_gemv(d, packed, xb)
+    y0 = torch.zeros((m, n), dtype=torch.float32, device="cuda")
+    goq.gemv(d, packed, dev(xb), m, y0, goq.F32)
+    torch.cuda.synchronize()
+    y0 = y0.cpu().numpy().astype(np.float64)
+    assert np.array_equal(y[1], y0[1])
+    for tok in (0, 2, m - 1):
+        assert 0 < np.linalg.norm(y[tok] - y0[tok]) <= 1e-6 * np.linalg.norm(y0[tok]), tok
+
+
 def test_e4m3_operand_gemm_reports_a_wait_that_runs_out(goq):
     """With one poll a wait the kernel gives up: the status word reads GOQ_ERR_TIMEOUT, and on a fresh scratch buffer the next call is right again."""
     from tests.gpu_util import dev, pack_weights
